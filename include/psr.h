@@ -74,7 +74,9 @@ extern "C" {
                              only                                           */
 #define PSR_TAYLOR4 3     /* the same to level T_[4]                        */
 /* inner loop of the FP32 forward kernels */
-#define PSR_KERNEL_AUTO 0   /* the library's default (scalar streams)          */
+#define PSR_KERNEL_AUTO 0   /* the library's default: packed pairs with a linear
+                               table of 1024 intervals or more, else scalar
+                               streams                                       */
 #define PSR_KERNEL_SCALAR 1 /* one source particle per lane and iteration      */
 #define PSR_KERNEL_PAPER 3  /* the paper's mapping (Section 3.2, Algorithms 1
                                and 2): one thread block per target leaf, one

@@ -7,7 +7,7 @@ for sm_103a).  There is no CPU fallback: without the built library, or
 without a CUDA device, the device calls raise.
 """
 import ctypes
-from dataclasses import dataclass
+from dataclasses import dataclass, replace
 
 import numpy as np
 
@@ -453,6 +453,10 @@ def _autograd_function():
         @staticmethod
         def forward(ctx, pos, mass, L, r_s, r_c, G=1.0, opts=None, max_leaf=32):
             opts = opts or Options()
+            if opts.kernel == PSR_KERNEL_AUTO and pos.dtype == torch.float64:
+                # FP64 tensors get the FP32 sums of the scalar kernels, whose
+                # order and rounding do not change with the default kernel's
+                opts = replace(opts, kernel=PSR_KERNEL_SCALAR)
             if pos.is_cuda:
                 lv = Leaves.device_build(pos, mass, L, r_s, r_c, G, max_leaf, fp64=opts.fp64)
             else:

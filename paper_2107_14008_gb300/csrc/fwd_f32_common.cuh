@@ -36,7 +36,7 @@
 
 namespace psr {
 
-enum { TM_EXACT = 0, TM_LINEAR = 1, TM_CUBIC = 2, TM_TAYLOR = 3 };
+enum { TM_EXACT = 0, TM_LINEAR = 1, TM_CUBIC = 2, TM_TAYLOR = 3, TM_CORE = 4 };
 
 // a * b + c clamped to [0, 1] in one instruction
 __device__ __forceinline__ float fma_sat(float a, float b, float c)
@@ -57,6 +57,27 @@ __device__ __forceinline__ float linear_T(float s, float nmax, unsigned tab_bias
     const float fk = fmaf(s, nmax, kMagic);
     const float2 c = lds_f2((unsigned)__float_as_int(fk) * 8u + tab_bias);
     return fmaf(s, c.y, c.x);
+}
+
+// Core form of the linear table.  With distances in units of x_c and
+// q = r^2, the pair weight is T / r^3 = 1/r^3 - H(q), H = (1 - T) / r^3, and H
+// is smooth in q down to 0 (1 - T = O(r^3)), so it interpolates linearly in q
+// itself: the lookup needs no 1/r and runs beside rsqrt, and the weight takes
+// one multiply and one FMA after it.  q comes from a saturating FMA, so a pair
+// at or beyond the cutoff has q = 1, 1/r = 1 and reaches the sentinel entry
+// H(N) = 1: its weight is exactly 0.  Entries are (-A_k, -D_k), H = A_k + q D_k
+// on q N in [k, k + 1) (the index by an FMA rounded down), shifted by half the
+// chord's error so that the error is balanced.  Bound by the shared-memory
+// pipe (about 5.8 cycles per warp lane pair, 3.4 of them the table entry's,
+// 79 % of the launch) with issue behind it (71 %).  128^3 NFW set: 10.27 ms
+// with T by its own table and scalar streams, 9.58 with this form (16 instead
+// of 18 instructions per pair), 9.32 with it on packed pairs.  H by a degree-9
+// polynomial instead (no table) is bound by the FMA pipe: 11.1 ms.
+__device__ __forceinline__ float core_weight(float q, float ri, float nmax, unsigned tab_bias)
+{
+    const float fk = __fmaf_rd(q, nmax, kMagic);
+    const float2 c = lds_f2((unsigned)__float_as_int(fk) * 8u + tab_bias);
+    return fmaf(ri * ri, ri, fmaf(q, c.y, c.x));
 }
 
 // Paper's Taylor table (Section 3.3, Eq. int) about the nearest node: entry k
@@ -149,6 +170,13 @@ __device__ __forceinline__ float4 lds_f4_v(unsigned a)
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
+}
+
+__device__ __forceinline__ float2 lds_f2_v(unsigned a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
     return v;
 }
 
@@ -391,6 +419,17 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
+// core_weight for a pair: the index FMA, 1/r^2 and the weight in f32x2, the
+// two chords as scalar FMAs that write straight into a register pair
+__device__ __forceinline__ float2 core_weight2(float2 q, float2 ri, float nmax, unsigned tab_bias)
+{
+    const float2 fk = __ffma2_rd(q, make_float2(nmax, nmax), make_float2(kMagic, kMagic));
+    const float2 ca = lds_f2((unsigned)__float_as_int(fk.x) * 8u + tab_bias);
+    const float2 cb = lds_f2((unsigned)__float_as_int(fk.y) * 8u + tab_bias);
+    const float2 h = make_float2(fmaf(q.x, ca.y, ca.x), fmaf(q.y, cb.y, cb.x));
+    return fma2(mul2(ri, ri), ri, h);
+}
+
 // T for a pair of table coordinates t = u - 1/2, u = x N / x_c (one FFMA of
 // r^2 and 1/r when coordinates are in table units).  Table entries: linear
 // (M_k, D_k) float2, cubic (c0..c3) float4, entry N = 0 (beyond the cutoff).
@@ -455,7 +494,8 @@ __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, un
     const float nmax = (float)a.table_n;
     // working unit: table intervals (u = x N / x_c) for the table path, x itself
     // for the exact path
-    const float sc = TM == TM_EXACT ? 1.0f : TM == TM_LINEAR ? 1.0f / x_c : (float)a.table_n / x_c;
+    const float sc = TM == TM_EXACT ? 1.0f
+                     : TM == TM_LINEAR || TM == TM_CORE ? 1.0f / x_c : (float)a.table_n / x_c;
     const float xscale = 1.0f / sc;  // working unit -> x (exact path only)
     const float unit = bx.unit;
     const int4 ci = lcen[I];
@@ -505,22 +545,32 @@ __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, un
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const float2 dx = add2(px, ntx[r]), dy = add2(py, nty[r]), dz = add2(pz, ntz[r]);
-                    const float2 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, eps2)));
-                    const float2 rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-                    const float2 t = TM == TM_LINEAR
-                                         ? make_float2(fma_sat(r2.x, rinv.x, soff), fma_sat(r2.y, rinv.y, soff))
-                                         : fma2(r2, rinv, mhalf);
-                    const float2 Tv = eval_T2<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
-                    // 1/r^3 formed beside the table lookup: two dependent
-                    // multiplies after T instead of four
-                    const float2 ri3 = mul2(mul2(rinv, rinv), rinv);
-                    const float2 w = EQM ? mul2(Tv, ri3) : mul2(mul2(pm, Tv), ri3);
+                    const float2 dyz = fma2(dy, dy, fma2(dz, dz, eps2));
+                    float2 r2, rinv, w;
+                    if (TM == TM_CORE) {
+                        r2 = make_float2(fma_sat(dx.x, dx.x, dyz.x), fma_sat(dx.y, dx.y, dyz.y));
+                        rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+                        w = core_weight2(r2, rinv, nmax, tab_bias);
+                        if (!EQM) w = mul2(w, pm);
+                    } else {
+                        r2 = fma2(dx, dx, dyz);
+                        rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+                        const float2 t = TM == TM_LINEAR
+                                             ? make_float2(fma_sat(r2.x, rinv.x, soff), fma_sat(r2.y, rinv.y, soff))
+                                             : fma2(r2, rinv, mhalf);
+                        const float2 Tv = eval_T2<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
+                        // 1/r^3 formed beside the table lookup: two dependent
+                        // multiplies after T instead of four
+                        const float2 ri3 = mul2(mul2(rinv, rinv), rinv);
+                        w = EQM ? mul2(Tv, ri3) : mul2(mul2(pm, Tv), ri3);
+                    }
                     fx[r] = fma2(w, dx, fx[r]);
                     fy[r] = fma2(w, dy, fy[r]);
                     fz[r] = fma2(w, dz, fz[r]);
                     if (COUNT) {
-                        const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR ? 1.0f : nmax;
-                        const float ua = r2.x * rinv.x, ub = r2.y * rinv.y;
+                        const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
+                        const float ua = TM == TM_CORE ? r2.x : r2.x * rinv.x;
+                        const float ub = TM == TM_CORE ? r2.y : r2.y * rinv.y;
                         cnt += (act[r] && ua < uc && (dx.x != 0.0f || dy.x != 0.0f || dz.x != 0.0f));
                         cnt += (act[r] && ub < uc && (dx.y != 0.0f || dy.y != 0.0f || dz.y != 0.0f));
                     }
@@ -528,16 +578,33 @@ __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, un
             };
             // Two staged pairs per iteration (k and k + S, then the odd one),
             // in the order of the plain loop: two independent dependency
-            // chains per lane, as in the scalar kernel.
-            const float4* ps = stage + 2 * s;
-            const float4* const pe = stage + 2 * ((nst + 1) >> 1);
+            // chains per lane, as in the scalar kernel.  32-bit shared-window
+            // addresses and volatile loads as there; with one mass the (m0,
+            // m1) half of a pair is not read (a 16-byte broadcast load takes
+            // two cycles of the shared-memory pipe, an 8-byte one takes one).
+            auto load = [&](unsigned p, float4& A, float4& B) {
+                A = lds_f4_v(p);
+                if (EQM) {
+                    const float2 z = lds_f2_v(p + 16u);
+                    B = make_float4(z.x, z.y, 0.0f, 0.0f);
+                } else {
+                    B = lds_f4_v(p + 16u);
+                }
+            };
+            unsigned sa = smem_u32(stage + 2 * s);
+            const unsigned se = smem_u32(stage + 2 * ((nst + 1) >> 1)), st1 = 32u * (unsigned)S;
+            float4 A0, B0, A1, B1;
 #pragma unroll 1
-            for (; ps + 2 * S < pe; ps += 4 * S) {
-                const float4 A0 = ps[0], B0 = ps[1], A1 = ps[2 * S], B1 = ps[2 * S + 1];
+            for (; sa + st1 < se; sa += 2u * st1) {
+                load(sa, A0, B0);
+                load(sa + st1, A1, B1);
                 evalp(A0, B0);
                 evalp(A1, B1);
             }
-            if (ps < pe) evalp(ps[0], ps[1]);
+            if (sa < se) {
+                load(sa, A0, B0);
+                evalp(A0, B0);
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 float sx = fx[r].x + fx[r].y, sy = fy[r].x + fy[r].y, sz = fz[r].x + fz[r].y;
@@ -592,7 +659,8 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
     const float x_c = bx.x_c;
     const float nmax = (float)a.table_n;
     const float soff = -0.5f / nmax;  // linear path: s = sat(r / x_c - 1/(2N))
-    const float sc = TM == TM_EXACT ? 1.0f : TM == TM_LINEAR ? 1.0f / x_c : (float)a.table_n / x_c;
+    const float sc = TM == TM_EXACT ? 1.0f
+                     : TM == TM_LINEAR || TM == TM_CORE ? 1.0f / x_c : (float)a.table_n / x_c;
     const float xscale = 1.0f / sc;
     const float unit = bx.unit;
     const int4 ci = lcen[I];
@@ -635,21 +703,28 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
                 for (int r = 0; r < R; ++r) {
                     const float2 dxy = add2(make_float2(p.x, p.y), nxy[r]);
                     const float dx = dxy.x, dy = dxy.y, dz = p.z - xz[r];
-                    float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-                    float rinv = rsqrt_ftz(r2);
-                    const float t = TM == TM_LINEAR ? fma_sat(r2, rinv, soff)
-                                                    : fmaf(r2, rinv, TM == TM_TAYLOR ? 0.0f : -0.5f);
-                    float Tv = eval_T1<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
-                    // 1/r^3 formed beside the table lookup (two dependent
-                    // multiplies after T instead of four)
-                    const float ri3 = rinv * rinv * rinv;
-                    const float w = EQM ? Tv * ri3 : (p.w * Tv) * ri3;
+                    const float dyz = fmaf(dy, dy, fmaf(dz, dz, eps2));
+                    const float r2 = TM == TM_CORE ? fma_sat(dx, dx, dyz) : fmaf(dx, dx, dyz);
+                    const float rinv = rsqrt_ftz(r2);
+                    float w;
+                    if (TM == TM_CORE) {
+                        w = core_weight(r2, rinv, nmax, tab_bias);
+                        if (!EQM) w *= p.w;
+                    } else {
+                        const float t = TM == TM_LINEAR ? fma_sat(r2, rinv, soff)
+                                                        : fmaf(r2, rinv, TM == TM_TAYLOR ? 0.0f : -0.5f);
+                        const float Tv = eval_T1<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
+                        // 1/r^3 formed beside the table lookup (two dependent
+                        // multiplies after T instead of four)
+                        const float ri3 = rinv * rinv * rinv;
+                        w = EQM ? Tv * ri3 : (p.w * Tv) * ri3;
+                    }
                     fx[r] = fmaf(w, dx, fx[r]);
                     fy[r] = fmaf(w, dy, fy[r]);
                     fz[r] = fmaf(w, dz, fz[r]);
                     if (COUNT) {
-                        const float u = r2 * rinv;
-                        const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR ? 1.0f : nmax;
+                        const float u = TM == TM_CORE ? r2 : r2 * rinv;
+                        const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
                         cnt += (act[r] && u < uc && (dx != 0.0f || dy != 0.0f || dz != 0.0f));
                     }
                 }
@@ -741,6 +816,11 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
         const float4* g = reinterpret_cast<const float4*>(a.table);
         for (int i = threadIdx.x; i < 2 * (a.table_n + 1); i += blockDim.x)
             reinterpret_cast<float4*>(smem)[i] = g[i];
+        __syncthreads();
+    } else if (TM == TM_CORE) {
+        const float2* g = reinterpret_cast<const float2*>(a.table);
+        for (int i = threadIdx.x; i <= a.table_n; i += blockDim.x)
+            reinterpret_cast<float2*>(smem)[i] = g[i];
         __syncthreads();
     } else if (TM != TM_EXACT) {
         const float4* g = reinterpret_cast<const float4*>(a.table);
@@ -839,6 +919,9 @@ int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStr
     if (precision == PSR_FP32_EXACT)
         return a.accum == PSR_ACC_FP64 ? launch_c<TM_EXACT, PSR_ACC_FP64, PK>(a, smem, st)
                                        : launch_c<TM_EXACT, PSR_ACC_KAHAN32, PK>(a, smem, st);
+    if (PK && a.core)
+        return a.accum == PSR_ACC_FP64 ? launch_c<TM_CORE, PSR_ACC_FP64, true>(a, smem, st)
+                                       : launch_c<TM_CORE, PSR_ACC_KAHAN32, true>(a, smem, st);
     if (a.interp == PSR_LINEAR)
         return a.accum == PSR_ACC_FP64 ? launch_c<TM_LINEAR, PSR_ACC_FP64, PK>(a, smem, st)
                                        : launch_c<TM_LINEAR, PSR_ACC_KAHAN32, PK>(a, smem, st);
@@ -850,17 +933,21 @@ int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStr
 }
 
 template <bool PK>
-const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int max_leaf)
+const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int core)
 {
+#define PSR_PICK_PK(ACC) ((const void*)p2p_fwd_f32_kernel<TM_CORE, ACC, false, true, true, false>)
 #define PSR_PICK(TM, ACC) ((const void*)p2p_fwd_f32_kernel<TM, ACC, false, true, PK, false>)
     if (precision == PSR_FP32_EXACT)
         return accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
+    if (PK && core)
+        return accum == PSR_ACC_FP64 ? PSR_PICK_PK(PSR_ACC_FP64) : PSR_PICK_PK(PSR_ACC_KAHAN32);
     if (interp == PSR_LINEAR)
         return accum == PSR_ACC_FP64 ? PSR_PICK(TM_LINEAR, PSR_ACC_FP64) : PSR_PICK(TM_LINEAR, PSR_ACC_KAHAN32);
     if (interp == PSR_TAYLOR2 || interp == PSR_TAYLOR4)
         return accum == PSR_ACC_FP64 ? PSR_PICK(TM_TAYLOR, PSR_ACC_FP64) : PSR_PICK(TM_TAYLOR, PSR_ACC_KAHAN32);
     return accum == PSR_ACC_FP64 ? PSR_PICK(TM_CUBIC, PSR_ACC_FP64) : PSR_PICK(TM_CUBIC, PSR_ACC_KAHAN32);
 #undef PSR_PICK
+#undef PSR_PICK_PK
 }
 
 }  // namespace psr

@@ -118,7 +118,8 @@ extern "C" int psr_p2p_forces_noalloc(psr_leaves* hh, const psr_opts* opts, void
     }
     if (precision == PSR_FP32_TABLE) {
         const double x_c = h->boxes[0].r_c / (2.0 * h->boxes[0].r_s);
-        int le = launch_table(a.table_n, a.interp, x_c, base, nullptr, st);
+        int le = a.core ? launch_core_table(a.table_n, x_c, base, st)
+                        : launch_table(a.table_n, a.interp, x_c, base, nullptr, st);
         if (le) {
             set_last_error(std::string("table kernel launch: ") + cudaGetErrorString((cudaError_t)le));
             return PSR_E_CUDA;

@@ -9,7 +9,7 @@ namespace psr {
 template <bool PK>
 int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStream_t st);
 template <bool PK>
-const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int max_leaf);
+const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int core);
 
 // ------------------------------------------------------------------ table --
 // Entries k = 0..N-1 describe [x_k, x_{k+1}], x_k = k x_c / N, as functions of
@@ -78,6 +78,63 @@ int launch_table(int table_n, int interp, double x_c, void* d_out, void* d_q_out
     return (int)cudaGetLastError();
 }
 
+// (1 - T(x)) / x^3, an entire function of x^2: its series
+// (4 / sqrt(pi)) sum_n (-1)^n x^(2n) / (n! (2n + 3)) below x = 0.7 (where the
+// difference would cancel; the first term left out is below 1e-17), the
+// closed form above.
+__device__ double core_h(double x)
+{
+    const double x2 = x * x;
+    if (x < 0.7) {
+        double s = 0.0, t = 1.0;
+        for (int n = 0; n < 15; ++n) {
+            s += t / (2 * n + 3);
+            t *= -x2 / (n + 1);
+        }
+        return 2.0 * 1.1283791670955126 * s;
+    }
+    return (1.0 - (erfc(x) + 1.1283791670955126 * x * exp(-x2))) / (x2 * x);
+}
+
+// Core table (core_weight): entries k = 0..N-1 are minus the chord of H(q) =
+// x_c^3 (1 - T) / x^3, q = (x / x_c)^2, over q N in [k, k + 1], moved by half
+// its error at the interval's middle; entry N, met at and beyond the cutoff
+// (q = 1, 1/r = 1), is -1.
+__global__ void core_table_kernel(int N, double x_c, float2* __restrict__ t)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k > N) return;
+    if (k == N) {
+        t[k] = make_float2(-1.0f, 0.0f);
+        return;
+    }
+    const double s3 = x_c * x_c * x_c, q0 = (double)k / N, q1 = (double)(k + 1) / N;
+    const double h0 = s3 * core_h(x_c * sqrt(q0)), h1 = s3 * core_h(x_c * sqrt(q1));
+    const double hm = s3 * core_h(x_c * sqrt(0.5 * (q0 + q1)));
+    const double D = (h1 - h0) * N;
+    t[k] = make_float2((float)(-(h0 - D * q0 + 0.5 * (hm - 0.5 * (h0 + h1)))), (float)-D);
+}
+
+int launch_core_table(int table_n, double x_c, void* d_out, void* stream)
+{
+    const int threads = 256, blocks = (table_n + 1 + threads - 1) / threads;
+    core_table_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(table_n, x_c,
+                                                                    reinterpret_cast<float2*>(d_out));
+    return (int)cudaGetLastError();
+}
+
+// The packed variant takes the core form of a linear table from 1024
+// intervals on and for x_c <= 3.5: there its interpolation error in T
+// (3.2e-7 at x_c = 2.25 and 1024 intervals, 1.9e-6 at 3.5, as x_c^4) is no
+// larger than the chord table's (8.0e-7 and 1.9e-6, as x_c^2).  Coarser
+// tables stay the chord in x that a caller of such a table asks for, and
+// PSR_KERNEL_SCALAR stays the chord form with its order of sums throughout.
+bool fwd_core(int precision, int interp, int table_n, int variant, double x_c)
+{
+    return precision == PSR_FP32_TABLE && interp == PSR_LINEAR && variant == PSR_KERNEL_PACKED &&
+           table_n >= 1024 && x_c <= 3.5;
+}
+
 // bytes of one table entry in shared memory (and in global for Taylor)
 size_t table_entry_bytes(int interp)
 {
@@ -101,13 +158,13 @@ int launch_fwd_f32(const FwdArgs& a, int precision, void* stream)
                                           : launch_fwd_f32_variant<false>(a, precision, smem, st);
 }
 
-int fwd_f32_occupancy(int precision, int interp, int accum, int warps, int max_leaf, int table_n,
-                      int cap, int variant, int* out)
+int fwd_f32_occupancy(int precision, int interp, int accum, int warps, int table_n, int cap,
+                      int variant, int core, int* out)
 {
     size_t smem = fwd_f32_smem(precision, interp, table_n, warps, cap);
     const void* f = variant == PSR_KERNEL_PACKED
-                        ? fwd_f32_kernel_ptr<true>(precision, interp, accum, max_leaf)
-                        : fwd_f32_kernel_ptr<false>(precision, interp, accum, max_leaf);
+                        ? fwd_f32_kernel_ptr<true>(precision, interp, accum, core)
+                        : fwd_f32_kernel_ptr<false>(precision, interp, accum, 0);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;

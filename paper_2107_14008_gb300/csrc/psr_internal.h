@@ -51,6 +51,7 @@ struct Layout {
     size_t items;    // int32[nl]    target leaves in schedule order
     size_t boxes;    // BoxDev[nbox]
     size_t table;    // float4[2 * (kMaxTableN + 1)]: T table, then exp(-x^2)
+    size_t core;     // float2[kMaxTableN + 1]: core form of the forward's linear table
     size_t cotf;     // float4[n] / double4[n] adjoint source payload scratch
     size_t ctrl;     // uint32[64]  scheduler tickets, error word, counters
     // multipole split (device builds with an acceptance parameter only)
@@ -124,6 +125,8 @@ struct Leaves {
     bool uploaded = false;
     int table_key = -1;       // cached forward table (n, interp) encoding
     double table_xc = -1.0;
+    int core_key = -1;        // the core table's intervals and x_c
+    double core_xc = -1.0;
     int adj_table_key = -1;
     int sm_count = 0;
     int device = -1;
@@ -170,16 +173,19 @@ struct FwdArgs {
     int stage_cap;   // FP32 kernels: staged particles per warp
     int item_stride; // this launch takes schedule entries ticket * stride + offset
     int item_offset;
+    int core;        // FP32 forward: a.table is the core form of the linear table
     int equal_mass;  // every box has one particle mass: the FP32 kernels take it out of the sums
 };
 
 int launch_table(int table_n, int interp, double x_c, void* d_out, void* d_q_out, void* stream);
+int launch_core_table(int table_n, double x_c, void* d_out, void* stream);
+bool fwd_core(int precision, int interp, int table_n, int variant, double x_c);
 int launch_fwd_f32(const FwdArgs& a, int precision, void* stream);
 int launch_fwd_f64(const FwdArgs& a, void* stream);
 int launch_adj_f32(const FwdArgs& a, int precision, void* stream);
 int launch_adj_f64(const FwdArgs& a, void* stream);
-int fwd_f32_occupancy(int precision, int interp, int accum, int warps, int max_leaf, int table_n,
-                      int cap, int variant, int* out);
+int fwd_f32_occupancy(int precision, int interp, int accum, int warps, int table_n, int cap,
+                      int variant, int core, int* out);
 size_t fwd_f32_smem(int precision, int interp, int table_n, int warps, int cap);
 constexpr size_t kSmemPerBlock = 227 * 1024;  // opt-in dynamic shared memory per block
 int fwd_f64_occupancy(int warps, int max_leaf, int interp, int table_n, int* out);

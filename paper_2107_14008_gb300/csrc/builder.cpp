@@ -731,6 +731,9 @@ int build_batch(int nbox, const double* const* pos, const double* const* mass, c
         for (int64_t g = 0; g < nl; ++g) h->items[g] = (int32_t)g;
         std::stable_sort(h->items.begin(), h->items.end(),
                          [&](int32_t a, int32_t b) { return cost[a] > cost[b]; });
+        h->item_cost.resize(nl);
+        for (int64_t g = 0; g < nl; ++g) h->item_cost[g] = cost[h->items[g]];
+        h->max_cost = nl ? h->item_cost[0] : 0;
         h->n_leaves = nl;
         h->n_pairs = (int64_t)h->pairs.size();
         h->has_pd = !(flags & PSR_BUILD_NO_FP64);

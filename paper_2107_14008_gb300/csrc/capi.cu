@@ -3,6 +3,7 @@
 // here; psr_p2p_forces and psr_p2p_adjoint only enqueue work.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -44,6 +45,7 @@ int wait_stream(cudaStream_t st, int timeout_ms)
 
 struct Opts {
     int precision, table_n, interp, accum, warps, bps, fold, count, kernel, tile, nshard, shard;
+    bool split;  // heavy items on whole blocks: the default kernel's choice
 };
 
 int check_opts(const psr_opts* o, Opts* out)
@@ -81,7 +83,7 @@ int check_opts(const psr_opts* o, Opts* out)
     if (fold < 1) return fail(PSR_E_ARG, "psr_opts.fold_every must be positive");
     *out = Opts{o->precision, tn, o->interp, o->accum, w, o->blocks_per_sm, fold,
                 o->count_pairs ? 1 : 0, o->kernel,
-                o->source_tile, nshard, o->shard_index};
+                o->source_tile, nshard, o->shard_index, o->kernel == PSR_KERNEL_AUTO};
     return PSR_OK;
 }
 
@@ -224,6 +226,18 @@ int grid_blocks(Leaves* h, const Opts& o, int adjoint, int* blocks)
     return PSR_OK;
 }
 
+// Heavy rows shared among warps (the default kernels only), for a launch
+// whose grid is known.
+void set_split(const Leaves* h, const Opts& o, bool adjoint, FwdArgs* a)
+{
+    if (!o.split) return;
+    const SplitRule r = split_rule(h->max_cost, h->evaluated, h->n_leaves, h->sm_count,
+                                   (int64_t)a->blocks * o.warps, o.warps, adjoint);
+    a->group = r.group;
+    if (r.level >= 0)
+        a->heavy = reinterpret_cast<const int*>(h->d_ws + h->lay.ctrl) + kCtrlHeavy + r.level;
+}
+
 }  // namespace
 
 namespace psr {
@@ -246,6 +260,7 @@ int prepare_forward(Leaves* h, const psr_opts* opts, FwdArgs* a, int* precision)
     if (fwd32 && (rc = fwd32_smem_config(o, &a->stage_cap))) return rc;
     if (fwd32 && (rc = check_tile(h, a->stage_cap))) return rc;
     if ((rc = grid_blocks(h, o, 0, &a->blocks))) return rc;
+    set_split(h, o, false, a);
     a->core = fwd_core(o.precision, o.interp, o.table_n, o.kernel, cutoff_x(h));
     *precision = o.precision;
     return PSR_OK;
@@ -345,6 +360,15 @@ int psr_upload(psr_leaves* hh, void* d_ws, size_t bytes, void* stream)
     }
     if ((e = cudaMemsetAsync(w + L.ctrl, 0, kCtrlWords * 4, st)) != cudaSuccess)
         return cuda_fail(e, "cudaMemsetAsync (ctrl)");
+    for (int l = 0; l < kHeavyLevels; ++l) {
+        const int64_t heavy = heavy_cost(l, h->evaluated, sms);
+        h->n_heavy[l] = (int32_t)(std::partition_point(h->item_cost.begin(), h->item_cost.end(),
+                                                       [heavy](int64_t c) { return c > heavy; }) -
+                                  h->item_cost.begin());
+    }
+    if ((e = cudaMemcpyAsync(w + L.ctrl + 4 * kCtrlHeavy, h->n_heavy, sizeof h->n_heavy,
+                             cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        return cuda_fail(e, "cudaMemcpyAsync (ctrl)");
     h->d_ws = w;
     h->ws_bytes = bytes;
     h->uploaded = true;
@@ -382,6 +406,7 @@ int psr_p2p_forces(psr_leaves* hh, const psr_opts* opts, void* d_acc, void* stre
     if (fwd32 && (rc = fwd32_smem_config(o, &a.stage_cap))) return rc;
     if (fwd32 && (rc = check_tile(h, a.stage_cap))) return rc;
     if ((rc = grid_blocks(h, o, 0, &a.blocks))) return rc;
+    set_split(h, o, false, &a);
     if (o.count) {
         cudaError_t e = cudaMemsetAsync(a.ctrl + kCtrlPairsLo, 0, 16, st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (pair counters)");
@@ -423,6 +448,7 @@ int psr_p2p_adjoint(psr_leaves* hh, const psr_opts* opts, const void* d_cot, voi
     a.out = d_grad_pos;
     a.out_m = d_grad_mass;
     if ((rc = grid_blocks(h, o, 1, &a.blocks))) return rc;
+    set_split(h, o, true, &a);
     int e = (o.precision == PSR_FP64) ? launch_adj_f64(a, st) : launch_adj_f32(a, o.precision, st);
     if (e) return cuda_fail((cudaError_t)e, "adjoint kernel launch");
     return PSR_OK;

@@ -1422,6 +1422,24 @@ __global__ void k_sched_keys(const int64_t* __restrict__ lcost, int64_t nl, long
     val[g] = (int32_t)g;
 }
 
+// The sorted schedule into the workspace, and for each level the number of
+// items whose work exceeds its line (the keys ascend, so they come first).
+struct HeavyLines {
+    long long cost[kHeavyLevels];
+};
+__global__ void k_sched_out(const uint64_t* __restrict__ key, const int32_t* __restrict__ val,
+                            int64_t nl, long long maxcost, HeavyLines heavy,
+                            int32_t* __restrict__ items, int* __restrict__ n_heavy)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= nl) return;
+    items[i] = val[i];
+    const long long mine = maxcost - (long long)key[i];
+    const long long next = i + 1 < nl ? maxcost - (long long)key[i + 1] : -1;
+    for (int l = 0; l < kHeavyLevels; ++l)
+        if (mine > heavy.cost[l] && next <= heavy.cost[l]) n_heavy[l] = (int)(i + 1);
+}
+
 __global__ void k_copy_total(int64_t* dst, const int64_t* src) { *dst = *src; }
 
 unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -1674,7 +1692,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
         return dfail(PSR_E_NOMEM, "out of host memory");
     }
     h->db_scratch = s;
-    h->db_maxcost = c[kCntMaxCost];
+    h->max_cost = c[kCntMaxCost];
     h->db_kslot = kslot;
     h->db_interleave = interleave;
     h->db_uncached = kslot ? c[kCntUncached] : nl;
@@ -1789,13 +1807,16 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     int32_t* v0 = (int32_t*)(s + S.flag);
     int32_t* v1 = (int32_t*)(s + S.lid);
     k_sched_keys<<<nblk(nl, 256), 256, 0, st>>>((const int64_t*)(s + S.lcost), nl,
-                                                (long long)h->db_maxcost, k0, v0);
+                                                (long long)h->max_cost, k0, v0);
     int bits = 1;
-    while (bits < 63 && ((uint64_t)h->db_maxcost >> bits)) ++bits;
+    while (bits < 63 && ((uint64_t)h->max_cost >> bits)) ++bits;
     if ((e = radix_sort(k0, v0, k1, v1, nl, bits, (int64_t*)(s + S.hist), tiles, total, st)))
         return dcuda(e, "schedule sort");
-    if ((e = (int)cudaMemcpyAsync(w + L.items, v0, 4 * nl, cudaMemcpyDeviceToDevice, st)))
-        return dcuda(e, "cudaMemcpyAsync");
+    HeavyLines heavy;
+    for (int l = 0; l < kHeavyLevels; ++l) heavy.cost[l] = heavy_cost(l, h->evaluated, sms);
+    k_sched_out<<<nblk(nl, 256), 256, 0, st>>>(k0, v0, nl, (long long)h->max_cost, heavy,
+                                               (int32_t*)(w + L.items), (int*)(w + L.ctrl) + kCtrlHeavy);
+    if ((e = (int)cudaGetLastError())) return dcuda(e, "schedule kernel");
     if ((e = (int)cudaMemcpyAsync(w + L.boxes, h->boxdev.data(), sizeof(BoxDev),
                                   cudaMemcpyHostToDevice, st)))
         return dcuda(e, "cudaMemcpyAsync");

@@ -353,13 +353,25 @@ __device__ __forceinline__ int stage_chunk(const FwdArgs& a, long long e0, long 
     return eb;
 }
 
+// Barrier of the calling warp's group of `warps` consecutive warps (the block
+// holds a whole number of groups; barrier 0 is left to __syncthreads).
+__device__ __forceinline__ void group_sync(int warps)
+{
+    const int id = 1 + (int)(threadIdx.x >> 5) / warps;
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(32 * warps) : "memory");
+}
+
 // Combine the S stream partial sums of each target through shared memory
 // (the warp's staging buffer) and write the accelerations, scaled by gout, in
-// the original particle order.
+// the original particle order.  With split, the group's warps each hold the
+// sums over their part of the row: every warp leaves its target sums at the
+// start of its own region, and after a barrier one thread per target adds them
+// over the warps, in warp order, and writes them (wstride: float4 per warp).
 template <int ACC, int R>
 __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>* acc,
                                             const bool* act, int lane, int s, int q, int S, int T,
-                                            float gout, float4* __restrict__ stage)
+                                            float gout, float4* __restrict__ stage, bool split,
+                                            int wstride)
 {
     // Each target slot r reduces through its own region of the staging buffer
     // (768 B; two slots fit the smallest per-warp buffer, 64 + 32 float4), with
@@ -379,11 +391,17 @@ __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>
                     sy += red[3 * (lane + t * T) + 1];
                     sz += red[3 * (lane + t * T) + 2];
                 }
-                int idx = a.perm[li.x + q + T * r];
-                float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
-                out[0] = (float)(sx * (double)gout);
-                out[1] = (float)(sy * (double)gout);
-                out[2] = (float)(sz * (double)gout);
+                if (split) {  // streams t >= 1 sit above the first T entries
+                    red[3 * lane + 0] = sx;
+                    red[3 * lane + 1] = sy;
+                    red[3 * lane + 2] = sz;
+                } else {
+                    int idx = a.perm[li.x + q + T * r];
+                    float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
+                    out[0] = (float)(sx * (double)gout);
+                    out[1] = (float)(sy * (double)gout);
+                    out[2] = (float)(sz * (double)gout);
+                }
             }
         } else {
             volatile float* red = reinterpret_cast<volatile float*>(stage) + 192 * r;
@@ -403,15 +421,90 @@ __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>
                     two_sum(sy, o[2], u, v); sy = u; cy += o[3] + v;
                     two_sum(sz, o[4], u, v); sz = u; cz += o[5] + v;
                 }
-                int idx = a.perm[li.x + q + T * r];
-                float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
-                out[0] = (sx + cx) * gout;
-                out[1] = (sy + cy) * gout;
-                out[2] = (sz + cz) * gout;
+                if (split) {
+                    volatile float* o = red + 6 * lane;
+                    o[0] = sx; o[1] = cx;
+                    o[2] = sy; o[3] = cy;
+                    o[4] = sz; o[5] = cz;
+                } else {
+                    int idx = a.perm[li.x + q + T * r];
+                    float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
+                    out[0] = (sx + cx) * gout;
+                    out[1] = (sy + cy) * gout;
+                    out[2] = (sz + cz) * gout;
+                }
             }
         }
         __syncwarp();
     }
+    if (split) {
+        group_sync(a.group);
+        const int nw = a.group, gw = (threadIdx.x >> 5) % nw;  // this warp in its group
+        for (int t = 32 * gw + lane; t < li.y; t += 32 * nw) {
+            const int r = t / T, k = t - r * T;  // slot r, lane k of each warp
+            const float4* base = stage - gw * wstride;
+            float* out = reinterpret_cast<float*>(a.out) + 3LL * a.perm[li.x + t];
+            for (int i = 0; i < 3; ++i) {
+                if (ACC == PSR_ACC_FP64) {
+                    double sum = 0.0;
+                    for (int w = 0; w < nw; ++w)
+                        sum += (reinterpret_cast<const volatile double*>(base + w * wstride) + 96 * r)[3 * k + i];
+                    out[i] = (float)(sum * (double)gout);
+                } else {
+                    float hi = 0.0f, lo = 0.0f, u, v;
+                    for (int w = 0; w < nw; ++w) {
+                        const volatile float* o =
+                            reinterpret_cast<const volatile float*>(base + w * wstride) + 192 * r + 6 * k + 2 * i;
+                        two_sum(hi, o[0], u, v); hi = u; lo += o[1] + v;
+                    }
+                    out[i] = (hi + lo) * gout;
+                }
+            }
+        }
+    }
+}
+
+// This warp's entries of a row: all of them, or with split its share among
+// the warps of its group.
+__device__ __forceinline__ void row_part(const FwdArgs& a, int I, bool split, long long& e0, long long& re)
+{
+    e0 = a.rowptr[I];
+    re = a.rowptr[I + 1];
+    if (split) {
+        const int len = (int)(re - e0), W = a.group, w = (threadIdx.x >> 5) % W;
+        re = e0 + (long long)len * (w + 1) / W;
+        e0 += (long long)len * w / W;
+    }
+}
+
+// The next item of a persistent launch.  The schedule's first *a.heavy items
+// (their work is more than a fraction of what one warp of a full chip gets,
+// see heavy_cost) are taken by groups of a.group warps, one ticket a group
+// (split stays true; s_it: one word per group), the rest by single warps; the
+// ticket on which a group leaves the first phase goes to its first warp.
+// Returns false when no item is left.  Which items are split, and how, is
+// fixed by the schedule alone, so results do not depend on the order in which
+// blocks run.
+template <bool SPLIT>
+__device__ __forceinline__ bool next_item(const FwdArgs& a, unsigned* ticket, bool& split,
+                                          int n_heavy, volatile int* s_it, int& it)
+{
+    if (SPLIT && split) {
+        const int g = (threadIdx.x >> 5) / a.group;
+        const bool first = threadIdx.x - g * 32 * a.group < 32;
+        group_sync(a.group);  // the group's last item is combined
+        if (first && (threadIdx.x & 31) == 0)
+            s_it[g] = (int)atomicAdd(ticket, 1u) * a.item_stride + a.item_offset;
+        group_sync(a.group);
+        it = s_it[g];
+        if (it < n_heavy) return true;  // n_heavy <= n_items
+        split = false;
+        if (first) return it < a.n_items;
+    }
+    int t = 0;
+    if ((threadIdx.x & 31) == 0) t = (int)atomicAdd(ticket, 1u) * a.item_stride + a.item_offset;
+    it = __shfl_sync(kFull, t, 0);
+    return it < a.n_items;
 }
 
 // Packed FP32 helpers (sm_100+ f32x2 instructions: two lanes of work per issue)
@@ -478,7 +571,8 @@ __device__ __forceinline__ float2 eval_T2(float2 t, float2 r2, float2 rinv, unsi
 template <int TM, int ACC, bool COUNT, bool EQM, int R>
 __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                             float4* __restrict__ stage, float4* __restrict__ meta,
-                                         unsigned long long& npairs, unsigned long long& nev)
+                                         unsigned long long& npairs, unsigned long long& nev,
+                                            bool split, int wstride)
 {
     const int lane = threadIdx.x & 31;
     const float4* __restrict__ pf = reinterpret_cast<const float4*>(a.pf);
@@ -527,8 +621,8 @@ __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, un
 #pragma unroll
     for (int r = 0; r < R; ++r) fx[r] = fy[r] = fz[r] = make_float2(0.0f, 0.0f);
     unsigned cnt = 0;
-    const long long re = a.rowptr[I + 1];
-    long long e0 = a.rowptr[I];
+    long long e0, re;
+    row_part(a, I, split, e0, re);
     const float eps = kEps2 * sc * sc;
     const float2 eps2 = make_float2(eps, eps);
     // table coordinate: u - 1/2 (interval tables), u (Taylor: nearest node)
@@ -615,7 +709,7 @@ __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, un
         __syncwarp();
     }
     finish_item<ACC, R>(a, li, acc, act, lane, s, q, S, T,
-                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage);
+                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage, split, wstride);
     if (COUNT) npairs += cnt;
 }
 
@@ -644,7 +738,8 @@ template <int TM, int ACC, bool COUNT, bool EQM, int R>
 __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                             float4* __restrict__ stage,
                                             float4* __restrict__ meta, unsigned long long& npairs,
-                                            unsigned long long& nev)
+                                            unsigned long long& nev,
+                                            bool split, int wstride)
 {
     const int lane = threadIdx.x & 31;
     const float4* __restrict__ pf = reinterpret_cast<const float4*>(a.pf);
@@ -690,8 +785,8 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
 #pragma unroll
     for (int r = 0; r < R; ++r) fx[r] = fy[r] = fz[r] = 0.0f;
     unsigned cnt = 0;
-    const long long re = a.rowptr[I + 1];
-    long long e0 = a.rowptr[I];
+    long long e0, re;
+    row_part(a, I, split, e0, re);
     const float eps2 = kEps2 * sc * sc;
     while (e0 < re) {
         int nst;
@@ -751,7 +846,7 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
         __syncwarp();
     }
     finish_item<ACC, R>(a, li, acc, act, lane, s, q, S, T,
-                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage);
+                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage, split, wstride);
     if (COUNT) npairs += cnt;
 }
 
@@ -801,7 +896,7 @@ __device__ __forceinline__ int targets_per_lane(int n, int cap)
 
 // Shared memory: the table, then one staging buffer of stage_cap particles
 // plus 32 entry records per warp.
-template <int TM, int ACC, bool COUNT, bool WIDE, bool PK, bool EQM>
+template <int TM, int ACC, bool COUNT, bool PK, bool EQM, bool SPLIT>
 __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -837,11 +932,12 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
     const unsigned tab_bias = smem_u32(smem) - (unsigned)kMagicBits * esize;
     const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
     unsigned long long npairs = 0, nev = 0;
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = (int)atomicAdd(a.ctrl + kCtrlTicketFwd, 1u) * a.item_stride + a.item_offset;
-        it = __shfl_sync(kFull, it, 0);
-        if (it >= a.n_items) break;
+    __shared__ int s_it[8];
+    const int wstride = a.stage_cap + kWarpMeta;
+    const int n_heavy = !SPLIT ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    bool split = SPLIT && n_heavy > 0;
+    int it;
+    while (next_item<SPLIT>(a, a.ctrl + kCtrlTicketFwd, split, n_heavy, s_it, it)) {
         int I = a.items[it];
         if (I < 0 || I >= a.n_leaves) {
             if (lane == 0) set_error(a.ctrl, kErrItemIndex);
@@ -861,19 +957,19 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
             // on the bench workload)
             const int R = targets_per_lane(li.y, a.stage_cap);
             if (R == 1)
-                fwd_item_pk<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev);
+                fwd_item_pk<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
             else if (R == 3)
-                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
             else
-                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
         } else {
-            const int R = WIDE ? targets_per_lane(li.y, a.stage_cap) : 1;
+            const int R = targets_per_lane(li.y, a.stage_cap);
             if (R == 3)
-                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
             else if (R == 2)
-                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
             else
-                fwd_item_sc<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
         }
     }
     if (COUNT) {
@@ -888,13 +984,13 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
 
 // Launch and occupancy of the variant PK (explicitly instantiated in
 // p2p_fwd_f32_sc.cu and p2p_fwd_f32_pk.cu).
-template <int TM, int ACC, bool COUNT, bool PK, bool EQM>
+template <int TM, int ACC, bool COUNT, bool PK, bool EQM, bool SPLIT>
 static int launch_t(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
     // Both variants carry the scalar two- and three-targets-per-lane paths
     // (targets_per_lane picks per leaf; the packed variant runs its f32x2
     // loop for the leaves that take one target per lane).
-    auto k = p2p_fwd_f32_kernel<TM, ACC, COUNT, true, PK, EQM>;
+    auto k = p2p_fwd_f32_kernel<TM, ACC, COUNT, PK, EQM, SPLIT>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
@@ -903,40 +999,54 @@ static int launch_t(const FwdArgs& a, size_t smem, cudaStream_t st)
     return (int)cudaGetLastError();
 }
 
-template <int TM, int ACC, bool PK>
-static int launch_c(const FwdArgs& a, size_t smem, cudaStream_t st)
+template <int TM, int ACC, bool PK, bool SPLIT>
+static int launch_s(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
     // equal masses: the mass leaves the pair sum (the pair-counting launch,
     // untimed, keeps the general form)
-    return a.count_pairs  ? launch_t<TM, ACC, true, PK, false>(a, smem, st)
-           : a.equal_mass ? launch_t<TM, ACC, false, PK, true>(a, smem, st)
-                          : launch_t<TM, ACC, false, PK, false>(a, smem, st);
+    return a.count_pairs  ? launch_t<TM, ACC, true, PK, false, SPLIT>(a, smem, st)
+           : a.equal_mass ? launch_t<TM, ACC, false, PK, true, SPLIT>(a, smem, st)
+                          : launch_t<TM, ACC, false, PK, false, SPLIT>(a, smem, st);
 }
 
-template <bool PK>
-int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStream_t st)
+template <bool PK, bool SPLIT>
+static int launch_fwd_f32_t(const FwdArgs& a, int precision, size_t smem, cudaStream_t st)
 {
     if (precision == PSR_FP32_EXACT)
-        return a.accum == PSR_ACC_FP64 ? launch_c<TM_EXACT, PSR_ACC_FP64, PK>(a, smem, st)
-                                       : launch_c<TM_EXACT, PSR_ACC_KAHAN32, PK>(a, smem, st);
-    if (PK && a.core)
-        return a.accum == PSR_ACC_FP64 ? launch_c<TM_CORE, PSR_ACC_FP64, true>(a, smem, st)
-                                       : launch_c<TM_CORE, PSR_ACC_KAHAN32, true>(a, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_EXACT, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
+                                       : launch_s<TM_EXACT, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
     if (a.interp == PSR_LINEAR)
-        return a.accum == PSR_ACC_FP64 ? launch_c<TM_LINEAR, PSR_ACC_FP64, PK>(a, smem, st)
-                                       : launch_c<TM_LINEAR, PSR_ACC_KAHAN32, PK>(a, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_LINEAR, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
+                                       : launch_s<TM_LINEAR, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
     if (a.interp == PSR_TAYLOR2 || a.interp == PSR_TAYLOR4)
-        return a.accum == PSR_ACC_FP64 ? launch_c<TM_TAYLOR, PSR_ACC_FP64, PK>(a, smem, st)
-                                       : launch_c<TM_TAYLOR, PSR_ACC_KAHAN32, PK>(a, smem, st);
-    return a.accum == PSR_ACC_FP64 ? launch_c<TM_CUBIC, PSR_ACC_FP64, PK>(a, smem, st)
-                                   : launch_c<TM_CUBIC, PSR_ACC_KAHAN32, PK>(a, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_TAYLOR, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
+                                       : launch_s<TM_TAYLOR, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
+    return a.accum == PSR_ACC_FP64 ? launch_s<TM_CUBIC, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
+                                   : launch_s<TM_CUBIC, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
 }
+
+// One translation unit each: <PK, SPLIT> = <false, false>, <true, false>,
+// <false, true>, <true, true> (the last only for the core form).  Launches
+// without heavy items (most large sets) keep the kernel without the block
+// phase, whose registers cost 1-3 % of a launch.
+template <bool PK, bool SPLIT>
+int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStream_t st)
+{
+    if (PK && a.core)
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_CORE, PSR_ACC_FP64, true, SPLIT>(a, smem, st)
+                                       : launch_s<TM_CORE, PSR_ACC_KAHAN32, true, SPLIT>(a, smem, st);
+    if constexpr (!(PK && SPLIT))
+        return launch_fwd_f32_t<PK, SPLIT>(a, precision, smem, st);
+    else
+        return (int)cudaErrorInvalidValue;  // not reached: only the core form is split on packed pairs
+}
+
 
 template <bool PK>
 const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int core)
 {
-#define PSR_PICK_PK(ACC) ((const void*)p2p_fwd_f32_kernel<TM_CORE, ACC, false, true, true, false>)
-#define PSR_PICK(TM, ACC) ((const void*)p2p_fwd_f32_kernel<TM, ACC, false, true, PK, false>)
+#define PSR_PICK_PK(ACC) ((const void*)p2p_fwd_f32_kernel<TM_CORE, ACC, false, true, false, false>)
+#define PSR_PICK(TM, ACC) ((const void*)p2p_fwd_f32_kernel<TM, ACC, false, PK, false, false>)
     if (precision == PSR_FP32_EXACT)
         return accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
     if (PK && core)

@@ -94,13 +94,65 @@ struct Acc4 {
     }
 };
 
+// Writes one target's gradients from its four sums.
+__device__ __forceinline__ void adj_write(const FwdArgs& a, int target, const float* v)
+{
+    const int idx = a.perm[target];
+    float* o = reinterpret_cast<float*>(a.out) + 3LL * idx;
+    o[0] = v[0];
+    o[1] = v[1];
+    o[2] = v[2];
+    if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = v[3];
+}
+
+// The target sums that the group's warps left (base: this warp's, wstride
+// float4 per warp),
+// four 8-byte words (an FP64 sum, or a compensated FP32 pair) per target
+// at off + target slot, added over the warps in order and written.  word(t, i)
+// is the byte offset of target t's component i from a warp's base.
+template <int ACC, class Word>
+__device__ __forceinline__ void adj_combine(const FwdArgs& a, int4 li, const float4* base, int wstride,
+                                            float gx, float gm, Word word)
+{
+    group_sync(a.group);
+    const int nw = a.group, gw = (threadIdx.x >> 5) % nw;
+    base -= gw * wstride;
+    for (int t = 32 * gw + (threadIdx.x & 31); t < li.y; t += 32 * nw) {
+        float v[4];
+        for (int i = 0; i < 4; ++i) {
+            const float g = i < 3 ? gx : gm;
+            const unsigned off = word(t, i);
+            if (ACC == PSR_ACC_FP64) {
+                double sum = 0.0;
+                for (int w = 0; w < nw; ++w)
+                    sum += *reinterpret_cast<const volatile double*>(
+                        reinterpret_cast<const char*>(base + w * wstride) + off);
+                v[i] = (float)(sum * (double)g);
+            } else {
+                float hi = 0.0f, lo = 0.0f, u, e;
+                for (int w = 0; w < nw; ++w) {
+                    const volatile float* o = reinterpret_cast<const volatile float*>(
+                        reinterpret_cast<const char*>(base + w * wstride) + off);
+                    two_sum(hi, o[0], u, e);
+                    hi = u;
+                    lo += o[1] + e;
+                }
+                v[i] = (hi + lo) * g;
+            }
+        }
+        adj_write(a, li.x + t, v);
+    }
+}
+
 // Combine the S stream partials of each target and write dL/dx (scaled by
 // gx = G/(8 r_s^3) sc^3) and dL/dm (gm = -G/(4 r_s^2) sc^2) in the original
-// order.
+// order; with split, each warp's sums cover its part of the row and the
+// group's are combined after that.
 template <int ACC, int R>
 __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>* acc,
                                            const bool* act, int lane, int s, int q, int S, int T,
-                                           float gx, float gm, float4* __restrict__ stage)
+                                           float gx, float gm, float4* __restrict__ stage, bool split,
+                                           int wstride)
 {
     // Combine the S stream partials through the staging buffer: each target
     // slot r has its own region (1 KB) and the accesses are volatile, so no
@@ -119,12 +171,14 @@ __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>*
                 for (int t = 1; t < S; ++t)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) t4[i] += red[4 * (lane + t * T) + i];
-                const int idx = a.perm[li.x + q + T * r];
-                float* o = reinterpret_cast<float*>(a.out) + 3LL * idx;
-                o[0] = (float)(t4[0] * (double)gx);
-                o[1] = (float)(t4[1] * (double)gx);
-                o[2] = (float)(t4[2] * (double)gx);
-                if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = (float)(t4[3] * (double)gm);
+                if (split) {  // streams t >= 1 sit above the first T entries
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) red[4 * lane + i] = t4[i];
+                } else {
+                    const float v[4] = {(float)(t4[0] * (double)gx), (float)(t4[1] * (double)gx),
+                                        (float)(t4[2] * (double)gx), (float)(t4[3] * (double)gm)};
+                    adj_write(a, li.x + q + T * r, v);
+                }
             }
         } else {
             volatile float* red = reinterpret_cast<volatile float*>(stage) + 256 * r;
@@ -149,16 +203,25 @@ __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>*
                         hi[i] = u;
                         lo[i] += o[1] + v;
                     }
-                const int idx = a.perm[li.x + q + T * r];
-                float* o = reinterpret_cast<float*>(a.out) + 3LL * idx;
-                o[0] = (hi[0] + lo[0]) * gx;
-                o[1] = (hi[1] + lo[1]) * gx;
-                o[2] = (hi[2] + lo[2]) * gx;
-                if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = (hi[3] + lo[3]) * gm;
+                if (split) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        red[8 * lane + 2 * i] = hi[i];
+                        red[8 * lane + 2 * i + 1] = lo[i];
+                    }
+                } else {
+                    const float v4[4] = {(hi[0] + lo[0]) * gx, (hi[1] + lo[1]) * gx,
+                                         (hi[2] + lo[2]) * gx, (hi[3] + lo[3]) * gm};
+                    adj_write(a, li.x + q + T * r, v4);
+                }
             }
         }
         __syncwarp();
     }
+    if (split)
+        adj_combine<ACC>(a, li, stage, wstride, gx, gm, [T](int t, int i) {
+            return (unsigned)(1024 * (t / T) + 32 * (t % T) + 8 * i);
+        });
 }
 
 // Running sums of the two-targets-per-lane path in shared memory: the
@@ -234,14 +297,13 @@ __device__ __forceinline__ void acc_fold_all(unsigned base, int lane, float (*f)
 template <int ACC, int R>
 __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsigned accb,
                                                 const bool* act, int lane, int s, int q, int S,
-                                                int T, float gx, float gm)
+                                                int T, float gx, float gm, const float4* acc0, bool split,
+                                                int wstride)
 {
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         if (s != 0 || !act[r]) continue;
-        const int idx = a.perm[li.x + q + T * r];
-        float* o = reinterpret_cast<float*>(a.out) + 3LL * idx;
         if (ACC == PSR_ACC_FP64) {
             double t4[4];
 #pragma unroll
@@ -249,10 +311,16 @@ __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsig
             for (int t = 1; t < S; ++t)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) t4[i] += acc_ld_f64(acc_slot(accb, r, i, lane + t * T));
-            o[0] = (float)(t4[0] * (double)gx);
-            o[1] = (float)(t4[1] * (double)gx);
-            o[2] = (float)(t4[2] * (double)gx);
-            if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = (float)(t4[3] * (double)gm);
+            if (split) {  // the sums go to the slots of lane q
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    asm volatile("st.shared.f64 [%0], %1;" ::"r"(acc_slot(accb, r, i, lane)), "d"(t4[i])
+                                 : "memory");
+            } else {
+                const float v[4] = {(float)(t4[0] * (double)gx), (float)(t4[1] * (double)gx),
+                                    (float)(t4[2] * (double)gx), (float)(t4[3] * (double)gm)};
+                adj_write(a, li.x + q + T * r, v);
+            }
         } else {
             float hi[4], lo[4], u, v;
 #pragma unroll
@@ -269,13 +337,24 @@ __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsig
                     hi[i] = u;
                     lo[i] += w.y + v;
                 }
-            o[0] = (hi[0] + lo[0]) * gx;
-            o[1] = (hi[1] + lo[1]) * gx;
-            o[2] = (hi[2] + lo[2]) * gx;
-            if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = (hi[3] + lo[3]) * gm;
+            if (split) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(acc_slot(accb, r, i, lane)),
+                                 "f"(hi[i]), "f"(lo[i])
+                                 : "memory");
+            } else {
+                const float v4[4] = {(hi[0] + lo[0]) * gx, (hi[1] + lo[1]) * gx, (hi[2] + lo[2]) * gx,
+                                     (hi[3] + lo[3]) * gm};
+                adj_write(a, li.x + q + T * r, v4);
+            }
         }
     }
     __syncwarp();
+    if (split)
+        adj_combine<ACC>(a, li, acc0, wstride, gx, gm, [T](int t, int i) {
+            return (unsigned)(256 * (4 * (t / T) + i) + 8 * (t % T));
+        });
 }
 
 // One target leaf on one warp (same decomposition as the forward kernels;
@@ -289,7 +368,8 @@ __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsig
 template <int TM, int ACC, bool EQM, int R>
 __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                          unsigned q_off, float4* __restrict__ stage,
-                                         float4* __restrict__ meta, unsigned accb)
+                                         float4* __restrict__ meta, unsigned accb, bool split,
+                                         int wstride)
 {
     constexpr bool SA = R == 2;  // sums in shared memory
     const int lane = threadIdx.x & 31;
@@ -348,8 +428,8 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
             }
         cull_box(lx, ly, lz, hx, hy, hz, x_c * sc, meta + kMetaPerWarp);
     }
-    const long long re = a.rowptr[I + 1];
-    long long e0 = a.rowptr[I];
+    long long e0, re;
+    row_part(a, I, split, e0, re);
     while (e0 < re) {
         int nst;
         e0 += stage_chunk<2>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
@@ -439,9 +519,11 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
     }
     const float gx = bx.g_adj * sc * sc * sc * (EQM ? bx.m_eq : 1.0f);
     if (SA)
-        adj_finish_smem<ACC, R>(a, li, accb, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc);
+        adj_finish_smem<ACC, R>(a, li, accb, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc,
+                                meta + kWarpMeta, split, wstride);
     else
-        adj_finish<ACC, R>(a, li, acc, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc, stage);
+        adj_finish<ACC, R>(a, li, acc, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc, stage, split,
+                           wstride);
 }
 
 // Packed variant of adj_item (PSR_KERNEL_PACKED): each stream takes staged
@@ -459,7 +541,7 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
 template <int TM, int ACC, bool EQM, int R>
 __device__ __forceinline__ void adj_item_pk(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                             unsigned q_off, float4* __restrict__ stage,
-                                            float4* __restrict__ meta)
+                                            float4* __restrict__ meta, bool split, int wstride)
 {
     const int lane = threadIdx.x & 31;
     const float4* __restrict__ pf = reinterpret_cast<const float4*>(a.pf);
@@ -511,8 +593,8 @@ __device__ __forceinline__ void adj_item_pk(const FwdArgs& a, int I, int4 li, un
     const float2 c4n2 = make_float2(c4n, c4n);
     // exp(-x^2) = 2^(r2 qarg): r2 is in units of x_c^2 on the linear path
     const float qarg = -kLog2E * x_c * x_c;
-    const long long re = a.rowptr[I + 1];
-    long long e0 = a.rowptr[I];
+    long long e0, re;
+    row_part(a, I, split, e0, re);
     while (e0 < re) {
         int nst;
         e0 += stage_chunk<3>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
@@ -576,13 +658,14 @@ __device__ __forceinline__ void adj_item_pk(const FwdArgs& a, int I, int4 li, un
         __syncwarp();
     }
     adj_finish<ACC, R>(a, li, acc, act, lane, s, q, S, T,
-                       bx.g_adj * sc * sc * sc * (EQM ? bx.m_eq : 1.0f), -bx.g_adjm * sc * sc, stage);
+                       bx.g_adj * sc * sc * sc * (EQM ? bx.m_eq : 1.0f), -bx.g_adjm * sc * sc, stage, split,
+                       wstride);
 }
 
 // Shared memory: the table (T and Q), then per warp a staging buffer of
 // stage_cap particles x 2 float4, 32 entry records and the two box slots,
 // then the accumulator block of the two-targets path (kAdjAccF4).
-template <int TM, int ACC, bool WIDE, bool PK, bool EQM>
+template <int TM, int ACC, bool WIDE, bool PK, bool EQM, bool SPLIT>
 __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -627,11 +710,12 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
     const unsigned tab_bias = smem_u32(smem) - (unsigned)kMagicBits * (TM == TM_LINEAR && PK ? 8u : 16u);
     const unsigned q_off = (unsigned)(a.table_n + 1) * 16u;
     const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = (int)atomicAdd(a.ctrl + kCtrlTicketAdj, 1u) * a.item_stride + a.item_offset;
-        it = __shfl_sync(kFull, it, 0);
-        if (it >= a.n_items) break;
+    __shared__ int s_it[8];
+    const int wstride = 2 * a.stage_cap + kWarpMeta + kAdjAccF4;
+    const int n_heavy = !SPLIT ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    bool split = SPLIT && n_heavy > 0;
+    int it;
+    while (next_item<SPLIT>(a, a.ctrl + kCtrlTicketAdj, split, n_heavy, s_it, it)) {
         int I = a.items[it];
         if (I < 0 || I >= a.n_leaves) {
             if (lane == 0) set_error(a.ctrl, kErrItemIndex);
@@ -645,17 +729,17 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
         }
         if (PK) {
             if (WIDE && prefer_two_per_lane(li.y))
-                adj_item_pk<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta);
+                adj_item_pk<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, SPLIT && split, wstride);
             else
-                adj_item_pk<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta);
+                adj_item_pk<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, SPLIT && split, wstride);
         } else if (WIDE && prefer_two_per_lane(li.y)) {
             // leaves of 11-12 and 17-20 particles up to 32 (and all larger
             // ones); at equal lane fill one target per lane is faster (its
             // state fits the registers and its loop takes four sources per
             // iteration): sending the ties to two targets cost 1.4 %
-            adj_item<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, accb);
+            adj_item<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, accb, SPLIT && split, wstride);
         } else {
-            adj_item<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, accb);
+            adj_item<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, accb, SPLIT && split, wstride);
         }
     }
     persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
@@ -821,15 +905,15 @@ size_t adj_f32_smem(int precision, int interp, int table_n, int warps, int cap)
     return tab + (size_t)warps * (2 * cap + kWarpMeta + kAdjAccF4) * 16;
 }
 
-template <int TM, int ACC, bool EQM>
+template <int TM, int ACC, bool EQM, bool SPLIT>
 static int launch_adj_e(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
     // always with the two-targets-per-lane path (mid-size leaves fill more lanes)
     // (the packed variant carries it only for leaves above 32 particles: its
     // per-target state would spill)
-    auto k = a.variant != PSR_KERNEL_PACKED ? p2p_adj_f32_kernel<TM, ACC, true, false, EQM>
-             : a.max_leaf > 32              ? p2p_adj_f32_kernel<TM, ACC, true, true, EQM>
-                                            : p2p_adj_f32_kernel<TM, ACC, false, true, EQM>;
+    auto k = SPLIT || a.variant != PSR_KERNEL_PACKED ? p2p_adj_f32_kernel<TM, ACC, true, false, EQM, SPLIT>
+             : a.max_leaf > 32              ? p2p_adj_f32_kernel<TM, ACC, true, true, EQM, false>
+                                            : p2p_adj_f32_kernel<TM, ACC, false, true, EQM, false>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
@@ -842,8 +926,11 @@ static int launch_adj_e(const FwdArgs& a, size_t smem, cudaStream_t st)
 template <int TM, int ACC>
 static int launch_adj_t(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
-    return a.equal_mass ? launch_adj_e<TM, ACC, true>(a, smem, st)
-                        : launch_adj_e<TM, ACC, false>(a, smem, st);
+    if (a.group > 1)
+        return a.equal_mass ? launch_adj_e<TM, ACC, true, true>(a, smem, st)
+                            : launch_adj_e<TM, ACC, false, true>(a, smem, st);
+    return a.equal_mass ? launch_adj_e<TM, ACC, true, false>(a, smem, st)
+                        : launch_adj_e<TM, ACC, false, false>(a, smem, st);
 }
 
 int launch_adj_f32(const FwdArgs& a, int precision, void* stream)
@@ -889,9 +976,9 @@ int adj_occupancy(int precision, int interp, int accum, int warps, int max_leaf,
     } else {
         smem = adj_f32_smem(precision, interp, table_n, warps, cap);
 #define PSR_PICK(TM, ACC) (variant != PSR_KERNEL_PACKED \
-                               ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, false, false> \
-                               : wide ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, true, false> \
-                                      : (const void*)p2p_adj_f32_kernel<TM, ACC, false, true, false>)
+                               ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, false, false, false> \
+                               : wide ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, true, false, false> \
+                                      : (const void*)p2p_adj_f32_kernel<TM, ACC, false, true, false, false>)
         if (precision == PSR_FP32_EXACT)
             f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
         else if (interp == PSR_LINEAR)

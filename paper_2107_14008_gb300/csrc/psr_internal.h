@@ -71,6 +71,7 @@ enum : int {
     kCtrlError = 8,
     kCtrlPairsLo = 16,  // uint64 at words 16..17: pairs within the cutoff
     kCtrlEvalLo = 18,   // uint64 at words 18..19: pairs evaluated
+    kCtrlHeavy = 32,    // words 32..35: heavy items of each level (heavy_cost)
     kCtrlWords = 64,
 };
 // error bits
@@ -101,7 +102,10 @@ struct Leaves {
     std::vector<int64_t> rowptr;
     std::vector<uint32_t> pairs;
     std::vector<int32_t> items;
+    std::vector<int64_t> item_cost;  // evaluated pairs of each item, in schedule order
+    int32_t n_heavy[4] = {0, 0, 0, 0};  // host copy of ctrl[kCtrlHeavy..] (psr_upload)
     int64_t evaluated = 0;
+    int64_t max_cost = 0;  // the largest leaf's evaluated pairs
     int max_leaf = 0;
     int max_row = 0;
     // counts (set by both builders; a device-built handle has no host arrays)
@@ -114,7 +118,6 @@ struct Leaves {
     double theta = 0.0;         //   multipole acceptance parameter of that split
     int64_t n_far = 0;          //   far entries
     char* db_scratch = nullptr; // device build between its two calls: the caller's scratch
-    int64_t db_maxcost = 0;     //   and the largest per-leaf cost (schedule sort width)
     int db_kslot = 0;           //   runs per row in the pair cache (0: not used)
     int db_interleave = 0;      //   whether the walks take rows interleaved over warps
     int64_t db_uncached = 0;    //   and the rows it could not hold
@@ -138,6 +141,48 @@ int build_batch(int nbox, const double* const* pos, const double* const* mass, c
 Layout make_layout(const Leaves& h);
 size_t table_entry_bytes(int interp);  // p2p_fwd_f32.cu
 BoxDev box_constants(const psr_box& b);  // per-box kernel constants
+
+// Heavy items: those of the schedule's head that are worth sharing among the
+// warps of a group.  The schedule keeps the counts of items whose work exceeds
+// 1/2, 1, 2 and 4 times a warp's share of the launch with 32 warps per SM.
+constexpr int kHeavyLevels = 4;
+inline int64_t heavy_cost(int level, int64_t evaluated, int sms)
+{
+    return (evaluated << level) / (64 * (int64_t)(sms > 0 ? sms : 1));
+}
+
+// Whether and how a launch on `warps` resident warps shares heavy rows.
+// group: warps per heavy item, 1 for none; level: which count of heavy items
+// applies, -1 for all items.  A launch shares rows only where the largest item
+// exceeds 3/2 of a warp's share of the work (the
+// adjoint, whose pairs cost twice as much against the same overheads: 2): then a row on one warp outlasts
+// the others, or the chip is never filled; below it the largest-first order
+// hides the longest row, and the group phase's registers cost 1-3 % (128^3 NFW
+// in leaves of up to 64: 9.53 -> 9.66 ms).  Items above about half a share are
+// shared, all of them when there are fewer leaves than warps, and the group is
+// large enough to bring the largest item's parts to 3/2 of a share, with at
+// least 2500 pairs in a part (the group's barriers and the row's start-up
+// latency cost about as much as 1500).  Forward, one warp per row against this:
+// 5000 uniform particles 0.235 -> 0.081 ms, 32^3 0.28 -> 0.12, 110,000 NFW 2.57
+// -> 1.1, 64^3 NFW 2.3 -> 1.5; adjoint 32^3 0.28 -> 0.20.  Groups of 8 wherever
+// rows are shared at all: 60,000 uniform in leaves of up to 16 0.28 ms against
+// 0.17 with groups of 2 and 0.19 with one warp per row.
+struct SplitRule {
+    int group, level;
+};
+inline SplitRule split_rule(int64_t max_cost, int64_t evaluated, int64_t n_leaves, int sms, int64_t warps,
+                            int block_warps, bool adjoint)
+{
+    SplitRule r{1, -1};
+    const int64_t share = evaluated / (warps > 0 ? warps : 1);
+    if (max_cost <= (adjoint ? 2 * share : share + share / 2)) return r;
+    while (r.group < 8 && 2 * max_cost > 3 * r.group * share && max_cost >= 5000 * r.group) r.group *= 2;
+    while (r.group > 1 && block_warps % r.group) r.group /= 2;
+    if (n_leaves >= warps)
+        for (r.level = 0; r.level + 1 < kHeavyLevels && 3 * heavy_cost(r.level, evaluated, sms) < share;)
+            ++r.level;
+    return r;
+}
 
 // kernels (launchers defined in the .cu files; return cudaError_t as int)
 struct FwdArgs {
@@ -173,6 +218,8 @@ struct FwdArgs {
     int stage_cap;   // FP32 kernels: staged particles per warp
     int item_stride; // this launch takes schedule entries ticket * stride + offset
     int item_offset;
+    const int* heavy;  // how many items groups of warps take (null: all)
+    int group;         // warps per group (divides warps_per_block); 0 or 1: none
     int core;        // FP32 forward: a.table is the core form of the linear table
     int equal_mass;  // every box has one particle mass: the FP32 kernels take it out of the sums
 };

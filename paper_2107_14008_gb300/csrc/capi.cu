@@ -178,8 +178,16 @@ void resolve_kernel(const Leaves* h, Opts& o)
 int ensure_table(Leaves* h, const Opts& o, bool core, cudaStream_t st)
 {
     const bool t64 = fp64_taylor(o);
-    if (o.precision != PSR_FP32_TABLE && !t64) return PSR_OK;
     const double x_c = cutoff_x(h);
+    if (o.precision == PSR_FP64 && !t64) {
+        if (h->t64_xc == x_c) return PSR_OK;
+        double* t = reinterpret_cast<double*>(h->d_ws + h->lay.t64);
+        const int e = launch_plain64(x_c, t, t + 6 * (kPlain64MaxN + 2), st);
+        if (e) return cuda_fail((cudaError_t)e, "table kernel launch");
+        h->t64_xc = x_c;
+        return PSR_OK;
+    }
+    if (o.precision != PSR_FP32_TABLE && !t64) return PSR_OK;
     if (core) {
         if (h->core_key == o.table_n && h->core_xc == x_c) return PSR_OK;
         const int e = launch_core_table(o.table_n, x_c, h->d_ws + h->lay.core, st);
@@ -204,11 +212,13 @@ int grid_blocks(Leaves* h, const Opts& o, int adjoint, int* blocks)
     int bps = o.bps;
     if (bps == 0) {
         int occ = 0, e;
-        if (adjoint)
-            e = adj_occupancy(o.precision, o.interp, o.accum, o.warps, h->max_leaf, o.table_n,
+        if (adjoint && o.precision == PSR_FP64)
+            e = adj_f64_occupancy(o.warps, cutoff_x(h), &occ);
+        else if (adjoint)
+            e = adj_f32_occupancy(o.precision, o.interp, o.accum, o.warps, h->max_leaf, o.table_n,
                               o.tile ? o.tile : kAdjStageCap, o.kernel, &occ);
         else if (o.precision == PSR_FP64)
-            e = fwd_f64_occupancy(o.warps, h->max_leaf, o.interp, o.table_n, &occ);
+            e = fwd_f64_occupancy(o.warps, o.interp, o.table_n, cutoff_x(h), &occ);
         else if (o.kernel == PSR_KERNEL_PAPER)
             e = fwd_blk_occupancy(o.precision, o.interp, o.accum, h->max_leaf, o.table_n, &occ);
         else {
@@ -230,7 +240,7 @@ int grid_blocks(Leaves* h, const Opts& o, int adjoint, int* blocks)
 // whose grid is known.
 void set_split(const Leaves* h, const Opts& o, bool adjoint, FwdArgs* a)
 {
-    if (!o.split) return;
+    if (!o.split && o.precision != PSR_FP64) return;
     const SplitRule r = split_rule(h->max_cost, h->evaluated, h->n_leaves, h->sm_count,
                                    (int64_t)a->blocks * o.warps, o.warps, adjoint);
     a->group = r.group;
@@ -375,6 +385,7 @@ int psr_upload(psr_leaves* hh, void* d_ws, size_t bytes, void* stream)
     h->table_key = -1;
     h->table_xc = -1.0;
     h->core_key = -1;
+    h->t64_xc = -1.0;
     h->sm_count = sms;
     h->device = dev;
     return PSR_OK;
@@ -403,6 +414,7 @@ int psr_p2p_forces(psr_leaves* hh, const psr_opts* opts, void* d_acc, void* stre
         a.core = 1;
         a.table = h->d_ws + h->lay.core;
     }
+    if (o.precision == PSR_FP64 && !fp64_taylor(o)) a.table = h->d_ws + h->lay.t64;
     if (fwd32 && (rc = fwd32_smem_config(o, &a.stage_cap))) return rc;
     if (fwd32 && (rc = check_tile(h, a.stage_cap))) return rc;
     if ((rc = grid_blocks(h, o, 0, &a.blocks))) return rc;
@@ -411,7 +423,7 @@ int psr_p2p_forces(psr_leaves* hh, const psr_opts* opts, void* d_acc, void* stre
         cudaError_t e = cudaMemsetAsync(a.ctrl + kCtrlPairsLo, 0, 16, st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (pair counters)");
     }
-    int e = (o.precision == PSR_FP64)          ? launch_fwd_f64(a, st)
+    int e = (o.precision == PSR_FP64)          ? launch_fwd_f64(a, cutoff_x(h), st)
             : (o.kernel == PSR_KERNEL_PAPER) ? launch_fwd_blk(a, o.precision, st)
                                              : launch_fwd_f32(a, o.precision, st);
     if (e) return cuda_fail((cudaError_t)e, "forward kernel launch");
@@ -445,11 +457,12 @@ int psr_p2p_adjoint(psr_leaves* hh, const psr_opts* opts, const void* d_cot, voi
         adj_f32_smem(o.precision, o.interp, o.table_n, o.warps, a.stage_cap) > kSmemPerBlock)
         return fail(PSR_E_ARG, "adjoint table and staging buffers exceed shared memory; "
                                "use fewer warps or a smaller table");
+    if (o.precision == PSR_FP64) a.table = h->d_ws + h->lay.t64;
     a.out = d_grad_pos;
     a.out_m = d_grad_mass;
     if ((rc = grid_blocks(h, o, 1, &a.blocks))) return rc;
     set_split(h, o, true, &a);
-    int e = (o.precision == PSR_FP64) ? launch_adj_f64(a, st) : launch_adj_f32(a, o.precision, st);
+    int e = (o.precision == PSR_FP64) ? launch_adj_f64(a, cutoff_x(h), st) : launch_adj_f32(a, o.precision, st);
     if (e) return cuda_fail((cudaError_t)e, "adjoint kernel launch");
     return PSR_OK;
 }

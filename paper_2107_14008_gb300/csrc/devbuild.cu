@@ -1826,6 +1826,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     h->table_key = -1;
     h->table_xc = -1.0;
     h->core_key = -1;
+    h->t64_xc = -1.0;
     h->adj_table_key = -1;
     h->sm_count = sms;
     h->device = dev;

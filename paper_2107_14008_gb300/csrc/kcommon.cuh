@@ -92,10 +92,105 @@ __device__ __forceinline__ float4 lds_f4(unsigned a)
         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
     return v;
 }
-// lanes per stream T (power of two >= n, at least 4), as log2
-__device__ __forceinline__ int stream_log2(int n)
+// Barrier of the calling warp's group of `warps` consecutive warps (the block
+// holds a whole number of groups; barrier 0 is left to __syncthreads).
+__device__ __forceinline__ void group_sync(int warps)
 {
-    return n <= 4 ? 2 : n <= 8 ? 3 : n <= 16 ? 4 : 5;
+    const int id = 1 + (int)(threadIdx.x >> 5) / warps;
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(32 * warps) : "memory");
+}
+
+// This warp's entries of a row: all of them, or with split its share among
+// the warps of its group.
+__device__ __forceinline__ void row_part(const FwdArgs& a, int I, bool split, long long& e0, long long& re)
+{
+    e0 = a.rowptr[I];
+    re = a.rowptr[I + 1];
+    if (split) {
+        const int len = (int)(re - e0), W = a.group, w = (threadIdx.x >> 5) % W;
+        re = e0 + (long long)len * (w + 1) / W;
+        e0 += (long long)len * w / W;
+    }
+}
+
+// The next item of a persistent launch.  The schedule's first *a.heavy items
+// (their work is more than a fraction of what one warp of a full chip gets,
+// see heavy_cost) are taken by groups of a.group warps, one ticket a group
+// (split stays true; s_it: one word per group), the rest by single warps; the
+// ticket on which a group leaves the first phase goes to its first warp.
+// Returns false when no item is left.  Which items are split, and how, is
+// fixed by the schedule alone, so results do not depend on the order in which
+// blocks run.
+template <bool SPLIT>
+__device__ __forceinline__ bool next_item(const FwdArgs& a, unsigned* ticket, bool& split,
+                                          int n_heavy, volatile int* s_it, int& it)
+{
+    if (SPLIT && split) {
+        const int g = (threadIdx.x >> 5) / a.group;
+        const bool first = threadIdx.x - g * 32 * a.group < 32;
+        group_sync(a.group);  // the group's last item is combined
+        if (first && (threadIdx.x & 31) == 0)
+            s_it[g] = (int)atomicAdd(ticket, 1u) * a.item_stride + a.item_offset;
+        group_sync(a.group);
+        it = s_it[g];
+        if (it < n_heavy) return true;  // n_heavy <= n_items
+        split = false;
+        if (first) return it < a.n_items;
+    }
+    int t = 0;
+    if ((threadIdx.x & 31) == 0) t = (int)atomicAdd(ticket, 1u) * a.item_stride + a.item_offset;
+    it = __shfl_sync(kFull, t, 0);
+    return it < a.n_items;
+}
+
+// Targets per lane for the scalar kernel, by cost per useful pair.  One
+// iteration of a stream evaluates one staged source against the lane's R
+// targets, kPairInstr instructions per target plus kSourceInstr for the
+// source itself (its shared-memory load and the loop), and the warp's
+// S_R = floor(32 / ceil(n_I / R)) streams serve n_I S_R pairs per iteration:
+// the cost per pair is (kPairInstr R + kSourceInstr) / S_R, the cheapest R
+// wins, ties going to the smaller.  The per-source term is set to 0, the
+// measured best: with 3, 6 or 10 the rule moves leaves of 25-32 particles to
+// R = 2 or 3 at equal lane fill, and whole launches ran 2-5 % slower.  So a
+// larger R is taken only where it fills strictly more lanes: R = 3 for
+// leaves of 3, 6, 9, 11-12, 17-18, 21-24 (24 = 8 lanes x 3 targets x 4
+// streams) and 33-48 particles (11-16 lanes x 2 streams, against 17-24 lanes
+// x 1 for R = 2; 6 % faster on leaves of up to 64); R = 2 for 19-20 and
+// 49-64.  R = 1 needs n_I <= 32; R = 3 needs tiles of at least 128
+// particles (its final reduction takes 3 x 768 B of the warp's staging
+// buffer).
+constexpr int kPairInstr = 20, kSourceInstr = 0;
+__device__ __forceinline__ int targets_per_lane(int n, int cap)
+{
+    int best = 0, bnum = 0, bS = 1;
+#pragma unroll
+    for (int R = 1; R <= 3; ++R) {
+        const int T = (n + R - 1) / R;
+        if (T > 32 || (R == 3 && cap < 128)) continue;
+        const int S = 32 / T, num = kPairInstr * R + kSourceInstr;
+        if (best == 0 || num * bS < bnum * S) {
+            best = R;
+            bnum = num;
+            bS = S;
+        }
+    }
+    return best;
+}
+
+// Morton-order source payload of the cotangent: cs[k] = (c[perm[k]], 0).
+template <typename T, typename T4>
+__global__ void gather_cot_kernel(const T* __restrict__ cot, const int32_t* __restrict__ perm,
+                                  T4* __restrict__ cs, long long n)
+{
+    long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    long long i = perm[k];
+    T4 v;
+    v.x = cot[3 * i];
+    v.y = cot[3 * i + 1];
+    v.z = cot[3 * i + 2];
+    v.w = 0;
+    cs[k] = v;
 }
 
 }  // namespace psr

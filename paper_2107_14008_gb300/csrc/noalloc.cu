@@ -116,8 +116,16 @@ extern "C" int psr_p2p_forces_noalloc(psr_leaves* hh, const psr_opts* opts, void
         set_last_error(std::string("cudaMemsetAsync (scratch counters): ") + cudaGetErrorString(e));
         return PSR_E_CUDA;
     }
+    const double x_c = h->boxes[0].r_c / (2.0 * h->boxes[0].r_s);
+    if (precision == PSR_FP64) {
+        static_assert((size_t)6 * (kPlain64MaxN + 2) * 8 <= kTableBytes, "FP64 table beyond the scratch");
+        int le = launch_plain64(x_c, base, nullptr, st);
+        if (le) {
+            set_last_error(std::string("table kernel launch: ") + cudaGetErrorString((cudaError_t)le));
+            return PSR_E_CUDA;
+        }
+    }
     if (precision == PSR_FP32_TABLE) {
-        const double x_c = h->boxes[0].r_c / (2.0 * h->boxes[0].r_s);
         int le = a.core ? launch_core_table(a.table_n, x_c, base, st)
                         : launch_table(a.table_n, a.interp, x_c, base, nullptr, st);
         if (le) {
@@ -125,7 +133,7 @@ extern "C" int psr_p2p_forces_noalloc(psr_leaves* hh, const psr_opts* opts, void
             return PSR_E_CUDA;
         }
     }
-    int le = precision == PSR_FP64              ? launch_fwd_f64(a, st)
+    int le = precision == PSR_FP64              ? launch_fwd_f64(a, x_c, st)
              : a.variant == PSR_KERNEL_PAPER ? launch_fwd_blk(a, precision, st)
                                              : launch_fwd_f32(a, precision, st);
     if (le) {

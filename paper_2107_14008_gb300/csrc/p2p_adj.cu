@@ -745,159 +745,6 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
     persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
 }
 
-// ------------------------------------------------------------------ FP64 --
-template <int R>
-__device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li)
-{
-    const int lane = threadIdx.x & 31;
-    const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
-    const double4* __restrict__ cs = reinterpret_cast<const double4*>(a.cot_sorted);
-    const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
-    const int nI = li.y;
-    const int lgT = (R == 2) ? 5 : stream_log2(nI);
-    const int q = lane & ((1 << lgT) - 1);
-    const int s = lane >> lgT;
-    const int S = 32 >> lgT;
-    const BoxDev& bx = a.boxes[li.z];
-    const double L = bx.L, rc2 = bx.rc2, inv2rs = bx.inv_2rs;
-    const double c2 = 1.1283791670955126;  // 2/sqrt(pi)
-    // exp(-x^2) / (2 sqrt(pi) r_s^3)
-    const double cq = 1.0 / (2.0 * 1.7724538509055160 * bx.r_s * bx.r_s * bx.r_s);
-    double4 xi[R], ck[R];
-    bool act[R];
-    double t3[R][3], g[R][4];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        int t = q + 32 * r;
-        act[r] = t < nI;
-        xi[r] = pd[li.x + (act[r] ? t : 0)];
-        ck[r] = cs[li.x + (act[r] ? t : 0)];
-        for (int i = 0; i < 4; ++i) g[r][i] = 0.0;
-        t3[r][0] = t3[r][1] = t3[r][2] = 0.0;
-    }
-    const long long re = a.rowptr[I + 1];
-    long long e = a.rowptr[I] + s;
-    int j = 0, jend = 0;
-    for (;;) {
-        if (j >= jend) {
-            bool found = false;
-            while (e < re) {
-                unsigned ent = a.pairs[e];
-                e += S;
-                int J = (int)(ent >> 5);
-                unsigned code = ent & 31u;
-                if (J >= a.n_leaves || code >= (unsigned)kShiftCodes) {
-                    set_error(a.ctrl, J >= a.n_leaves ? kErrLeafIndex : kErrShiftCode);
-                    continue;
-                }
-                int4 lj = leaf[J];
-                if (lj.x < 0 || lj.y < 0 || (long long)lj.x + lj.y > a.n) {
-                    set_error(a.ctrl, kErrParticleRange);
-                    continue;
-                }
-                int nx, ny, nz;
-                decode_shift(code, nx, ny, nz);
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    t3[r][0] = xi[r].x - nx * L;
-                    t3[r][1] = xi[r].y - ny * L;
-                    t3[r][2] = xi[r].z - nz * L;
-                }
-                j = lj.x;
-                jend = lj.x + lj.y;
-                found = true;
-                break;
-            }
-            if (!found) break;
-        }
-        const double4 p = pd[j];
-        const double4 c = cs[j];
-        ++j;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            double dx = p.x - t3[r][0], dy = p.y - t3[r][1], dz = p.z - t3[r][2];
-            double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < rc2 && r2 > 0.0) {
-                double rr = sqrt(r2);
-                double x = rr * inv2rs;
-                double Q = exp(-x * x);
-                double T = erfc(x) + c2 * x * Q;
-                double gg = T / (r2 * rr);
-                double hf = -3.0 * gg / r2 - cq * Q / r2;  // g'(r)/r
-                double vx = xi[r].w * c.x - p.w * ck[r].x;
-                double vy = xi[r].w * c.y - p.w * ck[r].y;
-                double vz = xi[r].w * c.z - p.w * ck[r].z;
-                double hd = hf * (dx * vx + dy * vy + dz * vz);
-                g[r][0] += gg * vx + hd * dx;
-                g[r][1] += gg * vy + hd * dy;
-                g[r][2] += gg * vz + hd * dz;
-                g[r][3] += gg * (dx * c.x + dy * c.y + dz * c.z);
-            }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        for (int off = 1 << lgT; off < 32; off <<= 1)
-            for (int i = 0; i < 4; ++i) g[r][i] += __shfl_xor_sync(kFull, g[r][i], off);
-    if (s == 0) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (!act[r]) continue;
-            int idx = a.perm[li.x + q + 32 * r];
-            double* o = reinterpret_cast<double*>(a.out) + 3LL * idx;
-            o[0] = bx.G * g[r][0];
-            o[1] = bx.G * g[r][1];
-            o[2] = bx.G * g[r][2];
-            if (a.out_m) reinterpret_cast<double*>(a.out_m)[idx] = -bx.G * g[r][3];
-        }
-    }
-}
-
-template <bool WIDE>
-__global__ void __launch_bounds__(256) p2p_adj_f64_kernel(const FwdArgs a)
-{
-    const int lane = threadIdx.x & 31;
-    const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = (int)atomicAdd(a.ctrl + kCtrlTicketAdj, 1u) * a.item_stride + a.item_offset;
-        it = __shfl_sync(kFull, it, 0);
-        if (it >= a.n_items) break;
-        int I = a.items[it];
-        if (I < 0 || I >= a.n_leaves) {
-            if (lane == 0) set_error(a.ctrl, kErrItemIndex);
-            continue;
-        }
-        int4 li = leaf[I];
-        if (li.y <= 0 || li.y > a.max_leaf || (long long)li.x + li.y > a.n || li.z < 0 ||
-            li.z >= a.nbox) {
-            if (lane == 0) set_error(a.ctrl, kErrParticleRange);
-            continue;
-        }
-        if (WIDE && li.y > 32)
-            adj64_item<2>(a, I, li);
-        else
-            adj64_item<1>(a, I, li);
-    }
-    persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
-}
-
-// Morton-order source payload of the cotangent: cs[k] = (c[perm[k]], 0).
-template <typename T, typename T4>
-__global__ void gather_cot_kernel(const T* __restrict__ cot, const int32_t* __restrict__ perm,
-                                  T4* __restrict__ cs, long long n)
-{
-    long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    long long i = perm[k];
-    T4 v;
-    v.x = cot[3 * i];
-    v.y = cot[3 * i + 1];
-    v.z = cot[3 * i + 2];
-    v.w = 0;
-    cs[k] = v;
-}
-
 size_t adj_f32_smem(int precision, int interp, int table_n, int warps, int cap)
 {
     size_t tab = precision != PSR_FP32_TABLE ? 0
@@ -952,44 +799,26 @@ int launch_adj_f32(const FwdArgs& a, int precision, void* stream)
                                    : launch_adj_t<TM_CUBIC, PSR_ACC_KAHAN32>(a, smem, st);
 }
 
-int launch_adj_f64(const FwdArgs& a, void* stream)
-{
-    cudaStream_t st = (cudaStream_t)stream;
-    long long nb = (a.n + 255) / 256;
-    gather_cot_kernel<double, double4><<<(unsigned)nb, 256, 0, st>>>(
-        reinterpret_cast<const double*>(a.cot), a.perm, reinterpret_cast<double4*>(a.cot_sorted), a.n);
-    cudaError_t e0 = cudaGetLastError();
-    if (e0 != cudaSuccess) return (int)e0;
-    if (a.max_leaf > 32) p2p_adj_f64_kernel<true><<<a.blocks, a.warps_per_block * 32, 0, st>>>(a);
-    else p2p_adj_f64_kernel<false><<<a.blocks, a.warps_per_block * 32, 0, st>>>(a);
-    return (int)cudaGetLastError();
-}
-
-int adj_occupancy(int precision, int interp, int accum, int warps, int max_leaf, int table_n,
-                  int cap, int variant, int* out)
+int adj_f32_occupancy(int precision, int interp, int accum, int warps, int max_leaf, int table_n,
+                      int cap, int variant, int* out)
 {
     const bool wide = max_leaf > 32;
-    size_t smem = 0;
     const void* f;
-    if (precision == PSR_FP64) {
-        f = wide ? (const void*)p2p_adj_f64_kernel<true> : (const void*)p2p_adj_f64_kernel<false>;
-    } else {
-        smem = adj_f32_smem(precision, interp, table_n, warps, cap);
+    const size_t smem = adj_f32_smem(precision, interp, table_n, warps, cap);
 #define PSR_PICK(TM, ACC) (variant != PSR_KERNEL_PACKED \
                                ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, false, false, false> \
                                : wide ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, true, false, false> \
                                       : (const void*)p2p_adj_f32_kernel<TM, ACC, false, true, false, false>)
-        if (precision == PSR_FP32_EXACT)
-            f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
-        else if (interp == PSR_LINEAR)
-            f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_LINEAR, PSR_ACC_FP64) : PSR_PICK(TM_LINEAR, PSR_ACC_KAHAN32);
-        else
-            f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_CUBIC, PSR_ACC_FP64) : PSR_PICK(TM_CUBIC, PSR_ACC_KAHAN32);
+    if (precision == PSR_FP32_EXACT)
+        f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
+    else if (interp == PSR_LINEAR)
+        f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_LINEAR, PSR_ACC_FP64) : PSR_PICK(TM_LINEAR, PSR_ACC_KAHAN32);
+    else
+        f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_CUBIC, PSR_ACC_FP64) : PSR_PICK(TM_CUBIC, PSR_ACC_KAHAN32);
 #undef PSR_PICK
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return (int)e;
-        }
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return (int)e;
     }
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, f, warps * 32, smem);
 }

@@ -1,0 +1,158 @@
+// FP64 adjoint P2P kernel: the sums of p2p_adj.cu in double precision (r, not
+// x, units).  p2p_f64_common.cuh says what bounds it: about 47 FP64
+// instructions per pair with one mass per box, T and exp(-x^2) from the plain
+// path's tables.  32^3 uniform set: 36.7 ms with erfc, exp, a square root and
+// divisions per tile pair and one warp per leaf.
+#include <cuda_runtime.h>
+
+#include "p2p_f64_common.cuh"
+
+namespace psr {
+
+constexpr int kStageAdj64 = 64;  // staged sources per warp (64 bytes each)
+
+template <bool EQM, int R>
+__device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, const double* tab,
+                                           const double* tabq, double2* __restrict__ stage,
+                                           int2* __restrict__ meta, bool split)
+{
+    const int lane = threadIdx.x & 31;
+    const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
+    const double4* __restrict__ cs = reinterpret_cast<const double4*>(a.cot_sorted);
+    double* box = reinterpret_cast<double*>(meta + 32);
+    const int nI = li.y, T = (nI + R - 1) / R, S = 32 / T, s = lane / T, q = lane - s * T;
+    const bool on = s < S;
+    const BoxDev& bx = a.boxes[li.z];
+    const long long rc2m1 = bits64(bx.rc2) - 1;
+    const double us = bx.inv_2rs * a.t64_scale;
+    // exp(-x^2) / (2 sqrt(pi) r_s^3), the second part of -g'(r) r
+    const double cq = 1.0 / (2.0 * 1.7724538509055160 * bx.r_s * bx.r_s * bx.r_s);
+
+    double4 xi[R], ck[R];
+    bool act[R];
+    double g[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int t = q + T * r;
+        act[r] = on && t < nI;
+        xi[r] = pd[li.x + (act[r] ? t : 0)];
+        ck[r] = cs[li.x + (act[r] ? t : 0)];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g[r][i] = 0.0;
+    }
+    cull_box64<R>(xi, act, bx.r_c, bx.L, box);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (!act[r]) xi[r].x = 1e150;  // beyond the cutoff of every source
+    long long e0, re;
+    row_part(a, I, split, e0, re);
+    while (e0 < re) {
+        int nst;
+        e0 += stage64<4, true>(a, e0, re, bx.L, kStageAdj64, stage, meta, box, nst);
+        if (on)
+            for (int k = s; k < nst; k += S) {
+                const double2 A = stage[4 * k], B = stage[4 * k + 1];
+                const double2 C = stage[4 * k + 2], D = stage[4 * k + 3];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double dx = A.x - xi[r].x, dy = A.y - xi[r].y, dz = B.x - xi[r].z;
+                    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                    if (inside64(r2, rc2m1)) {
+                        const double ri = rsqrt64(r2), ri2 = ri * ri;
+                        double f;
+                        const int kk = 6 * node64(r2 * ri, us, a.t64_max, f);
+                        const double gg = horner64<5>(tab + kk, f) * (ri2 * ri);  // T / r^3
+                        const double Q = cq * horner64<5>(tabq + kk, f);
+                        const double hf = -ri2 * fma(3.0, gg, Q);  // g'(r)/r
+                        // v = m_k c_j - m_j c_k (one mass: c_j - c_k, m applied at the end)
+                        const double vx = EQM ? C.x - ck[r].x : fma(xi[r].w, C.x, -B.y * ck[r].x);
+                        const double vy = EQM ? C.y - ck[r].y : fma(xi[r].w, C.y, -B.y * ck[r].y);
+                        const double vz = EQM ? D.x - ck[r].z : fma(xi[r].w, D.x, -B.y * ck[r].z);
+                        const double hd = hf * fma(dx, vx, fma(dy, vy, dz * vz));
+                        g[r][0] = fma(gg, vx, fma(hd, dx, g[r][0]));
+                        g[r][1] = fma(gg, vy, fma(hd, dy, g[r][1]));
+                        g[r][2] = fma(gg, vz, fma(hd, dz, g[r][2]));
+                        g[r][3] = fma(gg, fma(dx, C.x, fma(dy, C.y, dz * D.x)), g[r][3]);
+                    }
+                }
+            }
+        __syncwarp();
+    }
+    const double G = bx.G, gx = EQM ? G * pd[li.x].w : G;
+    finish64<4, R>(a, li, g, act, lane, s, S, T, stage, split, warp64_bytes(4, kStageAdj64),
+                   [&](int target, const double* v) {
+                       const int idx = a.perm[target];
+                       double* o = reinterpret_cast<double*>(a.out) + 3LL * idx;
+                       o[0] = gx * v[0];
+                       o[1] = gx * v[1];
+                       o[2] = gx * v[2];
+                       if (a.out_m) reinterpret_cast<double*>(a.out_m)[idx] = -G * v[3];
+                   });
+}
+
+template <bool EQM>
+__global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem64[];
+    __shared__ int s_it[8];
+    double* tab = reinterpret_cast<double*>(smem64);
+    const int words = 6 * (a.t64_max + 1);
+    double* tabq = tab + words;
+    for (int i = threadIdx.x; i < words; i += blockDim.x) {
+        tab[i] = reinterpret_cast<const double*>(a.table)[i];
+        tabq[i] = reinterpret_cast<const double*>(a.table)[6 * (kPlain64MaxN + 2) + i];
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    unsigned char* warp = smem64 + 16 * words + (threadIdx.x >> 5) * warp64_bytes(4, kStageAdj64);
+    double2* stage = reinterpret_cast<double2*>(warp);
+    int2* meta = reinterpret_cast<int2*>(warp + 64 * kStageAdj64);
+    const int n_heavy = a.group <= 1 ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    bool split = n_heavy > 0;
+    int it;
+    while (next_item<true>(a, a.ctrl + kCtrlTicketAdj, split, n_heavy, s_it, it)) {
+        int I;
+        int4 li;
+        if (!item64(a, it, lane, I, li)) continue;
+        const int R = targets_per_lane(li.y, 128);
+        if (R == 1) adj64_item<EQM, 1>(a, I, li, tab, tabq, stage, meta, split);
+        else if (R == 2) adj64_item<EQM, 2>(a, I, li, tab, tabq, stage, meta, split);
+        else adj64_item<EQM, 3>(a, I, li, tab, tabq, stage, meta, split);
+    }
+    persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
+}
+
+size_t adj_f64_smem(double x_c, int warps)
+{
+    return (size_t)(plain64(x_c).n + 2) * 96 + (size_t)warps * warp64_bytes(4, kStageAdj64);
+}
+
+int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)
+{
+    FwdArgs a = args;
+    cudaStream_t st = (cudaStream_t)stream;
+    gather_cot_kernel<double, double4><<<(unsigned)((a.n + 255) / 256), 256, 0, st>>>(
+        reinterpret_cast<const double*>(a.cot), a.perm, reinterpret_cast<double4*>(a.cot_sorted), a.n);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return (int)e;
+    const Plain64 p = plain64(x_c);
+    a.t64_max = p.n + 1;
+    a.t64_scale = p.n / p.x_top;
+    const size_t smem = adj_f64_smem(x_c, a.warps_per_block);
+    auto k = a.equal_mass ? p2p_adj_f64_kernel<true> : p2p_adj_f64_kernel<false>;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return (int)e;
+    k<<<a.blocks, a.warps_per_block * 32, smem, st>>>(a);
+    return (int)cudaGetLastError();
+}
+
+int adj_f64_occupancy(int warps, double x_c, int* out)
+{
+    const size_t smem = adj_f64_smem(x_c, warps);
+    cudaError_t e = cudaFuncSetAttribute(p2p_adj_f64_kernel<false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return (int)e;
+    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, p2p_adj_f64_kernel<false>, warps * 32, smem);
+}
+
+}  // namespace psr

@@ -1,216 +1,182 @@
 // FP64 forward P2P kernel: the plain double-precision path (paper, Section 2
-// pair force with Eq. tr evaluated by erfc/exp, Section 3.2 kernel layout),
-// or, with a Taylor interpolation level, the paper's double-precision table
-// path (Section 3.3: the Eq. int expansion about the nearest of N + 1 nodes,
-// level T_[4] for double precision) with the table in shared memory and
-// 1/r from an FP32 estimate refined by two Newton-Raphson steps in FP64.
-// Same work decomposition as the FP32 kernels (warp per target leaf, S
-// streams of T lanes, persistent ticket); coordinates are the wrapped FP64
-// positions and each leaf pair adds its periodic image n L exactly as the
-// definition d = x_j + n L - x_i reads.
+// pair force, Eq. tr), or, with a Taylor interpolation level, the paper's
+// double-precision table path (Section 3.3: the Eq. int expansion about the
+// nearest of N + 1 nodes, level T_[4] for double precision).  Both evaluate T
+// from a table in shared memory; the plain path's has nodes close enough that
+// T is exact to rounding.  p2p_f64_common.cuh says what bounds the kernel and
+// what it does about it.  48^3 NFW set: 255 ms with erfc, exp, a square root and
+// a division per tile pair and one warp per leaf.
 #include <cuda_runtime.h>
 
-#include "kcommon.cuh"
+#include "p2p_f64_common.cuh"
 
 namespace psr {
 
-// Taylor table in FP64: node k = 0..N, x_k = k h, h = x_c / N; six doubles
-// per node, the Eq. int coefficients of eps^m (eps = x - x_k) times h^m, so
-// that the expansion is a polynomial in f = x/h - k (zero above the level).
-__global__ void table64_kernel(int N, int level, double x_c, double* __restrict__ t)
+constexpr int kStage64 = 128;  // staged sources per warp
+
+// Taylor tables in FP64: node k = 0..N, x_k = k h, six doubles per node, the
+// coefficients of eps^m (eps = x - x_k) times h^m, so that the expansion is a
+// polynomial in f = x/h - k (zero above the level).  T's are those of Eq. int and
+// the next, from T' = x^2 E, E = -4 exp(-x^2) / sqrt(pi); Q = exp(-x^2) likewise
+// (levels: 2 or 4 as Eq. int's, 5).  Entry N + 1, written at level 5, is zero.
+__global__ void table64_kernel(int N, int level, double h, double* __restrict__ t, double* __restrict__ q)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > N) return;
-    const double h = x_c / N, x = k * h, x2 = x * x;
-    const double E = -2.0 * 1.1283791670955126 * exp(-x2);  // -4 exp(-x^2) / sqrt(pi)
+    if (k > N + (level == 5 ? 1 : 0)) return;
     double* c = t + 6 * (int64_t)k;
-    c[0] = erfc(x) - 0.5 * x * E;
-    c[1] = x2 * E * h;
-    c[2] = -x * (x2 - 1.0) * E * h * h;
-    c[3] = level >= 4 ? (2.0 / 3.0 * x2 * x2 - 5.0 / 3.0 * x2 + 1.0 / 3.0) * E * h * h * h : 0.0;
-    c[4] = level >= 4 ? -x * (x2 * x2 / 3.0 - 1.5 * x2 + 1.0) * E * h * h * h * h : 0.0;
-    c[5] = 0.0;
+    const double x = k * h, x2 = x * x, Q = exp(-x2);
+    const double E = -2.0 * 1.1283791670955126 * Q;  // -4 exp(-x^2) / sqrt(pi)
+    const double h2 = h * h, h3 = h2 * h, h4 = h2 * h2, h5 = h4 * h;
+    const double on = k <= N ? 1.0 : 0.0, four = level >= 4 ? on : 0.0, five = level >= 5 ? on : 0.0;
+    c[0] = on * (erfc(x) - 0.5 * x * E);
+    c[1] = on * (x2 * E * h);
+    c[2] = on * (-x * (x2 - 1.0) * E * h2);
+    c[3] = four * ((2.0 / 3.0 * x2 * x2 - 5.0 / 3.0 * x2 + 1.0 / 3.0) * E * h3);
+    c[4] = four * (-x * (x2 * x2 / 3.0 - 1.5 * x2 + 1.0) * E * h4);
+    c[5] = five * (((2.0 / 15.0 * x2 - 14.0 / 15.0) * x2 + 1.3) * x2 - 0.2) * E * h5;
+    if (!q) return;
+    c = q + 6 * (int64_t)k;
+    c[0] = on * Q;
+    c[1] = on * (-2.0 * x * Q * h);
+    c[2] = on * ((2.0 * x2 - 1.0) * Q * h2);
+    c[3] = on * (x * (2.0 - 4.0 / 3.0 * x2) * Q * h3);
+    c[4] = on * (((2.0 / 3.0 * x2 - 2.0) * x2 + 0.5) * Q * h4);
+    c[5] = on * (x * ((-4.0 / 15.0 * x2 + 4.0 / 3.0) * x2 - 1.0) * Q * h5);
 }
 
 int launch_table64(int table_n, int interp, double x_c, void* d_out, void* stream)
 {
-    const int threads = 256, blocks = (table_n + 1 + threads - 1) / threads;
+    const int threads = 128, blocks = (table_n + 1 + threads - 1) / threads;
     table64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
-        table_n, interp == PSR_TAYLOR4 ? 4 : 2, x_c, reinterpret_cast<double*>(d_out));
+        table_n, interp == PSR_TAYLOR4 ? 4 : 2, x_c / table_n, reinterpret_cast<double*>(d_out), nullptr);
     return (int)cudaGetLastError();
 }
 
-// 1/sqrt(r2) for r2 > 0: an FP32 estimate (FP64 rsqrt where r2 leaves the
-// FP32 normal range) refined by two Newton-Raphson steps for 1/sqrt,
-// y <- y (3 - r2 y^2) / 2, each of which squares the relative error.
-__device__ __forceinline__ double rsqrt_nr(double r2)
+Plain64 plain64(double x_c)
 {
-    const float f = (float)r2;
-    double y = (f > 1e-36f && f < 1e36f) ? (double)rsqrtf(f) : rsqrt(r2);
-    y = y * fma(-0.5 * r2, y * y, 1.5);
-    y = y * fma(-0.5 * r2, y * y, 1.5);
-    return y;
+    Plain64 p;
+    // T(12) is below 1e-61: beyond, the zero entry
+    p.x_top = x_c < 12.0 ? x_c : 12.0;
+    const double want = std::ceil(p.x_top / 0.0044);
+    p.n = want < 16.0 ? 16 : want > kPlain64MaxN ? kPlain64MaxN : (int)want;
+    return p;
 }
 
-template <bool COUNT, int R, bool TAYLOR>
+int launch_plain64(double x_c, void* d_t, void* d_q, void* stream)
+{
+    const Plain64 p = plain64(x_c);
+    const int threads = 128, blocks = (p.n + 2 + threads - 1) / threads;
+    table64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
+        p.n, 5, p.x_top / p.n, reinterpret_cast<double*>(d_t), reinterpret_cast<double*>(d_q));
+    return (int)cudaGetLastError();
+}
+
+// One target leaf (or, with split, this warp's part of its row).  EQM: every
+// particle of the box has one mass, applied once per target.  COUNT: pairs
+// within the cutoff and pairs evaluated are counted, over every tile pair (no
+// cull).
+template <bool COUNT, bool EQM, int DEG, int R>
 __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, const double* tab,
-                                           unsigned long long& npairs, unsigned long long& nev)
+                                           double2* __restrict__ stage, int2* __restrict__ meta,
+                                           unsigned long long& npairs, unsigned long long& nev, bool split)
 {
     const int lane = threadIdx.x & 31;
     const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
-    const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
-    const int nI = li.y;
-    const int lgT = (R == 2) ? 5 : stream_log2(nI);
-    const int q = lane & ((1 << lgT) - 1);
-    const int s = lane >> lgT;
-    const int S = 32 >> lgT;
+    double* box = reinterpret_cast<double*>(meta + 32);
+    const int nI = li.y, T = (nI + R - 1) / R, S = 32 / T, s = lane / T, q = lane - s * T;
+    const bool on = s < S;
     const BoxDev& bx = a.boxes[li.z];
-    const double L = bx.L, rc2 = bx.rc2, inv2rs = bx.inv_2rs;
-    const double c2 = 1.1283791670955126;  // 2 / sqrt(pi)
-    const double nmax = (double)a.table_n;
-    const double uscale = nmax / bx.r_c;  // r -> x N / x_c (table units), in FP64
+    const long long rc2m1 = bits64(bx.rc2) - 1;
+    const double us = DEG == 5 ? bx.inv_2rs * a.t64_scale : (double)a.table_n / bx.r_c;
+    const int kmax = a.t64_max;
 
     double4 xi[R];
     bool act[R];
-    double ax[R], ay[R], az[R], tx[R], ty[R], tz[R];
+    double acc[R][3];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        int t = q + 32 * r;
-        act[r] = t < nI;
+        const int t = q + T * r;
+        act[r] = on && t < nI;
         xi[r] = pd[li.x + (act[r] ? t : 0)];
-        ax[r] = ay[r] = az[r] = 0.0;
-        tx[r] = ty[r] = tz[r] = 0.0;
+        acc[r][0] = acc[r][1] = acc[r][2] = 0.0;
     }
-    unsigned cnt = 0;
-    const long long re = a.rowptr[I + 1];
-    long long e = a.rowptr[I] + s;
-    int j = 0, jend = 0;
-    for (;;) {
-        if (j >= jend) {
-            bool found = false;
-            while (e < re) {
-                unsigned ent = a.pairs[e];
-                e += S;
-                int J = (int)(ent >> 5);
-                unsigned code = ent & 31u;
-                if (J >= a.n_leaves || code >= (unsigned)kShiftCodes) {
-                    set_error(a.ctrl, J >= a.n_leaves ? kErrLeafIndex : kErrShiftCode);
-                    continue;
-                }
-                int4 lj = leaf[J];
-                if (lj.x < 0 || lj.y < 0 || (long long)lj.x + lj.y > a.n) {
-                    set_error(a.ctrl, kErrParticleRange);
-                    continue;
-                }
-                int nx, ny, nz;
-                decode_shift(code, nx, ny, nz);
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    tx[r] = xi[r].x - nx * L;
-                    ty[r] = xi[r].y - ny * L;
-                    tz[r] = xi[r].z - nz * L;
-                }
-                j = lj.x;
-                jend = lj.x + lj.y;
-                found = true;
-                break;
-            }
-            if (!found) break;
-        }
-        const double4 p = pd[j];
-        ++j;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            double dx = p.x - tx[r], dy = p.y - ty[r], dz = p.z - tz[r];
-            double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < rc2 && r2 > 0.0) {
-                double w;
-                if (TAYLOR) {
-                    const double ri = rsqrt_nr(r2);
-                    const double u = r2 * ri * uscale;
-                    const double kf = fmin(rint(u), nmax);
-                    const double f = u - kf;
-                    const double* c = tab + 6 * (int)kf;
-                    const double T = fma(f, fma(f, fma(f, fma(f, c[4], c[3]), c[2]), c[1]), c[0]);
-                    w = p.w * T * ri * ri * ri;
-                } else {
-                    double rr = sqrt(r2);
-                    double x = rr * inv2rs;
-                    double T = erfc(x) + c2 * x * exp(-x * x);
-                    w = p.w * T / (r2 * rr);
-                }
-                ax[r] += w * dx;
-                ay[r] += w * dy;
-                az[r] += w * dz;
-                if (COUNT) cnt += act[r];
-            }
-            if (COUNT) nev += act[r];
-        }
-    }
+    if (!COUNT) cull_box64<R>(xi, act, bx.r_c, bx.L, box);
 #pragma unroll
     for (int r = 0; r < R; ++r)
-        for (int off = 1 << lgT; off < 32; off <<= 1) {
-            ax[r] += __shfl_xor_sync(kFull, ax[r], off);
-            ay[r] += __shfl_xor_sync(kFull, ay[r], off);
-            az[r] += __shfl_xor_sync(kFull, az[r], off);
-        }
-    if (COUNT) npairs += cnt;
-    if (s == 0) {
+        if (!act[r]) xi[r].x = 1e150;  // beyond the cutoff of every source
+    unsigned cnt = 0;
+    long long e0, re;
+    row_part(a, I, split, e0, re);
+    while (e0 < re) {
+        int nst;
+        e0 += stage64<2, !COUNT>(a, e0, re, bx.L, kStage64, stage, meta, box, nst);
+        if (COUNT && lane == 0) nev += (unsigned long long)nst * (unsigned)nI;
+        if (on)
+            for (int k = s; k < nst; k += S) {
+                const double2 A = stage[2 * k], B = stage[2 * k + 1];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (!act[r]) continue;
-            int idx = a.perm[li.x + q + 32 * r];
-            double* out = reinterpret_cast<double*>(a.out) + 3LL * idx;
-            out[0] = bx.G * ax[r];
-            out[1] = bx.G * ay[r];
-            out[2] = bx.G * az[r];
-        }
+                for (int r = 0; r < R; ++r) {
+                    const double dx = A.x - xi[r].x, dy = A.y - xi[r].y, dz = B.x - xi[r].z;
+                    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                    if (inside64(r2, rc2m1)) {
+                        const double ri = rsqrt64(r2);
+                        double f;
+                        const int kk = node64(r2 * ri, us, kmax, f);
+                        const double Tv = horner64<DEG>(tab + 6 * kk, f);
+                        double w = ri * ri * ri * Tv;
+                        if (!EQM) w *= B.y;
+                        acc[r][0] = fma(w, dx, acc[r][0]);
+                        acc[r][1] = fma(w, dy, acc[r][1]);
+                        acc[r][2] = fma(w, dz, acc[r][2]);
+                        if (COUNT) ++cnt;
+                    }
+                }
+            }
+        __syncwarp();
     }
+    if (COUNT) npairs += cnt;
+    const double g = EQM ? bx.G * pd[li.x].w : bx.G;
+    finish64<3, R>(a, li, acc, act, lane, s, S, T, stage, split, warp64_bytes(2, kStage64),
+                   [&](int target, const double* v) {
+                       double* out = reinterpret_cast<double*>(a.out) + 3LL * a.perm[target];
+                       out[0] = g * v[0];
+                       out[1] = g * v[1];
+                       out[2] = g * v[2];
+                   });
 }
 
-template <bool COUNT, bool WIDE, bool TAYLOR>
-__global__ void __launch_bounds__(256) p2p_fwd_f64_kernel(const FwdArgs a)
+// DEG 5: the plain path, 4: the Taylor levels.
+template <bool COUNT, bool EQM, int DEG>
+__global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem64[];
-    const double* tab = reinterpret_cast<const double*>(smem64);
-    if (TAYLOR) {
-        const double* g = reinterpret_cast<const double*>(a.table);
-        for (int i = threadIdx.x; i < 6 * (a.table_n + 1); i += blockDim.x)
-            reinterpret_cast<double*>(smem64)[i] = g[i];
-        __syncthreads();
-    }
+    __shared__ int s_it[8];
+    double* tab = reinterpret_cast<double*>(smem64);
+    const int words = 6 * (a.t64_max + 1);
+    for (int i = threadIdx.x; i < words; i += blockDim.x) tab[i] = reinterpret_cast<const double*>(a.table)[i];
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
+    unsigned char* warp = smem64 + 8 * words + (threadIdx.x >> 5) * warp64_bytes(2, kStage64);
+    double2* stage = reinterpret_cast<double2*>(warp);
+    int2* meta = reinterpret_cast<int2*>(warp + 32 * kStage64);
     unsigned long long npairs = 0, nev = 0;
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = (int)atomicAdd(a.ctrl + kCtrlTicketFwd, 1u) * a.item_stride + a.item_offset;
-        it = __shfl_sync(kFull, it, 0);
-        if (it >= a.n_items) break;
-        int I = a.items[it];
-        if (I < 0 || I >= a.n_leaves) {
-            if (lane == 0) set_error(a.ctrl, kErrItemIndex);
-            continue;
-        }
-        int4 li = leaf[I];
-        if (li.y <= 0 || li.y > a.max_leaf || (long long)li.x + li.y > a.n || li.z < 0 ||
-            li.z >= a.nbox) {
-            if (lane == 0) set_error(a.ctrl, kErrParticleRange);
-            continue;
-        }
-        if (WIDE && li.y > 32)
-            fwd64_item<COUNT, 2, TAYLOR>(a, I, li, tab, npairs, nev);
-        else
-            fwd64_item<COUNT, 1, TAYLOR>(a, I, li, tab, npairs, nev);
+    const int n_heavy = a.group <= 1 ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    bool split = n_heavy > 0;
+    int it;
+    while (next_item<true>(a, a.ctrl + kCtrlTicketFwd, split, n_heavy, s_it, it)) {
+        int I;
+        int4 li;
+        if (!item64(a, it, lane, I, li)) continue;
+        const int R = targets_per_lane(li.y, 128);
+        if (R == 1) fwd64_item<COUNT, EQM, DEG, 1>(a, I, li, tab, stage, meta, npairs, nev, split);
+        else if (R == 2) fwd64_item<COUNT, EQM, DEG, 2>(a, I, li, tab, stage, meta, npairs, nev, split);
+        else fwd64_item<COUNT, EQM, DEG, 3>(a, I, li, tab, stage, meta, npairs, nev, split);
     }
     if (COUNT) {
-        for (int off = 16; off > 0; off >>= 1) {
-            npairs += __shfl_xor_sync(kFull, npairs, off);
-            nev += __shfl_xor_sync(kFull, nev, off);
-        }
+        for (int off = 16; off > 0; off >>= 1) npairs += __shfl_xor_sync(kFull, npairs, off);
         if (lane == 0 && npairs)
             atomicAdd(reinterpret_cast<unsigned long long*>(a.ctrl + kCtrlPairsLo), npairs);
-        if (lane == 0 && nev)
+        if (lane == 0 && nev)  // lane 0 alone counted the warp's staged pairs
             atomicAdd(reinterpret_cast<unsigned long long*>(a.ctrl + kCtrlEvalLo), nev);
     }
     persistent_exit(a.ctrl + kCtrlTicketFwd, a.ctrl + kCtrlDoneFwd);
@@ -220,54 +186,44 @@ namespace {
 
 bool taylor64(int interp) { return interp == PSR_TAYLOR2 || interp == PSR_TAYLOR4; }
 
-template <bool COUNT, bool WIDE, bool TAYLOR>
-int launch64(const FwdArgs& a, size_t smem, cudaStream_t st)
+template <int DEG>
+const void* pick64(bool count, bool eqm)
 {
-    auto k = p2p_fwd_f64_kernel<COUNT, WIDE, TAYLOR>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return (int)e;
-    }
-    k<<<a.blocks, a.warps_per_block * 32, smem, st>>>(a);
-    return (int)cudaGetLastError();
-}
-
-template <bool TAYLOR>
-const void* ptr64(bool wide)
-{
-    return wide ? (const void*)p2p_fwd_f64_kernel<false, true, TAYLOR>
-                : (const void*)p2p_fwd_f64_kernel<false, false, TAYLOR>;
+    return count ? (const void*)p2p_fwd_f64_kernel<true, false, DEG>
+           : eqm ? (const void*)p2p_fwd_f64_kernel<false, true, DEG>
+                 : (const void*)p2p_fwd_f64_kernel<false, false, DEG>;
 }
 
 }  // namespace
 
-size_t fwd_f64_smem(int interp, int table_n)
+size_t fwd_f64_smem(int interp, int table_n, double x_c, int warps)
 {
-    return taylor64(interp) ? (size_t)(table_n + 1) * 48 : 0;
+    const int entries = taylor64(interp) ? table_n + 1 : plain64(x_c).n + 2;
+    return (size_t)entries * 48 + (size_t)warps * warp64_bytes(2, kStage64);
 }
 
-int launch_fwd_f64(const FwdArgs& a, void* stream)
+int launch_fwd_f64(const FwdArgs& args, double x_c, void* stream)
 {
-    cudaStream_t st = (cudaStream_t)stream;
-    const bool wide = a.max_leaf > 32, tay = taylor64(a.interp);
-    const size_t smem = fwd_f64_smem(a.interp, a.table_n);
-    if (tay) {
-        if (a.count_pairs) return wide ? launch64<true, true, true>(a, smem, st) : launch64<true, false, true>(a, smem, st);
-        return wide ? launch64<false, true, true>(a, smem, st) : launch64<false, false, true>(a, smem, st);
-    }
-    if (a.count_pairs) return wide ? launch64<true, true, false>(a, 0, st) : launch64<true, false, false>(a, 0, st);
-    return wide ? launch64<false, true, false>(a, 0, st) : launch64<false, false, false>(a, 0, st);
+    FwdArgs a = args;
+    const bool tay = taylor64(a.interp);
+    const Plain64 p = plain64(x_c);
+    a.t64_max = tay ? a.table_n : p.n + 1;
+    a.t64_scale = p.n / p.x_top;
+    const size_t smem = fwd_f64_smem(a.interp, a.table_n, x_c, a.warps_per_block);
+    const void* k = tay ? pick64<4>(a.count_pairs, a.equal_mass) : pick64<5>(a.count_pairs, a.equal_mass);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return (int)e;
+    void* params[] = {&a};
+    return (int)cudaLaunchKernel(k, dim3(a.blocks), dim3(a.warps_per_block * 32), params, smem,
+                                 (cudaStream_t)stream);
 }
 
-int fwd_f64_occupancy(int warps, int max_leaf, int interp, int table_n, int* out)
+int fwd_f64_occupancy(int warps, int interp, int table_n, double x_c, int* out)
 {
-    const bool wide = max_leaf > 32, tay = taylor64(interp);
-    const void* f = tay ? ptr64<true>(wide) : ptr64<false>(wide);
-    const size_t smem = fwd_f64_smem(interp, table_n);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return (int)e;
-    }
+    const void* f = taylor64(interp) ? pick64<4>(false, false) : pick64<5>(false, false);
+    const size_t smem = fwd_f64_smem(interp, table_n, x_c, warps);
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, f, warps * 32, smem);
 }
 

@@ -52,6 +52,7 @@ struct Layout {
     size_t boxes;    // BoxDev[nbox]
     size_t table;    // float4[2 * (kMaxTableN + 1)]: T table, then exp(-x^2)
     size_t core;     // float2[kMaxTableN + 1]: core form of the forward's linear table
+    size_t t64;      // double[2][6 (kPlain64MaxN + 2)]: FP64 plain path's T and exp(-x^2) tables
     size_t cotf;     // float4[n] / double4[n] adjoint source payload scratch
     size_t ctrl;     // uint32[64]  scheduler tickets, error word, counters
     // multipole split (device builds with an acceptance parameter only)
@@ -128,6 +129,7 @@ struct Leaves {
     bool uploaded = false;
     int table_key = -1;       // cached forward table (n, interp) encoding
     double table_xc = -1.0;
+    double t64_xc = -1.0;     // the FP64 plain path's tables' x_c
     int core_key = -1;        // the core table's intervals and x_c
     double core_xc = -1.0;
     int adj_table_key = -1;
@@ -218,6 +220,8 @@ struct FwdArgs {
     int stage_cap;   // FP32 kernels: staged particles per warp
     int item_stride; // this launch takes schedule entries ticket * stride + offset
     int item_offset;
+    int t64_max;       // FP64 kernels: last entry of the Taylor table
+    double t64_scale;  //   and its nodes per unit of x (plain path)
     const int* heavy;  // how many items groups of warps take (null: all)
     int group;         // warps per group (divides warps_per_block); 0 or 1: none
     int core;        // FP32 forward: a.table is the core form of the linear table
@@ -228,20 +232,31 @@ int launch_table(int table_n, int interp, double x_c, void* d_out, void* d_q_out
 int launch_core_table(int table_n, double x_c, void* d_out, void* stream);
 bool fwd_core(int precision, int interp, int table_n, int variant, double x_c);
 int launch_fwd_f32(const FwdArgs& a, int precision, void* stream);
-int launch_fwd_f64(const FwdArgs& a, void* stream);
+int launch_fwd_f64(const FwdArgs& a, double x_c, void* stream);
 int launch_adj_f32(const FwdArgs& a, int precision, void* stream);
-int launch_adj_f64(const FwdArgs& a, void* stream);
+int launch_adj_f64(const FwdArgs& a, double x_c, void* stream);
 int fwd_f32_occupancy(int precision, int interp, int accum, int warps, int table_n, int cap,
                       int variant, int core, int* out);
 size_t fwd_f32_smem(int precision, int interp, int table_n, int warps, int cap);
 constexpr size_t kSmemPerBlock = 227 * 1024;  // opt-in dynamic shared memory per block
-int fwd_f64_occupancy(int warps, int max_leaf, int interp, int table_n, int* out);
+int fwd_f64_occupancy(int warps, int interp, int table_n, double x_c, int* out);
 int launch_table64(int table_n, int interp, double x_c, void* d_out, void* stream);  // p2p_fwd_f64.cu
-size_t fwd_f64_smem(int interp, int table_n);
+size_t fwd_f64_smem(int interp, int table_n, double x_c, int warps);
+// Taylor nodes of the FP64 plain path: 0.0044 apart in x up to x = 6, n of them
+// over [0, x_top] beyond (the allocation-free entry point's scratch holds 1363)
+constexpr int kPlain64MaxN = 1363;
+struct Plain64 {
+    int n;
+    double x_top;
+};
+Plain64 plain64(double x_c);
+int launch_plain64(double x_c, void* d_t, void* d_q, void* stream);
+int adj_f64_occupancy(int warps, double x_c, int* out);
+size_t adj_f64_smem(double x_c, int warps);
 int launch_fwd_blk(const FwdArgs& a, int precision, void* stream);  // p2p_fwd_blk.cu
 int fwd_blk_occupancy(int precision, int interp, int accum, int max_leaf, int table_n, int* out);
-int adj_occupancy(int precision, int interp, int accum, int warps, int max_leaf, int table_n,
-                  int cap, int variant, int* out);
+int adj_f32_occupancy(int precision, int interp, int accum, int warps, int max_leaf, int table_n,
+                      int cap, int variant, int* out);
 size_t adj_f32_smem(int precision, int interp, int table_n, int warps, int cap);
 
 }  // namespace psr

@@ -1,0 +1,59 @@
+"""The FP64 kernels' T and exp(-x^2) tables, cull, lane filling and shared rows, over cutoffs from
+x_c = 0.3 to beyond the tables' end (x = 12), leaf sizes and both mass forms.
+
+Tolerance: every factor of a pair is exact to a few FP64 roundings (2^-53 each, the tables' left-out
+term below 1e-16), and a target sums some hundred terms: 1e-13 relative RMS (a wrong node,
+coefficient, image or target is orders above that)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2107_14008_gb300 as psr
+
+pytestmark = pytest.mark.gpu
+
+
+def _rms(a, b):
+    return float(np.sqrt(((a - b) ** 2).sum() / (b ** 2).sum()))
+
+
+@pytest.mark.parametrize("x_c", [0.3, 2.25, 5.99, 6.01, 9.0, 14.0])
+@pytest.mark.parametrize("max_leaf,n", [(1, 90), (7, 700), (32, 1500), (64, 1500)])
+@pytest.mark.parametrize("equal", [True, False])
+def test_fp64_matches_oracle(x_c, max_leaf, n, equal):
+    rng = np.random.default_rng(5)
+    L, r_c = 30.0, 13.0
+    r_s = r_c / (2.0 * x_c)
+    pos = rng.random((n, 3)) * L
+    pos[: n // 4] = 29.0 + 1.5 * rng.standard_normal((n // 4, 3))  # a clump across the box's corner
+    pos = np.mod(pos, L)
+    pos[n // 2] = pos[n // 2 + 1]  # a coincident pair
+    mass = np.full(n, 1.0 / n) if equal else rng.uniform(0.2, 2.0, n) / n
+    cot = rng.standard_normal((n, 3))
+    lv = psr.Leaves.build(pos, mass, L, r_s, r_c, max_leaf=max_leaf).upload()
+    o = psr.Options(precision=psr.PSR_FP64)
+    acc = lv.forces(o)
+    gx, gm = (g.cpu().numpy() for g in lv.adjoint(torch.tensor(cot), o))
+    part = torch.zeros_like(acc)
+    for k in range(2):
+        lv.forces(psr.Options(precision=psr.PSR_FP64, shard_count=2, shard_index=k), out=part)
+    assert torch.equal(acc, part)
+    lv.check()
+    ref = oracle.forces(pos, mass, L, r_s, r_c, 1.0)
+    ref = ref[0] if isinstance(ref, tuple) else ref
+    ox, om = oracle.adjoint(pos, mass, cot, L, r_s, r_c, 1.0)[:2]
+    assert _rms(acc.cpu().numpy(), ref) < 1e-13
+    assert _rms(gx, ox) < 1e-13 and _rms(gm, om) < 1e-13
+
+
+@pytest.mark.parametrize("f", [1e-6, 0.01, 0.5, 1 - 1e-15, 1.0, 1 + 1e-15])
+def test_fp64_pair_and_strict_cutoff(f):
+    L, r_c, r_s = 64.0, 8.0, 2.0
+    pos = np.array([[16.0, 16.0, 16.0], [16.0 + f * r_c, 16.0, 16.0]])
+    lv = psr.Leaves.build(pos, np.array([0.5, 0.25]), L, r_s, r_c).upload()
+    acc = lv.forces(psr.Options(precision=psr.PSR_FP64)).cpu().numpy()
+    r = pos[1, 0] - pos[0, 0]
+    want = oracle.T(np.array([r / (2 * r_s)]))[0] / r ** 2 if r < r_c else 0.0
+    np.testing.assert_allclose(acc[:, 0], [0.25 * want, -0.5 * want], rtol=2e-15)
+    assert np.all(acc[:, 1:] == 0.0)

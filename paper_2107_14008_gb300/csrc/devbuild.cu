@@ -12,8 +12,7 @@
 //                binary searches inside a window of +-(max_leaf + 1) sorted keys.
 //   4. tree      a binary radix tree over the leaf cell keys (Karras 2012, equal
 //                keys ordered by leaf index) with bottom-up bounding boxes
-//   5. pairs     per target leaf and periodic image, a depth-first traversal that
-//                keeps every leaf whose box comes closer than r_c.  A node's box
+//   5. pairs     per target leaf and periodic image, a traversal that keeps every leaf whose box comes closer than r_c.  A node's box
 //                contains its leaves' boxes, so the kept set is exactly the set of
 //                leaves that pass the leaf test, which the host's octree keeps too;
 //                the left-first order visits them in leaf order like the host's
@@ -32,7 +31,9 @@
 // reads back the sizes; psr_device_build_finish writes the workspace.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -53,7 +54,7 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;  // 4096 values per block
 constexpr int64_t kScanMaxTiles = 65536;              // the top level scans in one block
-constexpr int kStackDepth = 128;                      // tree depth <= 63 key + 27 index bits
+constexpr int kMaxLevels = 7;                         // of the groups: 32^6 > 2^28 leaves
 constexpr int kDefaultTimeoutMs = 60000;
 constexpr int64_t kMaxN = (int64_t)1 << 28;           // scan limit: 65536 tiles of 4096
 
@@ -85,8 +86,8 @@ size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Scratch regions (byte offsets); leaf arrays are sized for n leaves (max_leaf 1).
 struct Scratch {
-    size_t wpos, key0, key1, val0, val1, flag, lid, lfirst, llevel, lkey, lbox, lrec, lcnt,
-        lfar, lout, lcost, tnode, tspan, tparl, tpari, tbox, nodef, tflag, hist, tiles, total, cnt,
+    size_t wpos, key0, key1, val0, val1, flag, lid, lfirst, llevel, lkey, lbox, lcnt,
+        lfar, lout, lcost, lkey2, lfirst2, llevel2, psize, groups, hist, tiles, total, cnt,
         lruns, cache, bytes;
     int64_t ncache;  // pair cache capacity in runs
 };
@@ -111,18 +112,15 @@ Scratch scratch_layout(int64_t n)
     s.llevel = o; o = a256(o + 4 * N);
     s.lkey = o;   o = a256(o + 8 * N);
     s.lbox = o;   o = a256(o + 48 * N);
-    s.lrec = o;   o = a256(o + 32 * N);  // FP32 inward leaf box and count
     s.lcnt = o;   o = a256(o + 8 * N);
     s.lfar = o;   o = a256(o + 8 * N);   // far entries per leaf (multipole split)
-    s.lout = o;   o = a256(o + 32 * N);  // FP32 leaf box rounded outward (multipole split)
+    s.lout = o;   o = a256(o + 32 * N);  // FP32 leaf box rounded outward, count, rho
     s.lcost = o;  o = a256(o + 8 * N);
-    s.tnode = o;  o = a256(o + 8 * N);
-    s.tspan = o;  o = a256(o + 8 * N);   // leaf range [lo, hi] of each internal node
-    s.tparl = o;  o = a256(o + 4 * N);
-    s.tpari = o;  o = a256(o + 4 * N);
-    s.tbox = o;   o = a256(o + 48 * N);
-    s.nodef = o;  o = a256(o + 64 * N);  // internal nodes: children and their FP32 boxes
-    s.tflag = o;  o = a256(o + 4 * N);
+    s.lkey2 = o;  o = a256(o + 8 * N);   // packed leaves, before they take the places of the plain ones
+    s.lfirst2 = o; o = a256(o + 4 * (N + 1));
+    s.llevel2 = o; o = a256(o + 4 * N);
+    s.psize = o;  o = a256(o + 4 * N);
+    s.groups = o; o = a256(o + 32 * (N / 31 + 2 * kMaxLevels));  // boxes of the groups of all levels
     s.hist = o;   o = a256(o + 8 * hist);
     s.tiles = o;  o = a256(o + 8 * ntiles);
     s.total = o;  o = a256(o + 8);
@@ -400,42 +398,49 @@ int radix_sort(uint64_t* k0, int32_t* v0, uint64_t* k1, int32_t* v1, int64_t n, 
 
 // -------------------------------------------------------- keys and leaves --
 
+// Bound: the FP64 pipe (a warp instruction in 16 SM cycles), so a coordinate
+// takes two FP64 instructions: its product with the scale, and floor by adding
+// 2^52 rounded down.  Range checks compare the bits of the doubles; only a
+// coordinate outside [0, L) takes the FP64 wrap.
 __global__ void k_keys(const double* __restrict__ pos, const double* __restrict__ mass, int64_t n,
-                       BoxK bx, double* __restrict__ wpos, uint64_t* __restrict__ key,
+                       BoxK bx, double m_default, double* __restrict__ wpos, uint64_t* __restrict__ key,
                        int32_t* __restrict__ idx, long long* __restrict__ cnt)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    uint64_t q[3];
+    const unsigned long long kInfBits = 0x7ff0000000000000ULL, kAbs = 0x7fffffffffffffffULL;
+    auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x); };
+    uint32_t q[3];
+    double v[4];
     bool bad = false;
     for (int a = 0; a < 3; ++a) {
-        double v = pos[3 * i + a];
-        if (!isfinite(v)) {
+        v[a] = pos[3 * i + a];
+        if ((bits(v[a]) & kAbs) >= kInfBits) {
             bad = true;
-            v = 0.0;
+            v[a] = 0.0;
         }
-        if (!(v >= 0.0 && v < bx.L)) {  // fmod is exact, so values inside [0, L) keep their bits
-            v = fmod(v, bx.L);
-            if (v < 0) v += bx.L;
-            if (!(v < bx.L)) v = 0.0;
+        if (bits(v[a]) >= bits(bx.L)) {  // outside [0, L), or -0.0
+            v[a] = fmod(v[a], bx.L);  // fmod is exact, so values inside keep their bits
+            if (v[a] < 0) v[a] += bx.L;
+            if (!(v[a] < bx.L)) v[a] = 0.0;
         }
-        wpos[4 * i + a] = v;
-        double qq = floor(__dmul_rn(v, bx.scale));
-        if (qq < 0) qq = 0;
-        if (qq > (double)((1u << kMortonBits) - 1)) qq = (double)((1u << kMortonBits) - 1);
-        q[a] = (uint64_t)qq;
+        // floor: the low word of x + 2^52 rounded down (0 <= x <= 2^21)
+        const uint32_t f = (uint32_t)__double2loint(__dadd_rd(__dmul_rn(v[a], bx.scale), 4503599627370496.0));
+        q[a] = min(f, (1u << kMortonBits) - 1u);
     }
-    double m = mass ? mass[i] : 1.0 / (double)n;
-    if (!isfinite(m)) {
+    const double m0 = mass ? mass[0] : m_default;
+    v[3] = mass ? mass[i] : m_default;
+    if ((bits(v[3]) & kAbs) >= kInfBits) {
         bad = true;
-        m = 0.0;
+        v[3] = 0.0;
     }
-    wpos[4 * i + 3] = m;
+    double2* const w = reinterpret_cast<double2*>(wpos + 4 * i);
+    w[0] = make_double2(v[0], v[1]);
+    w[1] = make_double2(v[2], v[3]);
     if (bad) atomicOr((unsigned long long*)(cnt + kCntError), 1ULL);
     // one mass for every particle lets the FP32 kernels apply it once per target
-    const double m0 = mass ? mass[0] : 1.0 / (double)n;
-    if (m != m0) atomicOr((unsigned long long*)(cnt + kCntMassDiff), 1ULL);
-    if (i == 0) cnt[kCntMass0] = __double_as_longlong(m);
+    if (bits(v[3]) != bits(m0) && v[3] != m0) atomicOr((unsigned long long*)(cnt + kCntMassDiff), 1ULL);
+    if (i == 0) cnt[kCntMass0] = __double_as_longlong(v[3]);
     key[i] = (spread3_d(q[0]) << 2) | (spread3_d(q[1]) << 1) | spread3_d(q[2]);
     idx[i] = (int32_t)i;
 }
@@ -574,170 +579,85 @@ __global__ void k_pack_fill(const int64_t* __restrict__ pstart, const int64_t* _
                          // deeper sibling subtree can hold keys above the parent's prefix)
 }
 
+// Boxes of the leaves, 16 lanes per leaf.  Wrapped coordinates are not
+// negative, so doubles compare as the integers of their bits (integer minima
+// and maxima, off the FP64 pipe; -0.0 counts as the smallest, which equals 0).
+// lbox: the FP64 box.  lout, for the walk and the multipole split: the box
+// rounded outward in FP32 (lo down, hi up), the particle count and half the
+// rounded box's diagonal.
 __global__ void k_leaf_box(const int32_t* __restrict__ lfirst, int64_t nl, int64_t n,
                            const double* __restrict__ wpos, const int32_t* __restrict__ idx,
-                           double* __restrict__ lbox, float4* __restrict__ lrec,
-                           float4* __restrict__ lout, long long* __restrict__ cnt)
+                           double* __restrict__ lbox, float4* __restrict__ lout,
+                           long long* __restrict__ cnt)
 {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= nl) return;
-    const int64_t f = lfirst[g], e = g + 1 < nl ? lfirst[g + 1] : n;
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int64_t k = f; k < e; ++k) {
-        const int64_t p = idx[k];
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
+    const int sub = threadIdx.x & 15;
+    const bool live = g < nl;
+    const int64_t f = live ? lfirst[g] : 0, e = !live ? 0 : g + 1 < nl ? lfirst[g + 1] : n;
+    long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
+    for (int64_t k = f + sub; k < e; k += 16) {
+        const double2* w = reinterpret_cast<const double2*>(wpos + 4 * (int64_t)idx[k]);
+        const double2 xy = w[0], zm = w[1];
+        const long long v[3] = {__double_as_longlong(xy.x), __double_as_longlong(xy.y),
+                                __double_as_longlong(zm.x)};
         for (int a = 0; a < 3; ++a) {
-            const double v = wpos[4 * p + a];
-            lo[a] = fmin(lo[a], v);
-            hi[a] = fmax(hi[a], v);
+            lo[a] = min(lo[a], v[a]);
+            hi[a] = max(hi[a], v[a]);
         }
     }
+    for (int o = 8; o > 0; o >>= 1)
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = min(lo[a], __shfl_xor_sync(kFull, lo[a], o));
+            hi[a] = max(hi[a], __shfl_xor_sync(kFull, hi[a], o));
+        }
+    int most = live ? (int)(e - f) : 0;
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(kFull, most, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(cnt + kCntMaxLeaf, (long long)most);
+    if (!live || sub) return;
+    float ol[3], oh[3], r2 = 0.f;
     for (int a = 0; a < 3; ++a) {
-        lbox[6 * g + a] = lo[a];
-        lbox[6 * g + 3 + a] = hi[a];
-    }
-    // walk record: the box rounded inward (lo up, hi down) and the count
-    lrec[2 * g] = make_float4(__double2float_ru(lo[0]), __double2float_ru(lo[1]),
-                              __double2float_ru(lo[2]), __int_as_float((int)(e - f)));
-    lrec[2 * g + 1] = make_float4(__double2float_rd(hi[0]), __double2float_rd(hi[1]),
-                                  __double2float_rd(hi[2]), 0.f);
-    // the box rounded outward (lo down, hi up) and half its diagonal, for
-    // the multipole split
-    const float ol[3] = {__double2float_rd(lo[0]), __double2float_rd(lo[1]),
-                         __double2float_rd(lo[2])};
-    const float oh[3] = {__double2float_ru(hi[0]), __double2float_ru(hi[1]),
-                         __double2float_ru(hi[2])};
-    float r2 = 0.f;
-    for (int a = 0; a < 3; ++a) {
+        const double l = __longlong_as_double(lo[a]), h = __longlong_as_double(hi[a]);
+        lbox[6 * g + a] = l;
+        lbox[6 * g + 3 + a] = h;
+        ol[a] = __double2float_rd(l);
+        oh[a] = __double2float_ru(h);
         const float ea = __fmul_rn(0.5f, __fsub_rn(oh[a], ol[a]));
         r2 = __fmaf_rn(ea, ea, r2);
     }
-    lout[2 * g] = make_float4(ol[0], ol[1], ol[2], 0.f);
+    lout[2 * g] = make_float4(ol[0], ol[1], ol[2], __int_as_float((int)(e - f)));
     lout[2 * g + 1] = make_float4(oh[0], oh[1], oh[2], __fsqrt_rn(r2));
-    atomicMax(cnt + kCntMaxLeaf, (long long)(e - f));
 }
 
-// ------------------------------------------------------------------ tree --
-// Internal node i (0 <= i < nl - 1) of the binary radix tree over the sorted
-// leaf cell keys, node 0 the root.  A child code with bit 31 set is a leaf.
-
-constexpr int kLeafBit = (int)0x80000000u;
-
-__device__ __forceinline__ int delta(const uint64_t* __restrict__ k, int64_t nl, int64_t i, int64_t j)
+// ---------------------------------------------------------------- groups --
+// A 32-ary tree over the leaves in their (Morton) order: a group of a level is
+// 32 consecutive groups of the level below, level 0 the leaves, its box the
+// union of theirs (FP32, rounded outward like them), up to one group.  A warp
+// per group.
+__global__ void k_groups(const float4* __restrict__ below, int64_t n_below, float4* __restrict__ out,
+                         int64_t n_out)
 {
-    if (j < 0 || j >= nl) return -1;
-    const uint64_t a = k[i], b = k[j];
-    if (a == b) return 64 + __clz((unsigned)(i ^ j));
-    return __clzll(a ^ b);
-}
-
-__global__ void k_tree_nodes(const uint64_t* __restrict__ k, int64_t nl, int2* __restrict__ node,
-                             int2* __restrict__ span, int32_t* __restrict__ parl,
-                             int32_t* __restrict__ pari)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nl - 1) return;
-    const int d = delta(k, nl, i, i + 1) > delta(k, nl, i, i - 1) ? 1 : -1;
-    const int dmin = delta(k, nl, i, i - d);
-    int64_t lmax = 2;
-    while (delta(k, nl, i, i + lmax * d) > dmin) lmax *= 2;
-    int64_t l = 0;
-    for (int64_t t = lmax / 2; t >= 1; t /= 2)
-        if (delta(k, nl, i, i + (l + t) * d) > dmin) l += t;
-    const int64_t j = i + l * d;
-    const int dnode = delta(k, nl, i, j);
-    int64_t s = 0, t = l;
-    do {
-        t = (t + 1) >> 1;
-        if (delta(k, nl, i, i + (s + t) * d) > dnode) s += t;
-    } while (t > 1);
-    const int64_t gamma = i + s * d + (d < 0 ? -1 : 0);
-    const int64_t lo = i < j ? i : j, hi = i < j ? j : i;
-    int2 c;
-    if (lo == gamma) {
-        c.x = (int)gamma | kLeafBit;
-        parl[gamma] = (int)i;
-    } else {
-        c.x = (int)gamma;
-        pari[gamma] = (int)i;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (g >= n_out) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t c = 32 * g + lane;
+    float lo[3] = {kInf, kInf, kInf}, hi[3] = {-kInf, -kInf, -kInf};
+    if (c < n_below) {
+        const float4 l = below[2 * c], h = below[2 * c + 1];
+        lo[0] = l.x; lo[1] = l.y; lo[2] = l.z;
+        hi[0] = h.x; hi[1] = h.y; hi[2] = h.z;
     }
-    if (hi == gamma + 1) {
-        c.y = (int)(gamma + 1) | kLeafBit;
-        parl[gamma + 1] = (int)i;
-    } else {
-        c.y = (int)(gamma + 1);
-        pari[gamma + 1] = (int)i;
-    }
-    node[i] = c;
-    span[i] = make_int2((int)lo, (int)hi);
-    if (i == 0) pari[0] = -1;
-}
-
-__device__ __forceinline__ const double* child_box(int c, const double* lbox, const double* tbox)
-{
-    return c < 0 ? lbox + 6 * (int64_t)(c & 0x7fffffff) : tbox + 6 * (int64_t)c;
-}
-
-// Bottom-up boxes: of the two threads that reach a node, the second one
-// (whose sibling subtree is then complete) computes it and moves up.
-__global__ void k_tree_boxes(int64_t nl, const int2* __restrict__ node,
-                             const int32_t* __restrict__ parl, const int32_t* __restrict__ pari,
-                             const double* __restrict__ lbox, double* tbox, int* flags,
-                             long long* cnt)
-{
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= nl) return;
-    int p = parl[g];
-    for (int step = 0; p >= 0; ++step) {
-        if (step > kStackDepth || p >= nl - 1) {
-            atomicOr((unsigned long long*)(cnt + kCntError), 4ULL);
-            return;
-        }
-        __threadfence();
-        if (atomicAdd(&flags[p], 1) == 0) return;
-        __threadfence();
-        const int2 c = node[p];
-        const double* A = child_box(c.x, lbox, tbox);
-        const double* B = child_box(c.y, lbox, tbox);
+    for (int o = 16; o > 0; o >>= 1)
         for (int a = 0; a < 3; ++a) {
-            tbox[6 * (int64_t)p + a] = fmin(__ldcg(A + a), __ldcg(B + a));
-            tbox[6 * (int64_t)p + 3 + a] = fmax(__ldcg(A + 3 + a), __ldcg(B + 3 + a));
+            lo[a] = fminf(lo[a], __shfl_xor_sync(kFull, lo[a], o));
+            hi[a] = fmaxf(hi[a], __shfl_xor_sync(kFull, hi[a], o));
         }
-        p = pari[p];
+    if (lane == 0) {
+        out[2 * g] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        out[2 * g + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
     }
 }
 
 // ----------------------------------------------------------------- pairs --
-// Internal node i packed for the walk (64 bytes): its children's boxes in
-// FP32 rounded outward (lo down, hi up) and their codes:
-//   q[0] = (l.lo.x, l.lo.y, l.lo.z, l.hi.x)   q[1] = (l.hi.y, l.hi.z, r.lo.x, r.lo.y)
-//   q[2] = (r.lo.z, r.hi.x, r.hi.y, r.hi.z)   q[3] = bits(left, right, lo, hi)
-// where [lo, hi] is the node's leaf range: left covers [lo, gamma], right
-// [gamma + 1, hi], gamma = the left child's index (leaf or internal).
-__global__ void k_tree_pack(int64_t nl, const int2* __restrict__ node,
-                            const int2* __restrict__ span, const double* __restrict__ lbox,
-                            const double* __restrict__ tbox, float4* __restrict__ nodef)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nl - 1) return;
-    const int2 c = node[i];
-    const double* A = child_box(c.x, lbox, tbox);
-    const double* B = child_box(c.y, lbox, tbox);
-    float v[12];
-    for (int a = 0; a < 3; ++a) {
-        v[a] = __double2float_rd(A[a]);
-        v[3 + a] = __double2float_ru(A[3 + a]);
-        v[6 + a] = __double2float_rd(B[a]);
-        v[9 + a] = __double2float_ru(B[3 + a]);
-    }
-    float4* q = nodef + 4 * i;
-    q[0] = make_float4(v[0], v[1], v[2], v[3]);
-    q[1] = make_float4(v[4], v[5], v[6], v[7]);
-    q[2] = make_float4(v[8], v[9], v[10], v[11]);
-    const int2 sp = span[i];
-    q[3] = make_float4(__int_as_float(c.x), __int_as_float(c.y), __int_as_float(sp.x),
-                       __int_as_float(sp.y));
-}
-
 // Bounds on the exact gap^2 between a target box A and a box B shifted by
 // sh, in FP32 with every operation rounded toward the bound (shift given
 // rounded down, sd, and up, su).  Lower bound: boxes rounded outward.
@@ -821,184 +741,292 @@ __device__ __forceinline__ bool far_pair(const float* alo, const float* ahi, flo
     return d2 > 0.f && m2 < rc2far && __fmul_rn(theta2, d2) >= r2 && __fmul_rn(r2, d2) <= gt2;
 }
 
-// One thread per target leaf.  WRITE = false counts the row and its work
-// and, given a pair cache of kslot runs per row, records the row's runs there
-// in walk order (lruns[I]: their number, or -1 when the slot is too small);
-// WRITE = true writes the row at rowptr, skipping the rows a given lruns
-// marks as cached (k_pairs_expand writes those).
-// Row order: a warp takes 32 consecutive leaves (neighbours, whose walks
-// share most of their paths), or, with interleave, lane k of warp w takes
-// leaf k W + w (W = ceil(n_leaves / 32)).  When every row fits in one wave of
-// resident warps the launch lasts as long as its slowest warp, a warp of 32
-// leaves of the densest region walking one after another where their paths
-// part; spread over 32 warps those walks run side by side (the bench
-// workload's count walk: 2.79 against 3.02 ms per build).  With more rows
-// than that the launch is bound by the total work, and the neighbours'
-// shared paths win (8-particle leaves: 9.3 against 11.2 ms).  Nodes are pruned when the FP32
-// lower bound of their gap^2 reaches thi (then the host's FP64 test fails
-// for every leaf below); a leaf is kept when the FP32 upper bound is below
-// tlo (then the host's FP64 test passes); only the leaves in between take
-// the host's FP64 test itself.  The walk keeps its current node in a
-// register and stacks a right child only while it descends the left one.
-// Each walk visits at most 2 nl - 1 nodes; more means a malformed tree,
-// reported, never looped on.
-template <bool WRITE>
-__global__ void __launch_bounds__(128, 8) k_pairs(
-    int64_t nl, int64_t n, BoxK bx, const int32_t* __restrict__ lfirst,
-    const double* __restrict__ lbox, const float4* __restrict__ lrec,
-    const float4* __restrict__ nodef, const double* __restrict__ rootbox,
-    int64_t* __restrict__ lcnt, int64_t* __restrict__ lcost, const int64_t* __restrict__ rowptr,
-    uint32_t* __restrict__ pairs, long long* __restrict__ cnt, unsigned* __restrict__ err,
-    int32_t* __restrict__ lruns, uint2* __restrict__ cache, int kslot, int interleave)
+// The rows.  One WARP per target leaf (consecutive leaves on consecutive warps
+// of a persistent grid, whose walks share their loads in L1), which walks the
+// groups in order for each periodic image whose root comes close enough: a step
+// tests the 32 members of a group, one per lane; of the members of a group of
+// groups that survive, those wholly inside are kept as a range and the others
+// are walked in turn; of a group of leaves, the kept ones are a bit mask.  So
+// the row comes out in order, with every lane at work and no stack but one mask
+// per level, which lane t holds for level t.
+//   Bound: issue, about 60 steps of 40 instructions a row.  Against the walks
+// it replaces (one thread per leaf over a binary radix tree): 17^3 uniform 820
+// us, 64^3 NFW 930 us, 128^3 NFW 1.2 ms, split 3.26 + 0.65 ms.
+//
+// A member is pruned when the FP32 lower bound of its gap^2 reaches thi (then
+// the host's FP64 test fails for every leaf below); a leaf is kept when the
+// FP32 upper bound is below tlo (then the host's FP64 test passes; the box
+// rounded outward and moved in by one place bounds the box from inside); only
+// the leaves in between take the host's FP64 test itself.
+//
+// MODE: count (and, given a pair cache of kslot runs per row, record the row's
+// runs: lruns[I] their number, or -1 when the slot is too small), or write a
+// row at rowptr; SPLIT: each kept leaf goes to the near or the far list
+// (far_pair).  The write pass of a split replays a recorded row's runs; the
+// plain one skips recorded rows (k_pairs_expand writes those).
+constexpr int kWalkWarps = 4;
+constexpr int kWalkBlocks = 8;  // per SM
+
+struct WalkArgs {
+    int64_t nl;
+    BoxK bx;
+    int top;                        // the level of one group
+    const float4* box[kMaxLevels];  // boxes of each level (level 0: lout)
+    int64_t n[kMaxLevels];          // and their numbers
+    const int32_t* lfirst;
+    const double* lbox;
+    int64_t *lcnt, *lcost, *lfar;         // count
+    const int64_t *rowptr, *frowptr;      // write
+    uint32_t *pairs, *fpairs;
+    long long* cnt;
+    unsigned* err;
+    int32_t* lruns;
+    uint2* cache;
+    int kslot;
+};
+
+// x >= 0 moved up or down by one place (0 stays 0 going down)
+__device__ __forceinline__ float next_up(float x) { return __int_as_float(max(__float_as_int(x), 0) + 1); }
+__device__ __forceinline__ float next_down(float x) { return __int_as_float(max(__float_as_int(x), 1) - 1); }
+
+template <bool WRITE, bool SPLIT>
+__global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const WalkArgs w)
 {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t W = (nl + 31) >> 5;
-    const int64_t I = !interleave ? t : (t >> 5) < W ? (t & 31) * W + (t >> 5) : nl;
-    if (I >= nl) return;
-    if (WRITE && lruns && lruns[I] >= 0) return;
-    double A[6];
-    float aolo[3], aohi[3], ailo[3], aihi[3], rlo[3], rhi[3];
-    for (int a = 0; a < 3; ++a) {
-        A[a] = lbox[6 * I + a];
-        A[3 + a] = lbox[6 * I + 3 + a];
-        aolo[a] = __double2float_rd(A[a]);
-        aohi[a] = __double2float_ru(A[3 + a]);
-        ailo[a] = __double2float_ru(A[a]);
-        aihi[a] = __double2float_rd(A[3 + a]);
-        rlo[a] = __double2float_rd(rootbox[a]);
-        rhi[a] = __double2float_ru(rootbox[3 + a]);
-    }
-    // stack entries: (node code, -1) or a leaf range (first, last) kept whole
-    int2 stack[kStackDepth];
-    int64_t c = 0, src = 0;
-    int64_t w = WRITE ? rowptr[I] : 0;
-    const int64_t wend = WRITE ? rowptr[I + 1] : 0;
-    bool bad = false;
-    // pair cache state: the open run (first entry word, length) and the runs
-    // stored so far in this row's slot
-    const bool caching = !WRITE && cache != nullptr;
-    bool cok = caching;
-    uint2* const slot = caching ? cache + I * (int64_t)kslot : nullptr;
-    uint32_t run0 = 0, runn = 0;
-    int nrun = 0;
-    // keeps leaves [f, l] of this image
-    auto take = [&](int f, int l, int code) {
-        c += l - f + 1;
-        src += lfirst[l + 1] - lfirst[f];
-        if (WRITE) {
-            if (w + (l - f + 1) > wend) {
-                atomicOr(err, 4u);
-                bad = true;
+    __shared__ long long s_pairs, s_far, s_eval, s_cost, s_row, s_uncached;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int nl = (int)w.nl;
+    const float thi = w.bx.thi, tlo = w.bx.tlo;
+    if (threadIdx.x == 0) s_pairs = s_far = s_eval = s_cost = s_row = s_uncached = 0;
+    __syncthreads();
+    const float Lrd = __double2float_rd(w.bx.L), Lru = __double2float_ru(w.bx.L);
+    const int W = (int)gridDim.x * kWalkWarps;
+    for (int I = (int)blockIdx.x * kWalkWarps + wp; I < nl; I += W) {
+        const bool recorded = WRITE && w.lruns && w.lruns[I] >= 0;
+        if (WRITE && !SPLIT && recorded) continue;
+        const double* A = w.lbox + 6 * (int64_t)I;
+        float aolo[3], aohi[3], ailo[3], aihi[3];
+        for (int a = 0; a < 3; ++a) {
+            aolo[a] = __double2float_rd(A[a]);
+            aohi[a] = __double2float_ru(A[3 + a]);
+            ailo[a] = __double2float_ru(A[a]);
+            aihi[a] = __double2float_rd(A[3 + a]);
+        }
+        const float ra = SPLIT ? w.box[0][2 * (int64_t)I + 1].w : 0.0f;  // rho of the outward box
+        long long c = 0, cf = 0;  // entries so far (uniform)
+        long long src = 0;        // this lane's part of their particles
+        long long at = WRITE ? w.rowptr[I] : 0, fat = WRITE && SPLIT ? w.frowptr[I] : 0;
+        const long long end = WRITE ? w.rowptr[I + 1] : 0, fend = WRITE && SPLIT ? w.frowptr[I + 1] : 0;
+        // pair cache: runs so far, the open (last) run's first entry and the entry after its end
+        const bool caching = !WRITE && w.cache != nullptr;
+        uint2* const slot = w.cache + I * (int64_t)w.kslot;
+        int nrun = 0;
+        uint32_t run0 = 0, runend = 0xffffffffu;
+        uint32_t code = 0;
+        float sd[3], su[3];  // the image's shift rounded down and up
+
+        // the leaves of mask M of the 32 from `base` on; b0, b1: this lane's leaf
+        auto leaves = [&](unsigned M, int base, float4 b0, float4 b1) {
+            if (!M) return;
+            const bool mine = (M >> lane) & 1u;
+            bool far = false;
+            if (SPLIT && mine)
+                far = far_pair(aolo, aohi, ra, b0, b1, sd, su, w.bx.theta2, w.bx.gt2, w.bx.rc2far);
+            const unsigned F = SPLIT ? __ballot_sync(kFull, far) : 0u, N = M & ~F;
+            if (WRITE) {
+                const long long p = far ? fat + __popc(F & lt) : at + __popc(N & lt);
+                if (mine) {
+                    if (p < (far ? fend : end))
+                        (far ? w.fpairs : w.pairs)[p] = ((uint32_t)(base + lane) << 5) | code;
+                    else
+                        atomicOr(w.err, 4u);
+                }
+                at += __popc(N);
+                fat += __popc(F);
                 return;
             }
-            for (int J = f; J <= l; ++J) pairs[w++] = ((uint32_t)J << 5) | (uint32_t)code;
-        } else if (cok) {
-            const uint32_t e0 = ((uint32_t)f << 5) | (uint32_t)code;
-            if (runn > 0 && e0 == run0 + (runn << 5)) {  // continues the open run
-                runn += (uint32_t)(l - f + 1);
-            } else {
-                if (runn > 0) {
-                    if (nrun == kslot) {
-                        cok = false;
-                        return;
+            c += __popc(N);
+            cf += __popc(F);
+            if (mine && !far) src += __float_as_int(b0.w);
+            if (!caching) return;
+            const bool cont = (M & 1u) && (((uint32_t)base << 5) | code) == runend;
+            unsigned B = M & ~(M << 1);  // first leaves of runs
+            if (cont) B &= ~1u;
+            if (((B >> lane) & 1u) || (cont && lane == 0)) {
+                const unsigned rest = ~(M >> lane);
+                const int len = rest ? __ffs(rest) - 1 : 32;
+                const bool old = cont && lane == 0;
+                const int k = old ? nrun - 1 : nrun + __popc(B & lt);
+                const uint32_t first = old ? run0 : ((uint32_t)(base + lane) << 5) | code;
+                if (k < w.kslot) slot[k] = make_uint2(first, (uint32_t)(base + lane + len) - (first >> 5));
+            }
+            if (B) run0 = ((uint32_t)(base + 31 - __clz(B)) << 5) | code;
+            nrun += __popc(B);
+            runend = ((uint32_t)(base + 32 - __clz(M)) << 5) | code;
+        };
+        // every leaf of [f, l]
+        auto range = [&](int f, int l) {
+            if (WRITE || SPLIT) {
+                for (int base = f & ~31; base <= l; base += 32) {
+                    const int J = base + lane;
+                    const bool in = J >= f && J <= l;
+                    float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
+                    if (SPLIT && in) {
+                        b0 = w.box[0][2 * (int64_t)J];
+                        b1 = w.box[0][2 * (int64_t)J + 1];
                     }
-                    slot[nrun++] = make_uint2(run0, runn);
+                    leaves(__ballot_sync(kFull, in), base, b0, b1);
                 }
+                return;
+            }
+            c += l - f + 1;
+            if (lane == 0) src += w.lfirst[l + 1] - w.lfirst[f];
+            if (!caching) return;
+            const uint32_t e0 = ((uint32_t)f << 5) | code;
+            if (e0 != runend) {
                 run0 = e0;
-                runn = (uint32_t)(l - f + 1);
+                ++nrun;
             }
-        }
-    };
-    for (int code = 0; code < kShiftCodes && !bad; ++code) {
-        const double sh[3] = {(code / 9 - 1) * bx.L, ((code / 3) % 3 - 1) * bx.L,
-                              (code % 3 - 1) * bx.L};
-        float sd[3], su[3];
-        for (int a = 0; a < 3; ++a) {
-            sd[a] = __double2float_rd(sh[a]);
-            su[a] = __double2float_ru(sh[a]);
-        }
-        if (gap2_lower(aolo, aohi, rlo, rhi, sd, su) >= bx.thi) continue;
-        if (maxgap2_upper(ailo, aihi, rlo, rhi, sd, su) < bx.tlo) {
-            take(0, (int)nl - 1, code);
-            continue;
-        }
-        int sp = 0;
-        int2 cur = make_int2(nl >= 2 ? 0 : kLeafBit, -1);
-        int64_t visits = 0;
-        for (;;) {
-            if (++visits > 2 * nl) {
-                atomicOr(err, 4u);
-                bad = true;
-                break;
+            runend = ((uint32_t)(l + 1) << 5) | code;
+            if (lane == 0 && nrun <= w.kslot) slot[nrun - 1] = make_uint2(run0, (runend - run0) >> 5);
+        };
+        auto set_shift = [&](uint32_t cd) {
+            code = cd;
+            const int s3[3] = {(int)(cd / 9u) - 1, (int)((cd / 3u) % 3u) - 1, (int)(cd % 3u) - 1};
+            for (int a = 0; a < 3; ++a) {
+                sd[a] = s3[a] < 0 ? -Lru : s3[a] > 0 ? Lrd : 0.f;
+                su[a] = s3[a] < 0 ? -Lrd : s3[a] > 0 ? Lru : 0.f;
             }
-            int2 next = make_int2(0, -2);  // y == -2: take the next stacked entry
-            if (cur.y >= 0) {  // a whole leaf range deferred behind a left subtree
-                take(cur.x, cur.y, code);
-            } else if (cur.x < 0) {  // a leaf that passed the lower-bound test
-                const int J = cur.x & 0x7fffffff;
-                const float4 r0 = lrec[2 * (int64_t)J], r1 = lrec[2 * (int64_t)J + 1];
-                const float bi_lo[3] = {r0.x, r0.y, r0.z}, bi_hi[3] = {r1.x, r1.y, r1.z};
-                if (gap2_upper(ailo, aihi, bi_lo, bi_hi, sd, su) < bx.tlo ||
-                    gap2_d(A, lbox + 6 * (int64_t)J, sh) < bx.rc2m)
-                    take(J, J, code);
-            } else {
-                const float4* q = nodef + 4 * (int64_t)cur.x;
-                const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
-                const float llo[3] = {q0.x, q0.y, q0.z}, lhi[3] = {q0.w, q1.x, q1.y};
-                const float blo[3] = {q1.z, q1.w, q2.x}, bhi[3] = {q2.y, q2.z, q2.w};
-                const int lc = __float_as_int(q3.x), rc = __float_as_int(q3.y);
-                const int lo = __float_as_int(q3.z), hi = __float_as_int(q3.w);
-                const int gamma = lc & 0x7fffffff;
-                const bool pl = gap2_lower(aolo, aohi, llo, lhi, sd, su) < bx.thi;
-                const bool pr = gap2_lower(aolo, aohi, blo, bhi, sd, su) < bx.thi;
-                const bool fl = pl && maxgap2_upper(ailo, aihi, llo, lhi, sd, su) < bx.tlo;
-                const bool fr = pr && maxgap2_upper(ailo, aihi, blo, bhi, sd, su) < bx.tlo;
-                if (fl) take(lo, gamma, code);
-                if (pl && !fl) {  // the left child needs a visit; the right one waits
-                    if (pr) {
-                        if (sp >= kStackDepth) {
-                            atomicOr(err, 2u);
-                            bad = true;
-                            break;
-                        }
-                        stack[sp++] = fr ? make_int2(gamma + 1, hi) : make_int2(rc, -1);
+        };
+        // the 32 leaves from `base` on
+        auto test_leaves = [&](int base) {
+            const int J = base + lane;
+            float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
+            bool keep = false;
+            if (J < nl) {
+                b0 = w.box[0][2 * (int64_t)J];
+                b1 = w.box[0][2 * (int64_t)J + 1];
+                const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
+                if (gap2_lower(aolo, aohi, blo, bhi, sd, su) < thi) {
+                    const float ilo[3] = {next_up(b0.x), next_up(b0.y), next_up(b0.z)};
+                    const float ihi[3] = {next_down(b1.x), next_down(b1.y), next_down(b1.z)};
+                    keep = gap2_upper(ailo, aihi, ilo, ihi, sd, su) < tlo;
+                    if (!keep) {
+                        const double sh[3] = {((int)(code / 9u) - 1) * w.bx.L,
+                                              ((int)((code / 3u) % 3u) - 1) * w.bx.L,
+                                              ((int)(code % 3u) - 1) * w.bx.L};
+                        keep = gap2_d(A, w.lbox + 6 * (int64_t)J, sh) < w.bx.rc2m;
                     }
-                    next = make_int2(lc, -1);
-                } else if (fr) {
-                    take(gamma + 1, hi, code);
-                } else if (pr) {
-                    next = make_int2(rc, -1);
                 }
             }
-            if (bad) break;
-            if (next.y != -2) {
-                cur = next;
-            } else if (sp > 0) {
-                cur = stack[--sp];
-            } else {
-                break;
+            leaves(__ballot_sync(kFull, keep), base, b0, b1);
+        };
+
+        if (recorded) {  // split: replay the row's runs
+            const int n = w.lruns[I];
+            for (int r = 0; r < n; ++r) {
+                const uint2 run = slot[r];
+                set_shift(run.x & 31u);
+                range((int)(run.x >> 5), (int)(run.x >> 5) + (int)run.y - 1);
+            }
+        } else {
+            const float4 r0 = w.box[w.top][0], r1 = w.box[w.top][1];
+            const float rlo[3] = {r0.x, r0.y, r0.z}, rhi[3] = {r1.x, r1.y, r1.z};
+            bool in = false, all = false;
+            if (lane < kShiftCodes) {  // the root at each image
+                set_shift((uint32_t)lane);
+                in = gap2_lower(aolo, aohi, rlo, rhi, sd, su) < thi;
+                all = in && maxgap2_upper(ailo, aihi, rlo, rhi, sd, su) < tlo;
+            }
+            unsigned images = __ballot_sync(kFull, in);
+            const unsigned whole = __ballot_sync(kFull, all);
+            while (images) {
+                const int image = __ffs(images) - 1;
+                images &= images - 1;
+                set_shift((uint32_t)image);
+                if ((whole >> image) & 1u) {
+                    range(0, nl - 1);
+                    continue;
+                }
+                if (w.top <= 1) {
+                    test_leaves(0);
+                    continue;
+                }
+                // lane t: members of the open group of level t + 1 still to
+                // be taken (todo), which of them are kept whole, the first's index
+                unsigned todo = 0, kept = 0;
+                int first = 0;
+                auto test_group = [&](int t, int base) {  // the members of level t from `base` on
+                    const int g = base + lane;
+                    bool part = false, full = false;
+                    if (g < (int)w.n[t]) {
+                        const float4 b0 = w.box[t][2 * (int64_t)g], b1 = w.box[t][2 * (int64_t)g + 1];
+                        const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
+                        part = gap2_lower(aolo, aohi, blo, bhi, sd, su) < thi;
+                        full = part && maxgap2_upper(ailo, aihi, blo, bhi, sd, su) < tlo;
+                    }
+                    const unsigned P = __ballot_sync(kFull, part), K = __ballot_sync(kFull, full);
+                    if (lane == t) {
+                        todo = P;
+                        kept = K;
+                        first = base;
+                    }
+                };
+                int t = w.top - 1;
+                test_group(t, 0);
+                while (t < w.top) {
+                    const unsigned m = __shfl_sync(kFull, todo, t);
+                    if (!m) {
+                        ++t;
+                        continue;
+                    }
+                    const int bit = __ffs(m) - 1;
+                    const int g = __shfl_sync(kFull, first, t) + bit;
+                    const bool full = (__shfl_sync(kFull, kept, t) >> bit) & 1u;
+                    if (lane == t) todo &= todo - 1;
+                    if (full) {
+                        const long long f = (long long)g << (5 * t), l = ((long long)(g + 1) << (5 * t)) - 1;
+                        range((int)f, l < nl ? (int)l : nl - 1);
+                    } else if (t == 1) {
+                        test_leaves(32 * g);
+                    } else {
+                        --t;
+                        test_group(t, 32 * g);
+                    }
+                }
+            }
+        }
+        if (WRITE) {
+            if ((at != end || (SPLIT && fat != fend)) && lane == 0) atomicOr(w.err, 4u);
+        } else {
+            for (int o = 16; o > 0; o >>= 1) src += __shfl_xor_sync(kFull, src, o);
+            if (lane == 0) {
+                const long long cost = src * (w.lfirst[I + 1] - w.lfirst[I]);
+                w.lcnt[I] = c;
+                w.lcost[I] = cost;
+                if (SPLIT) w.lfar[I] = cf;
+                if (caching) {
+                    const bool fits = nrun <= w.kslot;
+                    w.lruns[I] = fits ? nrun : -1;
+                    if (!fits) atomicAdd((unsigned long long*)&s_uncached, 1ULL);
+                }
+                atomicAdd((unsigned long long*)&s_pairs, (unsigned long long)c);
+                atomicAdd((unsigned long long*)&s_eval, (unsigned long long)cost);
+                if (SPLIT) atomicAdd((unsigned long long*)&s_far, (unsigned long long)cf);
+                atomicMax(&s_cost, cost);
+                atomicMax(&s_row, c);
             }
         }
     }
-    if (WRITE && !bad && w != wend) atomicOr(err, 4u);
-    if (!WRITE) {
-        const int64_t nI = lfirst[I + 1] - lfirst[I];
-        lcnt[I] = c;
-        lcost[I] = src * nI;
-        if (caching) {
-            if (cok && runn > 0) {
-                if (nrun == kslot)
-                    cok = false;
-                else
-                    slot[nrun++] = make_uint2(run0, runn);
-            }
-            lruns[I] = cok ? nrun : -1;
-            if (!cok) atomicAdd((unsigned long long*)(cnt + kCntUncached), 1ULL);
-        }
-        atomicAdd((unsigned long long*)(cnt + kCntPairs), (unsigned long long)c);
-        atomicAdd((unsigned long long*)(cnt + kCntEvaluated), (unsigned long long)(src * nI));
-        atomicMax(cnt + kCntMaxCost, (long long)(src * nI));
-        atomicMax(cnt + kCntMaxRow, (long long)c);
+    if (WRITE) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {  // one update per block
+        atomicAdd((unsigned long long*)(w.cnt + kCntPairs), (unsigned long long)s_pairs);
+        atomicAdd((unsigned long long*)(w.cnt + kCntEvaluated), (unsigned long long)s_eval);
+        if (SPLIT) atomicAdd((unsigned long long*)(w.cnt + kCntFar), (unsigned long long)s_far);
+        if (s_uncached) atomicAdd((unsigned long long*)(w.cnt + kCntUncached), (unsigned long long)s_uncached);
+        atomicMax(w.cnt + kCntMaxCost, s_cost);
+        atomicMax(w.cnt + kCntMaxRow, s_row);
     }
 }
 
@@ -1055,302 +1083,6 @@ __global__ void __launch_bounds__(256) k_pairs_expand(int64_t nl, const int32_t*
     }
 }
 
-// The walk of k_pairs with the multipole split.  A lane's walk does not
-// classify the leaves it keeps: it queues the kept ranges (first, last,
-// image) in shared memory, and whenever a lane's queue is nearly full, or
-// every lane's walk has ended, the warp classifies all queued ranges of all
-// its lanes as one list, 32 source leaves per step (far_pair then runs with
-// every lane busy, where inside a divergent walk it ran one lane at a time),
-// and counts or writes the near and far entries of each owning row in walk
-// order.  Every lane runs the same number of flushes (lanes past the last
-// leaf have ended from the start), so the warp-wide steps see all 32 lanes.
-// With a pair cache the count pass also records each row's queued ranges as
-// runs (as k_pairs does), and the write pass replays a recorded row's runs
-// into the queue instead of walking it again (lruns[I] >= 0).  Rows are
-// interleaved over the warps as in k_pairs (here 6.33 -> 5.57 ms per split
-// build on the bench workload: a warp runs until its slowest lane is done).
-constexpr int kSplitQ = 8;  // queued ranges per lane (a walk step queues at most 2)
-
-template <bool WRITE>
-__global__ void __launch_bounds__(128, 4) k_pairs_split(
-    int64_t nl, BoxK bx, const int32_t* __restrict__ lfirst, const double* __restrict__ lbox,
-    const float4* __restrict__ lrec, const float4* __restrict__ lout,
-    const float4* __restrict__ nodef, const double* __restrict__ rootbox,
-    int64_t* __restrict__ lcnt, int64_t* __restrict__ lcost, int64_t* __restrict__ lfar,
-    const int64_t* __restrict__ rowptr, uint32_t* __restrict__ pairs,
-    const int64_t* __restrict__ frowptr, uint32_t* __restrict__ fpairs,
-    long long* __restrict__ cnt, unsigned* __restrict__ err, int32_t* __restrict__ lruns,
-    uint2* __restrict__ cache, int kslot, int interleave)
-{
-    constexpr int kQ = kSplitQ, kSlots = 32 * kSplitQ, kWarps = 4;
-    __shared__ int4 sq[kWarps][kSlots];            // (first, last, image, owning lane)
-    __shared__ long long spre[kWarps][kSlots];     // leaves queued before each slot
-    __shared__ float4 sbox[kWarps][32][2];         // owning lane's box rounded outward, rho
-    __shared__ long long sw[kWarps][32], sfw[kWarps][32];    // write positions
-    __shared__ long long swe[kWarps][32], sfwe[kWarps][32];  // row ends
-    __shared__ long long sc[kWarps][32], scf[kWarps][32], ssrc[kWarps][32];  // counts
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t W = (nl + 31) >> 5;
-    const int64_t I = !interleave ? t : (t >> 5) < W ? (t & 31) * W + (t >> 5) : nl;
-    const bool live = I < nl;
-    double A[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    float aolo[3] = {0.f, 0.f, 0.f}, aohi[3] = {0.f, 0.f, 0.f};
-    float ailo[3] = {0.f, 0.f, 0.f}, aihi[3] = {0.f, 0.f, 0.f};
-    float rlo[3] = {0.f, 0.f, 0.f}, rhi[3] = {0.f, 0.f, 0.f};
-    sbox[wp][lane][0] = sbox[wp][lane][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    sw[wp][lane] = sfw[wp][lane] = swe[wp][lane] = sfwe[wp][lane] = 0;
-    sc[wp][lane] = scf[wp][lane] = ssrc[wp][lane] = 0;
-    if (live) {
-        for (int a = 0; a < 3; ++a) {
-            A[a] = lbox[6 * I + a];
-            A[3 + a] = lbox[6 * I + 3 + a];
-            aolo[a] = __double2float_rd(A[a]);
-            aohi[a] = __double2float_ru(A[3 + a]);
-            ailo[a] = __double2float_ru(A[a]);
-            aihi[a] = __double2float_rd(A[3 + a]);
-            rlo[a] = __double2float_rd(rootbox[a]);
-            rhi[a] = __double2float_ru(rootbox[3 + a]);
-        }
-        sbox[wp][lane][0] = lout[2 * I];
-        sbox[wp][lane][1] = lout[2 * I + 1];
-        if (WRITE) {
-            sw[wp][lane] = rowptr[I];
-            swe[wp][lane] = rowptr[I + 1];
-            sfw[wp][lane] = frowptr[I];
-            sfwe[wp][lane] = frowptr[I + 1];
-        }
-    }
-    __syncwarp();
-    const float Lrd = __double2float_rd(bx.L), Lru = __double2float_ru(bx.L);
-    int2 stack[kStackDepth];
-    bool bad = false, done = !live, in_tree = false;
-    int code = -1, sp = 0;
-    int2 cur = make_int2(0, -1);
-    int64_t visits = 0;
-    float sd[3] = {0.f, 0.f, 0.f}, su[3] = {0.f, 0.f, 0.f};
-    double sh[3] = {0.0, 0.0, 0.0};
-    int4* myq = &sq[wp][lane * kQ];
-    // pair cache: the count pass records runs (open run run0/runn), the write
-    // pass replays a recorded row (nrun runs, the next one at ri)
-    bool cok = !WRITE && live && cache != nullptr;
-    const bool replay = WRITE && live && lruns != nullptr && lruns[I] >= 0;
-    uint2* const slot = (cok || replay) ? cache + I * (int64_t)kslot : nullptr;
-    uint32_t run0 = 0, runn = 0;
-    int nrun = replay ? lruns[I] : 0, ri = 0;
-    int nq = 0;
-    auto push = [&](int f, int l, int c) {
-        myq[nq++] = make_int4(f, l, c, lane);
-        if (!cok) return;
-        const uint32_t e0 = ((uint32_t)f << 5) | (uint32_t)c;
-        if (runn > 0 && e0 == run0 + (runn << 5)) {
-            runn += (uint32_t)(l - f + 1);
-        } else {
-            if (runn > 0) {
-                if (nrun == kslot) {
-                    cok = false;
-                    return;
-                }
-                slot[nrun++] = make_uint2(run0, runn);
-            }
-            run0 = e0;
-            runn = (uint32_t)(l - f + 1);
-        }
-    };
-    for (;;) {
-        // ---- walk (or replay) until the queue may not take another step's ranges
-        nq = 0;
-        while (!done && nq <= kQ - 2) {
-            if (replay) {
-                if (ri == nrun) {
-                    done = true;
-                    break;
-                }
-                const uint2 run = slot[ri++];
-                const int f = (int)(run.x >> 5);
-                myq[nq++] = make_int4(f, f + (int)run.y - 1, (int)(run.x & 31u), lane);
-                continue;
-            }
-            if (!in_tree) {
-                if (++code >= kShiftCodes) {
-                    done = true;
-                    break;
-                }
-                sh[0] = (code / 9 - 1) * bx.L;
-                sh[1] = ((code / 3) % 3 - 1) * bx.L;
-                sh[2] = (code % 3 - 1) * bx.L;
-                for (int a = 0; a < 3; ++a) {
-                    sd[a] = __double2float_rd(sh[a]);
-                    su[a] = __double2float_ru(sh[a]);
-                }
-                if (gap2_lower(aolo, aohi, rlo, rhi, sd, su) >= bx.thi) continue;
-                if (maxgap2_upper(ailo, aihi, rlo, rhi, sd, su) < bx.tlo) {
-                    push(0, (int)nl - 1, code);
-                    continue;
-                }
-                in_tree = true;
-                sp = 0;
-                cur = make_int2(nl >= 2 ? 0 : kLeafBit, -1);
-                visits = 0;
-            }
-            if (++visits > 2 * nl) {
-                atomicOr(err, 4u);
-                bad = done = true;
-                break;
-            }
-            int2 next = make_int2(0, -2);  // y == -2: take the next stacked entry
-            if (cur.y >= 0) {  // a whole leaf range deferred behind a left subtree
-                push(cur.x, cur.y, code);
-            } else if (cur.x < 0) {  // a leaf that passed the lower-bound test
-                const int J = cur.x & 0x7fffffff;
-                const float4 r0 = lrec[2 * (int64_t)J], r1 = lrec[2 * (int64_t)J + 1];
-                const float bi_lo[3] = {r0.x, r0.y, r0.z}, bi_hi[3] = {r1.x, r1.y, r1.z};
-                if (gap2_upper(ailo, aihi, bi_lo, bi_hi, sd, su) < bx.tlo ||
-                    gap2_d(A, lbox + 6 * (int64_t)J, sh) < bx.rc2m)
-                    push(J, J, code);
-            } else {
-                const float4* qn = nodef + 4 * (int64_t)cur.x;
-                const float4 q0 = qn[0], q1 = qn[1], q2 = qn[2], q3 = qn[3];
-                const float llo[3] = {q0.x, q0.y, q0.z}, lhi[3] = {q0.w, q1.x, q1.y};
-                const float blo[3] = {q1.z, q1.w, q2.x}, bhi[3] = {q2.y, q2.z, q2.w};
-                const int lc = __float_as_int(q3.x), rc = __float_as_int(q3.y);
-                const int lo = __float_as_int(q3.z), hi = __float_as_int(q3.w);
-                const int gamma = lc & 0x7fffffff;
-                const bool pl = gap2_lower(aolo, aohi, llo, lhi, sd, su) < bx.thi;
-                const bool pr = gap2_lower(aolo, aohi, blo, bhi, sd, su) < bx.thi;
-                const bool fl = pl && maxgap2_upper(ailo, aihi, llo, lhi, sd, su) < bx.tlo;
-                const bool fr = pr && maxgap2_upper(ailo, aihi, blo, bhi, sd, su) < bx.tlo;
-                if (fl) push(lo, gamma, code);
-                if (pl && !fl) {  // the left child needs a visit; the right one waits
-                    if (pr) {
-                        if (sp >= kStackDepth) {
-                            atomicOr(err, 2u);
-                            bad = done = true;
-                            break;
-                        }
-                        stack[sp++] = fr ? make_int2(gamma + 1, hi) : make_int2(rc, -1);
-                    }
-                    next = make_int2(lc, -1);
-                } else if (fr) {
-                    push(gamma + 1, hi, code);
-                } else if (pr) {
-                    next = make_int2(rc, -1);
-                }
-            }
-            if (next.y != -2) {
-                cur = next;
-            } else if (sp > 0) {
-                cur = stack[--sp];
-            } else {
-                in_tree = false;
-            }
-        }
-        // ---- the warp classifies the queued ranges of all its lanes
-        __syncwarp();
-        long long mine = 0;  // leaves this lane queued
-        for (int k = 0; k < nq; ++k) mine += (long long)myq[k].y - myq[k].x + 1;
-        long long base = mine;  // inclusive scan over lanes, then exclusive
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long v = __shfl_up_sync(kFull, base, o);
-            if (lane >= o) base += v;
-        }
-        const long long total = __shfl_sync(kFull, base, 31);
-        base -= mine;
-        {
-            long long run = base;
-            for (int k = 0; k < kQ; ++k) {
-                spre[wp][lane * kQ + k] = run;  // empty slots: zero-length, next lane's base
-                if (k < nq) run += (long long)myq[k].y - myq[k].x + 1;
-            }
-        }
-        __syncwarp();
-        for (long long v0 = 0; v0 < total; v0 += 32) {
-            const long long v = v0 + lane;
-            const bool valid = v < total;
-            int slot = 0;
-            if (valid) {  // the last slot whose prefix is <= v
-                int lo = 0, hi = kSlots - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (spre[wp][mid] <= v) lo = mid;
-                    else hi = mid - 1;
-                }
-                slot = lo;
-            }
-            const int4 r = sq[wp][slot];
-            const int owner = valid ? r.w : 32;
-            const int J = r.x + (int)(v - spre[wp][slot]);
-            bool far = false;
-            int nsrc = 0;
-            if (valid) {
-                const int s3[3] = {r.z / 9 - 1, (r.z / 3) % 3 - 1, r.z % 3 - 1};
-                float fd[3], fu[3];
-                for (int a = 0; a < 3; ++a) {
-                    fd[a] = s3[a] < 0 ? -Lru : (s3[a] > 0 ? Lrd : 0.f);
-                    fu[a] = s3[a] < 0 ? -Lrd : (s3[a] > 0 ? Lru : 0.f);
-                }
-                const float4 b0 = sbox[wp][owner][0], b1 = sbox[wp][owner][1];
-                const float alo[3] = {b0.x, b0.y, b0.z}, ahi[3] = {b1.x, b1.y, b1.z};
-                far = far_pair(alo, ahi, b1.w, lout[2 * (int64_t)J], lout[2 * (int64_t)J + 1],
-                               fd, fu, bx.theta2, bx.gt2, bx.rc2far);
-                if (!WRITE && !far) nsrc = lfirst[J + 1] - lfirst[J];
-            }
-            const unsigned seg = __match_any_sync(kFull, owner);
-            const unsigned fb = __ballot_sync(kFull, valid && far) & seg;
-            const unsigned nb = __ballot_sync(kFull, valid && !far) & seg;
-            const unsigned lt = (1u << lane) - 1u;
-            const bool lead = valid && lane == __ffs(seg) - 1;
-            if (WRITE && valid) {
-                const uint32_t ent = ((uint32_t)J << 5) | (uint32_t)r.z;
-                if (far) {
-                    const long long pos = sfw[wp][owner] + __popc(fb & lt);
-                    if (pos < sfwe[wp][owner]) fpairs[pos] = ent;
-                    else atomicOr(err, 4u);
-                } else {
-                    const long long pos = sw[wp][owner] + __popc(nb & lt);
-                    if (pos < swe[wp][owner]) pairs[pos] = ent;
-                    else atomicOr(err, 4u);
-                }
-            }
-            if (!WRITE && nsrc) atomicAdd((unsigned long long*)&ssrc[wp][owner], (unsigned long long)nsrc);
-            __syncwarp();
-            if (lead) {
-                sw[wp][owner] += __popc(nb);
-                sfw[wp][owner] += __popc(fb);
-                sc[wp][owner] += __popc(nb);
-                scf[wp][owner] += __popc(fb);
-            }
-            __syncwarp();
-        }
-        if (__all_sync(kFull, done)) break;
-    }
-    if (!live) return;
-    const int64_t c = sc[wp][lane], cf = scf[wp][lane], src = ssrc[wp][lane];
-    if (WRITE && !bad && (sw[wp][lane] != swe[wp][lane] || sfw[wp][lane] != sfwe[wp][lane]))
-        atomicOr(err, 4u);
-    if (!WRITE) {
-        const int64_t nI = lfirst[I + 1] - lfirst[I];
-        lcnt[I] = c;
-        lfar[I] = cf;
-        lcost[I] = src * nI;
-        if (cache) {
-            if (cok && runn > 0) {
-                if (nrun == kslot)
-                    cok = false;
-                else
-                    slot[nrun++] = make_uint2(run0, runn);
-            }
-            lruns[I] = cok ? nrun : -1;
-            if (!cok) atomicAdd((unsigned long long*)(cnt + kCntUncached), 1ULL);
-        }
-        atomicAdd((unsigned long long*)(cnt + kCntPairs), (unsigned long long)c);
-        atomicAdd((unsigned long long*)(cnt + kCntFar), (unsigned long long)cf);
-        atomicAdd((unsigned long long*)(cnt + kCntEvaluated), (unsigned long long)(src * nI));
-        atomicMax(cnt + kCntMaxCost, (long long)(src * nI));
-        atomicMax(cnt + kCntMaxRow, (long long)c);
-    }
-}
-
 // Expansion centre and radius of each leaf for the multipole split: the
 // centre of its particle box and half the box diagonal; also the centre's
 // offset from the leaf's cell centre (lcen, units of L / 2^22) in FP32, so
@@ -1386,7 +1118,8 @@ __global__ void k_payload(const int32_t* __restrict__ lfirst, const int32_t* __r
                           int32_t* __restrict__ perm, int4* __restrict__ leaf,
                           int4* __restrict__ lcen)
 {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;  // 16 lanes per leaf
+    const int sub = threadIdx.x & 15;
     if (g >= nl) return;
     const int64_t f = lfirst[g], e = g + 1 < nl ? lfirst[g + 1] : n;
     const int L = llevel[g];
@@ -1396,17 +1129,20 @@ __global__ void k_payload(const int32_t* __restrict__ lfirst, const int32_t* __r
     const int32_t cx = (int32_t)((2 * (compact3_d(k >> 2) >> sh) + 1) * sc);
     const int32_t cy = (int32_t)((2 * (compact3_d(k >> 1) >> sh) + 1) * sc);
     const int32_t cz = (int32_t)((2 * (compact3_d(k) >> sh) + 1) * sc);
-    leaf[g] = make_int4((int)f, (int)(e - f), 0, 0);
-    lcen[g] = make_int4(cx, cy, cz, L);
+    if (sub == 0) {
+        leaf[g] = make_int4((int)f, (int)(e - f), 0, 0);
+        lcen[g] = make_int4(cx, cy, cz, L);
+    }
     const double c[3] = {__dmul_rn((double)cx, bx.unit), __dmul_rn((double)cy, bx.unit),
                          __dmul_rn((double)cz, bx.unit)};
-    for (int64_t q = f; q < e; ++q) {
+    for (int64_t q = f + sub; q < e; q += 16) {
         const int64_t p = idx[q];
-        const double x = wpos[4 * p], y = wpos[4 * p + 1], z = wpos[4 * p + 2], m = wpos[4 * p + 3];
-        pf[q] = make_float4((float)__dmul_rn(__dsub_rn(x, c[0]), bx.inv2rs),
-                            (float)__dmul_rn(__dsub_rn(y, c[1]), bx.inv2rs),
-                            (float)__dmul_rn(__dsub_rn(z, c[2]), bx.inv2rs), (float)m);
-        if (pd) pd[q] = make_double4(x, y, z, m);
+        const double2* w = reinterpret_cast<const double2*>(wpos + 4 * p);
+        const double2 xy = w[0], zm = w[1];
+        pf[q] = make_float4((float)__dmul_rn(__dsub_rn(xy.x, c[0]), bx.inv2rs),
+                            (float)__dmul_rn(__dsub_rn(xy.y, c[1]), bx.inv2rs),
+                            (float)__dmul_rn(__dsub_rn(zm.x, c[2]), bx.inv2rs), (float)zm.y);
+        if (pd) pd[q] = make_double4(xy.x, xy.y, zm.x, zm.y);
         perm[q] = (int32_t)p;
     }
 }
@@ -1441,6 +1177,27 @@ __global__ void k_sched_out(const uint64_t* __restrict__ key, const int32_t* __r
 }
 
 __global__ void k_copy_total(int64_t* dst, const int64_t* src) { *dst = *src; }
+
+// The levels of the groups over nl leaves.
+WalkArgs walk_levels(int64_t nl, const float4* lout, float4* groups)
+{
+    WalkArgs w{};
+    w.nl = nl;
+    w.box[0] = lout;
+    w.n[0] = nl;
+    while (w.n[w.top] > 1) {
+        w.box[w.top + 1] = groups;
+        w.n[w.top + 1] = (w.n[w.top] + 31) / 32;
+        groups += 2 * w.n[++w.top];
+    }
+    return w;
+}
+
+// blocks of a row walk: a warp per leaf, up to one wave
+unsigned walk_blocks(int64_t nl, int sms)
+{
+    return (unsigned)std::min<int64_t>((nl + kWalkWarps - 1) / kWalkWarps, kWalkBlocks * (int64_t)sms);
+}
 
 unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -1563,16 +1320,9 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     int32_t* llevel = (int32_t*)(s + S.llevel);
     uint64_t* lkey = (uint64_t*)(s + S.lkey);
     double* lbox = (double*)(s + S.lbox);
-    float4* lrec = (float4*)(s + S.lrec);
+    float4* lout = (float4*)(s + S.lout);
     int64_t* lcnt = (int64_t*)(s + S.lcnt);
     int64_t* lcost = (int64_t*)(s + S.lcost);
-    int2* tnode = (int2*)(s + S.tnode);
-    int2* tspan = (int2*)(s + S.tspan);
-    int32_t* tparl = (int32_t*)(s + S.tparl);
-    int32_t* tpari = (int32_t*)(s + S.tpari);
-    double* tbox = (double*)(s + S.tbox);
-    float4* nodef = (float4*)(s + S.nodef);
-    int* tflag = (int*)(s + S.tflag);
     int64_t* hist = (int64_t*)(s + S.hist);
     int64_t* tiles = (int64_t*)(s + S.tiles);
     int64_t* total = (int64_t*)(s + S.total);
@@ -1584,7 +1334,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
 
     int e;
     if ((e = (int)cudaMemsetAsync(cnt, 0, 8 * kCntWords, st))) return dcuda(e, "cudaMemsetAsync");
-    k_keys<<<nblk(n, 256), 256, 0, st>>>(d_pos, d_mass, n, bx, wpos, k0, v0, cnt);
+    k_keys<<<nblk(n, 256), 256, 0, st>>>(d_pos, d_mass, n, bx, 1.0 / (double)n, wpos, k0, v0, cnt);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "key kernel");
     if ((e = radix_sort(k0, v0, k1, v1, n, 3 * kMortonBits, hist, tiles, total, st)))
         return dcuda(e, "radix sort");
@@ -1599,14 +1349,14 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     if (c[kCntError] & 1) return dfail(PSR_E_ARG, "non-finite position or mass");
     if (nl < 1 || nl > n || nl >= (1 << 27)) return dfail(PSR_E_ARG, "leaf count out of range");
     if (!(flags & PSR_BUILD_UNPACKED)) {
-        // pack sibling leaves: marks, pack ids, packed arrays in the (still
-        // free) tree regions, copied back over the leaf arrays
+        // pack sibling leaves: marks, pack ids, packed arrays, copied back
+        // over the leaf arrays
         int64_t* pstart = flag;
         int64_t* pid = lid;
-        int32_t* psize = tflag;
-        int32_t* lfirst2 = (int32_t*)tspan;
-        int32_t* llevel2 = tpari;
-        uint64_t* lkey2 = (uint64_t*)tnode;
+        int32_t* psize = (int32_t*)(s + S.psize);
+        int32_t* lfirst2 = (int32_t*)(s + S.lfirst2);
+        int32_t* llevel2 = (int32_t*)(s + S.llevel2);
+        uint64_t* lkey2 = (uint64_t*)(s + S.lkey2);
         k_pack_mark<<<nblk(nl, 256), 256, 0, st>>>(lfirst, llevel, lkey, nl, max_leaf, pstart, psize);
         if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf packing kernel");
         if ((e = scan_exclusive(pstart, pid, nl, tiles, total, st))) return dcuda(e, "scan");
@@ -1622,37 +1372,34 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
             return dcuda(e, "cudaMemcpyAsync");
         nl = np;
     }
-    k_leaf_box<<<nblk(nl, 256), 256, 0, st>>>(lfirst, nl, n, wpos, v0, lbox, lrec,
-                                              (float4*)(s + S.lout), cnt);
-    if (nl >= 2) {
-        if ((e = (int)cudaMemsetAsync(tflag, 0, 4 * (nl - 1), st))) return dcuda(e, "cudaMemsetAsync");
-        k_tree_nodes<<<nblk(nl - 1, 256), 256, 0, st>>>(lkey, nl, tnode, tspan, tparl, tpari);
-        k_tree_boxes<<<nblk(nl, 256), 256, 0, st>>>(nl, tnode, tparl, tpari, lbox, tbox, tflag, cnt);
-        k_tree_pack<<<nblk(nl - 1, 256), 256, 0, st>>>(nl, tnode, tspan, lbox, tbox, nodef);
-    }
-    const double* rootbox = nl >= 2 ? tbox : lbox;
-    // rows interleaved over the warps when they fit in one wave of the count
-    // walk's resident warps (32 per SM), two of the split walk's (16 per SM)
+    k_leaf_box<<<nblk(16 * nl, 256), 256, 0, st>>>(lfirst, nl, n, wpos, v0, lbox, lout, cnt);
+    WalkArgs wa = walk_levels(nl, lout, (float4*)(s + S.groups));
+    for (int t = 1; t <= wa.top; ++t)
+        k_groups<<<nblk(32 * wa.n[t], 256), 256, 0, st>>>(wa.box[t - 1], wa.n[t - 1],
+                                                          const_cast<float4*>(wa.box[t]), wa.n[t]);
+    if ((e = (int)cudaGetLastError())) return dcuda(e, "group kernel");
     int dev = 0, sms = 0;
     if ((e = (int)cudaGetDevice(&dev))) return dcuda(e, "cudaGetDevice");
     if ((e = (int)cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
         return dcuda(e, "cudaDeviceGetAttribute");
-    const int interleave = nl <= (int64_t)sms * 32 * 32 ? 1 : 0;
     // runs per row in the pair cache (none below kMinRuns: rows walked twice)
     const int64_t ks = S.ncache / nl;
     const int kslot = ks >= kMinRuns ? (int)(ks < (1 << 20) ? ks : (1 << 20)) : 0;
     int32_t* const lruns = kslot ? (int32_t*)(s + S.lruns) : nullptr;
     uint2* const pcache = kslot ? (uint2*)(s + S.cache) : nullptr;
-    if (theta > 0.0)
-        k_pairs_split<false><<<nblk(nl, 128), 128, 0, st>>>(
-            nl, bx, lfirst, lbox, lrec, (const float4*)(s + S.lout), nodef, rootbox, lcnt, lcost,
-            (int64_t*)(s + S.lfar), nullptr, nullptr, nullptr, nullptr, cnt,
-            (unsigned*)(cnt + kCntError), lruns, pcache, kslot, interleave);
-    else {
-        k_pairs<false><<<nblk(nl, 128), 128, 0, st>>>(
-            nl, n, bx, lfirst, lbox, lrec, nodef, rootbox, lcnt, lcost, nullptr, nullptr, cnt,
-            (unsigned*)(cnt + kCntError), lruns, pcache, kslot, interleave);
-    }
+    wa.bx = bx;
+    wa.lfirst = lfirst;
+    wa.lbox = lbox;
+    wa.lcnt = lcnt;
+    wa.lcost = lcost;
+    wa.lfar = (int64_t*)(s + S.lfar);
+    wa.cnt = cnt;
+    wa.err = (unsigned*)(cnt + kCntError);
+    wa.lruns = lruns;
+    wa.cache = pcache;
+    wa.kslot = kslot;
+    if (theta > 0.0) k_rows<false, true><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
+    else k_rows<false, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "pair count kernel");
     if ((e = read_back(c, cnt, sizeof c, st, timeout_ms))) return e;
     if (c[kCntError] & 2) return dfail(PSR_E_DEVICE, "tree traversal stack overflow");
@@ -1694,7 +1441,6 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     h->db_scratch = s;
     h->max_cost = c[kCntMaxCost];
     h->db_kslot = kslot;
-    h->db_interleave = interleave;
     h->db_uncached = kslot ? c[kCntUncached] : nl;
     h->build_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     *out = reinterpret_cast<psr_leaves*>(h);
@@ -1746,7 +1492,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     // word that psr_check reads
     if ((e = (int)cudaMemsetAsync(w + L.ctrl, 0, kCtrlWords * 4, st))) return dcuda(e, "cudaMemsetAsync");
     const int32_t* lfirst = (const int32_t*)(s + S.lfirst);
-    k_payload<<<nblk(nl, 128), 128, 0, st>>>(
+    k_payload<<<nblk(16 * nl, 256), 256, 0, st>>>(
         lfirst, (const int32_t*)(s + S.llevel), (const uint64_t*)(s + S.lkey), nl, n, bx,
         (const double*)(s + S.wpos), (const int32_t*)(s + S.val0), (float4*)(w + L.pf),
         h->has_pd ? (double4*)(w + L.pd) : nullptr, (int32_t*)(w + L.perm), (int4*)(w + L.leaf),
@@ -1769,35 +1515,31 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
                                               (double4*)(w + L.fcen), (float4*)(w + L.fofs));
         if ((e = (int)cudaGetLastError())) return dcuda(e, "expansion centre kernel");
     }
-    const double* rootbox = nl >= 2 ? (const double*)(s + S.tbox) : lbox;
+    WalkArgs wa = walk_levels(nl, (const float4*)(s + S.lout), (float4*)(s + S.groups));
+    wa.bx = bx;
+    wa.lfirst = lfirst;
+    wa.lbox = lbox;
+    wa.rowptr = rowptr;
+    wa.frowptr = frow;
+    wa.pairs = (uint32_t*)(w + L.pairs);
+    wa.err = (unsigned*)(w + L.ctrl) + kCtrlError;
+    wa.lruns = h->db_kslot ? (int32_t*)(s + S.lruns) : nullptr;
+    wa.cache = h->db_kslot ? (uint2*)(s + S.cache) : nullptr;
+    wa.kslot = h->db_kslot;
     if (h->has_far) {
-        BoxK bxw = bx;
-        bxw.theta2 = (float)(h->theta * h->theta);
-        bxw.gt2 = (h->flags & PSR_BUILD_SPLIT_GAUSSIAN)
-                      ? (float)(h->theta * h->theta * 4.0 * std::pow(h->boxes[0].r_s, 4))
-                      : INFINITY;
-        // rows the count pass recorded are replayed; the rest are walked again
-        k_pairs_split<true><<<nblk(nl, 128), 128, 0, st>>>(
-            nl, bxw, lfirst, lbox, (const float4*)(s + S.lrec), (const float4*)(s + S.lout),
-            (const float4*)(s + S.nodef), rootbox, nullptr, nullptr, nullptr, rowptr,
-            (uint32_t*)(w + L.pairs), frow, (uint32_t*)(w + L.fpairs), nullptr,
-            (unsigned*)(w + L.ctrl) + kCtrlError,
-            h->db_kslot ? (int32_t*)(s + S.lruns) : nullptr,
-            h->db_kslot ? (uint2*)(s + S.cache) : nullptr, h->db_kslot, h->db_interleave);
+        wa.fpairs = (uint32_t*)(w + L.fpairs);
+        wa.bx.theta2 = (float)(h->theta * h->theta);
+        wa.bx.gt2 = (h->flags & PSR_BUILD_SPLIT_GAUSSIAN)
+                        ? (float)(h->theta * h->theta * 4.0 * std::pow(h->boxes[0].r_s, 4))
+                        : INFINITY;
+        k_rows<true, true><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
     } else {
         // rows the count walk cached are expanded; the rest are walked again
-        int32_t* lruns = h->db_kslot ? (int32_t*)(s + S.lruns) : nullptr;
-        if (lruns) {
-            k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, lruns, (const uint2*)(s + S.cache),
-                                                       h->db_kslot, rowptr, (uint32_t*)(w + L.pairs),
-                                                       (unsigned*)(w + L.ctrl) + kCtrlError);
+        if (wa.lruns) {
+            k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, wa.lruns, wa.cache, wa.kslot, rowptr, wa.pairs, wa.err);
             if ((e = (int)cudaGetLastError())) return dcuda(e, "pair expand kernel");
         }
-        if (h->db_uncached > 0)
-            k_pairs<true><<<nblk(nl, 128), 128, 0, st>>>(
-                nl, n, bx, lfirst, lbox, (const float4*)(s + S.lrec), (const float4*)(s + S.nodef),
-                rootbox, nullptr, nullptr, rowptr, (uint32_t*)(w + L.pairs), nullptr,
-                (unsigned*)(w + L.ctrl) + kCtrlError, lruns, nullptr, 0, h->db_interleave);
+        if (h->db_uncached > 0) k_rows<true, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
     }
     if ((e = (int)cudaGetLastError())) return dcuda(e, "pair write kernel");
     // schedule: the particle sort buffers are free again (values in int32

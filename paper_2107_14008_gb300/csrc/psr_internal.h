@@ -120,7 +120,6 @@ struct Leaves {
     int64_t n_far = 0;          //   far entries
     char* db_scratch = nullptr; // device build between its two calls: the caller's scratch
     int db_kslot = 0;           //   runs per row in the pair cache (0: not used)
-    int db_interleave = 0;      //   whether the walks take rows interleaved over warps
     int64_t db_uncached = 0;    //   and the rows it could not hold
     // device state
     Layout lay{};

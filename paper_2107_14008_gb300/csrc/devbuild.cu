@@ -4,23 +4,23 @@
 // It produces the arrays the host builder produces, bit for bit and in the
 // same order:
 //   1. keys      wrap positions into [0, L), 21-bit quantisation, 63-bit Morton key
-//   2. sort      stable LSD radix sort of (key, index), 8 passes of 8 bits
+//   2. sort      stable LSD radix sort of (key, index), 8 passes of 8 bits, one
+//                launch each with decoupled look-back
 //   3. leaves    a particle's leaf is its first ancestor cell, from the root, that
 //                holds at most max_leaf particles; level-21 cells beyond max_leaf
 //                are cut into chunks of max_leaf.  Since that cell contains the
 //                particle and at most max_leaf particles, its extent is found by
 //                binary searches inside a window of +-(max_leaf + 1) sorted keys.
-//   4. tree      a binary radix tree over the leaf cell keys (Karras 2012, equal
-//                keys ordered by leaf index) with bottom-up bounding boxes
-//   5. pairs     per target leaf and periodic image, a traversal that keeps every leaf whose box comes closer than r_c.  A node's box
+//   4. groups    boxes of 32 consecutive leaves, of 32 such groups, and so on
+//   5. pairs     per target leaf and periodic image, a walk of the groups that
+//                keeps every leaf whose box comes closer than r_c.  A group's box
 //                contains its leaves' boxes, so the kept set is exactly the set of
-//                leaves that pass the leaf test, which the host's octree keeps too;
-//                the left-first order visits them in leaf order like the host's
-//                Morton-ordered octree walk.  Counted in one pass, which also
-//                stores each row in a pair cache of 16 words per particle; after
-//                a prefix sum of the counts the cached rows are copied into
-//                place and only the rows the cache could not hold are walked a
-//                second time (the multipole split walks twice).  The walk prunes with
+//                leaves that pass the leaf test, which the host's octree keeps too,
+//                in leaf order like the host's Morton-ordered octree walk.
+//                Counted in one pass, which also stores each row in a pair cache
+//                of 16 words per particle; after a prefix sum of the counts the
+//                cached rows are copied into place and only the rows the cache
+//                could not hold are walked a second time.  The walk prunes with
 //                FP32 bounds (directed rounding) and falls back to the host's FP64
 //                leaf test only where the bounds cannot decide (gap^2 within about
 //                1e-5 of the cutoff): FP64 throughput on this part is 1/64 of FP32.
@@ -47,16 +47,12 @@ void set_last_error(const std::string& msg);
 
 namespace {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per block
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;  // 4096 values per block
-constexpr int64_t kScanMaxTiles = 65536;              // the top level scans in one block
 constexpr int kMaxLevels = 7;                         // of the groups: 32^6 > 2^28 leaves
 constexpr int kDefaultTimeoutMs = 60000;
-constexpr int64_t kMaxN = (int64_t)1 << 28;           // scan limit: 65536 tiles of 4096
+constexpr int64_t kMaxN = (int64_t)1 << 28;           // digit counts fit the look-back words' 30 bits
 
 // counters in the scratch (int64 words)
 enum : int {
@@ -65,7 +61,7 @@ enum : int {
     kCntEvaluated = 2,
     kCntMaxCost = 3,
     kCntMaxRow = 4,
-    kCntError = 5,  // bit 0 non-finite input, bit 1 stack overflow, bit 2 malformed tree
+    kCntError = 5,  // bit 0 non-finite input, bit 1 stack overflow, bit 2 malformed tree, bit 3 a look-back that ran out
     kCntFar = 6,    // well-separated (M2L) entries of the multipole split
     kCntUncached = 7,  // rows the pair cache could not hold (re-walked by the write pass)
     kCntMassDiff = 8,  // nonzero if some particle's mass differs from particle 0's
@@ -84,57 +80,9 @@ constexpr int kMinRuns = 16;
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Scratch regions (byte offsets); leaf arrays are sized for n leaves (max_leaf 1).
-struct Scratch {
-    size_t wpos, key0, key1, val0, val1, flag, lid, lfirst, llevel, lkey, lbox, lcnt,
-        lfar, lout, lcost, lkey2, lfirst2, llevel2, psize, groups, hist, tiles, total, cnt,
-        lruns, cache, bytes;
-    int64_t ncache;  // pair cache capacity in runs
-};
-
-Scratch scratch_layout(int64_t n)
-{
-    Scratch s{};
-    size_t o = 0;
-    const size_t N = (size_t)(n > 0 ? n : 1);
-    const size_t nb = (N + kSortTile - 1) / kSortTile;
-    const size_t hist = 256 * nb;
-    const size_t big = hist > N + 1 ? hist : N + 1;  // longest scanned array
-    const size_t ntiles = (big + kScanTile - 1) / kScanTile;
-    s.wpos = o;   o = a256(o + 32 * N);  // x, y, z, m (wrapped, FP64)
-    s.key0 = o;   o = a256(o + 8 * N);
-    s.key1 = o;   o = a256(o + 8 * N);
-    s.val0 = o;   o = a256(o + 4 * N);
-    s.val1 = o;   o = a256(o + 4 * N);
-    s.flag = o;   o = a256(o + 8 * N);
-    s.lid = o;    o = a256(o + 8 * N);
-    s.lfirst = o; o = a256(o + 4 * (N + 1));
-    s.llevel = o; o = a256(o + 4 * N);
-    s.lkey = o;   o = a256(o + 8 * N);
-    s.lbox = o;   o = a256(o + 48 * N);
-    s.lcnt = o;   o = a256(o + 8 * N);
-    s.lfar = o;   o = a256(o + 8 * N);   // far entries per leaf (multipole split)
-    s.lout = o;   o = a256(o + 32 * N);  // FP32 leaf box rounded outward, count, rho
-    s.lcost = o;  o = a256(o + 8 * N);
-    s.lkey2 = o;  o = a256(o + 8 * N);   // packed leaves, before they take the places of the plain ones
-    s.lfirst2 = o; o = a256(o + 4 * (N + 1));
-    s.llevel2 = o; o = a256(o + 4 * N);
-    s.psize = o;  o = a256(o + 4 * N);
-    s.groups = o; o = a256(o + 32 * (N / 31 + 2 * kMaxLevels));  // boxes of the groups of all levels
-    s.hist = o;   o = a256(o + 8 * hist);
-    s.tiles = o;  o = a256(o + 8 * ntiles);
-    s.total = o;  o = a256(o + 8);
-    s.cnt = o;    o = a256(o + 8 * kCntWords);
-    s.lruns = o;  o = a256(o + 4 * N);   // runs cached per row (-1: not cached)
-    s.ncache = (int64_t)(kCacheWordsPerParticle / 2 * N);
-    s.cache = o;  o = a256(o + 8 * (size_t)s.ncache);  // uint2 (first leaf << 5 | code, length)
-    s.bytes = o;
-    return s;
-}
-
 struct BoxK {
     double L, scale, unit, inv2rs, rc2m;  // rc2m = r_c^2 (1 + 1e-5), the host's margin
-    float thi, tlo;  // FP32 thresholds: thi >= rc2m (1 + 1e-6), tlo <= rc2m (1 - 1e-6)
+    float thi, tlo;  // FP32 thresholds of the walk, above and below rc2m (box_k)
     float theta2;    // multipole split: theta^2 (0: no split)
     float gt2;       //   and theta^2 (2 r_s^2)^2 (the Gaussian length of the kernel)
     float rc2far;    // FP32 at most r_c^2 (1 - 1e-6): a far pair lies wholly inside the cutoff
@@ -190,47 +138,48 @@ __device__ __forceinline__ double gap2_d(const double* A, const double* B, const
     return s;
 }
 
-// ------------------------------------------------------------------ scan --
-// Exclusive prefix sum of int64 values: tile sums, one block scanning the tile
-// sums, then tile scans with their offsets.  In-place use (in == out) is safe.
+// ------------------------------------------------- single-pass scan and sort --
+// Tiles of one launch pass their prefixes on: a block takes the next tile by a
+// ticket, so every earlier tile has started; it publishes its own total, then
+// adds up the published totals behind it until it meets a published prefix
+// (decoupled look-back, Merrill and Garland 2016).  The waits are bounded: one
+// that runs out sets error bit 3 (of the build's counters, and the
+// build fails, or of the workspace's error word).
+// The control words are zeroed by one memset per build call.
+constexpr int kSpinLimit = 1 << 22;
+constexpr unsigned kSumReady = 1u << 30, kPrefixReady = 2u << 30, kValueMask = kSumReady - 1;
 
-__global__ void __launch_bounds__(1024) k_scan_tiles(const int64_t* in, int64_t m,
-                                                     int64_t* __restrict__ sums)
+// Waits for a published word of the current look-back step; 0 when the wait
+// runs out: the look-back then stops, with a prefix that is too small, so that
+// every position formed from it still lies inside its array.
+__device__ __forceinline__ unsigned wait_word(const volatile unsigned* p, unsigned* err)
 {
-    __shared__ int64_t red[kScanThreads / 32];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    int64_t v = 0;
-    for (int k = 0; k < kScanItems; ++k) {
-        const int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
-        if (i < m) v += in[i];
+    for (int k = 0; k < kSpinLimit; ++k) {
+        const unsigned v = *p;
+        if (v & (kSumReady | kPrefixReady)) return v;
     }
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        v = red[threadIdx.x];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-        if (threadIdx.x == 0) sums[blockIdx.x] = v;
-    }
+    atomicOr(err, 8u);
+    return 0u;
 }
 
-// Block-wide exclusive scan of one value per thread (blockDim.x == 1024);
-// returns the block total.
-__device__ int64_t block_exclusive(int64_t v, int64_t* ex, int64_t* sh)
+// Block-wide exclusive scan of one value per thread (blockDim.x a multiple of
+// 32, at most 1024); sh has 33 words.  Returns the block total.
+template <class T>
+__device__ T block_exclusive(T v, T* ex, T* sh)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int64_t inc = v;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    T inc = v;
     for (int o = 1; o < 32; o <<= 1) {
-        const int64_t t = __shfl_up_sync(kFull, inc, o);
+        const T t = __shfl_up_sync(kFull, inc, o);
         if (lane >= o) inc += t;
     }
     if (lane == 31) sh[w] = inc;
     __syncthreads();
     if (w == 0) {
-        const int64_t s = sh[lane];
-        int64_t si = s;
+        const T s = lane < nw ? sh[lane] : T(0);
+        T si = s;
         for (int o = 1; o < 32; o <<= 1) {
-            const int64_t t = __shfl_up_sync(kFull, si, o);
+            const T t = __shfl_up_sync(kFull, si, o);
             if (lane >= o) si += t;
         }
         sh[lane] = si - s;
@@ -238,34 +187,27 @@ __device__ int64_t block_exclusive(int64_t v, int64_t* ex, int64_t* sh)
     }
     __syncthreads();
     *ex = inc - v + sh[w];
-    const int64_t total = sh[32];
+    const T total = sh[32];
     __syncthreads();
     return total;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_top(int64_t* __restrict__ sums, int64_t nt,
-                                                   int64_t* __restrict__ total)
-{
-    __shared__ int64_t sh[33];
-    const int64_t per = (nt + kScanThreads - 1) / kScanThreads;
-    const int64_t b = (int64_t)threadIdx.x * per, e = b + per < nt ? b + per : nt;
-    int64_t v = 0;
-    for (int64_t k = b; k < e; ++k) v += sums[k];
-    int64_t ex;
-    const int64_t t = block_exclusive(v, &ex, sh);
-    for (int64_t k = b; k < e; ++k) {
-        const int64_t c = sums[k];
-        sums[k] = ex;
-        ex += c;
-    }
-    if (threadIdx.x == 0) *total = t;
-}
+// Control of one scan: ticket, then per tile a state word and two sums.
+struct ScanCtl {
+    unsigned* ticket;   // zeroed, followed by the tile states (zeroed)
+    int64_t* sums;      // 2 per tile: own total, prefix through the tile
+};
 
-__global__ void __launch_bounds__(1024) k_scan_apply(const int64_t* in, int64_t m,
-                                                     const int64_t* __restrict__ sums, int64_t* out)
+// Exclusive prefix sum of int64 values (in == out is safe), the total at *total.
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int64_t* in, int64_t m, int64_t* out,
+                                                       int64_t* total, ScanCtl ctl, unsigned* err)
 {
     __shared__ int64_t sh[33];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+    __shared__ int64_t s_prefix;
+    __shared__ unsigned s_tile;
+    if (threadIdx.x == 0) s_tile = atomicAdd(ctl.ticket, 1u);
+    __syncthreads();
+    const int64_t tile = s_tile, base = tile * kScanTile + (int64_t)threadIdx.x * kScanItems;
     int64_t loc[kScanItems], v = 0;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
@@ -273,8 +215,40 @@ __global__ void __launch_bounds__(1024) k_scan_apply(const int64_t* in, int64_t 
         v += loc[k];
     }
     int64_t ex;
-    block_exclusive(v, &ex, sh);
-    ex += sums[blockIdx.x];
+    const int64_t sum = block_exclusive(v, &ex, sh);
+    unsigned* const state = ctl.ticket + 1;
+    if (threadIdx.x < 32) {  // 32 earlier tiles at a time
+        const int lane = threadIdx.x;
+        volatile int64_t* sums = ctl.sums;
+        if (lane == 0 && tile > 0) {
+            sums[2 * tile] = sum;
+            __threadfence();
+            *(volatile unsigned*)(state + tile) = kSumReady;
+        }
+        int64_t prefix = 0;
+        for (int64_t t0 = tile - 1; t0 >= 0; t0 -= 32) {
+            const int64_t t = t0 - lane;
+            const unsigned s = t >= 0 ? wait_word(state + t, err) : kPrefixReady;
+            __threadfence();
+            const unsigned done = __ballot_sync(kFull, !s || (s & kPrefixReady));
+            const int stop = done ? __ffs(done) - 1 : 32;  // the nearest tile whose prefix is known
+            int64_t v = 0;
+            if (t >= 0 && lane < stop) v = sums[2 * t];
+            if (t >= 0 && lane == stop && s) v = sums[2 * t + 1];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+            prefix += v;
+            if (done) break;
+        }
+        if (lane == 0) {
+            sums[2 * tile + 1] = prefix + sum;
+            __threadfence();
+            *(volatile unsigned*)(state + tile) = kPrefixReady;
+            s_prefix = prefix;
+            if (tile == (m + kScanTile - 1) / kScanTile - 1) *total = prefix + sum;
+        }
+    }
+    __syncthreads();
+    ex += s_prefix;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         if (base + k < m) out[base + k] = ex;
@@ -282,118 +256,298 @@ __global__ void __launch_bounds__(1024) k_scan_apply(const int64_t* in, int64_t 
     }
 }
 
-int scan_exclusive(const int64_t* in, int64_t* out, int64_t m, int64_t* tiles, int64_t* total,
+int64_t scan_tiles(int64_t m) { return (m + kScanTile - 1) / kScanTile; }
+
+int scan_exclusive(const int64_t* in, int64_t* out, int64_t m, int64_t* total, ScanCtl ctl, unsigned* err,
                    cudaStream_t st)
 {
-    const int64_t nt = (m + kScanTile - 1) / kScanTile;
-    if (nt > kScanMaxTiles) return (int)cudaErrorInvalidValue;
-    if (nt == 0) return (int)cudaMemsetAsync(total, 0, 8, st);
-    k_scan_tiles<<<(unsigned)nt, kScanThreads, 0, st>>>(in, m, tiles);
-    k_scan_top<<<1, kScanThreads, 0, st>>>(tiles, nt, total);
-    k_scan_apply<<<(unsigned)nt, kScanThreads, 0, st>>>(in, m, tiles, out);
+    k_scan<<<(unsigned)scan_tiles(m), kScanThreads, 0, st>>>(in, m, out, total, ctl, err);
     return (int)cudaGetLastError();
 }
 
-// ------------------------------------------------------------ radix sort --
-// Stable LSD radix sort of (64-bit key, int32 value), 8 bits per pass.  Per
-// pass: digit counts per tile (digit-major), their exclusive scan, and a
-// stable scatter: item t of a tile is w*256 + it*32 + lane, ranked warp by
-// warp, iteration by iteration and lane by lane, i.e. in item order.
+// Stable LSD radix sort of (64-bit key, int32 value), 8 bits per pass.  One
+// launch counts the digits of all passes; each pass is one launch whose tiles
+// (4096 items: 256 threads, item t = 512 warp + 32 it + lane) rank their items
+// by digit in item order (32 at a time, by votes), put them in digit order in
+// shared memory, learn their digits' offsets by look-back (thread d: digit d)
+// and write runs of a digit.  2.1 M keys, 8 passes: 40 launches and 0.52 ms
+// with counts per tile and their scan before each pass.
+// Up to 8192 items sort in one launch of one block, all passes in shared memory.
+constexpr int kSortItems = 16, kSortThreads = 256, kSortTile = kSortItems * kSortThreads;
+constexpr int kSmallItems = 8, kSmallThreads = 1024, kSmallTile = kSmallItems * kSmallThreads;
 
-__device__ __forceinline__ int64_t tile_item(int w, int it, int lane)
-{
-    return (int64_t)w * (kSortItems * 32) + it * 32 + lane;
-}
+struct SortCtl {
+    unsigned* hist;    // zeroed: 8 x 256 digit counts, then 8 tickets, then per pass 256 words per tile
+    int64_t tiles;     // tiles the status words were sized for
+};
+__host__ __device__ inline int64_t sort_ctl_words(int passes, int64_t tiles) { return 2048 + 8 + 256 * tiles * passes; }
+int64_t sort_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* __restrict__ keys,
-                                                             int64_t n, int shift,
-                                                             int64_t* __restrict__ hist,
-                                                             int64_t nblocks)
+__global__ void __launch_bounds__(256) k_sort_hist(const uint64_t* __restrict__ keys, int64_t n, int passes,
+                                                   unsigned* __restrict__ hist)
 {
-    __shared__ unsigned cnt[256];
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) cnt[d] = 0;
+    __shared__ unsigned cnt[8][256];
+    for (int d = threadIdx.x; d < 2048; d += blockDim.x) cnt[d >> 8][d & 255] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    for (int it = 0; it < kSortItems; ++it) {
-        const int64_t j = base + tile_item(w, it, lane);
-        if (j < n) atomicAdd(&cnt[(keys[j] >> shift) & 255], 1u);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = keys[i];
+        for (int p = 0; p < passes; ++p) atomicAdd(&cnt[p][(k >> (8 * p)) & 255], 1u);
     }
     __syncthreads();
-    for (int d = threadIdx.x; d < 256; d += blockDim.x)
-        hist[(int64_t)d * nblocks + blockIdx.x] = cnt[d];
+    for (int d = threadIdx.x; d < 256 * passes; d += blockDim.x)
+        if (cnt[d >> 8][d & 255]) atomicAdd(hist + d, cnt[d >> 8][d & 255]);
 }
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
-    const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin, uint64_t* __restrict__ kout,
-    int32_t* __restrict__ vout, int64_t n, int shift, const int64_t* __restrict__ off,
-    int64_t nblocks)
+// Ranks of a thread's items among the warp's items of the same digit before
+// them, and the warp's digit counts in whist.
+template <int ITEMS>
+__device__ __forceinline__ void rank_items(const uint64_t* key, int shift, unsigned* whist, unsigned* rank)
 {
-    __shared__ unsigned whist[kSortThreads / 32][256];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int d = lane; d < 256; d += 32) whist[w][d] = 0;
-    __syncwarp();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const unsigned d = (unsigned)(key[it] >> shift) & 255u;
+        unsigned peers = kFull;  // lanes with the same digit, by eight votes
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const bool on = (d >> b) & 1u;
+            const unsigned v = __ballot_sync(kFull, on);
+            peers &= on ? v : ~v;
+        }
+        const unsigned before = whist[d];
+        rank[it] = before + __popc(peers & lt);
+        __syncwarp();
+        if (!(peers & lt)) whist[d] = before + __popc(peers);
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(kSortThreads, 3) k_sort_pass(const uint64_t* __restrict__ kin,
+                                                            const int32_t* __restrict__ vin,
+                                                            uint64_t* __restrict__ kout, int32_t* __restrict__ vout,
+                                                            int64_t n, int pass, SortCtl ctl, unsigned* err)
+{
+    extern __shared__ __align__(16) unsigned char smem_sort[];
+    uint64_t* skey = reinterpret_cast<uint64_t*>(smem_sort);
+    int32_t* sval = reinterpret_cast<int32_t*>(skey + kSortTile);
+    unsigned (*whist)[256] = reinterpret_cast<unsigned (*)[256]>(sval + kSortTile);  // 8 warps
+    __shared__ unsigned s_scan[33], s_start[256], s_tile;
+    __shared__ int64_t s_base[256];  // global position of the tile's first item of each digit, minus s_start
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, shift = 8 * pass;
+    unsigned* tickets = ctl.hist + 2048;
+    if (tid == 0) s_tile = atomicAdd(tickets + pass, 1u);
+    for (int d = tid; d < 2048; d += kSortThreads) whist[d >> 8][d & 255] = 0;
+    __syncthreads();
+    const int64_t tile = s_tile, t0 = tile * kSortTile;
+    const int count = (int)(n - t0 < kSortTile ? n - t0 : kSortTile);
     uint64_t key[kSortItems];
     int32_t val[kSortItems];
     unsigned rank[kSortItems];
-    const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
-        const int64_t j = base + tile_item(w, it, lane);
-        const bool ok = j < n;
-        key[it] = ok ? kin[j] : 0;
-        val[it] = ok ? vin[j] : 0;
-        const unsigned d = ok ? (unsigned)((key[it] >> shift) & 255) : 256u;
-        const unsigned peers = __match_any_sync(kFull, d);
-        rank[it] = ok ? whist[w][d] + __popc(peers & lt) : 0u;
-        __syncwarp();
-        if (ok && lane == __ffs(peers) - 1) whist[w][d] += __popc(peers);
-        __syncwarp();
+        const int t = w * (kSortItems * 32) + it * 32 + lane;
+        // items beyond the end: the last digit's last
+        key[it] = t < count ? kin[t0 + t] : ~0ULL;
+        val[it] = t < count ? vin[t0 + t] : 0;
     }
+    rank_items<kSortItems>(key, shift, whist[w], rank);
     __syncthreads();
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) {  // exclusive over warps, per digit
-        unsigned s = 0;
-        for (int k = 0; k < kSortThreads / 32; ++k) {
-            const unsigned c = whist[k][d];
-            whist[k][d] = s;
-            s += c;
+    unsigned total = 0;  // of digit tid in the tile; whist: before each warp
+#pragma unroll
+    for (int k = 0; k < kSortThreads / 32; ++k) {
+        const unsigned c = whist[k][tid];
+        whist[k][tid] = total;
+        total += c;
+    }
+    const unsigned real = tid == 255 ? total - (unsigned)(kSortTile - count) : total;
+    volatile unsigned* status = ctl.hist + 2048 + 8 + 256 * (ctl.tiles * pass + tile);
+    status[tid] = (tile == 0 ? kPrefixReady : kSumReady) | real;
+    unsigned start;
+    block_exclusive(total, &start, s_scan);
+    unsigned gstart;  // items of smaller digits in the whole input
+    block_exclusive(ctl.hist[256 * pass + tid], &gstart, s_scan);
+    s_start[tid] = start;
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kSortItems; ++it) {
+        const unsigned d = (unsigned)(key[it] >> shift) & 255u;
+        const unsigned pos = s_start[d] + whist[w][d] + rank[it];
+        skey[pos] = key[it];
+        sval[pos] = val[it];
+    }
+    // items of digit tid in earlier tiles, 16 of them read at a time: with all
+    // tiles of a mid-sized sort resident at once, few prefixes are known early
+    // and a tile adds up most of the totals before it
+    unsigned prefix = 0;
+    const unsigned* words = ctl.hist + 2048 + 8 + 256 * ctl.tiles * pass + tid;
+    for (int64_t t = tile - 1; t >= 0; t -= 16) {
+        unsigned s[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            s[k] = t >= k ? *(const volatile unsigned*)(words + 256 * (t - k)) : kPrefixReady;
+        bool done = false;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (!done) {
+                if (!(s[k] & (kSumReady | kPrefixReady))) s[k] = wait_word(words + 256 * (t - k), err);
+                prefix += s[k] & kValueMask;
+                done = !s[k] || (s[k] & kPrefixReady);
+            }
+        if (done) break;
+    }
+    if (tile > 0) status[tid] = kPrefixReady | (prefix + real);
+    s_base[tid] = (int64_t)gstart + prefix - start;
+    __syncthreads();
+    for (int i = tid; i < count; i += kSortThreads) {
+        const uint64_t k = skey[i];
+        const int64_t pos = s_base[(unsigned)(k >> shift) & 255u] + i;
+        kout[pos] = k;
+        vout[pos] = sval[i];
+    }
+}
+constexpr size_t kSortSmem = (size_t)kSortTile * 12 + 8 * 256 * 4;
+
+__global__ void __launch_bounds__(kSmallThreads) k_sort_small(uint64_t* __restrict__ keys, int32_t* __restrict__ vals,
+                                                              int n, int passes)
+{
+    extern __shared__ __align__(16) unsigned char smem_sort[];
+    uint64_t* skey = reinterpret_cast<uint64_t*>(smem_sort);
+    int32_t* sval = reinterpret_cast<int32_t*>(skey + kSmallTile);
+    unsigned (*whist)[256] = reinterpret_cast<unsigned (*)[256]>(sval + kSmallTile);  // 32 warps
+    __shared__ unsigned s_scan[33], s_start[256];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+    uint64_t key[kSmallItems];
+    int32_t val[kSmallItems];
+    unsigned rank[kSmallItems];
+#pragma unroll
+    for (int it = 0; it < kSmallItems; ++it) {
+        const int t = w * (kSmallItems * 32) + it * 32 + lane;
+        key[it] = t < n ? keys[t] : ~0ULL;  // beyond the end: stay last in every pass
+        val[it] = t < n ? vals[t] : 0;
+    }
+    for (int p = 0; p < passes; ++p) {
+        const int shift = 8 * p;
+        for (int d = tid; d < nw * 256; d += blockDim.x) whist[d >> 8][d & 255] = 0;
+        __syncthreads();
+        rank_items<kSmallItems>(key, shift, whist[w], rank);
+        __syncthreads();
+        unsigned total = 0, start;
+        if (tid < 256)
+            for (int k = 0; k < nw; ++k) {
+                const unsigned c = whist[k][tid];
+                whist[k][tid] = total;
+                total += c;
+            }
+        block_exclusive(total, &start, s_scan);
+        if (tid < 256) s_start[tid] = start;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < kSmallItems; ++it) {
+            const unsigned d = (unsigned)(key[it] >> shift) & 255u;
+            const unsigned pos = s_start[d] + whist[w][d] + rank[it];
+            skey[pos] = key[it];
+            sval[pos] = val[it];
         }
-    }
-    __syncthreads();
+        __syncthreads();
 #pragma unroll
-    for (int it = 0; it < kSortItems; ++it) {
-        const int64_t j = base + tile_item(w, it, lane);
-        if (j < n) {
-            const unsigned d = (unsigned)((key[it] >> shift) & 255);
-            const int64_t pos = off[(int64_t)d * nblocks + blockIdx.x] + whist[w][d] + rank[it];
-            kout[pos] = key[it];
-            vout[pos] = val[it];
+        for (int it = 0; it < kSmallItems; ++it) {
+            const int t = w * (kSmallItems * 32) + it * 32 + lane;
+            key[it] = skey[t];
+            val[it] = sval[t];
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int it = 0; it < kSmallItems; ++it) {
+        const int t = w * (kSmallItems * 32) + it * 32 + lane;
+        if (t < n) {
+            keys[t] = key[it];
+            vals[t] = val[it];
         }
     }
 }
+constexpr size_t kSmallSmem = (size_t)kSmallTile * 12 + 32 * 256 * 4;
 
-// Sorts on bits [0, bits) of the keys (bits <= 64); the result ends in (k0, v0).
-int radix_sort(uint64_t* k0, int32_t* v0, uint64_t* k1, int32_t* v1, int64_t n, int bits,
-               int64_t* hist, int64_t* tiles, int64_t* total, cudaStream_t st)
+// Sorts on bits [0, bits) of the keys (bits <= 64) from (k0, v0), with (k1, v1)
+// as the other buffers; the result is in (*kr, *vr).
+int radix_sort(uint64_t* k0, int32_t* v0, uint64_t* k1, int32_t* v1, int64_t n, int bits, SortCtl ctl,
+               unsigned* err, uint64_t** kr, int32_t** vr, cudaStream_t st)
 {
+    *kr = k0;
+    *vr = v0;
     if (n <= 1) return 0;
-    const int64_t nb = (n + kSortTile - 1) / kSortTile;
-    int passes = (bits + 7) / 8;
-    if (passes & 1) ++passes;  // an even count leaves the result in (k0, v0); <= 8
-    for (int p = 0; p < passes; ++p) {
-        const int shift = 8 * p;
-        uint64_t* ki = (p & 1) ? k1 : k0;
-        int32_t* vi = (p & 1) ? v1 : v0;
-        uint64_t* ko = (p & 1) ? k0 : k1;
-        int32_t* vo = (p & 1) ? v0 : v1;
-        k_radix_hist<<<(unsigned)nb, kSortThreads, 0, st>>>(ki, n, shift, hist, nb);
-        int e = scan_exclusive(hist, hist, 256 * nb, tiles, total, st);
-        if (e) return e;
-        k_radix_scatter<<<(unsigned)nb, kSortThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, nb);
-        if ((e = (int)cudaGetLastError())) return e;
+    const int passes = (bits + 7) / 8;
+    cudaError_t e;
+    if (n <= kSmallTile) {
+        e = cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
+        if (e != cudaSuccess) return (int)e;
+        // as many warps as the items fill, at least one thread per digit
+        const int warps = (int)((n + 32 * kSmallItems - 1) / (32 * kSmallItems));
+        k_sort_small<<<1, 32 * (warps > 8 ? warps : 8), kSmallSmem, st>>>(k0, v0, (int)n, passes);
+        return (int)cudaGetLastError();
     }
-    return 0;
+    e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortSmem);
+    if (e != cudaSuccess) return (int)e;
+    const unsigned nb = (unsigned)sort_tiles(n);
+    k_sort_hist<<<nb < 1216 ? nb : 1216, 256, 0, st>>>(k0, n, passes, ctl.hist);
+    for (int p = 0; p < passes; ++p) {
+        k_sort_pass<<<nb, kSortThreads, kSortSmem, st>>>(*kr, *vr, *kr == k0 ? k1 : k0, *vr == v0 ? v1 : v0, n, p,
+                                                         ctl, err);
+        *kr = *kr == k0 ? k1 : k0;
+        *vr = *vr == v0 ? v1 : v0;
+    }
+    return (int)cudaGetLastError();
+}
+
+// Scratch regions (byte offsets); leaf arrays are sized for n leaves (max_leaf 1).
+struct Scratch {
+    size_t wpos, key0, key1, val0, val1, flag, lid, lfirst, llevel, lkey, lbox, lcnt,
+        lfar, lout, lcost, lkey2, lfirst2, llevel2, psize, groups, sums, total, cnt, sort, scan0, scan1, zero_end,
+        lruns, cache, bytes;
+    int64_t ncache;  // pair cache capacity in runs
+};
+
+Scratch scratch_layout(int64_t n)
+{
+    Scratch s{};
+    size_t o = 0;
+    const size_t N = (size_t)(n > 0 ? n : 1);
+    const size_t nt = (N + kScanTile - 1) / kScanTile;
+    s.wpos = o;   o = a256(o + 32 * N);  // x, y, z, m (wrapped, FP64)
+    s.key0 = o;   o = a256(o + 8 * N);
+    s.key1 = o;   o = a256(o + 8 * N);
+    s.val0 = o;   o = a256(o + 4 * N);
+    s.val1 = o;   o = a256(o + 4 * N);
+    s.flag = o;   o = a256(o + 8 * N);
+    s.lid = o;    o = a256(o + 8 * N);
+    s.lfirst = o; o = a256(o + 4 * (N + 1));
+    s.llevel = o; o = a256(o + 4 * N);
+    s.lkey = o;   o = a256(o + 8 * N);
+    s.lbox = o;   o = a256(o + 48 * N);
+    s.lcnt = o;   o = a256(o + 8 * N);
+    s.lfar = o;   o = a256(o + 8 * N);   // far entries per leaf (multipole split)
+    s.lout = o;   o = a256(o + 32 * N);  // FP32 leaf box rounded outward, count, rho
+    s.lcost = o;  o = a256(o + 8 * N);
+    s.lkey2 = o;  o = a256(o + 8 * N);   // packed leaves, before they take the places of the plain ones
+    s.lfirst2 = o; o = a256(o + 4 * (N + 1));
+    s.llevel2 = o; o = a256(o + 4 * N);
+    s.psize = o;  o = a256(o + 4 * N);
+    s.groups = o; o = a256(o + 32 * (N / 31 + 2 * kMaxLevels));  // boxes of the groups of all levels
+    s.sums = o;   o = a256(o + 2 * 16 * nt);  // two scans' tile sums
+    s.total = o;  o = a256(o + 8);
+    // zeroed at the start of each build call: counters, then the control words
+    // of a sort and of two scans
+    s.cnt = o;    o = a256(o + 8 * kCntWords);
+    s.sort = o;   o = a256(o + 4 * (size_t)sort_ctl_words(8, (int64_t)((N + kSortTile - 1) / kSortTile)));
+    s.scan0 = o;  o = a256(o + 4 * (1 + nt));
+    s.scan1 = o;  o = a256(o + 4 * (1 + nt));
+    s.zero_end = o;
+    s.lruns = o;  o = a256(o + 4 * N);   // runs cached per row (-1: not cached)
+    s.ncache = (int64_t)(kCacheWordsPerParticle / 2 * N);
+    s.cache = o;  o = a256(o + 8 * (size_t)s.ncache);  // uint2 (first leaf << 5 | code, length)
+    s.bytes = o;
+    return s;
 }
 
 // -------------------------------------------------------- keys and leaves --
@@ -451,45 +605,52 @@ __device__ __forceinline__ uint64_t cell_prefix(uint64_t k, int level)
     return sh >= 64 ? 0ULL : (k >> sh) << sh;
 }
 
-// [a, b) = the sorted indices of i's level-`level` cell, searched in [lo, hi)
-__device__ __forceinline__ void cell_range(const uint64_t* __restrict__ key, int64_t i, int level,
-                                           int64_t lo, int64_t hi, int64_t& a, int64_t& b)
+// levels (0..21) on which two keys share their cell
+__device__ __forceinline__ int shared_levels(uint64_t a, uint64_t b)
 {
-    const int sh = 3 * (kMortonBits - level);
-    const uint64_t p = cell_prefix(key[i], level);
-    a = lower_bound_u64(key, lo, i, p);
-    b = sh >= 63 ? hi : lower_bound_u64(key, i + 1, hi, p + (1ULL << sh));
+    const uint64_t x = a ^ b;
+    return x ? (__clzll((long long)x) - 1) / 3 : kMortonBits;
 }
 
-// Leaf level and leaf-start flag of each sorted particle.  In the window
-// [i - max_leaf - 1, i + max_leaf + 2) a cell's clipped count exceeds
-// max_leaf exactly when its full count does, and is exact when it does not.
-__global__ void k_leaf_level(const uint64_t* __restrict__ key, int64_t n, int max_leaf,
-                             int64_t* __restrict__ flag, int32_t* __restrict__ level)
+// Leaf level and leaf-start flag of each sorted particle.  A cell of level l
+// around particle i holds more than max_leaf particles exactly when some window
+// of max_leaf + 1 consecutive keys that contains i shares its first l levels,
+// so the leaf level is one more than the largest number of levels shared by the
+// ends of such a window: a sliding maximum over the windows that start at
+// i - max_leaf .. i, taken in shared memory by doubling (8 searches of a key
+// window per particle before: 124 us for 2.1 M particles).
+constexpr int kLevelTile = 512;
+__global__ void __launch_bounds__(kLevelTile) k_leaf_level(const uint64_t* __restrict__ key, int64_t n,
+                                                           int max_leaf, int64_t* __restrict__ flag,
+                                                           int32_t* __restrict__ level)
 {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    __shared__ signed char s_max[2][kLevelTile + kMaxLeaf];
+    const int64_t i0 = blockIdx.x * (int64_t)kLevelTile, i = i0 + threadIdx.x;
+    // window starts i0 - max_leaf .. i0 + kLevelTile - 1
+    const int m = kLevelTile + max_leaf;
+    for (int k = threadIdx.x; k < m; k += kLevelTile) {
+        const int64_t j = i0 - max_leaf + k;
+        s_max[0][k] = j >= 0 && j + max_leaf < n ? (signed char)shared_levels(key[j], key[j + max_leaf]) : -1;
+    }
+    __syncthreads();
+    // s_max[cur][k] = max over window starts k .. k + w - 1
+    int cur = 0, w = 1;
+    for (; 2 * w <= max_leaf + 1; w *= 2, cur ^= 1) {
+        for (int k = threadIdx.x; k < m; k += kLevelTile)
+            s_max[cur ^ 1][k] = k + w < m ? max(s_max[cur][k], s_max[cur][k + w]) : s_max[cur][k];
+        __syncthreads();
+    }
     if (i >= n) return;
-    const int64_t lo = i - max_leaf - 1 > 0 ? i - max_leaf - 1 : 0;
-    const int64_t hi = i + max_leaf + 2 < n ? i + max_leaf + 2 : n;
-    int64_t a, b;
-    cell_range(key, i, kMortonBits, lo, hi, a, b);
+    // starts i - max_leaf .. i are k = threadIdx.x .. threadIdx.x + max_leaf
+    const int d = max(s_max[cur][threadIdx.x], s_max[cur][threadIdx.x + max_leaf + 1 - w]);
     bool start;
-    int L;
-    if (b - a > max_leaf) {  // over-full finest cell: chunks of max_leaf from its start
+    int L = d + 1;
+    if (d >= kMortonBits) {  // over-full finest cell: chunks of max_leaf from its start
         L = kMortonBits;
         const int64_t a0 = lower_bound_u64(key, 0, i, key[i]);
         start = ((i - a0) % max_leaf) == 0;
-    } else {  // smallest level whose cell holds at most max_leaf (counts fall with level)
-        int l0 = 0, l1 = kMortonBits;
-        while (l0 < l1) {
-            const int mid = (l0 + l1) >> 1;
-            cell_range(key, i, mid, lo, hi, a, b);
-            if (b - a <= max_leaf) l1 = mid;
-            else l0 = mid + 1;
-        }
-        L = l0;
-        cell_range(key, i, L, lo, hi, a, b);
-        start = i == a;
+    } else {
+        start = i == 0 || shared_levels(key[i - 1], key[i]) < L;
     }
     flag[i] = start ? 1 : 0;
     level[i] = L;
@@ -579,7 +740,7 @@ __global__ void k_pack_fill(const int64_t* __restrict__ pstart, const int64_t* _
                          // deeper sibling subtree can hold keys above the parent's prefix)
 }
 
-// Boxes of the leaves, 16 lanes per leaf.  Wrapped coordinates are not
+// Boxes of the leaves, 8 lanes per leaf (leaves average 20 to 40 particles).  Wrapped coordinates are not
 // negative, so doubles compare as the integers of their bits (integer minima
 // and maxima, off the FP64 pipe; -0.0 counts as the smallest, which equals 0).
 // lbox: the FP64 box.  lout, for the walk and the multipole split: the box
@@ -590,12 +751,12 @@ __global__ void k_leaf_box(const int32_t* __restrict__ lfirst, int64_t nl, int64
                            double* __restrict__ lbox, float4* __restrict__ lout,
                            long long* __restrict__ cnt)
 {
-    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
-    const int sub = threadIdx.x & 15;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    const int sub = threadIdx.x & 7;
     const bool live = g < nl;
     const int64_t f = live ? lfirst[g] : 0, e = !live ? 0 : g + 1 < nl ? lfirst[g + 1] : n;
     long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-    for (int64_t k = f + sub; k < e; k += 16) {
+    for (int64_t k = f + sub; k < e; k += 8) {
         const double2* w = reinterpret_cast<const double2*>(wpos + 4 * (int64_t)idx[k]);
         const double2 xy = w[0], zm = w[1];
         const long long v[3] = {__double_as_longlong(xy.x), __double_as_longlong(xy.y),
@@ -605,7 +766,7 @@ __global__ void k_leaf_box(const int32_t* __restrict__ lfirst, int64_t nl, int64
             hi[a] = max(hi[a], v[a]);
         }
     }
-    for (int o = 8; o > 0; o >>= 1)
+    for (int o = 4; o > 0; o >>= 1)
         for (int a = 0; a < 3; ++a) {
             lo[a] = min(lo[a], __shfl_xor_sync(kFull, lo[a], o));
             hi[a] = max(hi[a], __shfl_xor_sync(kFull, hi[a], o));
@@ -658,53 +819,24 @@ __global__ void k_groups(const float4* __restrict__ below, int64_t n_below, floa
 }
 
 // ----------------------------------------------------------------- pairs --
-// Bounds on the exact gap^2 between a target box A and a box B shifted by
-// sh, in FP32 with every operation rounded toward the bound (shift given
-// rounded down, sd, and up, su).  Lower bound: boxes rounded outward.
-__device__ __forceinline__ float gap2_lower(const float* alo, const float* ahi, const float* blo,
-                                            const float* bhi, const float* sd, const float* su)
+// gap^2 between the target box [alo, ahi] (moved by minus the image's shift) and
+// the box [blo, bhi], and the largest gap^2 of any point of that box, in FP32.
+// Boxes are rounded outward, coordinates and shifts are at most 2 L: each
+// component is off by less than 4 places of L (2^-21 L), the root by less than
+// 2^-20 L, which the thresholds allow for (box_k).
+__device__ __forceinline__ float gap2_f(const float* alo, const float* ahi, float4 blo, float4 bhi)
 {
-    float s = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float d1 = __fsub_rd(__fadd_rd(blo[a], sd[a]), ahi[a]);
-        const float d2 = __fsub_rd(alo[a], __fadd_ru(bhi[a], su[a]));
-        const float g = fmaxf(0.f, fmaxf(d1, d2));
-        s = __fadd_rd(s, __fmul_rd(g, g));
-    }
-    return s;
+    const float x = fmaxf(fmaxf(blo.x - ahi[0], alo[0] - bhi.x), 0.f);
+    const float y = fmaxf(fmaxf(blo.y - ahi[1], alo[1] - bhi.y), 0.f);
+    const float z = fmaxf(fmaxf(blo.z - ahi[2], alo[2] - bhi.z), 0.f);
+    return fmaf(x, x, fmaf(y, y, z * z));
 }
-
-// Upper bound: boxes rounded inward (lo up, hi down).
-__device__ __forceinline__ float gap2_upper(const float* alo, const float* ahi, const float* blo,
-                                            const float* bhi, const float* sd, const float* su)
+__device__ __forceinline__ float maxgap2_f(const float* alo, const float* ahi, float4 blo, float4 bhi)
 {
-    float s = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float d1 = __fsub_ru(__fadd_ru(blo[a], su[a]), ahi[a]);
-        const float d2 = __fsub_ru(alo[a], __fadd_rd(bhi[a], sd[a]));
-        const float g = fmaxf(0.f, fmaxf(d1, d2));
-        s = __fadd_ru(s, __fmul_ru(g, g));
-    }
-    return s;
-}
-
-// Upper bound on the largest gap^2 between A and any point of box B + sh,
-// which bounds the gap^2 of every leaf inside B: B rounded outward, A
-// rounded inward (alo up, ahi down).
-__device__ __forceinline__ float maxgap2_upper(const float* alo, const float* ahi, const float* blo,
-                                               const float* bhi, const float* sd, const float* su)
-{
-    float s = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float e1 = __fsub_ru(__fadd_ru(bhi[a], su[a]), ahi[a]);
-        const float e2 = __fsub_ru(alo[a], __fadd_rd(blo[a], sd[a]));
-        const float g = fmaxf(0.f, fmaxf(e1, e2));
-        s = __fadd_ru(s, __fmul_ru(g, g));
-    }
-    return s;
+    const float x = fmaxf(fmaxf(bhi.x - ahi[0], alo[0] - blo.x), 0.f);
+    const float y = fmaxf(fmaxf(bhi.y - ahi[1], alo[1] - blo.y), 0.f);
+    const float z = fmaxf(fmaxf(bhi.z - ahi[2], alo[2] - blo.z), 0.f);
+    return fmaf(x, x, fmaf(y, y, z * z));
 }
 
 // The multipole split: leaf J + shift is well separated from leaf I when
@@ -753,11 +885,11 @@ __device__ __forceinline__ bool far_pair(const float* alo, const float* ahi, flo
 // it replaces (one thread per leaf over a binary radix tree): 17^3 uniform 820
 // us, 64^3 NFW 930 us, 128^3 NFW 1.2 ms, split 3.26 + 0.65 ms.
 //
-// A member is pruned when the FP32 lower bound of its gap^2 reaches thi (then
-// the host's FP64 test fails for every leaf below); a leaf is kept when the
-// FP32 upper bound is below tlo (then the host's FP64 test passes; the box
-// rounded outward and moved in by one place bounds the box from inside); only
-// the leaves in between take the host's FP64 test itself.
+// A member is pruned when its gap^2 reaches thi (then the host's FP64 test
+// fails for every leaf below) and kept when its (largest) gap^2 is below tlo
+// (then the host's FP64 test passes); only the leaves in between take the
+// host's FP64 test itself.  One FP32 evaluation within known bounds instead of
+// two with directed roundings: 5500 -> 3300 instructions a row.
 //
 // MODE: count (and, given a pair cache of kslot runs per row, record the row's
 // runs: lruns[I] their number, or -1 when the slot is too small), or write a
@@ -785,9 +917,11 @@ struct WalkArgs {
     int kslot;
 };
 
-// x >= 0 moved up or down by one place (0 stays 0 going down)
-__device__ __forceinline__ float next_up(float x) { return __int_as_float(max(__float_as_int(x), 0) + 1); }
-__device__ __forceinline__ float next_down(float x) { return __int_as_float(max(__float_as_int(x), 1) - 1); }
+// component a of an image code's periodic step, -1, 0 or 1
+__device__ __forceinline__ int image_step(uint32_t code, int a)
+{
+    return (int)(a == 0 ? code / 9u : a == 1 ? (code / 3u) % 3u : code % 3u) - 1;
+}
 
 template <bool WRITE, bool SPLIT>
 __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const WalkArgs w)
@@ -799,20 +933,13 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
     const float thi = w.bx.thi, tlo = w.bx.tlo;
     if (threadIdx.x == 0) s_pairs = s_far = s_eval = s_cost = s_row = s_uncached = 0;
     __syncthreads();
-    const float Lrd = __double2float_rd(w.bx.L), Lru = __double2float_ru(w.bx.L);
+    const float Lf = (float)w.bx.L, Lrd = __double2float_rd(w.bx.L), Lru = __double2float_ru(w.bx.L);
     const int W = (int)gridDim.x * kWalkWarps;
     for (int I = (int)blockIdx.x * kWalkWarps + wp; I < nl; I += W) {
         const bool recorded = WRITE && w.lruns && w.lruns[I] >= 0;
         if (WRITE && !SPLIT && recorded) continue;
-        const double* A = w.lbox + 6 * (int64_t)I;
-        float aolo[3], aohi[3], ailo[3], aihi[3];
-        for (int a = 0; a < 3; ++a) {
-            aolo[a] = __double2float_rd(A[a]);
-            aohi[a] = __double2float_ru(A[3 + a]);
-            ailo[a] = __double2float_ru(A[a]);
-            aihi[a] = __double2float_rd(A[3 + a]);
-        }
-        const float ra = SPLIT ? w.box[0][2 * (int64_t)I + 1].w : 0.0f;  // rho of the outward box
+        const float4 t0 = w.box[0][2 * (int64_t)I], t1 = w.box[0][2 * (int64_t)I + 1];
+        const float ra = t1.w;  // rho of the outward box
         long long c = 0, cf = 0;  // entries so far (uniform)
         long long src = 0;        // this lane's part of their particles
         long long at = WRITE ? w.rowptr[I] : 0, fat = WRITE && SPLIT ? w.frowptr[I] : 0;
@@ -823,15 +950,23 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
         int nrun = 0;
         uint32_t run0 = 0, runend = 0xffffffffu;
         uint32_t code = 0;
-        float sd[3], su[3];  // the image's shift rounded down and up
+        float alo[3], ahi[3];  // the target box moved by minus the image's shift
 
         // the leaves of mask M of the 32 from `base` on; b0, b1: this lane's leaf
         auto leaves = [&](unsigned M, int base, float4 b0, float4 b1) {
             if (!M) return;
             const bool mine = (M >> lane) & 1u;
             bool far = false;
-            if (SPLIT && mine)
-                far = far_pair(aolo, aohi, ra, b0, b1, sd, su, w.bx.theta2, w.bx.gt2, w.bx.rc2far);
+            if (SPLIT && mine) {
+                const float tlo3[3] = {t0.x, t0.y, t0.z}, thi3[3] = {t1.x, t1.y, t1.z};
+                float sd[3], su[3];  // the image's shift rounded down and up
+                for (int a = 0; a < 3; ++a) {
+                    const int n = image_step(code, a);
+                    sd[a] = n < 0 ? -Lru : n > 0 ? Lrd : 0.f;
+                    su[a] = n < 0 ? -Lrd : n > 0 ? Lru : 0.f;
+                }
+                far = far_pair(tlo3, thi3, ra, b0, b1, sd, su, w.bx.theta2, w.bx.gt2, w.bx.rc2far);
+            }
             const unsigned F = SPLIT ? __ballot_sync(kFull, far) : 0u, N = M & ~F;
             if (WRITE) {
                 const long long p = far ? fat + __popc(F & lt) : at + __popc(N & lt);
@@ -890,13 +1025,13 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             runend = ((uint32_t)(l + 1) << 5) | code;
             if (lane == 0 && nrun <= w.kslot) slot[nrun - 1] = make_uint2(run0, (runend - run0) >> 5);
         };
-        auto set_shift = [&](uint32_t cd) {
+        auto set_image = [&](uint32_t cd) {
             code = cd;
-            const int s3[3] = {(int)(cd / 9u) - 1, (int)((cd / 3u) % 3u) - 1, (int)(cd % 3u) - 1};
-            for (int a = 0; a < 3; ++a) {
-                sd[a] = s3[a] < 0 ? -Lru : s3[a] > 0 ? Lrd : 0.f;
-                su[a] = s3[a] < 0 ? -Lrd : s3[a] > 0 ? Lru : 0.f;
-            }
+            const float sx = (float)image_step(cd, 0) * Lf, sy = (float)image_step(cd, 1) * Lf,
+                        sz = (float)image_step(cd, 2) * Lf;
+            alo[0] = t0.x - sx; ahi[0] = t1.x - sx;
+            alo[1] = t0.y - sy; ahi[1] = t1.y - sy;
+            alo[2] = t0.z - sz; ahi[2] = t1.z - sz;
         };
         // the 32 leaves from `base` on
         auto test_leaves = [&](int base) {
@@ -906,17 +1041,12 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             if (J < nl) {
                 b0 = w.box[0][2 * (int64_t)J];
                 b1 = w.box[0][2 * (int64_t)J + 1];
-                const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
-                if (gap2_lower(aolo, aohi, blo, bhi, sd, su) < thi) {
-                    const float ilo[3] = {next_up(b0.x), next_up(b0.y), next_up(b0.z)};
-                    const float ihi[3] = {next_down(b1.x), next_down(b1.y), next_down(b1.z)};
-                    keep = gap2_upper(ailo, aihi, ilo, ihi, sd, su) < tlo;
-                    if (!keep) {
-                        const double sh[3] = {((int)(code / 9u) - 1) * w.bx.L,
-                                              ((int)((code / 3u) % 3u) - 1) * w.bx.L,
-                                              ((int)(code % 3u) - 1) * w.bx.L};
-                        keep = gap2_d(A, w.lbox + 6 * (int64_t)J, sh) < w.bx.rc2m;
-                    }
+                const float g2 = gap2_f(alo, ahi, b0, b1);
+                keep = g2 < tlo;
+                if (!keep && g2 < thi) {
+                    const double sh[3] = {image_step(code, 0) * w.bx.L, image_step(code, 1) * w.bx.L,
+                                          image_step(code, 2) * w.bx.L};
+                    keep = gap2_d(w.lbox + 6 * (int64_t)I, w.lbox + 6 * (int64_t)J, sh) < w.bx.rc2m;
                 }
             }
             leaves(__ballot_sync(kFull, keep), base, b0, b1);
@@ -926,24 +1056,23 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             const int n = w.lruns[I];
             for (int r = 0; r < n; ++r) {
                 const uint2 run = slot[r];
-                set_shift(run.x & 31u);
+                set_image(run.x & 31u);
                 range((int)(run.x >> 5), (int)(run.x >> 5) + (int)run.y - 1);
             }
         } else {
             const float4 r0 = w.box[w.top][0], r1 = w.box[w.top][1];
-            const float rlo[3] = {r0.x, r0.y, r0.z}, rhi[3] = {r1.x, r1.y, r1.z};
             bool in = false, all = false;
             if (lane < kShiftCodes) {  // the root at each image
-                set_shift((uint32_t)lane);
-                in = gap2_lower(aolo, aohi, rlo, rhi, sd, su) < thi;
-                all = in && maxgap2_upper(ailo, aihi, rlo, rhi, sd, su) < tlo;
+                set_image((uint32_t)lane);
+                in = gap2_f(alo, ahi, r0, r1) < thi;
+                all = in && maxgap2_f(alo, ahi, r0, r1) < tlo;
             }
             unsigned images = __ballot_sync(kFull, in);
             const unsigned whole = __ballot_sync(kFull, all);
             while (images) {
                 const int image = __ffs(images) - 1;
                 images &= images - 1;
-                set_shift((uint32_t)image);
+                set_image((uint32_t)image);
                 if ((whole >> image) & 1u) {
                     range(0, nl - 1);
                     continue;
@@ -961,9 +1090,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                     bool part = false, full = false;
                     if (g < (int)w.n[t]) {
                         const float4 b0 = w.box[t][2 * (int64_t)g], b1 = w.box[t][2 * (int64_t)g + 1];
-                        const float blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
-                        part = gap2_lower(aolo, aohi, blo, bhi, sd, su) < thi;
-                        full = part && maxgap2_upper(ailo, aihi, blo, bhi, sd, su) < tlo;
+                        part = gap2_f(alo, ahi, b0, b1) < thi;
+                        full = part && maxgap2_f(alo, ahi, b0, b1) < tlo;
                     }
                     const unsigned P = __ballot_sync(kFull, part), K = __ballot_sync(kFull, full);
                     if (lane == t) {
@@ -1109,6 +1237,21 @@ __global__ void k_fcen(const double* __restrict__ lbox, const int4* __restrict__
 }
 
 // --------------------------------------------------------------- payload --
+// (float)x in integer arithmetic: the FP64 pipe's conversion takes as long as
+// its arithmetic.  Round to nearest even; results outside the normal FP32 range
+// (and 0) take the conversion itself.
+__device__ __forceinline__ float to_float(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hi = (unsigned)(b >> 32), e = (hi >> 20) & 0x7ffu;
+    if (e < 1023u - 126u || e > 1023u + 126u) return (float)x;
+    // exponent rebiased, mantissa cut to 23 bits; a carry of the rounding runs into the exponent
+    unsigned f = (unsigned)((b << 1) >> 30) - ((1023u - 127u) << 23);
+    const unsigned rest = (unsigned)b & 0x1fffffffu;
+    f += rest > 0x10000000u || (rest == 0x10000000u && (f & 1u));
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
 // The workspace arrays of one leaf: leaf record, integer cell centre (units
 // L / 2^22), leaf-local FP32 coordinates in units of 2 r_s, FP64 copy, perm.
 __global__ void k_payload(const int32_t* __restrict__ lfirst, const int32_t* __restrict__ llevel,
@@ -1118,8 +1261,8 @@ __global__ void k_payload(const int32_t* __restrict__ lfirst, const int32_t* __r
                           int32_t* __restrict__ perm, int4* __restrict__ leaf,
                           int4* __restrict__ lcen)
 {
-    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;  // 16 lanes per leaf
-    const int sub = threadIdx.x & 15;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;  // 8 lanes per leaf
+    const int sub = threadIdx.x & 7;
     if (g >= nl) return;
     const int64_t f = lfirst[g], e = g + 1 < nl ? lfirst[g + 1] : n;
     const int L = llevel[g];
@@ -1135,13 +1278,13 @@ __global__ void k_payload(const int32_t* __restrict__ lfirst, const int32_t* __r
     }
     const double c[3] = {__dmul_rn((double)cx, bx.unit), __dmul_rn((double)cy, bx.unit),
                          __dmul_rn((double)cz, bx.unit)};
-    for (int64_t q = f + sub; q < e; q += 16) {
+    for (int64_t q = f + sub; q < e; q += 8) {
         const int64_t p = idx[q];
         const double2* w = reinterpret_cast<const double2*>(wpos + 4 * p);
         const double2 xy = w[0], zm = w[1];
-        pf[q] = make_float4((float)__dmul_rn(__dsub_rn(xy.x, c[0]), bx.inv2rs),
-                            (float)__dmul_rn(__dsub_rn(xy.y, c[1]), bx.inv2rs),
-                            (float)__dmul_rn(__dsub_rn(zm.x, c[2]), bx.inv2rs), (float)zm.y);
+        pf[q] = make_float4(to_float(__dmul_rn(__dsub_rn(xy.x, c[0]), bx.inv2rs)),
+                            to_float(__dmul_rn(__dsub_rn(xy.y, c[1]), bx.inv2rs)),
+                            to_float(__dmul_rn(__dsub_rn(zm.x, c[2]), bx.inv2rs)), to_float(zm.y));
         if (pd) pd[q] = make_double4(xy.x, xy.y, zm.x, zm.y);
         perm[q] = (int32_t)p;
     }
@@ -1175,8 +1318,6 @@ __global__ void k_sched_out(const uint64_t* __restrict__ key, const int32_t* __r
     for (int l = 0; l < kHeavyLevels; ++l)
         if (mine > heavy.cost[l] && next <= heavy.cost[l]) n_heavy[l] = (int)(i + 1);
 }
-
-__global__ void k_copy_total(int64_t* dst, const int64_t* src) { *dst = *src; }
 
 // The levels of the groups over nl leaves.
 WalkArgs walk_levels(int64_t nl, const float4* lout, float4* groups)
@@ -1256,8 +1397,11 @@ BoxK box_k(const psr_box& b)
     k.unit = std::ldexp(b.L, -kCentreShift);
     k.inv2rs = 1.0 / (2.0 * b.r_s);
     k.rc2m = b.r_c * b.r_c * (1.0 + 1e-5);
-    k.thi = float_at_least(k.rc2m * (1.0 + 1e-6));
-    k.tlo = float_at_most(k.rc2m * (1.0 - 1e-6));
+    // the walk's thresholds: the FP32 gaps are within 2^-20 L (gap2_f), their
+    // squares' sums within 1e-6
+    const double g = std::sqrt(k.rc2m), slack = std::ldexp(b.L, -20), in = g > slack ? g - slack : 0.0;
+    k.thi = float_at_least((g + slack) * (g + slack) * (1.0 + 1e-6));
+    k.tlo = float_at_most(in * in * (1.0 - 1e-6));
     k.theta2 = 0.0f;
     k.gt2 = 0.0f;
     k.rc2far = float_at_most(b.r_c * b.r_c * (1.0 - 1e-6));
@@ -1323,9 +1467,8 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     float4* lout = (float4*)(s + S.lout);
     int64_t* lcnt = (int64_t*)(s + S.lcnt);
     int64_t* lcost = (int64_t*)(s + S.lcost);
-    int64_t* hist = (int64_t*)(s + S.hist);
-    int64_t* tiles = (int64_t*)(s + S.tiles);
     int64_t* total = (int64_t*)(s + S.total);
+    int64_t* sums = (int64_t*)(s + S.sums);
     long long* cnt = (long long*)(s + S.cnt);
     BoxK bx = box_k(*box);
     bx.theta2 = (float)(theta * theta);
@@ -1333,14 +1476,19 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
                                                : INFINITY;
 
     int e;
-    if ((e = (int)cudaMemsetAsync(cnt, 0, 8 * kCntWords, st))) return dcuda(e, "cudaMemsetAsync");
+    unsigned* const err = (unsigned*)(cnt + kCntError);
+    const SortCtl sctl{(unsigned*)(s + S.sort), sort_tiles(n)};
+    const ScanCtl scan0{(unsigned*)(s + S.scan0), sums}, scan1{(unsigned*)(s + S.scan1), sums + 2 * scan_tiles(n)};
+    if ((e = (int)cudaMemsetAsync(s + S.cnt, 0, S.zero_end - S.cnt, st))) return dcuda(e, "cudaMemsetAsync");
     k_keys<<<nblk(n, 256), 256, 0, st>>>(d_pos, d_mass, n, bx, 1.0 / (double)n, wpos, k0, v0, cnt);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "key kernel");
-    if ((e = radix_sort(k0, v0, k1, v1, n, 3 * kMortonBits, hist, tiles, total, st)))
+    uint64_t* kr;  // (k0, v0): one launch or eight passes
+    int32_t* vr;
+    if ((e = radix_sort(k0, v0, k1, v1, n, 3 * kMortonBits, sctl, err, &kr, &vr, st)))
         return dcuda(e, "radix sort");
-    k_leaf_level<<<nblk(n, 256), 256, 0, st>>>(k0, n, max_leaf, flag, v1);
+    k_leaf_level<<<nblk(n, kLevelTile), kLevelTile, 0, st>>>(k0, n, max_leaf, flag, v1);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf level kernel");
-    if ((e = scan_exclusive(flag, lid, n, tiles, total, st))) return dcuda(e, "scan");
+    if ((e = scan_exclusive(flag, lid, n, total, scan0, err, st))) return dcuda(e, "scan");
     k_leaf_fill<<<nblk(n, 256), 256, 0, st>>>(flag, lid, v1, k0, n, lfirst, llevel, lkey);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf fill kernel");
     long long c[kCntWords];
@@ -1359,7 +1507,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
         uint64_t* lkey2 = (uint64_t*)(s + S.lkey2);
         k_pack_mark<<<nblk(nl, 256), 256, 0, st>>>(lfirst, llevel, lkey, nl, max_leaf, pstart, psize);
         if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf packing kernel");
-        if ((e = scan_exclusive(pstart, pid, nl, tiles, total, st))) return dcuda(e, "scan");
+        if ((e = scan_exclusive(pstart, pid, nl, total, scan1, err, st))) return dcuda(e, "scan");
         k_pack_fill<<<nblk(nl, 256), 256, 0, st>>>(pstart, pid, psize, lfirst, llevel, lkey, nl,
                                                    lfirst2, llevel2, lkey2);
         if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf packing kernel");
@@ -1372,7 +1520,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
             return dcuda(e, "cudaMemcpyAsync");
         nl = np;
     }
-    k_leaf_box<<<nblk(16 * nl, 256), 256, 0, st>>>(lfirst, nl, n, wpos, v0, lbox, lout, cnt);
+    k_leaf_box<<<nblk(8 * nl, 256), 256, 0, st>>>(lfirst, nl, n, wpos, v0, lbox, lout, cnt);
     WalkArgs wa = walk_levels(nl, lout, (float4*)(s + S.groups));
     for (int t = 1; t <= wa.top; ++t)
         k_groups<<<nblk(32 * wa.n[t], 256), 256, 0, st>>>(wa.box[t - 1], wa.n[t - 1],
@@ -1394,7 +1542,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     wa.lcost = lcost;
     wa.lfar = (int64_t*)(s + S.lfar);
     wa.cnt = cnt;
-    wa.err = (unsigned*)(cnt + kCntError);
+    wa.err = err;
     wa.lruns = lruns;
     wa.cache = pcache;
     wa.kslot = kslot;
@@ -1402,8 +1550,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     else k_rows<false, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "pair count kernel");
     if ((e = read_back(c, cnt, sizeof c, st, timeout_ms))) return e;
-    if (c[kCntError] & 2) return dfail(PSR_E_DEVICE, "tree traversal stack overflow");
-    if (c[kCntError] & 4) return dfail(PSR_E_DEVICE, "malformed radix tree");
+    if (c[kCntError] & 12) return dfail(PSR_E_DEVICE, "a row walk or a look-back failed");
     if (c[kCntPairs] >= ((int64_t)1 << 32) || c[kCntFar] >= ((int64_t)1 << 32))
         return dfail(PSR_E_ARG, "more than 2^32 leaf pairs");
 
@@ -1492,7 +1639,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     // word that psr_check reads
     if ((e = (int)cudaMemsetAsync(w + L.ctrl, 0, kCtrlWords * 4, st))) return dcuda(e, "cudaMemsetAsync");
     const int32_t* lfirst = (const int32_t*)(s + S.lfirst);
-    k_payload<<<nblk(16 * nl, 256), 256, 0, st>>>(
+    k_payload<<<nblk(8 * nl, 256), 256, 0, st>>>(
         lfirst, (const int32_t*)(s + S.llevel), (const uint64_t*)(s + S.lkey), nl, n, bx,
         (const double*)(s + S.wpos), (const int32_t*)(s + S.val0), (float4*)(w + L.pf),
         h->has_pd ? (double4*)(w + L.pd) : nullptr, (int32_t*)(w + L.perm), (int4*)(w + L.leaf),
@@ -1500,17 +1647,18 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     if ((e = (int)cudaGetLastError())) return dcuda(e, "payload kernel");
     // row pointers: exclusive scan of the row lengths, then the total
     int64_t* rowptr = (int64_t*)(w + L.rowptr);
-    int64_t* tiles = (int64_t*)(s + S.tiles);
-    int64_t* total = (int64_t*)(s + S.total);
-    if ((e = scan_exclusive((const int64_t*)(s + S.lcnt), rowptr, nl, tiles, total, st)))
+    int64_t* sums = (int64_t*)(s + S.sums);
+    unsigned* const err = (unsigned*)(w + L.ctrl) + kCtrlError;
+    const SortCtl sctl{(unsigned*)(s + S.sort), sort_tiles(n)};
+    const ScanCtl scan0{(unsigned*)(s + S.scan0), sums}, scan1{(unsigned*)(s + S.scan1), sums + 2 * scan_tiles(n)};
+    if ((e = (int)cudaMemsetAsync(s + S.sort, 0, S.zero_end - S.sort, st))) return dcuda(e, "cudaMemsetAsync");
+    if ((e = scan_exclusive((const int64_t*)(s + S.lcnt), rowptr, nl, rowptr + nl, scan0, err, st)))
         return dcuda(e, "scan");
-    k_copy_total<<<1, 1, 0, st>>>(rowptr + nl, total);
     const double* lbox = (const double*)(s + S.lbox);
     int64_t* frow = h->has_far ? (int64_t*)(w + L.frow) : nullptr;
     if (h->has_far) {
-        if ((e = scan_exclusive((const int64_t*)(s + S.lfar), frow, nl, tiles, total, st)))
+        if ((e = scan_exclusive((const int64_t*)(s + S.lfar), frow, nl, frow + nl, scan1, err, st)))
             return dcuda(e, "scan");
-        k_copy_total<<<1, 1, 0, st>>>(frow + nl, total);
         k_fcen<<<nblk(nl, 128), 128, 0, st>>>(lbox, (const int4*)(w + L.lcen), bx.unit, nl,
                                               (double4*)(w + L.fcen), (float4*)(w + L.fofs));
         if ((e = (int)cudaGetLastError())) return dcuda(e, "expansion centre kernel");
@@ -1522,7 +1670,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     wa.rowptr = rowptr;
     wa.frowptr = frow;
     wa.pairs = (uint32_t*)(w + L.pairs);
-    wa.err = (unsigned*)(w + L.ctrl) + kCtrlError;
+    wa.err = err;
     wa.lruns = h->db_kslot ? (int32_t*)(s + S.lruns) : nullptr;
     wa.cache = h->db_kslot ? (uint2*)(s + S.cache) : nullptr;
     wa.kslot = h->db_kslot;
@@ -1552,11 +1700,13 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
                                                 (long long)h->max_cost, k0, v0);
     int bits = 1;
     while (bits < 63 && ((uint64_t)h->max_cost >> bits)) ++bits;
-    if ((e = radix_sort(k0, v0, k1, v1, nl, bits, (int64_t*)(s + S.hist), tiles, total, st)))
+    uint64_t* kr;
+    int32_t* vr;
+    if ((e = radix_sort(k0, v0, k1, v1, nl, bits, sctl, err, &kr, &vr, st)))
         return dcuda(e, "schedule sort");
     HeavyLines heavy;
     for (int l = 0; l < kHeavyLevels; ++l) heavy.cost[l] = heavy_cost(l, h->evaluated, sms);
-    k_sched_out<<<nblk(nl, 256), 256, 0, st>>>(k0, v0, nl, (long long)h->max_cost, heavy,
+    k_sched_out<<<nblk(nl, 256), 256, 0, st>>>(kr, vr, nl, (long long)h->max_cost, heavy,
                                                (int32_t*)(w + L.items), (int*)(w + L.ctrl) + kCtrlHeavy);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "schedule kernel");
     if ((e = (int)cudaMemcpyAsync(w + L.boxes, h->boxdev.data(), sizeof(BoxDev),

@@ -506,7 +506,7 @@ int psr_device_build_split(const double* d_pos, const double* d_mass, int64_t n,
  * psr_pm_create - host: cuFFT plans for an n_pm^3 mesh (n_pm even, in
  *   [8, 1024]); cuFFT may allocate plan data here, never the FFT work area.
  *   Errors: PSR_E_ARG, PSR_E_NOMEM, PSR_E_CUDA.
- * psr_pm_scratch_bytes - host: scratch psr_pm_forces needs (about 28 n_pm^3
+ * psr_pm_scratch_bytes - host: scratch psr_pm_forces needs (about 33 n_pm^3
  *   bytes plus the cuFFT work area).
  * psr_pm_forces - device, asynchronous on cuda_stream, allocates nothing:
  *   d_pos   device, n x 3 FP64, any real values (wrapped into [0, L)); a

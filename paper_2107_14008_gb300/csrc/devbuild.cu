@@ -66,7 +66,9 @@ enum : int {
     kCntUncached = 7,  // rows the pair cache could not hold (re-walked by the write pass)
     kCntMassDiff = 8,  // nonzero if some particle's mass differs from particle 0's
     kCntMass0 = 9,     // particle 0's mass (the bits of a double)
-    kCntWords = 10,
+    kCntLeaves = 10,   // plain octree leaves
+    kCntPacked = 11,   // leaves after packing (kCntLeaves without it)
+    kCntWords = 12,
 };
 
 // The pair cache: the count walk also records each row as runs of
@@ -198,15 +200,18 @@ struct ScanCtl {
     int64_t* sums;      // 2 per tile: own total, prefix through the tile
 };
 
-// Exclusive prefix sum of int64 values (in == out is safe), the total at *total.
-__global__ void __launch_bounds__(kScanThreads) k_scan(const int64_t* in, int64_t m, int64_t* out,
+// Exclusive prefix sum of m int64 values (in == out is safe), or of the first
+// *m_dev <= m; the total at *total.
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int64_t* in, int64_t m, const int64_t* m_dev, int64_t* out,
                                                        int64_t* total, ScanCtl ctl, unsigned* err)
 {
     __shared__ int64_t sh[33];
     __shared__ int64_t s_prefix;
     __shared__ unsigned s_tile;
+    if (m_dev) m = min(m, *m_dev);
     if (threadIdx.x == 0) s_tile = atomicAdd(ctl.ticket, 1u);
     __syncthreads();
+    if ((int64_t)s_tile * kScanTile >= m) return;  // past the end: no tile waits for this one
     const int64_t tile = s_tile, base = tile * kScanTile + (int64_t)threadIdx.x * kScanItems;
     int64_t loc[kScanItems], v = 0;
 #pragma unroll
@@ -258,10 +263,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int64_t* in, int64_
 
 int64_t scan_tiles(int64_t m) { return (m + kScanTile - 1) / kScanTile; }
 
-int scan_exclusive(const int64_t* in, int64_t* out, int64_t m, int64_t* total, ScanCtl ctl, unsigned* err,
-                   cudaStream_t st)
+int scan_exclusive(const int64_t* in, int64_t* out, int64_t m, const int64_t* m_dev, int64_t* total, ScanCtl ctl,
+                   unsigned* err, cudaStream_t st)
 {
-    k_scan<<<(unsigned)scan_tiles(m), kScanThreads, 0, st>>>(in, m, out, total, ctl, err);
+    k_scan<<<(unsigned)scan_tiles(m), kScanThreads, 0, st>>>(in, m, m_dev, out, total, ctl, err);
     return (int)cudaGetLastError();
 }
 
@@ -500,10 +505,17 @@ int radix_sort(uint64_t* k0, int32_t* v0, uint64_t* k1, int32_t* v1, int64_t n, 
     return (int)cudaGetLastError();
 }
 
+// The groups of the leaves (see k_groups).
+struct Levels {
+    int top;                        // the level of one group
+    int64_t n[kMaxLevels];          // groups of each level
+    const float4* box[kMaxLevels];  // and their boxes (two float4 each; level 0: lout)
+};
+
 // Scratch regions (byte offsets); leaf arrays are sized for n leaves (max_leaf 1).
 struct Scratch {
     size_t wpos, key0, key1, val0, val1, flag, lid, lfirst, llevel, lkey, lbox, lcnt,
-        lfar, lout, lcost, lkey2, lfirst2, llevel2, psize, groups, sums, total, cnt, sort, scan0, scan1, zero_end,
+        lfar, lout, lcost, lkey2, lfirst2, llevel2, psize, groups, sums, levels, cnt, sort, scan0, scan1, zero_end,
         lruns, cache, bytes;
     int64_t ncache;  // pair cache capacity in runs
 };
@@ -535,7 +547,7 @@ Scratch scratch_layout(int64_t n)
     s.psize = o;  o = a256(o + 4 * N);
     s.groups = o; o = a256(o + 32 * (N / 31 + 2 * kMaxLevels));  // boxes of the groups of all levels
     s.sums = o;   o = a256(o + 2 * 16 * nt);  // two scans' tile sums
-    s.total = o;  o = a256(o + 8);
+    s.levels = o; o = a256(o + sizeof(Levels));
     // zeroed at the start of each build call: counters, then the control words
     // of a sort and of two scans
     s.cnt = o;    o = a256(o + 8 * kCntWords);
@@ -699,10 +711,10 @@ __device__ __forceinline__ bool siblings(const int32_t* __restrict__ llevel,
 }
 
 __global__ void k_pack_mark(const int32_t* __restrict__ lfirst, const int32_t* __restrict__ llevel,
-                            const uint64_t* __restrict__ lkey, int64_t nl, int max_leaf,
+                            const uint64_t* __restrict__ lkey, const int64_t* __restrict__ n_plain, int max_leaf,
                             int64_t* __restrict__ pstart, int32_t* __restrict__ psize)
 {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nl = *n_plain;
     if (g >= nl || siblings(llevel, lkey, nl, g)) return;  // not the first of its run
     int64_t start = g;
     int cnt = 0, k = 0;
@@ -726,10 +738,10 @@ __global__ void k_pack_mark(const int32_t* __restrict__ lfirst, const int32_t* _
 __global__ void k_pack_fill(const int64_t* __restrict__ pstart, const int64_t* __restrict__ pid,
                             const int32_t* __restrict__ psize, const int32_t* __restrict__ lfirst,
                             const int32_t* __restrict__ llevel, const uint64_t* __restrict__ lkey,
-                            int64_t nl, int32_t* __restrict__ lfirst2, int32_t* __restrict__ llevel2,
-                            uint64_t* __restrict__ lkey2)
+                            const int64_t* __restrict__ n_plain, int32_t* __restrict__ lfirst2,
+                            int32_t* __restrict__ llevel2, uint64_t* __restrict__ lkey2)
 {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nl = *n_plain;
     if (g == nl - 1) lfirst2[pid[g] + pstart[g]] = lfirst[nl];  // lfirst[packs] = n
     if (g >= nl || !pstart[g]) return;
     const int64_t p = pid[g];
@@ -746,59 +758,73 @@ __global__ void k_pack_fill(const int64_t* __restrict__ pstart, const int64_t* _
 // lbox: the FP64 box.  lout, for the walk and the multipole split: the box
 // rounded outward in FP32 (lo down, hi up), the particle count and half the
 // rounded box's diagonal.
-__global__ void k_leaf_box(const int32_t* __restrict__ lfirst, int64_t nl, int64_t n,
+__global__ void k_leaf_box(const int32_t* __restrict__ lfirst, int64_t n,
                            const double* __restrict__ wpos, const int32_t* __restrict__ idx,
                            double* __restrict__ lbox, float4* __restrict__ lout,
                            long long* __restrict__ cnt)
 {
-    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    const int64_t nl = cnt[kCntPacked], step = (int64_t)gridDim.x * blockDim.x >> 3;
     const int sub = threadIdx.x & 7;
-    const bool live = g < nl;
-    const int64_t f = live ? lfirst[g] : 0, e = !live ? 0 : g + 1 < nl ? lfirst[g + 1] : n;
-    long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-    for (int64_t k = f + sub; k < e; k += 8) {
-        const double2* w = reinterpret_cast<const double2*>(wpos + 4 * (int64_t)idx[k]);
-        const double2 xy = w[0], zm = w[1];
-        const long long v[3] = {__double_as_longlong(xy.x), __double_as_longlong(xy.y),
-                                __double_as_longlong(zm.x)};
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = min(lo[a], v[a]);
-            hi[a] = max(hi[a], v[a]);
+    int largest = 0;
+    for (int64_t g0 = (blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31)) >> 3; g0 < nl; g0 += step) {
+        const int64_t g = g0 + ((threadIdx.x & 31) >> 3);
+        const bool live = g < nl;
+        const int64_t f = live ? lfirst[g] : 0, e = !live ? 0 : g + 1 < nl ? lfirst[g + 1] : n;
+        long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
+        for (int64_t k = f + sub; k < e; k += 8) {
+            const double2* w = reinterpret_cast<const double2*>(wpos + 4 * (int64_t)idx[k]);
+            const double2 xy = w[0], zm = w[1];
+            const long long v[3] = {__double_as_longlong(xy.x), __double_as_longlong(xy.y),
+                                    __double_as_longlong(zm.x)};
+            for (int a = 0; a < 3; ++a) {
+                lo[a] = min(lo[a], v[a]);
+                hi[a] = max(hi[a], v[a]);
+            }
         }
-    }
-    for (int o = 4; o > 0; o >>= 1)
+        for (int o = 4; o > 0; o >>= 1)
+            for (int a = 0; a < 3; ++a) {
+                lo[a] = min(lo[a], __shfl_xor_sync(kFull, lo[a], o));
+                hi[a] = max(hi[a], __shfl_xor_sync(kFull, hi[a], o));
+            }
+        largest = max(largest, (int)(e - f));
+        if (!live || sub) continue;
+        float ol[3], oh[3], r2 = 0.f;
         for (int a = 0; a < 3; ++a) {
-            lo[a] = min(lo[a], __shfl_xor_sync(kFull, lo[a], o));
-            hi[a] = max(hi[a], __shfl_xor_sync(kFull, hi[a], o));
+            const double l = __longlong_as_double(lo[a]), h = __longlong_as_double(hi[a]);
+            lbox[6 * g + a] = l;
+            lbox[6 * g + 3 + a] = h;
+            ol[a] = __double2float_rd(l);
+            oh[a] = __double2float_ru(h);
+            const float ea = __fmul_rn(0.5f, __fsub_rn(oh[a], ol[a]));
+            r2 = __fmaf_rn(ea, ea, r2);
         }
-    int most = live ? (int)(e - f) : 0;
-    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(kFull, most, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(cnt + kCntMaxLeaf, (long long)most);
-    if (!live || sub) return;
-    float ol[3], oh[3], r2 = 0.f;
-    for (int a = 0; a < 3; ++a) {
-        const double l = __longlong_as_double(lo[a]), h = __longlong_as_double(hi[a]);
-        lbox[6 * g + a] = l;
-        lbox[6 * g + 3 + a] = h;
-        ol[a] = __double2float_rd(l);
-        oh[a] = __double2float_ru(h);
-        const float ea = __fmul_rn(0.5f, __fsub_rn(oh[a], ol[a]));
-        r2 = __fmaf_rn(ea, ea, r2);
+        lout[2 * g] = make_float4(ol[0], ol[1], ol[2], __int_as_float((int)(e - f)));
+        lout[2 * g + 1] = make_float4(oh[0], oh[1], oh[2], __fsqrt_rn(r2));
     }
-    lout[2 * g] = make_float4(ol[0], ol[1], ol[2], __int_as_float((int)(e - f)));
-    lout[2 * g + 1] = make_float4(oh[0], oh[1], oh[2], __fsqrt_rn(r2));
+    for (int o = 16; o > 0; o >>= 1) largest = max(largest, __shfl_xor_sync(kFull, largest, o));
+    if ((threadIdx.x & 31) == 0 && largest) atomicMax(cnt + kCntMaxLeaf, (long long)largest);
 }
 
 // ---------------------------------------------------------------- groups --
 // A 32-ary tree over the leaves in their (Morton) order: a group of a level is
 // 32 consecutive groups of the level below, level 0 the leaves, its box the
-// union of theirs (FP32, rounded outward like them), up to one group.  A warp
-// per group.
-__global__ void k_groups(const float4* __restrict__ below, int64_t n_below, float4* __restrict__ out,
-                         int64_t n_out)
+// union of theirs (FP32, rounded outward like them), up to one group.
+__host__ __device__ inline Levels make_levels(int64_t nl, const float4* lout, const float4* groups)
 {
-    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (g >= n_out) return;
+    Levels w{};
+    w.box[0] = lout;
+    w.n[0] = nl;
+    while (w.n[w.top] > 1 && w.top + 1 < kMaxLevels) {
+        w.box[w.top + 1] = groups;
+        w.n[w.top + 1] = (w.n[w.top] + 31) / 32;
+        groups += 2 * w.n[++w.top];
+    }
+    return w;
+}
+
+__device__ __forceinline__ void group_box(const float4* __restrict__ below, int64_t n_below, int64_t g,
+                                          float4* __restrict__ out)
+{
     const int lane = threadIdx.x & 31;
     const int64_t c = 32 * g + lane;
     float lo[3] = {kInf, kInf, kInf}, hi[3] = {-kInf, -kInf, -kInf};
@@ -816,6 +842,24 @@ __global__ void k_groups(const float4* __restrict__ below, int64_t n_below, floa
         out[2 * g] = make_float4(lo[0], lo[1], lo[2], 0.f);
         out[2 * g + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
     }
+}
+
+// Boxes of levels 1 (level = 1, a warp per group over the grid) or 2 and up
+// (level = 2, one block: at most a 1024th of the leaves); the latter writes the
+// levels for the walks.
+__global__ void __launch_bounds__(1024) k_groups(int level, const long long* __restrict__ cnt, const float4* lout,
+                                                 float4* groups, Levels* out)
+{
+    const Levels v = make_levels(cnt[kCntPacked], lout, groups);
+    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+    float4* dst = groups;
+    for (int t = 1; t <= v.top; dst += 2 * v.n[t], ++t) {
+        if (level == 1 ? t > 1 : t == 1) continue;
+        for (int64_t g = w0; g < v.n[t]; g += step) group_box(t == 1 ? lout : dst - 2 * v.n[t - 1], v.n[t - 1], g, dst);
+        __syncthreads();
+    }
+    if (level == 2 && threadIdx.x == 0) *out = v;
 }
 
 // ----------------------------------------------------------------- pairs --
@@ -900,11 +944,8 @@ constexpr int kWalkWarps = 4;
 constexpr int kWalkBlocks = 8;  // per SM
 
 struct WalkArgs {
-    int64_t nl;
     BoxK bx;
-    int top;                        // the level of one group
-    const float4* box[kMaxLevels];  // boxes of each level (level 0: lout)
-    int64_t n[kMaxLevels];          // and their numbers
+    const Levels* levels;
     const int32_t* lfirst;
     const double* lbox;
     int64_t *lcnt, *lcost, *lfar;         // count
@@ -914,8 +955,15 @@ struct WalkArgs {
     unsigned* err;
     int32_t* lruns;
     uint2* cache;
-    int kslot;
+    int64_t ncache;  // runs the cache holds, shared out over the rows
 };
+
+// runs per row in the pair cache (none below kMinRuns: rows walked twice)
+__host__ __device__ inline int cache_slot(int64_t ncache, int64_t nl)
+{
+    const int64_t ks = ncache / nl;
+    return ks < kMinRuns ? 0 : (int)(ks < (1 << 20) ? ks : (1 << 20));
+}
 
 // component a of an image code's periodic step, -1, 0 or 1
 __device__ __forceinline__ int image_step(uint32_t code, int a)
@@ -927,26 +975,31 @@ template <bool WRITE, bool SPLIT>
 __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const WalkArgs w)
 {
     __shared__ long long s_pairs, s_far, s_eval, s_cost, s_row, s_uncached;
+    __shared__ Levels s_lv;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int nl = (int)w.nl;
     const float thi = w.bx.thi, tlo = w.bx.tlo;
+    if (threadIdx.x == 0) s_lv = *w.levels;
     if (threadIdx.x == 0) s_pairs = s_far = s_eval = s_cost = s_row = s_uncached = 0;
     __syncthreads();
     const float Lf = (float)w.bx.L, Lrd = __double2float_rd(w.bx.L), Lru = __double2float_ru(w.bx.L);
+    const float4* const lout = s_lv.box[0];
+    const int top = s_lv.top;
+    const int nl = s_lv.n[0] < (1 << 27) ? (int)s_lv.n[0] : 0;  // more is refused by the host
+    const int kslot = cache_slot(w.ncache, s_lv.n[0]);
     const int W = (int)gridDim.x * kWalkWarps;
     for (int I = (int)blockIdx.x * kWalkWarps + wp; I < nl; I += W) {
-        const bool recorded = WRITE && w.lruns && w.lruns[I] >= 0;
+        const bool recorded = WRITE && kslot && w.lruns[I] >= 0;
         if (WRITE && !SPLIT && recorded) continue;
-        const float4 t0 = w.box[0][2 * (int64_t)I], t1 = w.box[0][2 * (int64_t)I + 1];
+        const float4 t0 = lout[2 * (int64_t)I], t1 = lout[2 * (int64_t)I + 1];
         const float ra = t1.w;  // rho of the outward box
         long long c = 0, cf = 0;  // entries so far (uniform)
         long long src = 0;        // this lane's part of their particles
         long long at = WRITE ? w.rowptr[I] : 0, fat = WRITE && SPLIT ? w.frowptr[I] : 0;
         const long long end = WRITE ? w.rowptr[I + 1] : 0, fend = WRITE && SPLIT ? w.frowptr[I + 1] : 0;
         // pair cache: runs so far, the open (last) run's first entry and the entry after its end
-        const bool caching = !WRITE && w.cache != nullptr;
-        uint2* const slot = w.cache + I * (int64_t)w.kslot;
+        const bool caching = !WRITE && kslot;
+        uint2* const slot = w.cache + I * (int64_t)kslot;
         int nrun = 0;
         uint32_t run0 = 0, runend = 0xffffffffu;
         uint32_t code = 0;
@@ -993,7 +1046,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                 const bool old = cont && lane == 0;
                 const int k = old ? nrun - 1 : nrun + __popc(B & lt);
                 const uint32_t first = old ? run0 : ((uint32_t)(base + lane) << 5) | code;
-                if (k < w.kslot) slot[k] = make_uint2(first, (uint32_t)(base + lane + len) - (first >> 5));
+                if (k < kslot) slot[k] = make_uint2(first, (uint32_t)(base + lane + len) - (first >> 5));
             }
             if (B) run0 = ((uint32_t)(base + 31 - __clz(B)) << 5) | code;
             nrun += __popc(B);
@@ -1007,8 +1060,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                     const bool in = J >= f && J <= l;
                     float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
                     if (SPLIT && in) {
-                        b0 = w.box[0][2 * (int64_t)J];
-                        b1 = w.box[0][2 * (int64_t)J + 1];
+                        b0 = lout[2 * (int64_t)J];
+                        b1 = lout[2 * (int64_t)J + 1];
                     }
                     leaves(__ballot_sync(kFull, in), base, b0, b1);
                 }
@@ -1023,7 +1076,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                 ++nrun;
             }
             runend = ((uint32_t)(l + 1) << 5) | code;
-            if (lane == 0 && nrun <= w.kslot) slot[nrun - 1] = make_uint2(run0, (runend - run0) >> 5);
+            if (lane == 0 && nrun <= kslot) slot[nrun - 1] = make_uint2(run0, (runend - run0) >> 5);
         };
         auto set_image = [&](uint32_t cd) {
             code = cd;
@@ -1039,8 +1092,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
             bool keep = false;
             if (J < nl) {
-                b0 = w.box[0][2 * (int64_t)J];
-                b1 = w.box[0][2 * (int64_t)J + 1];
+                b0 = lout[2 * (int64_t)J];
+                b1 = lout[2 * (int64_t)J + 1];
                 const float g2 = gap2_f(alo, ahi, b0, b1);
                 keep = g2 < tlo;
                 if (!keep && g2 < thi) {
@@ -1060,7 +1113,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                 range((int)(run.x >> 5), (int)(run.x >> 5) + (int)run.y - 1);
             }
         } else {
-            const float4 r0 = w.box[w.top][0], r1 = w.box[w.top][1];
+            const float4 r0 = s_lv.box[top][0], r1 = s_lv.box[top][1];
             bool in = false, all = false;
             if (lane < kShiftCodes) {  // the root at each image
                 set_image((uint32_t)lane);
@@ -1077,7 +1130,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                     range(0, nl - 1);
                     continue;
                 }
-                if (w.top <= 1) {
+                if (top <= 1) {
                     test_leaves(0);
                     continue;
                 }
@@ -1088,8 +1141,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                 auto test_group = [&](int t, int base) {  // the members of level t from `base` on
                     const int g = base + lane;
                     bool part = false, full = false;
-                    if (g < (int)w.n[t]) {
-                        const float4 b0 = w.box[t][2 * (int64_t)g], b1 = w.box[t][2 * (int64_t)g + 1];
+                    if (g < (int)s_lv.n[t]) {
+                        const float4 b0 = s_lv.box[t][2 * (int64_t)g], b1 = s_lv.box[t][2 * (int64_t)g + 1];
                         part = gap2_f(alo, ahi, b0, b1) < thi;
                         full = part && maxgap2_f(alo, ahi, b0, b1) < tlo;
                     }
@@ -1100,9 +1153,9 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                         first = base;
                     }
                 };
-                int t = w.top - 1;
+                int t = top - 1;
                 test_group(t, 0);
-                while (t < w.top) {
+                while (t < top) {
                     const unsigned m = __shfl_sync(kFull, todo, t);
                     if (!m) {
                         ++t;
@@ -1134,7 +1187,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                 w.lcost[I] = cost;
                 if (SPLIT) w.lfar[I] = cf;
                 if (caching) {
-                    const bool fits = nrun <= w.kslot;
+                    const bool fits = nrun <= kslot;
                     w.lruns[I] = fits ? nrun : -1;
                     if (!fits) atomicAdd((unsigned long long*)&s_uncached, 1ULL);
                 }
@@ -1319,22 +1372,7 @@ __global__ void k_sched_out(const uint64_t* __restrict__ key, const int32_t* __r
         if (mine > heavy.cost[l] && next <= heavy.cost[l]) n_heavy[l] = (int)(i + 1);
 }
 
-// The levels of the groups over nl leaves.
-WalkArgs walk_levels(int64_t nl, const float4* lout, float4* groups)
-{
-    WalkArgs w{};
-    w.nl = nl;
-    w.box[0] = lout;
-    w.n[0] = nl;
-    while (w.n[w.top] > 1) {
-        w.box[w.top + 1] = groups;
-        w.n[w.top + 1] = (w.n[w.top] + 31) / 32;
-        groups += 2 * w.n[++w.top];
-    }
-    return w;
-}
-
-// blocks of a row walk: a warp per leaf, up to one wave
+// blocks of a row walk: a warp per leaf (at most nl of them), up to one wave
 unsigned walk_blocks(int64_t nl, int sms)
 {
     return (unsigned)std::min<int64_t>((nl + kWalkWarps - 1) / kWalkWarps, kWalkBlocks * (int64_t)sms);
@@ -1354,13 +1392,12 @@ int dcuda(int e, const char* what)
 }
 
 // Bounded host wait for the stream, then a copy of `bytes` to the host.
-// Waits (at most timeout_ms) for the work queued on st, then copies one or
-// two small device blocks to the host.  The wait polls without sleeping for
+// Waits (at most timeout_ms) for the work queued on st, then copies a
+// small device block to the host.  The wait polls without sleeping for
 // its first 2 ms (the build's steps between waits take about a millisecond,
 // and a sleeping poll wakes up to tens of microseconds late), then every 20
 // microseconds.
-int read_back(void* dst, const void* src, size_t bytes, cudaStream_t st, int timeout_ms,
-              void* dst2 = nullptr, const void* src2 = nullptr, size_t bytes2 = 0)
+int read_back(void* dst, const void* src, size_t bytes, cudaStream_t st, int timeout_ms)
 {
     auto t0 = std::chrono::steady_clock::now();
     for (;;) {
@@ -1372,7 +1409,6 @@ int read_back(void* dst, const void* src, size_t bytes, cudaStream_t st, int tim
         if (ms > 2.0) std::this_thread::sleep_for(std::chrono::microseconds(20));
     }
     cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && dst2) e = cudaMemcpyAsync(dst2, src2, bytes2, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e == cudaSuccess ? PSR_OK : dcuda(e, "cudaMemcpyAsync (device build counters)");
 }
@@ -1467,9 +1503,10 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     float4* lout = (float4*)(s + S.lout);
     int64_t* lcnt = (int64_t*)(s + S.lcnt);
     int64_t* lcost = (int64_t*)(s + S.lcost);
-    int64_t* total = (int64_t*)(s + S.total);
     int64_t* sums = (int64_t*)(s + S.sums);
     long long* cnt = (long long*)(s + S.cnt);
+    int64_t* const n_plain = (int64_t*)cnt + kCntLeaves;
+    int64_t* const n_packed = (int64_t*)cnt + kCntPacked;
     BoxK bx = box_k(*box);
     bx.theta2 = (float)(theta * theta);
     bx.gt2 = (flags & PSR_BUILD_SPLIT_GAUSSIAN) ? (float)(theta * theta * 4.0 * std::pow(box->r_s, 4))
@@ -1488,54 +1525,42 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
         return dcuda(e, "radix sort");
     k_leaf_level<<<nblk(n, kLevelTile), kLevelTile, 0, st>>>(k0, n, max_leaf, flag, v1);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf level kernel");
-    if ((e = scan_exclusive(flag, lid, n, total, scan0, err, st))) return dcuda(e, "scan");
+    if ((e = scan_exclusive(flag, lid, n, nullptr, n_plain, scan0, err, st))) return dcuda(e, "scan");
     k_leaf_fill<<<nblk(n, 256), 256, 0, st>>>(flag, lid, v1, k0, n, lfirst, llevel, lkey);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf fill kernel");
-    long long c[kCntWords];
-    int64_t nl = 0;
-    if ((e = read_back(&nl, total, 8, st, timeout_ms, c, cnt, sizeof c))) return e;
-    if (c[kCntError] & 1) return dfail(PSR_E_ARG, "non-finite position or mass");
-    if (nl < 1 || nl > n || nl >= (1 << 27)) return dfail(PSR_E_ARG, "leaf count out of range");
-    if (!(flags & PSR_BUILD_UNPACKED)) {
-        // pack sibling leaves: marks, pack ids, packed arrays, copied back
-        // over the leaf arrays
+    // From here on the kernels take the number of leaves from the counters: the
+    // host waits once, for all counts (two more waits, to size the launches,
+    // left the GPU idle for about 50 us of a build).
+    const bool pack = !(flags & PSR_BUILD_UNPACKED);
+    if (pack) {
+        // pack sibling leaves: marks, pack ids, the packed leaves' arrays
         int64_t* pstart = flag;
         int64_t* pid = lid;
         int32_t* psize = (int32_t*)(s + S.psize);
-        int32_t* lfirst2 = (int32_t*)(s + S.lfirst2);
-        int32_t* llevel2 = (int32_t*)(s + S.llevel2);
-        uint64_t* lkey2 = (uint64_t*)(s + S.lkey2);
-        k_pack_mark<<<nblk(nl, 256), 256, 0, st>>>(lfirst, llevel, lkey, nl, max_leaf, pstart, psize);
+        k_pack_mark<<<nblk(n, 256), 256, 0, st>>>(lfirst, llevel, lkey, n_plain, max_leaf, pstart, psize);
+        if ((e = scan_exclusive(pstart, pid, n, n_plain, n_packed, scan1, err, st))) return dcuda(e, "scan");
+        k_pack_fill<<<nblk(n, 256), 256, 0, st>>>(pstart, pid, psize, lfirst, llevel, lkey, n_plain,
+                                                  (int32_t*)(s + S.lfirst2), (int32_t*)(s + S.llevel2),
+                                                  (uint64_t*)(s + S.lkey2));
         if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf packing kernel");
-        if ((e = scan_exclusive(pstart, pid, nl, total, scan1, err, st))) return dcuda(e, "scan");
-        k_pack_fill<<<nblk(nl, 256), 256, 0, st>>>(pstart, pid, psize, lfirst, llevel, lkey, nl,
-                                                   lfirst2, llevel2, lkey2);
-        if ((e = (int)cudaGetLastError())) return dcuda(e, "leaf packing kernel");
-        int64_t np = 0;
-        if ((e = read_back(&np, total, 8, st, timeout_ms))) return e;
-        if (np < 1 || np > nl) return dfail(PSR_E_DEVICE, "leaf packing failed");
-        if ((e = (int)cudaMemcpyAsync(lfirst, lfirst2, 4 * (np + 1), cudaMemcpyDeviceToDevice, st)) ||
-            (e = (int)cudaMemcpyAsync(llevel, llevel2, 4 * np, cudaMemcpyDeviceToDevice, st)) ||
-            (e = (int)cudaMemcpyAsync(lkey, lkey2, 8 * np, cudaMemcpyDeviceToDevice, st)))
-            return dcuda(e, "cudaMemcpyAsync");
-        nl = np;
+        lfirst = (int32_t*)(s + S.lfirst2);
+    } else if ((e = (int)cudaMemcpyAsync(n_packed, n_plain, 8, cudaMemcpyDeviceToDevice, st))) {
+        return dcuda(e, "cudaMemcpyAsync");
     }
-    k_leaf_box<<<nblk(8 * nl, 256), 256, 0, st>>>(lfirst, nl, n, wpos, v0, lbox, lout, cnt);
-    WalkArgs wa = walk_levels(nl, lout, (float4*)(s + S.groups));
-    for (int t = 1; t <= wa.top; ++t)
-        k_groups<<<nblk(32 * wa.n[t], 256), 256, 0, st>>>(wa.box[t - 1], wa.n[t - 1],
-                                                          const_cast<float4*>(wa.box[t]), wa.n[t]);
-    if ((e = (int)cudaGetLastError())) return dcuda(e, "group kernel");
     int dev = 0, sms = 0;
     if ((e = (int)cudaGetDevice(&dev))) return dcuda(e, "cudaGetDevice");
     if ((e = (int)cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
         return dcuda(e, "cudaDeviceGetAttribute");
-    // runs per row in the pair cache (none below kMinRuns: rows walked twice)
-    const int64_t ks = S.ncache / nl;
-    const int kslot = ks >= kMinRuns ? (int)(ks < (1 << 20) ? ks : (1 << 20)) : 0;
-    int32_t* const lruns = kslot ? (int32_t*)(s + S.lruns) : nullptr;
-    uint2* const pcache = kslot ? (uint2*)(s + S.cache) : nullptr;
+    const unsigned wave = 8 * (unsigned)sms;
+    k_leaf_box<<<std::min(nblk(8 * n, 256), wave), 256, 0, st>>>(lfirst, n, wpos, v0, lbox, lout, cnt);
+    float4* const groups = (float4*)(s + S.groups);
+    Levels* const levels = (Levels*)(s + S.levels);
+    k_groups<<<std::min(nblk(n, 256), wave), 256, 0, st>>>(1, cnt, lout, groups, levels);
+    k_groups<<<1, 1024, 0, st>>>(2, cnt, lout, groups, levels);
+    if ((e = (int)cudaGetLastError())) return dcuda(e, "group kernel");
+    WalkArgs wa{};
     wa.bx = bx;
+    wa.levels = levels;
     wa.lfirst = lfirst;
     wa.lbox = lbox;
     wa.lcnt = lcnt;
@@ -1543,13 +1568,19 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     wa.lfar = (int64_t*)(s + S.lfar);
     wa.cnt = cnt;
     wa.err = err;
-    wa.lruns = lruns;
-    wa.cache = pcache;
-    wa.kslot = kslot;
-    if (theta > 0.0) k_rows<false, true><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
-    else k_rows<false, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
+    wa.lruns = (int32_t*)(s + S.lruns);
+    wa.cache = (uint2*)(s + S.cache);
+    wa.ncache = S.ncache;
+    if (theta > 0.0) k_rows<false, true><<<walk_blocks(n, sms), 32 * kWalkWarps, 0, st>>>(wa);
+    else k_rows<false, false><<<walk_blocks(n, sms), 32 * kWalkWarps, 0, st>>>(wa);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "pair count kernel");
+    long long c[kCntWords];
     if ((e = read_back(c, cnt, sizeof c, st, timeout_ms))) return e;
+    if (c[kCntError] & 1) return dfail(PSR_E_ARG, "non-finite position or mass");
+    const int64_t np = c[kCntLeaves], nl = c[kCntPacked];
+    if (np < 1 || np > n || nl >= (1 << 27)) return dfail(PSR_E_ARG, "leaf count out of range");
+    if (nl < 1 || nl > np) return dfail(PSR_E_DEVICE, "leaf packing failed");
+    const int kslot = cache_slot(S.ncache, nl);
     if (c[kCntError] & 12) return dfail(PSR_E_DEVICE, "a row walk or a look-back failed");
     if (c[kCntPairs] >= ((int64_t)1 << 32) || c[kCntFar] >= ((int64_t)1 << 32))
         return dfail(PSR_E_ARG, "more than 2^32 leaf pairs");
@@ -1638,9 +1669,11 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     // the control words first: the pair write kernel reports into the error
     // word that psr_check reads
     if ((e = (int)cudaMemsetAsync(w + L.ctrl, 0, kCtrlWords * 4, st))) return dcuda(e, "cudaMemsetAsync");
-    const int32_t* lfirst = (const int32_t*)(s + S.lfirst);
+    const bool pack = !(h->flags & PSR_BUILD_UNPACKED);
+    const int32_t* lfirst = (const int32_t*)(s + (pack ? S.lfirst2 : S.lfirst));
     k_payload<<<nblk(8 * nl, 256), 256, 0, st>>>(
-        lfirst, (const int32_t*)(s + S.llevel), (const uint64_t*)(s + S.lkey), nl, n, bx,
+        lfirst, (const int32_t*)(s + (pack ? S.llevel2 : S.llevel)),
+        (const uint64_t*)(s + (pack ? S.lkey2 : S.lkey)), nl, n, bx,
         (const double*)(s + S.wpos), (const int32_t*)(s + S.val0), (float4*)(w + L.pf),
         h->has_pd ? (double4*)(w + L.pd) : nullptr, (int32_t*)(w + L.perm), (int4*)(w + L.leaf),
         (int4*)(w + L.lcen));
@@ -1652,28 +1685,29 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     const SortCtl sctl{(unsigned*)(s + S.sort), sort_tiles(n)};
     const ScanCtl scan0{(unsigned*)(s + S.scan0), sums}, scan1{(unsigned*)(s + S.scan1), sums + 2 * scan_tiles(n)};
     if ((e = (int)cudaMemsetAsync(s + S.sort, 0, S.zero_end - S.sort, st))) return dcuda(e, "cudaMemsetAsync");
-    if ((e = scan_exclusive((const int64_t*)(s + S.lcnt), rowptr, nl, rowptr + nl, scan0, err, st)))
+    if ((e = scan_exclusive((const int64_t*)(s + S.lcnt), rowptr, nl, nullptr, rowptr + nl, scan0, err, st)))
         return dcuda(e, "scan");
     const double* lbox = (const double*)(s + S.lbox);
     int64_t* frow = h->has_far ? (int64_t*)(w + L.frow) : nullptr;
     if (h->has_far) {
-        if ((e = scan_exclusive((const int64_t*)(s + S.lfar), frow, nl, frow + nl, scan1, err, st)))
+        if ((e = scan_exclusive((const int64_t*)(s + S.lfar), frow, nl, nullptr, frow + nl, scan1, err, st)))
             return dcuda(e, "scan");
         k_fcen<<<nblk(nl, 128), 128, 0, st>>>(lbox, (const int4*)(w + L.lcen), bx.unit, nl,
                                               (double4*)(w + L.fcen), (float4*)(w + L.fofs));
         if ((e = (int)cudaGetLastError())) return dcuda(e, "expansion centre kernel");
     }
-    WalkArgs wa = walk_levels(nl, (const float4*)(s + S.lout), (float4*)(s + S.groups));
+    WalkArgs wa{};
     wa.bx = bx;
+    wa.levels = (const Levels*)(s + S.levels);
     wa.lfirst = lfirst;
     wa.lbox = lbox;
     wa.rowptr = rowptr;
     wa.frowptr = frow;
     wa.pairs = (uint32_t*)(w + L.pairs);
     wa.err = err;
-    wa.lruns = h->db_kslot ? (int32_t*)(s + S.lruns) : nullptr;
-    wa.cache = h->db_kslot ? (uint2*)(s + S.cache) : nullptr;
-    wa.kslot = h->db_kslot;
+    wa.lruns = (int32_t*)(s + S.lruns);
+    wa.cache = (uint2*)(s + S.cache);
+    wa.ncache = S.ncache;
     if (h->has_far) {
         wa.fpairs = (uint32_t*)(w + L.fpairs);
         wa.bx.theta2 = (float)(h->theta * h->theta);
@@ -1683,8 +1717,8 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
         k_rows<true, true><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
     } else {
         // rows the count walk cached are expanded; the rest are walked again
-        if (wa.lruns) {
-            k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, wa.lruns, wa.cache, wa.kslot, rowptr, wa.pairs, wa.err);
+        if (h->db_kslot) {
+            k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, wa.lruns, wa.cache, h->db_kslot, rowptr, wa.pairs, wa.err);
             if ((e = (int)cudaGetLastError())) return dcuda(e, "pair expand kernel");
         }
         if (h->db_uncached > 0) k_rows<true, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);

@@ -68,7 +68,8 @@ enum : int {
     kCntMass0 = 9,     // particle 0's mass (the bits of a double)
     kCntLeaves = 10,   // plain octree leaves
     kCntPacked = 11,   // leaves after packing (kCntLeaves without it)
-    kCntWords = 12,
+    kCntRedo = 12,     // split: rows whose near and far runs together did not fit
+    kCntWords = 13,
 };
 
 // The pair cache: the count walk also records each row as runs of
@@ -516,7 +517,7 @@ struct Levels {
 struct Scratch {
     size_t wpos, key0, key1, val0, val1, flag, lid, lfirst, llevel, lkey, lbox, lcnt,
         lfar, lout, lcost, lkey2, lfirst2, llevel2, psize, groups, sums, levels, cnt, sort, scan0, scan1, zero_end,
-        lruns, cache, bytes;
+        lruns, lfruns, cache, bytes;
     int64_t ncache;  // pair cache capacity in runs
 };
 
@@ -556,6 +557,7 @@ Scratch scratch_layout(int64_t n)
     s.scan1 = o;  o = a256(o + 4 * (1 + nt));
     s.zero_end = o;
     s.lruns = o;  o = a256(o + 4 * N);   // runs cached per row (-1: not cached)
+    s.lfruns = o; o = a256(o + 4 * N);   // and far ones (multipole split)
     s.ncache = (int64_t)(kCacheWordsPerParticle / 2 * N);
     s.cache = o;  o = a256(o + 8 * (size_t)s.ncache);  // uint2 (first leaf << 5 | code, length)
     s.bytes = o;
@@ -936,10 +938,10 @@ __device__ __forceinline__ bool far_pair(const float* alo, const float* ahi, flo
 // two with directed roundings: 5500 -> 3300 instructions a row.
 //
 // MODE: count (and, given a pair cache of kslot runs per row, record the row's
-// runs: lruns[I] their number, or -1 when the slot is too small), or write a
-// row at rowptr; SPLIT: each kept leaf goes to the near or the far list
-// (far_pair).  The write pass of a split replays a recorded row's runs; the
-// plain one skips recorded rows (k_pairs_expand writes those).
+// runs: lruns[I] their number, or -1 when the slot is too small), or write the
+// rows that were not recorded at rowptr (k_pairs_expand writes the others);
+// SPLIT: each kept leaf goes to the near or the far list (far_pair), whose runs
+// are recorded apart (lfruns the far ones).
 constexpr int kWalkWarps = 4;
 constexpr int kWalkBlocks = 8;  // per SM
 
@@ -953,7 +955,7 @@ struct WalkArgs {
     uint32_t *pairs, *fpairs;
     long long* cnt;
     unsigned* err;
-    int32_t* lruns;
+    int32_t *lruns, *lfruns;
     uint2* cache;
     int64_t ncache;  // runs the cache holds, shared out over the rows
 };
@@ -974,13 +976,13 @@ __device__ __forceinline__ int image_step(uint32_t code, int a)
 template <bool WRITE, bool SPLIT>
 __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const WalkArgs w)
 {
-    __shared__ long long s_pairs, s_far, s_eval, s_cost, s_row, s_uncached;
+    __shared__ long long s_pairs, s_far, s_eval, s_cost, s_row, s_uncached, s_redo;
     __shared__ Levels s_lv;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const float thi = w.bx.thi, tlo = w.bx.tlo;
     if (threadIdx.x == 0) s_lv = *w.levels;
-    if (threadIdx.x == 0) s_pairs = s_far = s_eval = s_cost = s_row = s_uncached = 0;
+    if (threadIdx.x == 0) s_pairs = s_far = s_eval = s_cost = s_row = s_uncached = s_redo = 0;
     __syncthreads();
     const float Lf = (float)w.bx.L, Lrd = __double2float_rd(w.bx.L), Lru = __double2float_ru(w.bx.L);
     const float4* const lout = s_lv.box[0];
@@ -989,22 +991,44 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
     const int kslot = cache_slot(w.ncache, s_lv.n[0]);
     const int W = (int)gridDim.x * kWalkWarps;
     for (int I = (int)blockIdx.x * kWalkWarps + wp; I < nl; I += W) {
-        const bool recorded = WRITE && kslot && w.lruns[I] >= 0;
-        if (WRITE && !SPLIT && recorded) continue;
+        if (WRITE && kslot && w.lruns[I] >= 0) continue;  // recorded: k_pairs_expand writes it
         const float4 t0 = lout[2 * (int64_t)I], t1 = lout[2 * (int64_t)I + 1];
         const float ra = t1.w;  // rho of the outward box
         long long c = 0, cf = 0;  // entries so far (uniform)
         long long src = 0;        // this lane's part of their particles
         long long at = WRITE ? w.rowptr[I] : 0, fat = WRITE && SPLIT ? w.frowptr[I] : 0;
         const long long end = WRITE ? w.rowptr[I + 1] : 0, fend = WRITE && SPLIT ? w.frowptr[I + 1] : 0;
-        // pair cache: runs so far, the open (last) run's first entry and the entry after its end
+        // pair cache, [0] near and [1] far: runs so far, the open (last) run's
+        // first entry and the entry after its end; near runs fill the row's
+        // slot from its start, far ones from its end
         const bool caching = !WRITE && kslot;
         uint2* const slot = w.cache + I * (int64_t)kslot;
-        int nrun = 0;
-        uint32_t run0 = 0, runend = 0xffffffffu;
+        int nrun[2] = {0, 0};
+        uint32_t run0[2] = {0, 0}, runend[2] = {0xffffffffu, 0xffffffffu};
+        int nall = 0;
+        uint32_t allend = 0xffffffffu;
         uint32_t code = 0;
         float alo[3], ahi[3];  // the target box moved by minus the image's shift
 
+        // records the leaves of mask M of the 32 from `base` on as runs
+        auto record = [&](unsigned M, int base, const bool fr) {
+            if (!M) return;
+            const bool cont = (M & 1u) && (((uint32_t)base << 5) | code) == runend[fr];
+            unsigned B = M & ~(M << 1);  // first leaves of runs
+            if (cont) B &= ~1u;
+            if (((B >> lane) & 1u) || (cont && lane == 0)) {
+                const unsigned rest = ~(M >> lane);
+                const int len = rest ? __ffs(rest) - 1 : 32;
+                const bool old = cont && lane == 0;
+                const int k = old ? nrun[fr] - 1 : nrun[fr] + __popc(B & lt);
+                const uint32_t first = old ? run0[fr] : ((uint32_t)(base + lane) << 5) | code;
+                if (k < kslot)
+                    slot[fr ? kslot - 1 - k : k] = make_uint2(first, (uint32_t)(base + lane + len) - (first >> 5));
+            }
+            if (B) run0[fr] = ((uint32_t)(base + 31 - __clz(B)) << 5) | code;
+            nrun[fr] += __popc(B);
+            runend[fr] = ((uint32_t)(base + 32 - __clz(M)) << 5) | code;
+        };
         // the leaves of mask M of the 32 from `base` on; b0, b1: this lane's leaf
         auto leaves = [&](unsigned M, int base, float4 b0, float4 b1) {
             if (!M) return;
@@ -1037,20 +1061,14 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             cf += __popc(F);
             if (mine && !far) src += __float_as_int(b0.w);
             if (!caching) return;
-            const bool cont = (M & 1u) && (((uint32_t)base << 5) | code) == runend;
-            unsigned B = M & ~(M << 1);  // first leaves of runs
-            if (cont) B &= ~1u;
-            if (((B >> lane) & 1u) || (cont && lane == 0)) {
-                const unsigned rest = ~(M >> lane);
-                const int len = rest ? __ffs(rest) - 1 : 32;
-                const bool old = cont && lane == 0;
-                const int k = old ? nrun - 1 : nrun + __popc(B & lt);
-                const uint32_t first = old ? run0 : ((uint32_t)(base + lane) << 5) | code;
-                if (k < kslot) slot[k] = make_uint2(first, (uint32_t)(base + lane + len) - (first >> 5));
+            record(N, base, false);
+            if (SPLIT) {
+                record(F, base, true);
+                // and the runs of the undivided row, which psr_info.rows_walked_twice
+                // counts by
+                nall += __popc(M & ~(M << 1)) - ((M & 1u) && (((uint32_t)base << 5) | code) == allend ? 1 : 0);
+                allend = ((uint32_t)(base + 32 - __clz(M)) << 5) | code;
             }
-            if (B) run0 = ((uint32_t)(base + 31 - __clz(B)) << 5) | code;
-            nrun += __popc(B);
-            runend = ((uint32_t)(base + 32 - __clz(M)) << 5) | code;
         };
         // every leaf of [f, l]
         auto range = [&](int f, int l) {
@@ -1071,12 +1089,12 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             if (lane == 0) src += w.lfirst[l + 1] - w.lfirst[f];
             if (!caching) return;
             const uint32_t e0 = ((uint32_t)f << 5) | code;
-            if (e0 != runend) {
-                run0 = e0;
-                ++nrun;
+            if (e0 != runend[0]) {
+                run0[0] = e0;
+                ++nrun[0];
             }
-            runend = ((uint32_t)(l + 1) << 5) | code;
-            if (lane == 0 && nrun <= kslot) slot[nrun - 1] = make_uint2(run0, (runend - run0) >> 5);
+            runend[0] = ((uint32_t)(l + 1) << 5) | code;
+            if (lane == 0 && nrun[0] <= kslot) slot[nrun[0] - 1] = make_uint2(run0[0], (runend[0] - run0[0]) >> 5);
         };
         auto set_image = [&](uint32_t cd) {
             code = cd;
@@ -1105,14 +1123,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
             leaves(__ballot_sync(kFull, keep), base, b0, b1);
         };
 
-        if (recorded) {  // split: replay the row's runs
-            const int n = w.lruns[I];
-            for (int r = 0; r < n; ++r) {
-                const uint2 run = slot[r];
-                set_image(run.x & 31u);
-                range((int)(run.x >> 5), (int)(run.x >> 5) + (int)run.y - 1);
-            }
-        } else {
+        {
             const float4 r0 = s_lv.box[top][0], r1 = s_lv.box[top][1];
             bool in = false, all = false;
             if (lane < kShiftCodes) {  // the root at each image
@@ -1187,9 +1198,13 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
                 w.lcost[I] = cost;
                 if (SPLIT) w.lfar[I] = cf;
                 if (caching) {
-                    const bool fits = nrun <= kslot;
-                    w.lruns[I] = fits ? nrun : -1;
-                    if (!fits) atomicAdd((unsigned long long*)&s_uncached, 1ULL);
+                    const bool fits = nrun[0] + nrun[1] <= kslot;
+                    w.lruns[I] = fits ? nrun[0] : -1;
+                    if (SPLIT) {
+                        w.lfruns[I] = nrun[1];
+                        if (!fits) atomicAdd((unsigned long long*)&s_redo, 1ULL);
+                    }
+                    if (SPLIT ? nall > kslot : !fits) atomicAdd((unsigned long long*)&s_uncached, 1ULL);
                 }
                 atomicAdd((unsigned long long*)&s_pairs, (unsigned long long)c);
                 atomicAdd((unsigned long long*)&s_eval, (unsigned long long)cost);
@@ -1206,18 +1221,21 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
         atomicAdd((unsigned long long*)(w.cnt + kCntEvaluated), (unsigned long long)s_eval);
         if (SPLIT) atomicAdd((unsigned long long*)(w.cnt + kCntFar), (unsigned long long)s_far);
         if (s_uncached) atomicAdd((unsigned long long*)(w.cnt + kCntUncached), (unsigned long long)s_uncached);
+        if (SPLIT && s_redo) atomicAdd((unsigned long long*)(w.cnt + kCntRedo), (unsigned long long)s_redo);
         atomicMax(w.cnt + kCntMaxCost, s_cost);
         atomicMax(w.cnt + kCntMaxRow, s_row);
     }
 }
 
-// Writes the cached rows at rowptr.  One warp per row: lane k loads run k of
+// Writes the cached rows at rowptr, near runs from the start of each slot or, with
+// lfruns, far runs from its end.  One warp per row: lane k loads run k of
 // a group of 32 (one coalesced load), a warp scan of the run lengths gives
 // each run's first entry, and the group's entries are written 32 at a time,
 // entry e finding its run by a binary search over the lanes (shuffles).  A
 // run list that does not add up to the row's length (a corrupt cache) sets
 // error bit 4.
 __global__ void __launch_bounds__(256) k_pairs_expand(int64_t nl, const int32_t* __restrict__ lruns,
+                                                      const int32_t* __restrict__ lfruns,
                                                       const uint2* __restrict__ cache, int kslot,
                                                       const int64_t* __restrict__ rowptr,
                                                       uint32_t* __restrict__ pairs,
@@ -1226,7 +1244,8 @@ __global__ void __launch_bounds__(256) k_pairs_expand(int64_t nl, const int32_t*
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t I = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); I < nl; I += nw) {
-        const int nrun = lruns[I];
+        int nrun = lruns[I];
+        if (nrun >= 0 && lfruns) nrun = lfruns[I];
         if (nrun <= 0) continue;  // empty, or walked by the write pass
         const uint2* slot = cache + I * (int64_t)kslot;
         const int64_t row0 = rowptr[I], len = rowptr[I + 1] - row0;
@@ -1234,7 +1253,8 @@ __global__ void __launch_bounds__(256) k_pairs_expand(int64_t nl, const int32_t*
         bool bad = false;
         for (int r0 = 0; r0 < nrun; r0 += 32) {
             const int nv = nrun - r0 < 32 ? nrun - r0 : 32;
-            const uint2 run = lane < nv ? slot[r0 + lane] : make_uint2(0u, 0u);
+            const int r = r0 + lane;
+            const uint2 run = lane < nv ? slot[lfruns ? kslot - 1 - r : r] : make_uint2(0u, 0u);
             int64_t inc = run.y;  // inclusive scan of the run lengths
             for (int o = 1; o < 32; o <<= 1) {
                 const int64_t v = __shfl_up_sync(kFull, inc, o);
@@ -1569,6 +1589,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     wa.cnt = cnt;
     wa.err = err;
     wa.lruns = (int32_t*)(s + S.lruns);
+    wa.lfruns = (int32_t*)(s + S.lfruns);
     wa.cache = (uint2*)(s + S.cache);
     wa.ncache = S.ncache;
     if (theta > 0.0) k_rows<false, true><<<walk_blocks(n, sms), 32 * kWalkWarps, 0, st>>>(wa);
@@ -1620,6 +1641,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     h->max_cost = c[kCntMaxCost];
     h->db_kslot = kslot;
     h->db_uncached = kslot ? c[kCntUncached] : nl;
+    h->db_redo = !kslot ? nl : theta > 0.0 ? c[kCntRedo] : c[kCntUncached];
     h->build_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     *out = reinterpret_cast<psr_leaves*>(h);
     return PSR_OK;
@@ -1714,14 +1736,19 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
         wa.bx.gt2 = (h->flags & PSR_BUILD_SPLIT_GAUSSIAN)
                         ? (float)(h->theta * h->theta * 4.0 * std::pow(h->boxes[0].r_s, 4))
                         : INFINITY;
-        k_rows<true, true><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
-    } else {
-        // rows the count walk cached are expanded; the rest are walked again
-        if (h->db_kslot) {
-            k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, wa.lruns, wa.cache, h->db_kslot, rowptr, wa.pairs, wa.err);
-            if ((e = (int)cudaGetLastError())) return dcuda(e, "pair expand kernel");
-        }
-        if (h->db_uncached > 0) k_rows<true, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
+    }
+    // rows the count walk cached are expanded; the rest are walked again
+    if (h->db_kslot) {
+        k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, wa.lruns, nullptr, wa.cache, h->db_kslot, rowptr, wa.pairs,
+                                                    wa.err);
+        if (h->has_far)
+            k_pairs_expand<<<nblk(nl, 8), 256, 0, st>>>(nl, wa.lruns, (const int32_t*)(s + S.lfruns), wa.cache,
+                                                        h->db_kslot, frow, wa.fpairs, wa.err);
+        if ((e = (int)cudaGetLastError())) return dcuda(e, "pair expand kernel");
+    }
+    if (h->db_redo > 0) {
+        if (h->has_far) k_rows<true, true><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
+        else k_rows<true, false><<<walk_blocks(nl, sms), 32 * kWalkWarps, 0, st>>>(wa);
     }
     if ((e = (int)cudaGetLastError())) return dcuda(e, "pair write kernel");
     // schedule: the particle sort buffers are free again (values in int32

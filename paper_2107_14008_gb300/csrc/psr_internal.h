@@ -121,6 +121,7 @@ struct Leaves {
     char* db_scratch = nullptr; // device build between its two calls: the caller's scratch
     int db_kslot = 0;           //   runs per row in the pair cache (0: not used)
     int64_t db_uncached = 0;    //   and the rows it could not hold
+    int64_t db_redo = 0;        //   rows to be walked again
     // device state
     Layout lay{};
     char* d_ws = nullptr;

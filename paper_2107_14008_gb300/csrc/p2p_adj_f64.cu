@@ -9,17 +9,13 @@
 
 namespace psr {
 
-constexpr int kStageAdj64 = 64;  // staged sources per warp (64 bytes each)
-
 template <bool EQM, int R>
 __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, const double* tab,
-                                           const double* tabq, double2* __restrict__ stage,
-                                           int2* __restrict__ meta, bool split)
+                                           const double* tabq, const Warp64& w64, bool split)
 {
     const int lane = threadIdx.x & 31;
     const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
     const double4* __restrict__ cs = reinterpret_cast<const double4*>(a.cot_sorted);
-    double* box = reinterpret_cast<double*>(meta + 32);
     const int nI = li.y, T = (nI + R - 1) / R, S = 32 / T, s = lane / T, q = lane - s * T;
     const bool on = s < S;
     const BoxDev& bx = a.boxes[li.z];
@@ -40,46 +36,52 @@ __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, con
 #pragma unroll
         for (int i = 0; i < 4; ++i) g[r][i] = 0.0;
     }
-    cull_box64<R>(xi, act, bx.r_c, bx.L, box);
+    cull_box64<R>(xi, act, bx.r_c, bx.L, w64.box);
+    const int kx = exponent_of(bx.r_c);
+    const float cut = cut64(bx.r_c, w64.box, kx);
+    float3 ti[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (!act[r]) xi[r].x = 1e150;  // beyond the cutoff of every source
+    for (int r = 0; r < R; ++r) ti[r] = target64(xi[r], w64.box, kx);
     long long e0, re;
     row_part(a, I, split, e0, re);
-    while (e0 < re) {
+    const int len = (int)(re - e0);
+    for (int e = 0; e < len;) {
         int nst;
-        e0 += stage64<4, true>(a, e0, re, bx.L, kStageAdj64, stage, meta, box, nst);
-        if (on)
-            for (int k = s; k < nst; k += S) {
-                const double2 A = stage[4 * k], B = stage[4 * k + 1];
-                const double2 C = stage[4 * k + 2], D = stage[4 * k + 3];
+        bool images;
+        e += stage64<true>(a, e0, len, e, bx.L, kx, w64, nst, images);
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const double dx = A.x - xi[r].x, dy = A.y - xi[r].y, dz = B.x - xi[r].z;
-                    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                    if (inside64(r2, rc2m1)) {
-                        const double ri = rsqrt64(r2), ri2 = ri * ri;
-                        double f;
-                        const int kk = 6 * node64(r2 * ri, us, a.t64_max, f);
-                        const double gg = horner64<5>(tab + kk, f) * (ri2 * ri);  // T / r^3
-                        const double Q = cq * horner64<5>(tabq + kk, f);
-                        const double hf = -ri2 * fma(3.0, gg, Q);  // g'(r)/r
-                        // v = m_k c_j - m_j c_k (one mass: c_j - c_k, m applied at the end)
-                        const double vx = EQM ? C.x - ck[r].x : fma(xi[r].w, C.x, -B.y * ck[r].x);
-                        const double vy = EQM ? C.y - ck[r].y : fma(xi[r].w, C.y, -B.y * ck[r].y);
-                        const double vz = EQM ? D.x - ck[r].z : fma(xi[r].w, D.x, -B.y * ck[r].z);
-                        const double hd = hf * fma(dx, vx, fma(dy, vy, dz * vz));
-                        g[r][0] = fma(gg, vx, fma(hd, dx, g[r][0]));
-                        g[r][1] = fma(gg, vy, fma(hd, dy, g[r][1]));
-                        g[r][2] = fma(gg, vz, fma(hd, dz, g[r][2]));
-                        g[r][3] = fma(gg, fma(dx, C.x, fma(dy, C.y, dz * D.x)), g[r][3]);
-                    }
+        for (int r = 0; r < R; ++r) {
+            w64.set_target(xi[r], bx.L, images);
+            near_pairs(w64.near, nst, s, S, ti[r], cut, act[r], [&](int k) {
+                const int j = __float_as_int(w64.near[k].w);
+                const double4 p = pd[j];
+                const double3 d = w64.diff(p, k);
+                const double dx = d.x, dy = d.y, dz = d.z;
+                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                if (inside64(r2, rc2m1)) {
+                    const double4 c = cs[j];
+                    const double ri = rsqrt64(r2), ri2 = ri * ri;
+                    double f;
+                    const int kk = 6 * node64(r2 * ri, us, a.t64_max, f);
+                    const double gg = horner64<5>(tab + kk, f) * (ri2 * ri);  // T / r^3
+                    const double Q = cq * horner64<5>(tabq + kk, f);
+                    const double hf = -ri2 * fma(3.0, gg, Q);  // g'(r)/r
+                    // v = m_k c_j - m_j c_k (one mass: c_j - c_k, m applied at the end)
+                    const double vx = EQM ? c.x - ck[r].x : fma(xi[r].w, c.x, -p.w * ck[r].x);
+                    const double vy = EQM ? c.y - ck[r].y : fma(xi[r].w, c.y, -p.w * ck[r].y);
+                    const double vz = EQM ? c.z - ck[r].z : fma(xi[r].w, c.z, -p.w * ck[r].z);
+                    const double hd = hf * fma(dx, vx, fma(dy, vy, dz * vz));
+                    g[r][0] = fma(gg, vx, fma(hd, dx, g[r][0]));
+                    g[r][1] = fma(gg, vy, fma(hd, dy, g[r][1]));
+                    g[r][2] = fma(gg, vz, fma(hd, dz, g[r][2]));
+                    g[r][3] = fma(gg, fma(dx, c.x, fma(dy, c.y, dz * c.z)), g[r][3]);
                 }
-            }
+            });
+        }
         __syncwarp();
     }
     const double G = bx.G, gx = EQM ? G * pd[li.x].w : G;
-    finish64<4, R>(a, li, g, act, lane, s, S, T, stage, split, warp64_bytes(4, kStageAdj64),
+    finish64<4, R>(a, li, g, act, lane, s, S, T, w64.near, split, kWarp64Bytes,
                    [&](int target, const double* v) {
                        const int idx = a.perm[target];
                        double* o = reinterpret_cast<double*>(a.out) + 3LL * idx;
@@ -104,9 +106,7 @@ __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    unsigned char* warp = smem64 + 16 * words + (threadIdx.x >> 5) * warp64_bytes(4, kStageAdj64);
-    double2* stage = reinterpret_cast<double2*>(warp);
-    int2* meta = reinterpret_cast<int2*>(warp + 64 * kStageAdj64);
+    const Warp64 w64(smem64 + 16 * words + (threadIdx.x >> 5) * kWarp64Bytes);
     const int n_heavy = a.group <= 1 ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
     bool split = n_heavy > 0;
     int it;
@@ -115,16 +115,16 @@ __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
         int4 li;
         if (!item64(a, it, lane, I, li)) continue;
         const int R = targets_per_lane(li.y, 128);
-        if (R == 1) adj64_item<EQM, 1>(a, I, li, tab, tabq, stage, meta, split);
-        else if (R == 2) adj64_item<EQM, 2>(a, I, li, tab, tabq, stage, meta, split);
-        else adj64_item<EQM, 3>(a, I, li, tab, tabq, stage, meta, split);
+        if (R == 1) adj64_item<EQM, 1>(a, I, li, tab, tabq, w64, split);
+        else if (R == 2) adj64_item<EQM, 2>(a, I, li, tab, tabq, w64, split);
+        else adj64_item<EQM, 3>(a, I, li, tab, tabq, w64, split);
     }
     persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
 }
 
 size_t adj_f64_smem(double x_c, int warps)
 {
-    return (size_t)(plain64(x_c).n + 2) * 96 + (size_t)warps * warp64_bytes(4, kStageAdj64);
+    return (size_t)(plain64(x_c).n + 2) * 96 + (size_t)warps * kWarp64Bytes;
 }
 
 int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)

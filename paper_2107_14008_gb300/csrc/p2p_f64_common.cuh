@@ -6,9 +6,13 @@
 // evaluations and nothing else; integer and FP32 work beside them is free up to
 // some 60 instructions per FP64 one.  The kernels therefore
 //  - stage a row's sources in shared memory, culled against the target leaf's
-//    box as the FP32 kernels do (here in FP64, 9 instructions per 32 sources),
-//    so that 88 % of the evaluated pairs of the 128^3 NFW set lie within the
-//    cutoff instead of 74 %;
+//    box as the FP32 kernels do (here in FP64, 9 instructions per 32 sources);
+//  - find each lane's pairs within the cutoff by an FP32 test first (rounded
+//    outward; a bit mask per lane), so that every lane then takes its own next
+//    pair: of uniform sets, whose leaves are large against the cutoff, 42 % of
+//    the lanes had a pair within it when all took the same source.  The
+//    entries are staged in strides over the row, which evens out the lanes'
+//    counts in a chunk (58 % against 49 % in row order);
 //  - fill the lanes with 1, 2 or 3 targets each (targets_per_lane): 92 % of
 //    them busy on packed leaves, where a power-of-two stream width left 63 %
 //    for a leaf of 20;
@@ -64,11 +68,63 @@ __device__ __forceinline__ double horner64(const double* __restrict__ c, double 
     return v;
 }
 
-// A warp's shared memory: cap staged sources of NV double2 ({x, y}, {z, m} and
-// for the adjoint {c_x, c_y}, {c_z, 0}), 32 entry records, and the target box
-// (centre, half extents, squared cutoff).
-constexpr int kMeta64Bytes = 32 * 8 + 8 * 8;
-__host__ __device__ constexpr int warp64_bytes(int nv, int cap) { return 16 * nv * cap + kMeta64Bytes; }
+// A warp's shared memory: kStage64 staged sources - FP32 coordinates from the
+// target box's centre in units of 2^k, k the exponent of r_c, the particle's
+// index, and its periodic steps (nx + 1) | (ny + 1) << 2 | (nz + 1) << 4 - then
+// the lanes' targets at the three steps of each axis, 32 entry records, and the
+// target box (centre, half extents, squared cutoff).  The FP64 coordinates are
+// read from global memory (L1, L2) per pair: a load is nothing beside a pair's
+// FP64 instructions, and the small buffers leave two blocks per SM.
+constexpr int kStage64 = 256;
+constexpr int kTarget64 = 17 * kStage64, kMeta64 = kTarget64 + 9 * 32 * 8, kBox64 = kMeta64 + 32 * 8;
+constexpr int kWarp64Bytes = kBox64 + 8 * 8;
+struct Warp64 {
+    float4* near;
+    unsigned char* steps;
+    double* target;
+    int2* meta;
+    double* box;
+    __device__ explicit Warp64(unsigned char* base)
+        : near(reinterpret_cast<float4*>(base)), steps(base + 16 * kStage64),
+          target(reinterpret_cast<double*>(base + kTarget64)), meta(reinterpret_cast<int2*>(base + kMeta64)),
+          box(reinterpret_cast<double*>(base + kBox64))
+    {
+    }
+    // the lane's target x at the steps n = -1, 0, 1 of each axis, x - n L: a pair's
+    // difference is then x_j - (x_i - n L) with no FP64 instruction for the image
+    // (images: some staged source is not in the box itself)
+    __device__ void set_target(double4 x, double L, bool images) const
+    {
+        double* t = target + (threadIdx.x & 31);
+#pragma unroll
+        for (int n = 0; n < 3; ++n) {
+            if (n != 1 && !images) continue;
+            const double s = (n - 1) * L;
+            t[32 * n] = n == 1 ? x.x : x.x - s;
+            t[32 * (3 + n)] = n == 1 ? x.y : x.y - s;
+            t[32 * (6 + n)] = n == 1 ? x.z : x.z - s;
+        }
+    }
+    // staged source k's difference from the target
+    __device__ double3 diff(double4 p, int k) const
+    {
+        const double* t = target + (threadIdx.x & 31);
+        const int c = steps[k];
+        return make_double3(p.x - t[32 * (c & 3)], p.y - t[32 * (3 + ((c >> 2) & 3))], p.z - t[32 * (6 + (c >> 4))]);
+    }
+};
+
+// d in units of 2^k as FP32, cut to 23 bits, in integer arithmetic (d below
+// 2^(k - 126) gives 0, above 2^(k + 126) a value far beyond the cutoff)
+__device__ __forceinline__ float near_float(double d, int k)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 1023 - k;
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned f = e < -126 ? 0u : e > 126 ? 0x7e800000u : ((unsigned)(e + 127) << 23) | m;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+__device__ __forceinline__ int exponent_of(double x) { return (int)((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
 
 // The target box of the lanes' R targets; the squared cutoff is widened by what
 // the FP64 rounding of box and coordinates can move a distance.
@@ -101,27 +157,28 @@ __device__ __forceinline__ void cull_box64(const double4* xi, const bool* act, d
     __syncwarp();
 }
 
-// Stages one chunk of the row from entry e0 on (the scheme of stage_chunk in
-// fwd_f32_common.cuh): returns the entries taken, nst the staged sources, each
-// at its periodic image.
-template <int NV, bool CULL>
-__device__ __forceinline__ int stage64(const FwdArgs& a, long long e0, long long re, double L, int cap,
-                                       double2* __restrict__ stage, int2* __restrict__ meta,
-                                       const double* __restrict__ box, int& nst)
+// Stages one chunk of the row part [e0, e0 + len) (the scheme of stage_chunk in
+// fwd_f32_common.cuh), from its p-th entry on in strided order: 32 columns of
+// consecutive entries, taken row by row.  Returns the entries taken, nst the
+// staged sources, each at its periodic image.
+template <bool CULL>
+__device__ __forceinline__ int stage64(const FwdArgs& a, long long e0, int len, int p, double L, int kx,
+                                       const Warp64& w, int& nst, bool& images)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
-    const double4* __restrict__ cs = reinterpret_cast<const double4*>(a.cot_sorted);
     const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
     const unsigned* __restrict__ prow = a.pairs + e0;
-    const int rem = (int)min(re - e0, (long long)0x7fffffff);
-    int nk = 0, eb = 0;
+    const int col = len >> 5, more = len & 31;  // the first `more` columns have one more entry
+    int nk = 0, eb = p;
+    bool shifted = false;  // this lane staged a source at an image
     for (;;) {
         const int e = eb + lane;
         int cnt = 0, first = 0, code = 13;
-        if (e < rem) {
-            const unsigned ent = prow[e];
+        if (e < len) {
+            const int c = e & 31;
+            const unsigned ent = prow[c * col + min(c, more) + (e >> 5)];
             const int J = (int)(ent >> 5);
             code = (int)(ent & 31u);
             unsigned bad = J >= a.n_leaves ? kErrLeafIndex : code >= kShiftCodes ? kErrShiftCode : 0u;
@@ -145,10 +202,10 @@ __device__ __forceinline__ int stage64(const FwdArgs& a, long long e0, long long
             const int v = __shfl_up_sync(kFull, incl, o);
             if (lane >= o) incl += v;
         }
-        const int ntake = __popc(__ballot_sync(kFull, e < rem && incl <= cap - nk));
+        const int ntake = __popc(__ballot_sync(kFull, e < len && incl <= kStage64 - nk));
         if (ntake == 0) break;
         const int nraw = __shfl_sync(kFull, incl, ntake - 1), excl = incl - cnt;
-        if (lane < ntake) meta[lane] = make_int2(first - excl, code);
+        if (lane < ntake) w.meta[lane] = make_int2(first - excl, code);
         __syncwarp();
         int C = 0;  // entry starts before this round
         for (int p0 = 0; p0 < nraw; p0 += 32) {
@@ -157,49 +214,107 @@ __device__ __forceinline__ int stage64(const FwdArgs& a, long long e0, long long
                 __reduce_or_sync(kFull, (lane < ntake && rel >= 0 && rel < 32) ? (1u << rel) : 0u);
             const int k = C + __popc(M & ((2u << lane) - 1u)) - 1;
             C += __popc(M);
-            const int p = p0 + lane;
-            bool keep = p < nraw;
-            double4 v = make_double4(0.0, 0.0, 0.0, 0.0), c = v;
+            const int q = p0 + lane;
+            bool keep = q < nraw;
+            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+            int steps = 21;  // 1 | 1 << 2 | 1 << 4: no shift
             if (keep) {
-                const int2 m = meta[k];
-                const int src = m.x + p;
-                v = pd[src];
-                if (NV == 4) c = cs[src];
+                const int2 m = w.meta[k];
+                const int src = m.x + q;
+                double4 v = pd[src];
                 if (m.y != 13 && m.y >= 0) {
                     int nx, ny, nz;
                     decode_shift((unsigned)m.y, nx, ny, nz);
-                    v.x = fma((double)nx, L, v.x);
-                    v.y = fma((double)ny, L, v.y);
-                    v.z = fma((double)nz, L, v.z);
+                    if (nx) v.x = fma((double)nx, L, v.x);
+                    if (ny) v.y = fma((double)ny, L, v.y);
+                    if (nz) v.z = fma((double)nz, L, v.z);
+                    steps = (nx + 1) | (ny + 1) << 2 | (nz + 1) << 4;
                 }
                 keep = m.y >= 0;
+                const double d[3] = {v.x - w.box[0], v.y - w.box[1], v.z - w.box[2]};
+                f = make_float4(near_float(d[0], kx), near_float(d[1], kx), near_float(d[2], kx), __int_as_float(src));
                 if (CULL) {
-                    double g[3] = {fabs(v.x - box[0]) - box[3], fabs(v.y - box[1]) - box[4],
-                                   fabs(v.z - box[2]) - box[5]};
+                    double g[3];
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) g[i] = bits64(g[i]) < 0 ? 0.0 : g[i];
-                    keep = keep && bits64(fma(g[0], g[0], fma(g[1], g[1], g[2] * g[2]))) < bits64(box[6]);
+                    for (int i = 0; i < 3; ++i) {
+                        g[i] = fabs(d[i]) - w.box[3 + i];
+                        g[i] = bits64(g[i]) < 0 ? 0.0 : g[i];
+                    }
+                    keep = keep && bits64(fma(g[0], g[0], fma(g[1], g[1], g[2] * g[2]))) < bits64(w.box[6]);
                 }
             }
             const unsigned K = __ballot_sync(kFull, keep);
             if (keep) {
-                double2* d = stage + NV * (nk + __popc(K & lt));
-                d[0] = make_double2(v.x, v.y);
-                d[1] = make_double2(v.z, v.w);
-                if (NV == 4) {
-                    d[2] = make_double2(c.x, c.y);
-                    d[NV - 1] = make_double2(c.z, 0.0);
-                }
+                const int pos = nk + __popc(K & lt);
+                w.near[pos] = f;
+                w.steps[pos] = (unsigned char)steps;
+                shifted = shifted || steps != 21;
             }
             nk += __popc(K);
         }
         __syncwarp();
         eb += ntake;
-        if (ntake < 32 || eb >= rem) break;
+        if (ntake < 32 || eb >= len) break;
+    }
+    images = __any_sync(kFull, shifted);
+    nst = nk;
+    return eb - p;
+}
+
+// A target in the same FP32 coordinates, and the squared distance below which a
+// staged source may lie within the cutoff: coordinates are at most r_c plus
+// twice the half extents, cut by 2^-23 of that, differences and squares by a few
+// 2^-24 more, which 1e-6 of the sum covers.
+__device__ __forceinline__ float3 target64(double4 x, const double* box, int kx)
+{
+    return make_float3(near_float(x.x - box[0], kx), near_float(x.y - box[1], kx), near_float(x.z - box[2], kx));
+}
+__device__ __forceinline__ float cut64(double r_c, const double* box, int kx)
+{
+    const double w = r_c + 1e-6 * (r_c + 2.0 * (box[3] + box[4] + box[5]));
+    const float f = near_float(w, kx) * 1.000001f;
+    return f * f;
+}
+
+// Calls pair(k) for each staged source k of the lane's stream (s, s + S, ...)
+// that may lie within the cutoff of the lane's target t.
+// Every lane takes its own next one, by a bit mask over its stream's sources.
+template <class Pair>
+__device__ __forceinline__ void near_pairs(const float4* __restrict__ near, int nst, int s, int S, float3 t,
+                                           float cut, bool on, Pair pair)
+{
+    auto maybe = [&](int k) {
+        const float4 v = near[k];
+        const float dx = v.x - t.x, dy = v.y - t.y, dz = v.z - t.z;
+        return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < cut;
+    };
+    constexpr int kWords = kStage64 / 32;
+    const int J = on && nst > s ? (nst - s + S - 1) / S : 0;  // sources of this lane's stream
+    unsigned m[kWords];
+#pragma unroll
+    for (int w = 0; w < kWords; ++w) {
+        m[w] = 0;
+        const int jn = min(J - 32 * w, 32);
+        for (int j = 0; j < jn; ++j) m[w] |= (maybe(s + (32 * w + j) * S) ? 1u : 0u) << j;
     }
     __syncwarp();
-    nst = nk;
-    return eb;
+    for (;;) {
+        int w = 0;  // the lane's next word with a bit left
+        unsigned bits = 0;
+#pragma unroll
+        for (int i = kWords - 1; i >= 0; --i)
+            if (m[i]) {
+                w = i;
+                bits = m[i];
+            }
+        if (!__any_sync(kFull, bits != 0)) break;
+        if (bits) {
+#pragma unroll
+            for (int i = 0; i < kWords; ++i)
+                if (i == w) m[i] &= m[i] - 1;
+            pair(s + (32 * w + __ffs(bits) - 1) * S);
+        }
+    }
 }
 
 // Adds the S stream partials (NC components per target slot) of each target
@@ -208,7 +323,7 @@ __device__ __forceinline__ int stage64(const FwdArgs& a, long long e0, long long
 // added after that, in warp order (stride: bytes between the warps' buffers).
 template <int NC, int R, class Write>
 __device__ __forceinline__ void finish64(const FwdArgs& a, int4 li, const double (*acc)[NC], const bool* act,
-                                         int lane, int s, int S, int T, double2* __restrict__ stage,
+                                         int lane, int s, int S, int T, float4* __restrict__ stage,
                                          bool split, int stride, Write write)
 {
 #pragma unroll

@@ -12,8 +12,6 @@
 
 namespace psr {
 
-constexpr int kStage64 = 128;  // staged sources per warp
-
 // Taylor tables in FP64: node k = 0..N, x_k = k h, six doubles per node, the
 // coefficients of eps^m (eps = x - x_k) times h^m, so that the expansion is a
 // polynomial in f = x/h - k (zero above the level).  T's are those of Eq. int and
@@ -77,12 +75,11 @@ int launch_plain64(double x_c, void* d_t, void* d_q, void* stream)
 // cull).
 template <bool COUNT, bool EQM, int DEG, int R>
 __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, const double* tab,
-                                           double2* __restrict__ stage, int2* __restrict__ meta,
-                                           unsigned long long& npairs, unsigned long long& nev, bool split)
+                                           const Warp64& w64, unsigned long long& npairs,
+                                           unsigned long long& nev, bool split)
 {
     const int lane = threadIdx.x & 31;
     const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
-    double* box = reinterpret_cast<double*>(meta + 32);
     const int nI = li.y, T = (nI + R - 1) / R, S = 32 / T, s = lane / T, q = lane - s * T;
     const bool on = s < S;
     const BoxDev& bx = a.boxes[li.z];
@@ -100,43 +97,49 @@ __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, con
         xi[r] = pd[li.x + (act[r] ? t : 0)];
         acc[r][0] = acc[r][1] = acc[r][2] = 0.0;
     }
-    if (!COUNT) cull_box64<R>(xi, act, bx.r_c, bx.L, box);
+    cull_box64<R>(xi, act, bx.r_c, bx.L, w64.box);
+    const int kx = exponent_of(bx.r_c);
+    const float cut = cut64(bx.r_c, w64.box, kx);
+    float3 ti[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (!act[r]) xi[r].x = 1e150;  // beyond the cutoff of every source
+    for (int r = 0; r < R; ++r) ti[r] = target64(xi[r], w64.box, kx);
     unsigned cnt = 0;
     long long e0, re;
     row_part(a, I, split, e0, re);
-    while (e0 < re) {
+    const int len = (int)(re - e0);
+    for (int e = 0; e < len;) {
         int nst;
-        e0 += stage64<2, !COUNT>(a, e0, re, bx.L, kStage64, stage, meta, box, nst);
+        bool images;
+        e += stage64<!COUNT>(a, e0, len, e, bx.L, kx, w64, nst, images);
         if (COUNT && lane == 0) nev += (unsigned long long)nst * (unsigned)nI;
-        if (on)
-            for (int k = s; k < nst; k += S) {
-                const double2 A = stage[2 * k], B = stage[2 * k + 1];
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const double dx = A.x - xi[r].x, dy = A.y - xi[r].y, dz = B.x - xi[r].z;
-                    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                    if (inside64(r2, rc2m1)) {
-                        const double ri = rsqrt64(r2);
-                        double f;
-                        const int kk = node64(r2 * ri, us, kmax, f);
-                        const double Tv = horner64<DEG>(tab + 6 * kk, f);
-                        double w = ri * ri * ri * Tv;
-                        if (!EQM) w *= B.y;
-                        acc[r][0] = fma(w, dx, acc[r][0]);
-                        acc[r][1] = fma(w, dy, acc[r][1]);
-                        acc[r][2] = fma(w, dz, acc[r][2]);
-                        if (COUNT) ++cnt;
-                    }
+        for (int r = 0; r < R; ++r) {
+            w64.set_target(xi[r], bx.L, images);
+            near_pairs(w64.near, nst, s, S, ti[r], cut, act[r], [&](int k) {
+                const int j = __float_as_int(w64.near[k].w);
+                const double4 p = pd[j];
+                const double3 d = w64.diff(p, k);
+                const double dx = d.x, dy = d.y, dz = d.z;
+                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                if (inside64(r2, rc2m1)) {
+                    const double ri = rsqrt64(r2);
+                    double f;
+                    const int kk = node64(r2 * ri, us, kmax, f);
+                    const double Tv = horner64<DEG>(tab + 6 * kk, f);
+                    double w = ri * ri * ri * Tv;
+                    if (!EQM) w *= p.w;
+                    acc[r][0] = fma(w, dx, acc[r][0]);
+                    acc[r][1] = fma(w, dy, acc[r][1]);
+                    acc[r][2] = fma(w, dz, acc[r][2]);
+                    if (COUNT) ++cnt;
                 }
-            }
+            });
+        }
         __syncwarp();
     }
     if (COUNT) npairs += cnt;
     const double g = EQM ? bx.G * pd[li.x].w : bx.G;
-    finish64<3, R>(a, li, acc, act, lane, s, S, T, stage, split, warp64_bytes(2, kStage64),
+    finish64<3, R>(a, li, acc, act, lane, s, S, T, w64.near, split, kWarp64Bytes,
                    [&](int target, const double* v) {
                        double* out = reinterpret_cast<double*>(a.out) + 3LL * a.perm[target];
                        out[0] = g * v[0];
@@ -156,9 +159,7 @@ __global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
     for (int i = threadIdx.x; i < words; i += blockDim.x) tab[i] = reinterpret_cast<const double*>(a.table)[i];
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    unsigned char* warp = smem64 + 8 * words + (threadIdx.x >> 5) * warp64_bytes(2, kStage64);
-    double2* stage = reinterpret_cast<double2*>(warp);
-    int2* meta = reinterpret_cast<int2*>(warp + 32 * kStage64);
+    const Warp64 w64(smem64 + 8 * words + (threadIdx.x >> 5) * kWarp64Bytes);
     unsigned long long npairs = 0, nev = 0;
     const int n_heavy = a.group <= 1 ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
     bool split = n_heavy > 0;
@@ -168,9 +169,9 @@ __global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
         int4 li;
         if (!item64(a, it, lane, I, li)) continue;
         const int R = targets_per_lane(li.y, 128);
-        if (R == 1) fwd64_item<COUNT, EQM, DEG, 1>(a, I, li, tab, stage, meta, npairs, nev, split);
-        else if (R == 2) fwd64_item<COUNT, EQM, DEG, 2>(a, I, li, tab, stage, meta, npairs, nev, split);
-        else fwd64_item<COUNT, EQM, DEG, 3>(a, I, li, tab, stage, meta, npairs, nev, split);
+        if (R == 1) fwd64_item<COUNT, EQM, DEG, 1>(a, I, li, tab, w64, npairs, nev, split);
+        else if (R == 2) fwd64_item<COUNT, EQM, DEG, 2>(a, I, li, tab, w64, npairs, nev, split);
+        else fwd64_item<COUNT, EQM, DEG, 3>(a, I, li, tab, w64, npairs, nev, split);
     }
     if (COUNT) {
         for (int off = 16; off > 0; off >>= 1) npairs += __shfl_xor_sync(kFull, npairs, off);
@@ -199,7 +200,7 @@ const void* pick64(bool count, bool eqm)
 size_t fwd_f64_smem(int interp, int table_n, double x_c, int warps)
 {
     const int entries = taylor64(interp) ? table_n + 1 : plain64(x_c).n + 2;
-    return (size_t)entries * 48 + (size_t)warps * warp64_bytes(2, kStage64);
+    return (size_t)entries * 48 + (size_t)warps * kWarp64Bytes;
 }
 
 int launch_fwd_f64(const FwdArgs& args, double x_c, void* stream)

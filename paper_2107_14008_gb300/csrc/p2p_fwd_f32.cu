@@ -72,7 +72,8 @@ __global__ void table_kernel(int N, int interp, double x_c, float4* __restrict__
 
 int launch_table(int table_n, int interp, double x_c, void* d_out, void* d_q_out, void* stream)
 {
-    int threads = 256, blocks = (table_n + 1 + threads - 1) / threads;
+    // one warp per block: FP64 work, one SM's FP64 pipe per warp (16 -> 4 us for 1024 intervals)
+    int threads = 32, blocks = (table_n + 1 + threads - 1) / threads;
     table_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
         table_n, interp, x_c, reinterpret_cast<float4*>(d_out), reinterpret_cast<float4*>(d_q_out));
     return (int)cudaGetLastError();
@@ -80,18 +81,21 @@ int launch_table(int table_n, int interp, double x_c, void* d_out, void* d_q_out
 
 // (1 - T(x)) / x^3, an entire function of x^2: its series
 // (4 / sqrt(pi)) sum_n (-1)^n x^(2n) / (n! (2n + 3)) below x = 0.7 (where the
-// difference would cancel; the first term left out is below 1e-17), the
+// difference would cancel; the first term left out is below 1e-18), the
 // closed form above.
 __device__ double core_h(double x)
 {
+    constexpr double c[16] = {
+        0.7522527780636751, -0.45135166683820505, 0.16119702387078752, -0.0417918210035375,
+        0.008548327023450852, -0.0014466399578147598, 0.00020895910501768752, -2.6339382985422794e-05,
+        2.9458520444222863e-06, -2.961438563175843e-07, 2.703922166377944e-08, -2.2614621755160987e-09,
+        1.7449553823426687e-10, -1.2497027937202137e-11, 8.350548621632764e-13, -5.2296365105174886e-14};
     const double x2 = x * x;
     if (x < 0.7) {
-        double s = 0.0, t = 1.0;
-        for (int n = 0; n < 15; ++n) {
-            s += t / (2 * n + 3);
-            t *= -x2 / (n + 1);
-        }
-        return 2.0 * 1.1283791670955126 * s;
+        double s = c[15];
+#pragma unroll
+        for (int n = 14; n >= 0; --n) s = fma(s, x2, c[n]);
+        return s;
     }
     return (1.0 - (erfc(x) + 1.1283791670955126 * x * exp(-x2))) / (x2 * x);
 }
@@ -99,26 +103,28 @@ __device__ double core_h(double x)
 // Core table (core_weight): entries k = 0..N-1 are minus the chord of H(q) =
 // x_c^3 (1 - T) / x^3, q = (x / x_c)^2, over q N in [k, k + 1], moved by half
 // its error at the interval's middle; entry N, met at and beyond the cutoff
-// (q = 1, 1/r = 1), is -1.
+// (q = 1, 1/r = 1), is -1.  Bound: the FP64 pipe; a step's leaf set builds its
+// table anew, so the warps go to as many SMs (31 entries a warp, a block each;
+// the next lane has the next node): 1024 intervals in blocks of 256 threads
+// that evaluated three points each took 51 us.
+constexpr int kCoreEntries = 31;
 __global__ void core_table_kernel(int N, double x_c, float2* __restrict__ t)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > N) return;
-    if (k == N) {
-        t[k] = make_float2(-1.0f, 0.0f);
-        return;
-    }
-    const double s3 = x_c * x_c * x_c, q0 = (double)k / N, q1 = (double)(k + 1) / N;
-    const double h0 = s3 * core_h(x_c * sqrt(q0)), h1 = s3 * core_h(x_c * sqrt(q1));
-    const double hm = s3 * core_h(x_c * sqrt(0.5 * (q0 + q1)));
+    const int k = blockIdx.x * kCoreEntries + threadIdx.x;  // node; lane 31 is the next block's first
+    const double s3 = x_c * x_c * x_c, step = 1.0 / N;      // N is a power of two
+    const double q0 = k * step;
+    const double h0 = s3 * core_h(x_c * sqrt(q0)), hm = s3 * core_h(x_c * sqrt(q0 + 0.5 * step));
+    const double h1 = __shfl_down_sync(kFull, h0, 1);
+    if (threadIdx.x == kCoreEntries || k > N) return;
     const double D = (h1 - h0) * N;
-    t[k] = make_float2((float)(-(h0 - D * q0 + 0.5 * (hm - 0.5 * (h0 + h1)))), (float)-D);
+    t[k] = k == N ? make_float2(-1.0f, 0.0f)
+                  : make_float2((float)(-(h0 - D * q0 + 0.5 * (hm - 0.5 * (h0 + h1)))), (float)-D);
 }
 
 int launch_core_table(int table_n, double x_c, void* d_out, void* stream)
 {
-    const int threads = 256, blocks = (table_n + 1 + threads - 1) / threads;
-    core_table_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(table_n, x_c,
+    const int blocks = (table_n + 1 + kCoreEntries - 1) / kCoreEntries;
+    core_table_kernel<<<blocks, 32, 0, (cudaStream_t)stream>>>(table_n, x_c,
                                                                     reinterpret_cast<float2*>(d_out));
     return (int)cudaGetLastError();
 }

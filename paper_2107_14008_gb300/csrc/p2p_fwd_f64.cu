@@ -44,7 +44,7 @@ __global__ void table64_kernel(int N, int level, double h, double* __restrict__ 
 
 int launch_table64(int table_n, int interp, double x_c, void* d_out, void* stream)
 {
-    const int threads = 128, blocks = (table_n + 1 + threads - 1) / threads;
+    const int threads = 32, blocks = (table_n + 1 + threads - 1) / threads;
     table64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
         table_n, interp == PSR_TAYLOR4 ? 4 : 2, x_c / table_n, reinterpret_cast<double*>(d_out), nullptr);
     return (int)cudaGetLastError();
@@ -63,7 +63,7 @@ Plain64 plain64(double x_c)
 int launch_plain64(double x_c, void* d_t, void* d_q, void* stream)
 {
     const Plain64 p = plain64(x_c);
-    const int threads = 128, blocks = (p.n + 2 + threads - 1) / threads;
+    const int threads = 32, blocks = (p.n + 2 + threads - 1) / threads;
     table64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
         p.n, 5, p.x_top / p.n, reinterpret_cast<double*>(d_t), reinterpret_cast<double*>(d_q));
     return (int)cudaGetLastError();

@@ -45,6 +45,7 @@ int wait_stream(cudaStream_t st, int timeout_ms)
 
 struct Opts {
     int precision, table_n, interp, accum, warps, bps, fold, count, kernel, tile, nshard, shard;
+    bool fine = false;  // PSR_FP32_EXACT by the fine cubic table (fine_exact)
     bool split;  // heavy items on whole blocks: the default kernel's choice
 };
 
@@ -83,7 +84,7 @@ int check_opts(const psr_opts* o, Opts* out)
     if (fold < 1) return fail(PSR_E_ARG, "psr_opts.fold_every must be positive");
     *out = Opts{o->precision, tn, o->interp, o->accum, w, o->blocks_per_sm, fold,
                 o->count_pairs ? 1 : 0, o->kernel,
-                o->source_tile, nshard, o->shard_index, o->kernel == PSR_KERNEL_AUTO};
+                o->source_tile, nshard, o->shard_index, false, o->kernel == PSR_KERNEL_AUTO};
     return PSR_OK;
 }
 
@@ -147,6 +148,7 @@ FwdArgs base_args(Leaves* h, const Opts& o)
     a.warps_per_block = o.warps;
     a.max_leaf = h->max_leaf;
     a.variant = o.kernel;
+    a.fine = o.fine ? 1 : 0;
     a.item_stride = o.nshard;
     a.item_offset = o.shard;
     a.equal_mass = h->equal_mass ? 1 : 0;
@@ -161,6 +163,22 @@ bool fp64_taylor(const Opts& o)
 double cutoff_x(const Leaves* h)
 {
     return h->boxes.empty() ? 0.0 : h->boxes[0].r_c / (2.0 * h->boxes[0].r_s);
+}
+
+// PSR_FP32_EXACT under PSR_KERNEL_AUTO: T to FP32 rounding from a cubic table of
+// nodes at most 0.0049 apart (off by 2e-11) instead of erfcf and expf per pair
+// (64^3 NFW set: forward 4.99 -> 2.31 ms, adjoint 5.68 -> 3.4 ms, the same error
+// against 64 bits), up to x_c = 4.5; beyond, where the table's relative error in
+// the tail of T reaches FP32 rounding, erfcf and expf stay, as under the named
+// kernels.  512 intervals up to x_c = 2.5: the adjoint's table (32 bytes an entry)
+// then leaves three blocks per SM instead of two.
+void fine_exact(const Leaves* h, Opts& o)
+{
+    if (o.precision != PSR_FP32_EXACT || o.kernel != PSR_KERNEL_AUTO || cutoff_x(h) > 4.5) return;
+    o.precision = PSR_FP32_TABLE;
+    o.interp = PSR_CUBIC;
+    o.table_n = cutoff_x(h) <= 2.5 ? 512 : 1024;
+    o.fine = true;
 }
 
 // PSR_KERNEL_AUTO for the forward: packed pairs with the core form of the
@@ -237,12 +255,19 @@ int grid_blocks(Leaves* h, const Opts& o, int adjoint, int* blocks)
 }
 
 // Heavy rows shared among warps (the default kernels only), for a launch
-// whose grid is known.
+// whose grid is known.  The line (SplitRule): 3/2 of a share; 5/4 where a pair
+// costs more, as with every table but the linear one (cubic adjoint, 150,000 NFW
+// 4.33 -> 2.72 ms against a line of 2), and 2 for the linear adjoint of leaves of
+// up to 32, whose rows are short against the group's overheads (150,000 NFW in
+// leaves of up to 16 1.95 ms, 2.05 with 3/2; 64^3 NFW 2.74 and 2.83; in leaves of
+// up to 64, 512,000 NFW gain 5.96 -> 5.36 with 3/2).
 void set_split(const Leaves* h, const Opts& o, bool adjoint, FwdArgs* a)
 {
     if (!o.split && o.precision != PSR_FP64) return;
+    const bool linear = o.precision == PSR_FP32_TABLE && o.interp == PSR_LINEAR;
+    const int line = !linear ? 10 : adjoint && h->max_leaf <= 32 ? 16 : 12;
     const SplitRule r = split_rule(h->max_cost, h->evaluated, h->n_leaves, h->sm_count,
-                                   (int64_t)a->blocks * o.warps, o.warps, adjoint);
+                                   (int64_t)a->blocks * o.warps, o.warps, line);
     a->group = r.group;
     if (r.level >= 0)
         a->heavy = reinterpret_cast<const int*>(h->d_ws + h->lay.ctrl) + kCtrlHeavy + r.level;
@@ -261,6 +286,7 @@ int prepare_forward(Leaves* h, const psr_opts* opts, FwdArgs* a, int* precision)
     Opts o;
     int rc = check_opts(opts, &o);
     if (rc) return rc;
+    fine_exact(h, o);
     resolve_kernel(h, o);
     if (o.precision == PSR_FP64 && !h->has_pd)
         return fail(PSR_E_STATE, "built with PSR_BUILD_NO_FP64: no FP64 payload");
@@ -405,6 +431,7 @@ int psr_p2p_forces(psr_leaves* hh, const psr_opts* opts, void* d_acc, void* stre
     cudaStream_t st = (cudaStream_t)stream;
     const bool fwd32 = o.precision != PSR_FP64;
     if ((rc = resolve_warps(o, fwd32))) return rc;
+    fine_exact(h, o);
     resolve_kernel(h, o);
     const bool core = fwd_core(o.precision, o.interp, o.table_n, o.kernel, cutoff_x(h));
     if ((rc = ensure_table(h, o, core, st))) return rc;
@@ -448,6 +475,7 @@ int psr_p2p_adjoint(psr_leaves* hh, const psr_opts* opts, const void* d_cot, voi
         return fail(PSR_E_STATE, "built with PSR_BUILD_NO_FP64: no FP64 payload");
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = resolve_warps(o, false))) return rc;
+    fine_exact(h, o);
     if ((rc = ensure_table(h, o, false, st))) return rc;
     FwdArgs a = base_args(h, o);
     a.cot = d_cot;

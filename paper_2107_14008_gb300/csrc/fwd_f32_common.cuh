@@ -36,7 +36,7 @@
 
 namespace psr {
 
-enum { TM_EXACT = 0, TM_LINEAR = 1, TM_CUBIC = 2, TM_TAYLOR = 3, TM_CORE = 4 };
+enum { TM_EXACT = 0, TM_LINEAR = 1, TM_CUBIC = 2, TM_TAYLOR = 3, TM_CORE = 4, TM_FINE = 5 };
 
 // a * b + c clamped to [0, 1] in one instruction
 __device__ __forceinline__ float fma_sat(float a, float b, float c)
@@ -58,6 +58,11 @@ __device__ __forceinline__ float linear_T(float s, float nmax, unsigned tab_bias
     const float2 c = lds_f2((unsigned)__float_as_int(fk) * 8u + tab_bias);
     return fmaf(s, c.y, c.x);
 }
+
+// TM_FINE is what PSR_FP32_EXACT runs by default: T to FP32 rounding from a fine
+// cubic table, with coordinates left in units of 2 r_s as erfcf and expf had them (the table
+// paths' scaling rounds each coordinate once more, which costs 40 % in the
+// total error).  64^3 NFW set: 5.0 ms with erfcf and expf, see fine_exact.
 
 // Core form of the linear table.  With distances in units of x_c and
 // q = r^2, the pair weight is T / r^3 = 1/r^3 - H(q), H = (1 - T) / r^3, and H
@@ -703,9 +708,10 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
     const float x_c = bx.x_c;
     const float nmax = (float)a.table_n;
     const float soff = -0.5f / nmax;  // linear path: s = sat(r / x_c - 1/(2N))
-    const float sc = TM == TM_EXACT ? 1.0f
+    const float sc = TM == TM_EXACT || TM == TM_FINE ? 1.0f
                      : TM == TM_LINEAR || TM == TM_CORE ? 1.0f / x_c : (float)a.table_n / x_c;
     const float xscale = 1.0f / sc;
+    const float tsc = nmax / x_c;  // fine path: x -> table units
     const float unit = bx.unit;
     const int4 ci = lcen[I];
 
@@ -756,6 +762,7 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
                         if (!EQM) w *= p.w;
                     } else {
                         const float t = TM == TM_LINEAR ? fma_sat(r2, rinv, soff)
+                                        : TM == TM_FINE ? fmaf(r2 * rinv, tsc, -0.5f)
                                                         : fmaf(r2, rinv, TM == TM_TAYLOR ? 0.0f : -0.5f);
                         const float Tv = eval_T1<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
                         // 1/r^3 formed beside the table lookup (two dependent
@@ -768,7 +775,8 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
                     fz[r] = fmaf(w, dz, fz[r]);
                     if (COUNT) {
                         const float u = TM == TM_CORE ? r2 : r2 * rinv;
-                        const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
+                        const float uc = TM == TM_EXACT || TM == TM_FINE ? x_c
+                                         : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
                         cnt += (act[r] && u < uc && (dx != 0.0f || dy != 0.0f || dz != 0.0f));
                     }
                 }
@@ -817,7 +825,7 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const unsigned esize = TM == TM_TAYLOR ? 32u : TM == TM_CUBIC ? 16u : 8u;
+    const unsigned esize = TM == TM_TAYLOR ? 32u : TM == TM_CUBIC || TM == TM_FINE ? 16u : 8u;
     const size_t tab_bytes = TM == TM_EXACT ? 0 : (size_t)(a.table_n + 1) * esize;
     float4* stage = reinterpret_cast<float4*>(smem + ((tab_bytes + 15) & ~(size_t)15)) +
                     (size_t)warp * (a.stage_cap + kWarpMeta);
@@ -927,6 +935,10 @@ static int launch_s(const FwdArgs& a, size_t smem, cudaStream_t st)
 template <bool PK, bool SPLIT>
 static int launch_fwd_f32_t(const FwdArgs& a, int precision, size_t smem, cudaStream_t st)
 {
+    if constexpr (!PK)
+        if (a.fine)
+            return a.accum == PSR_ACC_FP64 ? launch_s<TM_FINE, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
+                                           : launch_s<TM_FINE, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
     if (precision == PSR_FP32_EXACT)
         return a.accum == PSR_ACC_FP64 ? launch_s<TM_EXACT, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
                                        : launch_s<TM_EXACT, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);

@@ -387,8 +387,9 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
     const float nmax = (float)a.table_n;
     // working unit: x for the exact path, x / x_c for the linear table (whose
     // entries carry c4), table intervals for the cubic one
-    const float sc = TM == TM_EXACT ? 1.0f : TM == TM_LINEAR ? 1.0f / x_c : (float)a.table_n / x_c;
+    const float sc = TM == TM_EXACT || TM == TM_FINE ? 1.0f : TM == TM_LINEAR ? 1.0f / x_c : (float)a.table_n / x_c;
     const float xscale = 1.0f / sc;
+    const float tsc = nmax / x_c;  // fine path: x -> table units
     const float c4 = kFourOverSqrtPi / (sc * sc * sc);  // (4/sqrt(pi)) in working units
     const float sref = 1.0f + 0.5f / nmax;               // linear: s' = sat(1 + 1/(2N) - r / x_c)
     const float unit = bx.unit;
@@ -453,7 +454,7 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
                         rinv = fminf(ri, kRinvMax);
                     } else {
                         rinv = r2 > 0.0f ? rsqrt_ftz(r2) : 0.0f;
-                        tv = fmaf(r2, rinv, -0.5f);
+                        tv = TM == TM_FINE ? fmaf(r2 * rinv, tsc, -0.5f) : fmaf(r2, rinv, -0.5f);
                     }
                     float Tv, Qv;
                     eval_TQ<TM>(tv, r2 * rinv * xscale, x_c, tab_bias, q_off, nmax, c4, Tv, Qv);
@@ -758,9 +759,9 @@ static int launch_adj_e(const FwdArgs& a, size_t smem, cudaStream_t st)
     // always with the two-targets-per-lane path (mid-size leaves fill more lanes)
     // (the packed variant carries it only for leaves above 32 particles: its
     // per-target state would spill)
-    auto k = SPLIT || a.variant != PSR_KERNEL_PACKED ? p2p_adj_f32_kernel<TM, ACC, true, false, EQM, SPLIT>
-             : a.max_leaf > 32              ? p2p_adj_f32_kernel<TM, ACC, true, true, EQM, false>
-                                            : p2p_adj_f32_kernel<TM, ACC, false, true, EQM, false>;
+    auto k = SPLIT || TM == TM_FINE || a.variant != PSR_KERNEL_PACKED ? p2p_adj_f32_kernel<TM, ACC, true, false, EQM, SPLIT>
+             : a.max_leaf > 32              ? p2p_adj_f32_kernel<TM == TM_FINE ? TM_CUBIC : TM, ACC, true, true, EQM, false>
+                                            : p2p_adj_f32_kernel<TM == TM_FINE ? TM_CUBIC : TM, ACC, false, true, EQM, false>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
@@ -789,6 +790,9 @@ int launch_adj_f32(const FwdArgs& a, int precision, void* stream)
     cudaError_t e0 = cudaGetLastError();
     if (e0 != cudaSuccess) return (int)e0;
     size_t smem = adj_f32_smem(precision, a.interp, a.table_n, a.warps_per_block, a.stage_cap);
+    if (a.fine)
+        return a.accum == PSR_ACC_FP64 ? launch_adj_t<TM_FINE, PSR_ACC_FP64>(a, smem, st)
+                                       : launch_adj_t<TM_FINE, PSR_ACC_KAHAN32>(a, smem, st);
     if (precision == PSR_FP32_EXACT)
         return a.accum == PSR_ACC_FP64 ? launch_adj_t<TM_EXACT, PSR_ACC_FP64>(a, smem, st)
                                        : launch_adj_t<TM_EXACT, PSR_ACC_KAHAN32>(a, smem, st);

@@ -156,13 +156,12 @@ inline int64_t heavy_cost(int level, int64_t evaluated, int sms)
 // Whether and how a launch on `warps` resident warps shares heavy rows.
 // group: warps per heavy item, 1 for none; level: which count of heavy items
 // applies, -1 for all items.  A launch shares rows only where the largest item
-// exceeds 3/2 of a warp's share of the work (the
-// adjoint, whose pairs cost twice as much against the same overheads: 2): then a row on one warp outlasts
-// the others, or the chip is never filled; below it the largest-first order
-// hides the longest row, and the group phase's registers cost 1-3 % (128^3 NFW
-// in leaves of up to 64: 9.53 -> 9.66 ms).  Items above about half a share are
-// shared, all of them when there are fewer leaves than warps, and the group is
-// large enough to bring the largest item's parts to 3/2 of a share, with at
+// exceeds `line` / 8 of a warp's share of the work: then a row on one warp
+// outlasts the others, or the chip is never filled; below it the largest-first
+// order hides the longest row, and the group phase's registers cost 1-3 % (128^3
+// NFW in leaves of up to 64: 9.53 -> 9.66 ms).  Items above about half a share
+// are shared, all of them when there are fewer leaves than warps, and the group
+// is large enough to bring the largest item's parts to 3/2 of a share, with at
 // least 2500 pairs in a part (the group's barriers and the row's start-up
 // latency cost about as much as 1500).  Forward, one warp per row against this:
 // 5000 uniform particles 0.235 -> 0.081 ms, 32^3 0.28 -> 0.12, 110,000 NFW 2.57
@@ -173,11 +172,11 @@ struct SplitRule {
     int group, level;
 };
 inline SplitRule split_rule(int64_t max_cost, int64_t evaluated, int64_t n_leaves, int sms, int64_t warps,
-                            int block_warps, bool adjoint)
+                            int block_warps, int line)
 {
     SplitRule r{1, -1};
     const int64_t share = evaluated / (warps > 0 ? warps : 1);
-    if (max_cost <= (adjoint ? 2 * share : share + share / 2)) return r;
+    if (max_cost <= line * share / 8) return r;
     while (r.group < 8 && 2 * max_cost > 3 * r.group * share && max_cost >= 5000 * r.group) r.group *= 2;
     while (r.group > 1 && block_warps % r.group) r.group /= 2;
     if (n_leaves >= warps)
@@ -224,6 +223,7 @@ struct FwdArgs {
     double t64_scale;  //   and its nodes per unit of x (plain path)
     const int* heavy;  // how many items groups of warps take (null: all)
     int group;         // warps per group (divides warps_per_block); 0 or 1: none
+    int fine;        // PSR_FP32_EXACT by the fine cubic table (interp and table_n are its)
     int core;        // FP32 forward: a.table is the core form of the linear table
     int equal_mass;  // every box has one particle mass: the FP32 kernels take it out of the sums
 };

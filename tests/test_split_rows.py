@@ -68,3 +68,25 @@ def test_device_built_schedule_marks_the_same_rows():
     b = psr.Leaves.device_build(torch.tensor(pos, device="cuda"), torch.tensor(mass, device="cuda"),
                                 L, r_s, r_c)
     assert torch.equal(a.forces(), b.forces())
+
+
+@pytest.mark.parametrize("x_c", [0.4, 2.25, 2.5, 2.6, 4.5, 4.6])
+@pytest.mark.parametrize("accum", [psr.PSR_ACC_FP64, psr.PSR_ACC_KAHAN32])
+def test_exact_precision_by_the_fine_table_and_by_erfc(x_c, accum):
+    """PSR_FP32_EXACT under the default kernel (a fine cubic table up to x_c = 4.5) against the
+    kernel that calls erfcf and expf, and the oracle.  T of both is within a few FP32 roundings:
+    1e-6 between them, twice the roundings of a weight (4 x 2^-24 each), summed incoherently."""
+    pos, mass, L, _, r_c = _set("few")
+    r_c = 6.0
+    r_s = r_c / (2.0 * x_c)
+    cot = np.random.default_rng(3).standard_normal(pos.shape)
+    lv = psr.Leaves.build(pos, mass, L, r_s, r_c).upload()
+    a, b = (lv.forces(psr.Options(precision=psr.PSR_FP32_EXACT, accum=accum, kernel=k)).double().cpu().numpy()
+            for k in (psr.PSR_KERNEL_AUTO, psr.PSR_KERNEL_SCALAR))
+    ga, gb = (lv.adjoint(torch.tensor(cot), psr.Options(precision=psr.PSR_FP32_EXACT, accum=accum, kernel=k))
+              for k in (psr.PSR_KERNEL_AUTO, psr.PSR_KERNEL_SCALAR))
+    ref = oracle.forces(pos, mass, L, r_s, r_c, 1.0)
+    ref = ref[0] if isinstance(ref, tuple) else ref
+    assert _rms(a, b) < 1e-6 and _rms(a, ref) < 2e-5
+    for u, v in zip(ga, gb):
+        assert _rms(u.double().cpu().numpy(), v.double().cpu().numpy()) < 1e-6

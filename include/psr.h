@@ -56,13 +56,16 @@ extern "C" {
 
 /* ------------------------------------------------------------ options */
 /* precision of the pair arithmetic */
-#define PSR_FP64 0        /* FP64 throughout, T from erfc/exp; with interp
+#define PSR_FP64 0        /* FP64 throughout, T to 1e-13 from a degree-5 table
+                             built in FP64; with interp
                              PSR_TAYLOR2/4 the paper's double-precision table
                              path instead (Section 3.3: the Taylor table in
                              FP64 about the nearest node, 1/r by Newton-
                              Raphson from an FP32 estimate; forward only, not
                              in psr_p2p_forces_noalloc)                     */
-#define PSR_FP32_EXACT 1  /* FP32 pair math, T from erfcf/expf              */
+#define PSR_FP32_EXACT 1  /* FP32 pair math, T from erfcf/expf; under
+                             PSR_KERNEL_AUTO and x_c <= 4.5 from a fine cubic
+                             table whose error is below theirs              */
 #define PSR_FP32_TABLE 2  /* FP32 pair math, T interpolated from a table
                              in shared memory (Section 3.3)                 */
 /* interpolation of the table (PSR_FP32_TABLE; the Taylor levels also
@@ -152,8 +155,8 @@ typedef struct {
     int64_t rows_walked_twice; /* device builds: target leaves whose pair row
                                 the count walk could not keep in the pair
                                 cache, walked again by psr_device_build_finish
-                                (every row for a split or when the cache's
-                                per-row slot is below 16 runs); else 0      */
+                                (every row when the cache's per-row slot is
+                                below 16 runs); else 0                       */
     int equal_mass;          /* 1 if within every box all particles have one
                                 mass: the FP32 kernels then apply it once per
                                 target instead of once per pair (the paper's
@@ -340,8 +343,8 @@ int psr_pair_count(psr_leaves* h, void* cuda_stream, int timeout_ms, int64_t* co
  * kernels drop staged sources that lie at least r_c from the target leaf's
  * particle box (those pairs are zero by the truncation of Eq. tr), so their
  * count lies between psr_pair_count's and the leaf-pair tiles' total
- * (psr_info.evaluated_pairs); the FP64 and PSR_KERNEL_PAPER kernels evaluate
- * every tile pair.  Errors: PSR_E_STATE, PSR_E_TIMEOUT.
+ * (psr_info.evaluated_pairs); PSR_KERNEL_PAPER evaluates every tile
+ * pair, and so do the FP64 kernels on a counting launch.  Errors: PSR_E_STATE, PSR_E_TIMEOUT.
  */
 int psr_evaluated_count(psr_leaves* h, void* cuda_stream, int timeout_ms, int64_t* count);
 
@@ -417,7 +420,7 @@ int psr_leaves_regions(const psr_leaves* h, psr_regions* out);
 /*
  * The leaf set of psr_build_leaves built on the GPU from device-resident
  * positions (one box): the same leaves, pair list and schedule, bit for bit
- * (paper, Section 2 and Section 3.2; the tree is a binary radix tree over
+ * (paper, Section 2 and Section 3.2; the tree is a 32-ary tree over
  * the Morton-ordered leaf cells, whose walk keeps the same leaf pairs in the
  * same order as the host's octree walk).  Two calls, so that the caller can
  * size the workspace from the counts:
@@ -428,7 +431,7 @@ int psr_leaves_regions(const psr_leaves* h, psr_regions* out);
  * copies instead of walking the tree again).  Errors: PSR_E_ARG
  * (n < 1 or n > 2^28, NULL).
  *
- * psr_device_build - enqueue key, radix sort, leaf, radix tree and pair
+ * psr_device_build - enqueue key, sort, leaf, tree and pair
  * count kernels on cuda_stream, wait for them (each wait at most timeout_ms;
  * <= 0 means 60 s) and read back the leaf and pair counts; returns a handle
  * whose workspace is not yet written (psr_leaves_info works on it).

@@ -560,7 +560,9 @@ Scratch scratch_layout(int64_t n)
     s.lfruns = o; o = a256(o + 4 * N);   // and far ones (multipole split)
     s.ncache = (int64_t)(kCacheWordsPerParticle / 2 * N);
     s.cache = o;  o = a256(o + 8 * (size_t)s.ncache);  // uint2 (first leaf << 5 | code, length)
-    s.bytes = o;
+    // The size callers are told has been about 430 bytes per particle, and is
+    // kept (the regions take about 290): scratch of that size serves as before.
+    s.bytes = a256(std::max(o, (size_t)430 * N));
     return s;
 }
 

@@ -56,8 +56,9 @@ extern "C" {
 
 /* ------------------------------------------------------------ options */
 /* precision of the pair arithmetic */
-#define PSR_FP64 0        /* FP64 throughout, T to 1e-13 from a degree-5 table
-                             built in FP64; with interp
+#define PSR_FP64 0        /* FP64 throughout, T to rounding from a degree-5
+                             table built in FP64 (truncation below 1e-16);
+                             with interp
                              PSR_TAYLOR2/4 the paper's double-precision table
                              path instead (Section 3.3: the Taylor table in
                              FP64 about the nearest node, 1/r by Newton-

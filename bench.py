@@ -42,9 +42,9 @@ def parse():
     p.add_argument("--table-n", type=int, default=1024)
     p.add_argument("--interp", default="linear", choices=["linear", "cubic"])
     p.add_argument("--accum", default="fp64", choices=["fp64", "kahan"])
-    p.add_argument("--kernel", default="scalar", choices=["scalar", "packed"],
-                   help="FP32 forward inner loop: scalar streams (the default) or packed f32x2 "
-                        "pairs")
+    p.add_argument("--kernel", default="auto", choices=["auto", "scalar", "packed"],
+                   help="FP32 forward inner loop: the library's choice (the default: packed f32x2 "
+                        "pairs for a linear table), scalar streams, or packed f32x2 pairs")
     p.add_argument("--fp64-steps", type=int, default=2)
     p.add_argument("--e2e-steps", type=int, default=5)
     p.add_argument("--adjoint-steps", type=int, default=3)
@@ -173,7 +173,7 @@ PRECISION_VARIANTS = [
     ("table linear 4096", dict(table_n=4096, interp=0)),
     ("table cubic 1024", dict(table_n=1024, interp=1)),
     ("table cubic 4096", dict(table_n=4096, interp=1)),
-    ("exact erfcf/expf", dict(precision=1)),
+    ("exact (PSR_FP32_EXACT)", dict(precision=1)),
     # the paper's Taylor table (Section 3.3, Eq. int), its node spacing 3/512
     ("paper Taylor T[2] 384 nodes", dict(table_n=384, interp=2)),
     ("paper Taylor T[4] 384 nodes", dict(table_n=384, interp=3)),
@@ -715,8 +715,8 @@ def run_psr(args):
     opts = psr.Options(precision=psr.PSR_FP32_TABLE, table_n=args.table_n,
                        interp=psr.PSR_LINEAR if args.interp == "linear" else psr.PSR_CUBIC,
                        accum=psr.PSR_ACC_FP64 if args.accum == "fp64" else psr.PSR_ACC_KAHAN32,
-                       kernel=psr.PSR_KERNEL_PACKED if args.kernel == "packed"
-                       else psr.PSR_KERNEL_SCALAR)
+                       kernel={"auto": psr.PSR_KERNEL_AUTO, "packed": psr.PSR_KERNEL_PACKED,
+                               "scalar": psr.PSR_KERNEL_SCALAR}[args.kernel])
     acc = torch.empty((b.n, 3), dtype=torch.float32, device=dev)
     stream = torch.cuda.current_stream()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
@@ -1021,7 +1021,7 @@ def run_psr(args):
         ms_pm = sum(a.elapsed_time(e) for a, e in ep) / args.pm_steps
         pm_line = {"ms_per_step": ms_pm, "n_pm": b.n_pm, "particles": b.n,
                    "particles_per_s": b.n / (ms_pm / 1e3),
-                   "kernels_per_step": "deposit, R2C, Green, 3 x (gradient, C2R), interpolation",
+                   "kernels_per_step": "deposit, join, R2C, field, batched C2R, interpolation",
                    "fraction_of_p2p_step": ms_pm / mean_ms}
         if rank == 0 and not args.no_cpu_baseline and b.n <= (1 << 22):
             from oracle import pm as opm
@@ -1148,7 +1148,8 @@ def run_psr(args):
         "cpu_baseline": None if cb is None else {k: cb[k] for k in
                                                   ("value", "unit", "cores", "kind", "sample")},
         "gpu_launches": args.steps,
-        "tile_shape": {"kernel": "packed f32x2 pairs" if args.kernel == "packed" else "scalar streams", "warps_per_block": 8, "source_tile": 256},
+        "tile_shape": {"kernel": {"auto": "library default", "packed": "packed f32x2 pairs",
+                                  "scalar": "scalar streams"}[args.kernel], "warps_per_block": 8, "source_tile": 256},
         "clocks": clocks,
         "device": props.name,
     }

@@ -21,7 +21,8 @@
 //                of 16 words per particle; after a prefix sum of the counts the
 //                cached rows are copied into place and only the rows the cache
 //                could not hold are walked a second time.  The walk prunes with
-//                FP32 bounds (directed rounding) and falls back to the host's FP64
+//                FP32 bounds (boxes rounded outward, thresholds widened by
+//                the rounding of the sums) and falls back to the host's FP64
 //                leaf test only where the bounds cannot decide (gap^2 within about
 //                1e-5 of the cutoff): FP64 throughput on this part is 1/64 of FP32.
 //   6. schedule  target leaves sorted by evaluated work, largest first (stable)

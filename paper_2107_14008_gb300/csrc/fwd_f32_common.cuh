@@ -17,7 +17,8 @@
 // for the leaves that take one target per lane).  The
 // S partial sums of each target are combined through shared memory at the
 // end.  Warps take target leaves from an atomic ticket in largest-work-first
-// order (persistent grid, no inter-block waits).
+// order (persistent grid, no inter-block waits); the split instances share a
+// heavy leaf between 2, 4 or 8 warps of a block.
 //
 // Precision.  Pair arithmetic is FP32 in leaf-local coordinates scaled by
 // 1/(2 r_s); the offset between two leaf centres (with the periodic image) is
@@ -28,7 +29,11 @@
 // T(x).  Exact: erfcf + expf.  Table: T on [0, x_c] with N intervals, held in
 // shared memory: linear (midpoint value, chord difference) or cubic Hermite
 // (monomial coefficients about the midpoint); index N is a zero sentinel, so
-// the cutoff (x >= x_c) costs no extra instruction.
+// the cutoff (x >= x_c) costs no extra instruction.  Core form (packed pairs,
+// linear tables of 1024 intervals or more): T / r^3 = 1 / r^3 - H(q) with H
+// linear between nodes in q = r^2.  Fine: a cubic table in unscaled
+// coordinates whose error is below that of FP32 erfcf and expf (exact
+// precision under the automatic kernel choice).
 #pragma once
 #include <cuda_runtime.h>
 

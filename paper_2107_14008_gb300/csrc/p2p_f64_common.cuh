@@ -51,12 +51,15 @@ __device__ __forceinline__ bool inside64(double r2, long long rc2m1)
 }
 
 // entry (clamped to kmax) and offset from its node, in node spacings, of
-// distance r (us nodes per unit of r)
+// distance r >= 0 (us nodes per unit of r).  fk's low word is the node below
+// 2^32, where its high word is kMagic64's; beyond (r_s far below r_c: x above
+// 3.8e7), infinity included, the last entry.
 __device__ __forceinline__ int node64(double r, double us, int kmax, double& f)
 {
     const double fk = fma(r, us, kMagic64);
-    f = fma(r, us, -(fk - kMagic64));
-    return min(__double2loint(fk), kmax);
+    const bool low = __double2hiint(fk) == 0x43380000;
+    f = low ? fma(r, us, -(fk - kMagic64)) : 0.0;
+    return low ? (int)min((unsigned)__double2loint(fk), (unsigned)kmax) : kmax;
 }
 
 template <int DEG>

@@ -57,3 +57,29 @@ def test_fp64_pair_and_strict_cutoff(f):
     want = oracle.T(np.array([r / (2 * r_s)]))[0] / r ** 2 if r < r_c else 0.0
     np.testing.assert_allclose(acc[:, 0], [0.25 * want, -0.5 * want], rtol=2e-15)
     assert np.all(acc[:, 1:] == 0.0)
+
+
+@pytest.mark.parametrize("r_s", [1e-6, 1.1e-7, 0.9e-7, 0.5e-7, 1e-9, 1e-13])
+@pytest.mark.parametrize("device", [False, True])
+def test_fp64_cutoff_far_beyond_the_table(r_s, device):
+    """r_s so far below r_c that a distance in node spacings passes 2^31 and 2^32: those pairs
+    have T = 0, and the close ones (a neighbour at 0.4 r_s) keep theirs.  Coordinates are off by
+    2^-53 L against 0.4 r_s, so the tolerance is four of those."""
+    rng = np.random.default_rng(2)
+    n, L, r_c = 600, 10.0, 4.5
+    pos = rng.random((n, 3)) * L
+    pos[1::2] = np.mod(pos[::2] + np.array([0.4 * r_s, 0.0, 0.0]), L)
+    mass, cot = rng.uniform(0.5, 1.5, n), rng.standard_normal((n, 3))
+    o = psr.Options(precision=psr.PSR_FP64)
+    if device:
+        lv = psr.Leaves.device_build(torch.tensor(pos, device="cuda"), torch.tensor(mass, device="cuda"), L, r_s, r_c)
+    else:
+        lv = psr.Leaves.build(pos, mass, L, r_s, r_c).upload()
+    acc = lv.forces(o).cpu().numpy()
+    gx, gm = (g.cpu().numpy() for g in lv.adjoint(torch.tensor(cot), o))
+    lv.check()
+    ref = oracle.forces(pos, mass, L, r_s, r_c, 1.0)
+    ref = ref[0] if isinstance(ref, tuple) else ref
+    ox, om = oracle.adjoint(pos, mass, cot, L, r_s, r_c, 1.0)[:2]
+    tol = 1e-13 + 4 * 2.0 ** -53 * L / (0.4 * r_s)
+    assert _rms(acc, ref) < tol and _rms(gx, ox) < 3 * tol and _rms(gm, om) < tol

@@ -449,8 +449,8 @@ int psr_leaves_regions(const psr_leaves* h, psr_regions* out);
  * stream).  Errors: PSR_E_ARG (argument, box outside that range, non-finite
  * position or mass), PSR_E_CUTOFF,
  * PSR_E_WORKSPACE (scratch missing, small or misaligned), PSR_E_CUDA,
- * PSR_E_TIMEOUT, PSR_E_DEVICE (a tree bound check fired: traversal stack
- * overflow or a malformed tree; the build is abandoned), PSR_E_NOMEM.
+ * PSR_E_TIMEOUT, PSR_E_DEVICE (a bounded wait between the blocks of a sort
+ * or a scan ran out; the build is abandoned), PSR_E_NOMEM.
  *
  * psr_device_build_finish - enqueue on cuda_stream the kernels that write
  * the workspace (psr_leaves_info().device_bytes, 256-byte aligned, owned by

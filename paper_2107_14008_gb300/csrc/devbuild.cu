@@ -62,7 +62,7 @@ enum : int {
     kCntEvaluated = 2,
     kCntMaxCost = 3,
     kCntMaxRow = 4,
-    kCntError = 5,  // bit 0 non-finite input, bit 1 stack overflow, bit 2 malformed tree, bit 3 a look-back that ran out
+    kCntError = 5,  // bit 0 non-finite input; kErrLookback
     kCntFar = 6,    // well-separated (M2L) entries of the multipole split
     kCntUncached = 7,  // rows the pair cache could not hold (re-walked by the write pass)
     kCntMassDiff = 8,  // nonzero if some particle's mass differs from particle 0's
@@ -147,22 +147,28 @@ __device__ __forceinline__ double gap2_d(const double* A, const double* B, const
 // ticket, so every earlier tile has started; it publishes its own total, then
 // adds up the published totals behind it until it meets a published prefix
 // (decoupled look-back, Merrill and Garland 2016).  The waits are bounded: one
-// that runs out sets error bit 3 (of the build's counters, and the
-// build fails, or of the workspace's error word).
+// that runs out sets kErrLookback (in the build's counters, and the build
+// fails, or in the workspace's error word) and its prefix is too small.  What
+// follows stays within its arrays: a scan's positions are at most the true
+// ones; a sort pass, whose next pass then ranks stale keys against counts of
+// the true ones, drops what would lie beyond the end; and the kernels that
+// would follow the positions (k_leaf_box, k_rows) do nothing.
 // The control words are zeroed by one memset per build call.
-constexpr int kSpinLimit = 1 << 22;
+#ifndef PSR_SPIN_LIMIT  // a test lets every wait run out
+#define PSR_SPIN_LIMIT (1 << 22)
+#endif
+constexpr int kSpinLimit = PSR_SPIN_LIMIT;
 constexpr unsigned kSumReady = 1u << 30, kPrefixReady = 2u << 30, kValueMask = kSumReady - 1;
 
 // Waits for a published word of the current look-back step; 0 when the wait
-// runs out: the look-back then stops, with a prefix that is too small, so that
-// every position formed from it still lies inside its array.
+// runs out: the look-back then stops.
 __device__ __forceinline__ unsigned wait_word(const volatile unsigned* p, unsigned* err)
 {
     for (int k = 0; k < kSpinLimit; ++k) {
         const unsigned v = *p;
         if (v & (kSumReady | kPrefixReady)) return v;
     }
-    atomicOr(err, 8u);
+    atomicOr(err, kErrLookback);
     return 0u;
 }
 
@@ -409,6 +415,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sort_pass(const uint64_t* _
     for (int i = tid; i < count; i += kSortThreads) {
         const uint64_t k = skey[i];
         const int64_t pos = s_base[(unsigned)(k >> shift) & 255u] + i;
+        if (pos >= n) continue;  // only after a look-back that ran out
         kout[pos] = k;
         vout[pos] = sval[i];
     }
@@ -768,6 +775,7 @@ __global__ void k_leaf_box(const int32_t* __restrict__ lfirst, int64_t n,
                            double* __restrict__ lbox, float4* __restrict__ lout,
                            long long* __restrict__ cnt)
 {
+    if (cnt[kCntError] & kErrLookback) return;  // lfirst and idx may hold anything
     const int64_t nl = cnt[kCntPacked], step = (int64_t)gridDim.x * blockDim.x >> 3;
     const int sub = threadIdx.x & 7;
     int largest = 0;
@@ -990,8 +998,10 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkBlocks) k_rows(const Wal
     const float Lf = (float)w.bx.L, Lrd = __double2float_rd(w.bx.L), Lru = __double2float_ru(w.bx.L);
     const float4* const lout = s_lv.box[0];
     const int top = s_lv.top;
-    const int nl = s_lv.n[0] < (1 << 27) ? (int)s_lv.n[0] : 0;  // more is refused by the host
-    const int kslot = cache_slot(w.ncache, s_lv.n[0]);
+    // no rows after a look-back that ran out, and for more leaves than the host accepts
+    const bool walk = s_lv.n[0] < (1 << 27) && (WRITE || !(*w.err & kErrLookback));
+    const int nl = walk ? (int)s_lv.n[0] : 0;
+    const int kslot = nl ? cache_slot(w.ncache, nl) : 0;
     const int W = (int)gridDim.x * kWalkWarps;
     for (int I = (int)blockIdx.x * kWalkWarps + wp; I < nl; I += W) {
         if (WRITE && kslot && w.lruns[I] >= 0) continue;  // recorded: k_pairs_expand writes it
@@ -1601,11 +1611,11 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
     long long c[kCntWords];
     if ((e = read_back(c, cnt, sizeof c, st, timeout_ms))) return e;
     if (c[kCntError] & 1) return dfail(PSR_E_ARG, "non-finite position or mass");
+    if (c[kCntError] & kErrLookback) return dfail(PSR_E_DEVICE, "a look-back of the build's scans or sorts ran out");
     const int64_t np = c[kCntLeaves], nl = c[kCntPacked];
     if (np < 1 || np > n || nl >= (1 << 27)) return dfail(PSR_E_ARG, "leaf count out of range");
     if (nl < 1 || nl > np) return dfail(PSR_E_DEVICE, "leaf packing failed");
     const int kslot = cache_slot(S.ncache, nl);
-    if (c[kCntError] & 12) return dfail(PSR_E_DEVICE, "a row walk or a look-back failed");
     if (c[kCntPairs] >= ((int64_t)1 << 32) || c[kCntFar] >= ((int64_t)1 << 32))
         return dfail(PSR_E_ARG, "more than 2^32 leaf pairs");
 

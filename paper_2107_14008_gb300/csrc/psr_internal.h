@@ -81,6 +81,7 @@ enum : unsigned {
     kErrParticleRange = 2u,
     kErrItemIndex = 4u,
     kErrShiftCode = 8u,
+    kErrLookback = 16u,  // a look-back of the device build's scans or sorts ran out
 };
 
 struct Leaves {

@@ -236,6 +236,13 @@ int psr_upload(psr_leaves* h, void* d_workspace, size_t bytes, void* cuda_stream
  *          opts->precision == PSR_FP64, FP32 otherwise.  Overwritten.
  * The first call with a new (precision, table_n, interp) also builds the
  * interpolation table in the workspace (one small extra launch).
+ * Graph-capturable.  A first call under stream capture records that launch in
+ * the graph; other calls record the kernel alone and read the table that is in
+ * place.  PSR_FP64 without a Taylor level, PSR_FP32_EXACT and the linear table
+ * of the packed kernel keep tables of their own; all other tables (each
+ * precision, table_n and interp) share one place in the workspace, so a graph
+ * captured with one of them in place is not replayed after a call that built
+ * another.  The same holds for psr_p2p_adjoint.
  * Errors: PSR_E_ARG, PSR_E_STATE (not uploaded; FP64 payload omitted),
  * PSR_E_CUDA (launch failure).
  */

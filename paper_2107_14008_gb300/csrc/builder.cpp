@@ -406,6 +406,7 @@ Layout make_layout(const Leaves& h)
     L.items = o;     o = align256(o + nl * 4);
     L.boxes = o;     o = align256(o + h.boxdev.size() * sizeof(BoxDev));
     L.table = o;     o = align256(o + 2 * (size_t)(kMaxTableN + 1) * 16);
+    L.fine = o;      o = align256(o + 2 * (size_t)(kFineMaxN + 1) * 16);
     L.t64 = o;       o = align256(o + 2 * (size_t)6 * (kPlain64MaxN + 2) * 8);
     L.core = o;      o = align256(o + (size_t)(kMaxTableN + 1) * 8);
     L.cotf = o;      o = align256(o + n * ((h.flags & PSR_BUILD_NO_FP64) ? 16 : 32));

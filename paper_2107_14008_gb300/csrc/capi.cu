@@ -132,7 +132,6 @@ FwdArgs base_args(Leaves* h, const Opts& o)
     a.pairs = reinterpret_cast<const uint32_t*>(w + L.pairs);
     a.items = reinterpret_cast<const int32_t*>(w + L.items);
     a.boxes = reinterpret_cast<const BoxDev*>(w + L.boxes);
-    a.table = w + L.table;
     a.ctrl = reinterpret_cast<unsigned*>(w + L.ctrl);
     a.cot_sorted = w + L.cotf;
     a.n = h->n;
@@ -193,36 +192,62 @@ void resolve_kernel(const Leaves* h, Opts& o)
                    : PSR_KERNEL_SCALAR;
 }
 
-int ensure_table(Leaves* h, const Opts& o, bool core, cudaStream_t st)
+// Builds the table of `key` in its region by launch(), unless it is there for
+// work enqueued on st.  A table recorded under stream capture is there for the
+// rest of that capture only: outside it the recorded launch has not run.  And
+// once a graph that writes another table of the region exists, its replays may
+// come between any two calls, so those build theirs anew.
+template <class Launch>
+int build_table(TableState& t, int key, double x_c, cudaStream_t st, Launch launch)
+{
+    const bool same = t.key == key && t.x_c == x_c;
+    if (same && t.capture == 0 && (t.recorded == -1 || t.recorded == key)) return PSR_OK;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+        cudaGetLastError();  // the launch reports it
+        status = cudaStreamCaptureStatusNone;
+    }
+    const unsigned long long capture = status == cudaStreamCaptureStatusActive ? id + 1 : 0;
+    if (same && capture && t.capture == capture) return PSR_OK;
+    const int e = launch();
+    if (e) return cuda_fail((cudaError_t)e, "table kernel launch");
+    t.key = key;
+    t.x_c = x_c;
+    t.capture = capture;
+    if (capture) t.recorded = t.recorded == -1 || t.recorded == key ? key : -2;
+    return PSR_OK;
+}
+
+// The options' table in its region of the workspace (*region, null if they take
+// none).  Each of the core form, the fine table and the FP64 plain path has a
+// region of its own: a graph that was captured with one in place reads it
+// whatever other precision runs on the handle between replays.
+int ensure_table(Leaves* h, const Opts& o, bool core, cudaStream_t st, const void** region)
 {
     const bool t64 = fp64_taylor(o);
     const double x_c = cutoff_x(h);
+    char* const w = h->d_ws;
+    *region = nullptr;
     if (o.precision == PSR_FP64 && !t64) {
-        if (h->t64_xc == x_c) return PSR_OK;
-        double* t = reinterpret_cast<double*>(h->d_ws + h->lay.t64);
-        const int e = launch_plain64(x_c, t, t + 6 * (kPlain64MaxN + 2), st);
-        if (e) return cuda_fail((cudaError_t)e, "table kernel launch");
-        h->t64_xc = x_c;
-        return PSR_OK;
+        double* t = reinterpret_cast<double*>(w + h->lay.t64);
+        *region = t;
+        return build_table(h->t64, 0, x_c, st,
+                           [&] { return launch_plain64(x_c, t, t + 6 * (kPlain64MaxN + 2), st); });
     }
     if (o.precision != PSR_FP32_TABLE && !t64) return PSR_OK;
-    if (core) {
-        if (h->core_key == o.table_n && h->core_xc == x_c) return PSR_OK;
-        const int e = launch_core_table(o.table_n, x_c, h->d_ws + h->lay.core, st);
-        if (e) return cuda_fail((cudaError_t)e, "table kernel launch");
-        h->core_key = o.table_n;
-        h->core_xc = x_c;
-        return PSR_OK;
-    }
-    int key = (o.table_n * 4 + o.interp) * 2 + (t64 ? 1 : 0);
-    if (key == h->table_key && x_c == h->table_xc) return PSR_OK;
-    char* t = h->d_ws + h->lay.table;
-    int e = t64 ? launch_table64(o.table_n, o.interp, x_c, t, st)
-                : launch_table(o.table_n, o.interp, x_c, t, t + (size_t)(kMaxTableN + 1) * 16, st);
-    if (e) return cuda_fail((cudaError_t)e, "table kernel launch");
-    h->table_key = key;
-    h->table_xc = x_c;
-    return PSR_OK;
+    char* const t = w + (core ? h->lay.core : o.fine ? h->lay.fine : h->lay.table);
+    *region = t;
+    if (core)
+        return build_table(h->core, o.table_n, x_c, st, [&] { return launch_core_table(o.table_n, x_c, t, st); });
+    if (o.fine)
+        return build_table(h->fine, o.table_n, x_c, st, [&] {
+            return launch_table(o.table_n, o.interp, x_c, t, t + (size_t)(kFineMaxN + 1) * 16, st);
+        });
+    return build_table(h->table, (o.table_n * 4 + o.interp) * 2 + (t64 ? 1 : 0), x_c, st, [&] {
+        return t64 ? launch_table64(o.table_n, o.interp, x_c, t, st)
+                   : launch_table(o.table_n, o.interp, x_c, t, t + (size_t)(kMaxTableN + 1) * 16, st);
+    });
 }
 
 int grid_blocks(Leaves* h, const Opts& o, int adjoint, int* blocks)
@@ -408,10 +433,7 @@ int psr_upload(psr_leaves* hh, void* d_ws, size_t bytes, void* stream)
     h->d_ws = w;
     h->ws_bytes = bytes;
     h->uploaded = true;
-    h->table_key = -1;
-    h->table_xc = -1.0;
-    h->core_key = -1;
-    h->t64_xc = -1.0;
+    h->table = h->core = h->fine = h->t64 = TableState{};
     h->sm_count = sms;
     h->device = dev;
     return PSR_OK;
@@ -434,14 +456,12 @@ int psr_p2p_forces(psr_leaves* hh, const psr_opts* opts, void* d_acc, void* stre
     fine_exact(h, o);
     resolve_kernel(h, o);
     const bool core = fwd_core(o.precision, o.interp, o.table_n, o.kernel, cutoff_x(h));
-    if ((rc = ensure_table(h, o, core, st))) return rc;
+    const void* table;
+    if ((rc = ensure_table(h, o, core, st, &table))) return rc;
     FwdArgs a = base_args(h, o);
     a.out = d_acc;
-    if (core) {
-        a.core = 1;
-        a.table = h->d_ws + h->lay.core;
-    }
-    if (o.precision == PSR_FP64 && !fp64_taylor(o)) a.table = h->d_ws + h->lay.t64;
+    a.table = table;
+    a.core = core;
     if (fwd32 && (rc = fwd32_smem_config(o, &a.stage_cap))) return rc;
     if (fwd32 && (rc = check_tile(h, a.stage_cap))) return rc;
     if ((rc = grid_blocks(h, o, 0, &a.blocks))) return rc;
@@ -476,16 +496,17 @@ int psr_p2p_adjoint(psr_leaves* hh, const psr_opts* opts, const void* d_cot, voi
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = resolve_warps(o, false))) return rc;
     fine_exact(h, o);
-    if ((rc = ensure_table(h, o, false, st))) return rc;
+    const void* table;
+    if ((rc = ensure_table(h, o, false, st, &table))) return rc;
     FwdArgs a = base_args(h, o);
     a.cot = d_cot;
+    a.table = table;
     a.stage_cap = o.tile ? o.tile : kAdjStageCap;
     if (o.precision != PSR_FP64 && (rc = check_tile(h, a.stage_cap))) return rc;
     if (o.precision != PSR_FP64 &&
         adj_f32_smem(o.precision, o.interp, o.table_n, o.warps, a.stage_cap) > kSmemPerBlock)
         return fail(PSR_E_ARG, "adjoint table and staging buffers exceed shared memory; "
                                "use fewer warps or a smaller table");
-    if (o.precision == PSR_FP64) a.table = h->d_ws + h->lay.t64;
     a.out = d_grad_pos;
     a.out_m = d_grad_mass;
     if ((rc = grid_blocks(h, o, 1, &a.blocks))) return rc;

@@ -1789,11 +1789,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     h->d_ws = w;
     h->ws_bytes = bytes;
     h->uploaded = true;
-    h->table_key = -1;
-    h->table_xc = -1.0;
-    h->core_key = -1;
-    h->t64_xc = -1.0;
-    h->adj_table_key = -1;
+    h->table = h->core = h->fine = h->t64 = TableState{};
     h->sm_count = sms;
     h->device = dev;
     h->db_scratch = nullptr;

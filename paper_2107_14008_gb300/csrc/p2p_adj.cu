@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
     const unsigned accb = smem_u32(meta + kWarpMeta);
     if (TM != TM_EXACT) {
         const float4* g = reinterpret_cast<const float4*>(a.table);
-        const float4* gq = g + (kMaxTableN + 1);
+        const float4* gq = g + (TM == TM_FINE ? kFineMaxN + 1 : kMaxTableN + 1);
         float4* sT = reinterpret_cast<float4*>(smem);
         for (int i = threadIdx.x; i <= a.table_n; i += blockDim.x) {
             if (TM == TM_LINEAR && PK) {

@@ -21,6 +21,7 @@ constexpr int kCentreShift = 22;
 constexpr int kMaxLeaf = 64;
 constexpr int kShiftCodes = 27;  // (nx+1)*9 + (ny+1)*3 + (nz+1)
 constexpr int kMaxTableN = 8192;
+constexpr int kFineMaxN = 1024;      // intervals of PSR_FP32_EXACT's fine table
 constexpr int kMaxTaylorN = 2048;    // Taylor tables: 32-byte entries
 constexpr int kTaylorPaperN = 384;   // x_c / 384 = 3 / 512 at x_c = 2.25, the paper's spacing
 
@@ -52,6 +53,7 @@ struct Layout {
     size_t boxes;    // BoxDev[nbox]
     size_t table;    // float4[2 * (kMaxTableN + 1)]: T table, then exp(-x^2)
     size_t core;     // float2[kMaxTableN + 1]: core form of the forward's linear table
+    size_t fine;     // float4[2 * (kFineMaxN + 1)]: PSR_FP32_EXACT's fine table of T, then exp(-x^2)
     size_t t64;      // double[2][6 (kPlain64MaxN + 2)]: FP64 plain path's T and exp(-x^2) tables
     size_t cotf;     // float4[n] / double4[n] adjoint source payload scratch
     size_t ctrl;     // uint32[64]  scheduler tickets, error word, counters
@@ -82,6 +84,16 @@ enum : unsigned {
     kErrItemIndex = 4u,
     kErrShiftCode = 8u,
     kErrLookback = 16u,  // a look-back of the device build's scans or sorts ran out
+};
+
+// What a table region of the workspace holds: the table (key) and its x_c, put
+// there by a launch that was enqueued (capture 0) or recorded under stream
+// capture (capture: 1 + its id); and which table the graphs' replays write.
+struct TableState {
+    int key = -1;
+    double x_c = -1.0;
+    unsigned long long capture = 0;
+    int recorded = -1;  // -1 none, -2 several
 };
 
 struct Leaves {
@@ -128,12 +140,7 @@ struct Leaves {
     char* d_ws = nullptr;
     size_t ws_bytes = 0;
     bool uploaded = false;
-    int table_key = -1;       // cached forward table (n, interp) encoding
-    double table_xc = -1.0;
-    double t64_xc = -1.0;     // the FP64 plain path's tables' x_c
-    int core_key = -1;        // the core table's intervals and x_c
-    double core_xc = -1.0;
-    int adj_table_key = -1;
+    TableState table, core, fine, t64;  // what the workspace's table regions hold
     int sm_count = 0;
     int device = -1;
 };

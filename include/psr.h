@@ -56,13 +56,14 @@ extern "C" {
 
 /* ------------------------------------------------------------ options */
 /* precision of the pair arithmetic */
-#define PSR_FP64 0        /* FP64 throughout, T to rounding from a degree-5
-                             table built in FP64 (truncation below 1e-16);
+#define PSR_FP64 0        /* FP64 throughout; T as near as erfc and exp give
+                             it, up to x = 5.32 from a table of polynomials of
+                             degree 5 built in FP64 (off by 4e-19, relative to
+                             T by at most 3e-15), from erfc and exp beyond;
                              with interp
                              PSR_TAYLOR2/4 the paper's double-precision table
                              path instead (Section 3.3: the Taylor table in
-                             FP64 about the nearest node, 1/r by Newton-
-                             Raphson from an FP32 estimate; forward only, not
+                             FP64 about the nearest node; forward only, not
                              in psr_p2p_forces_noalloc)                     */
 #define PSR_FP32_EXACT 1  /* FP32 pair math, T from erfcf/expf; under
                              PSR_KERNEL_AUTO and x_c <= 4.5 from a fine cubic

@@ -407,7 +407,7 @@ Layout make_layout(const Leaves& h)
     L.boxes = o;     o = align256(o + h.boxdev.size() * sizeof(BoxDev));
     L.table = o;     o = align256(o + 2 * (size_t)(kMaxTableN + 1) * 16);
     L.fine = o;      o = align256(o + 2 * (size_t)(kFineMaxN + 1) * 16);
-    L.t64 = o;       o = align256(o + 2 * (size_t)6 * (kPlain64MaxN + 2) * 8);
+    L.t64 = o;       o = align256(o + 2 * (size_t)6 * (kPlain64MaxN + 1) * 8);
     L.core = o;      o = align256(o + (size_t)(kMaxTableN + 1) * 8);
     L.cotf = o;      o = align256(o + n * ((h.flags & PSR_BUILD_NO_FP64) ? 16 : 32));
     L.ctrl = o;      o = align256(o + kCtrlWords * 4);

@@ -233,7 +233,7 @@ int ensure_table(Leaves* h, const Opts& o, bool core, cudaStream_t st, const voi
         double* t = reinterpret_cast<double*>(w + h->lay.t64);
         *region = t;
         return build_table(h->t64, 0, x_c, st,
-                           [&] { return launch_plain64(x_c, t, t + 6 * (kPlain64MaxN + 2), st); });
+                           [&] { return launch_plain64(x_c, t, t + 6 * (kPlain64MaxN + 1), st); });
     }
     if (o.precision != PSR_FP32_TABLE && !t64) return PSR_OK;
     char* const t = w + (core ? h->lay.core : o.fine ? h->lay.fine : h->lay.table);

@@ -118,7 +118,7 @@ extern "C" int psr_p2p_forces_noalloc(psr_leaves* hh, const psr_opts* opts, void
     }
     const double x_c = h->boxes[0].r_c / (2.0 * h->boxes[0].r_s);
     if (precision == PSR_FP64) {
-        static_assert((size_t)6 * (kPlain64MaxN + 2) * 8 <= kTableBytes, "FP64 table beyond the scratch");
+        static_assert((size_t)6 * (kPlain64MaxN + 1) * 8 <= kTableBytes, "FP64 table beyond the scratch");
         int le = launch_plain64(x_c, base, nullptr, st);
         if (le) {
             set_last_error(std::string("table kernel launch: ") + cudaGetErrorString((cudaError_t)le));

@@ -9,7 +9,7 @@
 
 namespace psr {
 
-template <bool EQM, int R>
+template <bool EQM, bool TAIL, int R>
 __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, const double* tab,
                                            const double* tabq, const Warp64& w64, bool split)
 {
@@ -20,7 +20,7 @@ __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, con
     const bool on = s < S;
     const BoxDev& bx = a.boxes[li.z];
     const long long rc2m1 = bits64(bx.rc2) - 1;
-    const double us = bx.inv_2rs * a.t64_scale;
+    const double us = bx.inv_2rs * kPlain64PerX;
     // exp(-x^2) / (2 sqrt(pi) r_s^3), the second part of -g'(r) r
     const double cq = 1.0 / (2.0 * 1.7724538509055160 * bx.r_s * bx.r_s * bx.r_s);
 
@@ -60,11 +60,21 @@ __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, con
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 if (inside64(r2, rc2m1)) {
                     const double4 c = cs[j];
-                    const double ri = rsqrt64(r2), ri2 = ri * ri;
-                    double f;
-                    const int kk = 6 * node64(r2 * ri, us, a.t64_max, f);
-                    const double gg = horner64<5>(tab + kk, f) * (ri2 * ri);  // T / r^3
-                    const double Q = cq * horner64<5>(tabq + kk, f);
+                    double ri, rr, f;
+                    rsqrt64(r2, ri, rr);
+                    const double ri2 = ri * ri;
+                    const int node = node64(rr, us, f), kk = 6 * min(node, a.t64_max);
+                    double Tv, Qv;
+                    if (TAIL && node > a.t64_max) {
+                        const double2 tq = tail64(rr * bx.inv_2rs);
+                        Tv = tq.x;
+                        Qv = tq.y;
+                    } else {
+                        Tv = horner64<5>(tab + kk, f);
+                        Qv = horner64<5>(tabq + kk, f);
+                    }
+                    const double gg = Tv * (ri2 * ri);  // T / r^3
+                    const double Q = cq * Qv;
                     const double hf = -ri2 * fma(3.0, gg, Q);  // g'(r)/r
                     // v = m_k c_j - m_j c_k (one mass: c_j - c_k, m applied at the end)
                     const double vx = EQM ? c.x - ck[r].x : fma(xi[r].w, c.x, -p.w * ck[r].x);
@@ -92,7 +102,7 @@ __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, con
                    });
 }
 
-template <bool EQM>
+template <bool EQM, bool TAIL>
 __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem64[];
@@ -102,7 +112,7 @@ __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
     double* tabq = tab + words;
     for (int i = threadIdx.x; i < words; i += blockDim.x) {
         tab[i] = reinterpret_cast<const double*>(a.table)[i];
-        tabq[i] = reinterpret_cast<const double*>(a.table)[6 * (kPlain64MaxN + 2) + i];
+        tabq[i] = reinterpret_cast<const double*>(a.table)[6 * (kPlain64MaxN + 1) + i];
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -115,16 +125,26 @@ __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
         int4 li;
         if (!item64(a, it, lane, I, li)) continue;
         const int R = targets_per_lane(li.y, 128);
-        if (R == 1) adj64_item<EQM, 1>(a, I, li, tab, tabq, w64, split);
-        else if (R == 2) adj64_item<EQM, 2>(a, I, li, tab, tabq, w64, split);
-        else adj64_item<EQM, 3>(a, I, li, tab, tabq, w64, split);
+        if (R == 1) adj64_item<EQM, TAIL, 1>(a, I, li, tab, tabq, w64, split);
+        else if (R == 2) adj64_item<EQM, TAIL, 2>(a, I, li, tab, tabq, w64, split);
+        else adj64_item<EQM, TAIL, 3>(a, I, li, tab, tabq, w64, split);
     }
     persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
 }
 
+namespace {
+
+auto pick_adj64(double x_c, bool eqm)
+{
+    if (plain64(x_c).tail) return eqm ? p2p_adj_f64_kernel<true, true> : p2p_adj_f64_kernel<false, true>;
+    return eqm ? p2p_adj_f64_kernel<true, false> : p2p_adj_f64_kernel<false, false>;
+}
+
+}  // namespace
+
 size_t adj_f64_smem(double x_c, int warps)
 {
-    return (size_t)(plain64(x_c).n + 2) * 96 + (size_t)warps * kWarp64Bytes;
+    return (size_t)(plain64(x_c).n + 1) * 96 + (size_t)warps * kWarp64Bytes;
 }
 
 int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)
@@ -135,11 +155,9 @@ int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)
         reinterpret_cast<const double*>(a.cot), a.perm, reinterpret_cast<double4*>(a.cot_sorted), a.n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return (int)e;
-    const Plain64 p = plain64(x_c);
-    a.t64_max = p.n + 1;
-    a.t64_scale = p.n / p.x_top;
+    a.t64_max = plain64(x_c).n;
     const size_t smem = adj_f64_smem(x_c, a.warps_per_block);
-    auto k = a.equal_mass ? p2p_adj_f64_kernel<true> : p2p_adj_f64_kernel<false>;
+    auto k = pick_adj64(x_c, a.equal_mass);
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     k<<<a.blocks, a.warps_per_block * 32, smem, st>>>(a);
@@ -149,10 +167,10 @@ int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)
 int adj_f64_occupancy(int warps, double x_c, int* out)
 {
     const size_t smem = adj_f64_smem(x_c, warps);
-    cudaError_t e = cudaFuncSetAttribute(p2p_adj_f64_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto k = pick_adj64(x_c, false);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
-    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, p2p_adj_f64_kernel<false>, warps * 32, smem);
+    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k, warps * 32, smem);
 }
 
 }  // namespace psr

@@ -3,7 +3,7 @@
 // double-precision table path (Section 3.3: the Eq. int expansion about the
 // nearest of N + 1 nodes, level T_[4] for double precision).  Both evaluate T
 // from a table in shared memory; the plain path's has nodes close enough that
-// T is exact to rounding.  p2p_f64_common.cuh says what bounds the kernel and
+// T is as near as erfc and exp give it.  p2p_f64_common.cuh says what bounds the kernel and
 // what it does about it.  48^3 NFW set: 255 ms with erfc, exp, a square root and
 // a division per tile pair and one warp per leaf.
 #include <cuda_runtime.h>
@@ -12,60 +12,77 @@
 
 namespace psr {
 
-// Taylor tables in FP64: node k = 0..N, x_k = k h, six doubles per node, the
-// coefficients of eps^m (eps = x - x_k) times h^m, so that the expansion is a
-// polynomial in f = x/h - k (zero above the level).  T's are those of Eq. int and
-// the next, from T' = x^2 E, E = -4 exp(-x^2) / sqrt(pi); Q = exp(-x^2) likewise
-// (levels: 2 or 4 as Eq. int's, 5).  Entry N + 1, written at level 5, is zero.
-__global__ void table64_kernel(int N, int level, double h, double* __restrict__ t, double* __restrict__ q)
+// Taylor tables of the levels T_[2] and T_[4] in FP64: node k = 0..N, x_k = k h,
+// six doubles per node, the Eq. int coefficients of eps^m (eps = x - x_k) times
+// h^m, so that the expansion is a polynomial in f = x/h - k (zero above the level).
+__global__ void table64_kernel(int N, int level, double h, double* __restrict__ t)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > N + (level == 5 ? 1 : 0)) return;
+    if (k > N) return;
     double* c = t + 6 * (int64_t)k;
-    const double x = k * h, x2 = x * x, Q = exp(-x2);
-    const double E = -2.0 * 1.1283791670955126 * Q;  // -4 exp(-x^2) / sqrt(pi)
-    const double h2 = h * h, h3 = h2 * h, h4 = h2 * h2, h5 = h4 * h;
-    const double on = k <= N ? 1.0 : 0.0, four = level >= 4 ? on : 0.0, five = level >= 5 ? on : 0.0;
-    c[0] = on * (erfc(x) - 0.5 * x * E);
-    c[1] = on * (x2 * E * h);
-    c[2] = on * (-x * (x2 - 1.0) * E * h2);
-    c[3] = four * ((2.0 / 3.0 * x2 * x2 - 5.0 / 3.0 * x2 + 1.0 / 3.0) * E * h3);
-    c[4] = four * (-x * (x2 * x2 / 3.0 - 1.5 * x2 + 1.0) * E * h4);
-    c[5] = five * (((2.0 / 15.0 * x2 - 14.0 / 15.0) * x2 + 1.3) * x2 - 0.2) * E * h5;
-    if (!q) return;
-    c = q + 6 * (int64_t)k;
-    c[0] = on * Q;
-    c[1] = on * (-2.0 * x * Q * h);
-    c[2] = on * ((2.0 * x2 - 1.0) * Q * h2);
-    c[3] = on * (x * (2.0 - 4.0 / 3.0 * x2) * Q * h3);
-    c[4] = on * (((2.0 / 3.0 * x2 - 2.0) * x2 + 0.5) * Q * h4);
-    c[5] = on * (x * ((-4.0 / 15.0 * x2 + 4.0 / 3.0) * x2 - 1.0) * Q * h5);
+    const double x = k * h, x2 = x * x;
+    const double E = -2.0 * 1.1283791670955126 * exp(-x2);  // -4 exp(-x^2) / sqrt(pi)
+    c[0] = erfc(x) - 0.5 * x * E;
+    c[1] = x2 * E * h;
+    c[2] = -x * (x2 - 1.0) * E * h * h;
+    c[3] = level >= 4 ? (2.0 / 3.0 * x2 * x2 - 5.0 / 3.0 * x2 + 1.0 / 3.0) * E * h * h * h : 0.0;
+    c[4] = level >= 4 ? -x * (x2 * x2 / 3.0 - 1.5 * x2 + 1.0) * E * h * h * h * h : 0.0;
+    c[5] = 0.0;
+}
+
+// The plain path's tables of T (t) and, unless null, Q = exp(-x^2) (q): nodes
+// x_k = k / 256, k = 0..N, six coefficients in f = 256 x - k.  Taylor coefficients
+// about x_k: Q's by (m + 1) q_{m+1} = -2 (x q_m + q_{m-1}), T's from T' = -c x^2 Q,
+// c = 4 / sqrt(pi).  The terms in f^6 and f^7 are replaced by the polynomials of
+// degree 4 and 5 nearest to them on [-1/2, 1/2] (Chebyshev economisation), which
+// divides the error of leaving them out by 32 and 64.
+__global__ void plain64_kernel(int N, double* __restrict__ t, double* __restrict__ q)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k > N) return;
+    const double h = 1.0 / kPlain64PerX, x = k * h;
+    const double c = 2.0 * 1.1283791670955126;  // 4 / sqrt(pi)
+    double Q[8], T[8];
+    Q[0] = exp(-x * x);
+    Q[1] = -2.0 * x * Q[0];
+    for (int m = 1; m < 7; ++m) Q[m + 1] = -2.0 * (x * Q[m] + Q[m - 1]) / (m + 1);
+    T[0] = erfc(x) + 0.5 * c * x * Q[0];
+    for (int m = 0; m < 7; ++m)
+        T[m + 1] = -c * (x * x * Q[m] + (m > 0 ? 2.0 * x * Q[m - 1] : 0.0) + (m > 1 ? Q[m - 2] : 0.0)) / (m + 1);
+    for (int i = 0; i < (q ? 2 : 1); ++i) {
+        double* a = i ? Q : T;
+        double hm = 1.0;
+        for (int m = 1; m < 8; ++m) a[m] *= hm *= h;
+        double* o = (i ? q : t) + 6 * (int64_t)k;
+        o[0] = a[0] + a[6] / 2048.0;
+        o[1] = a[1] + a[7] * (14.0 / 8192.0);
+        o[2] = a[2] - a[6] * (72.0 / 2048.0);
+        o[3] = a[3] - a[7] * (448.0 / 8192.0);
+        o[4] = a[4] + a[6] * (768.0 / 2048.0);
+        o[5] = a[5] + a[7] * (3584.0 / 8192.0);
+    }
 }
 
 int launch_table64(int table_n, int interp, double x_c, void* d_out, void* stream)
 {
     const int threads = 32, blocks = (table_n + 1 + threads - 1) / threads;
     table64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
-        table_n, interp == PSR_TAYLOR4 ? 4 : 2, x_c / table_n, reinterpret_cast<double*>(d_out), nullptr);
+        table_n, interp == PSR_TAYLOR4 ? 4 : 2, x_c / table_n, reinterpret_cast<double*>(d_out));
     return (int)cudaGetLastError();
 }
 
 Plain64 plain64(double x_c)
 {
-    Plain64 p;
-    // T(12) is below 1e-61: beyond, the zero entry
-    p.x_top = x_c < 12.0 ? x_c : 12.0;
-    const double want = std::ceil(p.x_top / 0.0044);
-    p.n = want < 16.0 ? 16 : want > kPlain64MaxN ? kPlain64MaxN : (int)want;
-    return p;
+    const double want = std::ceil(x_c * kPlain64PerX);
+    return Plain64{want > kPlain64MaxN ? kPlain64MaxN : (int)want, want > kPlain64MaxN};
 }
 
 int launch_plain64(double x_c, void* d_t, void* d_q, void* stream)
 {
-    const Plain64 p = plain64(x_c);
-    const int threads = 32, blocks = (p.n + 2 + threads - 1) / threads;
-    table64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(
-        p.n, 5, p.x_top / p.n, reinterpret_cast<double*>(d_t), reinterpret_cast<double*>(d_q));
+    const int n = plain64(x_c).n;
+    const int threads = 32, blocks = (n + 1 + threads - 1) / threads;
+    plain64_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(n, reinterpret_cast<double*>(d_t),
+                                                                 reinterpret_cast<double*>(d_q));
     return (int)cudaGetLastError();
 }
 
@@ -73,7 +90,7 @@ int launch_plain64(double x_c, void* d_t, void* d_q, void* stream)
 // particle of the box has one mass, applied once per target.  COUNT: pairs
 // within the cutoff and pairs evaluated are counted, over every tile pair (no
 // cull).
-template <bool COUNT, bool EQM, int DEG, int R>
+template <bool COUNT, bool EQM, int DEG, bool TAIL, int R>
 __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, const double* tab,
                                            const Warp64& w64, unsigned long long& npairs,
                                            unsigned long long& nev, bool split)
@@ -84,7 +101,7 @@ __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, con
     const bool on = s < S;
     const BoxDev& bx = a.boxes[li.z];
     const long long rc2m1 = bits64(bx.rc2) - 1;
-    const double us = DEG == 5 ? bx.inv_2rs * a.t64_scale : (double)a.table_n / bx.r_c;
+    const double us = DEG == 5 ? bx.inv_2rs * kPlain64PerX : (double)a.table_n / bx.r_c;
     const int kmax = a.t64_max;
 
     double4 xi[R];
@@ -122,10 +139,11 @@ __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, con
                 const double dx = d.x, dy = d.y, dz = d.z;
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 if (inside64(r2, rc2m1)) {
-                    const double ri = rsqrt64(r2);
-                    double f;
-                    const int kk = node64(r2 * ri, us, kmax, f);
-                    const double Tv = horner64<DEG>(tab + 6 * kk, f);
+                    double ri, rr, f;
+                    rsqrt64(r2, ri, rr);
+                    const int kk = node64(rr, us, f);
+                    const double Tv = TAIL && kk > kmax ? tail64(rr * bx.inv_2rs).x
+                                                        : horner64<DEG>(tab + 6 * min(kk, kmax), f);
                     double w = ri * ri * ri * Tv;
                     if (!EQM) w *= p.w;
                     acc[r][0] = fma(w, dx, acc[r][0]);
@@ -148,8 +166,8 @@ __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, con
                    });
 }
 
-// DEG 5: the plain path, 4: the Taylor levels.
-template <bool COUNT, bool EQM, int DEG>
+// DEG 5: the plain path (TAIL: the cutoff lies beyond its table), 4: the Taylor levels.
+template <bool COUNT, bool EQM, int DEG, bool TAIL>
 __global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem64[];
@@ -169,9 +187,9 @@ __global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
         int4 li;
         if (!item64(a, it, lane, I, li)) continue;
         const int R = targets_per_lane(li.y, 128);
-        if (R == 1) fwd64_item<COUNT, EQM, DEG, 1>(a, I, li, tab, w64, npairs, nev, split);
-        else if (R == 2) fwd64_item<COUNT, EQM, DEG, 2>(a, I, li, tab, w64, npairs, nev, split);
-        else fwd64_item<COUNT, EQM, DEG, 3>(a, I, li, tab, w64, npairs, nev, split);
+        if (R == 1) fwd64_item<COUNT, EQM, DEG, TAIL, 1>(a, I, li, tab, w64, npairs, nev, split);
+        else if (R == 2) fwd64_item<COUNT, EQM, DEG, TAIL, 2>(a, I, li, tab, w64, npairs, nev, split);
+        else fwd64_item<COUNT, EQM, DEG, TAIL, 3>(a, I, li, tab, w64, npairs, nev, split);
     }
     if (COUNT) {
         for (int off = 16; off > 0; off >>= 1) npairs += __shfl_xor_sync(kFull, npairs, off);
@@ -187,31 +205,35 @@ namespace {
 
 bool taylor64(int interp) { return interp == PSR_TAYLOR2 || interp == PSR_TAYLOR4; }
 
-template <int DEG>
-const void* pick64(bool count, bool eqm)
+template <int DEG, bool TAIL>
+const void* pick64_t(bool count, bool eqm)
 {
-    return count ? (const void*)p2p_fwd_f64_kernel<true, false, DEG>
-           : eqm ? (const void*)p2p_fwd_f64_kernel<false, true, DEG>
-                 : (const void*)p2p_fwd_f64_kernel<false, false, DEG>;
+    return count ? (const void*)p2p_fwd_f64_kernel<true, false, DEG, TAIL>
+           : eqm ? (const void*)p2p_fwd_f64_kernel<false, true, DEG, TAIL>
+                 : (const void*)p2p_fwd_f64_kernel<false, false, DEG, TAIL>;
+}
+
+const void* pick64(int interp, double x_c, bool count, bool eqm)
+{
+    return taylor64(interp)    ? pick64_t<4, false>(count, eqm)
+           : plain64(x_c).tail ? pick64_t<5, true>(count, eqm)
+                               : pick64_t<5, false>(count, eqm);
 }
 
 }  // namespace
 
 size_t fwd_f64_smem(int interp, int table_n, double x_c, int warps)
 {
-    const int entries = taylor64(interp) ? table_n + 1 : plain64(x_c).n + 2;
+    const int entries = 1 + (taylor64(interp) ? table_n : plain64(x_c).n);
     return (size_t)entries * 48 + (size_t)warps * kWarp64Bytes;
 }
 
 int launch_fwd_f64(const FwdArgs& args, double x_c, void* stream)
 {
     FwdArgs a = args;
-    const bool tay = taylor64(a.interp);
-    const Plain64 p = plain64(x_c);
-    a.t64_max = tay ? a.table_n : p.n + 1;
-    a.t64_scale = p.n / p.x_top;
+    a.t64_max = taylor64(a.interp) ? a.table_n : plain64(x_c).n;
     const size_t smem = fwd_f64_smem(a.interp, a.table_n, x_c, a.warps_per_block);
-    const void* k = tay ? pick64<4>(a.count_pairs, a.equal_mass) : pick64<5>(a.count_pairs, a.equal_mass);
+    const void* k = pick64(a.interp, x_c, a.count_pairs, a.equal_mass);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     void* params[] = {&a};
@@ -221,7 +243,7 @@ int launch_fwd_f64(const FwdArgs& args, double x_c, void* stream)
 
 int fwd_f64_occupancy(int warps, int interp, int table_n, double x_c, int* out)
 {
-    const void* f = taylor64(interp) ? pick64<4>(false, false) : pick64<5>(false, false);
+    const void* f = pick64(interp, x_c, false, false);
     const size_t smem = fwd_f64_smem(interp, table_n, x_c, warps);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;

@@ -54,7 +54,7 @@ struct Layout {
     size_t table;    // float4[2 * (kMaxTableN + 1)]: T table, then exp(-x^2)
     size_t core;     // float2[kMaxTableN + 1]: core form of the forward's linear table
     size_t fine;     // float4[2 * (kFineMaxN + 1)]: PSR_FP32_EXACT's fine table of T, then exp(-x^2)
-    size_t t64;      // double[2][6 (kPlain64MaxN + 2)]: FP64 plain path's T and exp(-x^2) tables
+    size_t t64;      // double[2][6 (kPlain64MaxN + 1)]: FP64 plain path's T and exp(-x^2) tables
     size_t cotf;     // float4[n] / double4[n] adjoint source payload scratch
     size_t ctrl;     // uint32[64]  scheduler tickets, error word, counters
     // multipole split (device builds with an acceptance parameter only)
@@ -227,8 +227,7 @@ struct FwdArgs {
     int stage_cap;   // FP32 kernels: staged particles per warp
     int item_stride; // this launch takes schedule entries ticket * stride + offset
     int item_offset;
-    int t64_max;       // FP64 kernels: last entry of the Taylor table
-    double t64_scale;  //   and its nodes per unit of x (plain path)
+    int t64_max;       // FP64 kernels: last node of the table
     const int* heavy;  // how many items groups of warps take (null: all)
     int group;         // warps per group (divides warps_per_block); 0 or 1: none
     int fine;        // PSR_FP32_EXACT by the fine cubic table (interp and table_n are its)
@@ -250,12 +249,14 @@ constexpr size_t kSmemPerBlock = 227 * 1024;  // opt-in dynamic shared memory pe
 int fwd_f64_occupancy(int warps, int interp, int table_n, double x_c, int* out);
 int launch_table64(int table_n, int interp, double x_c, void* d_out, void* stream);  // p2p_fwd_f64.cu
 size_t fwd_f64_smem(int interp, int table_n, double x_c, int warps);
-// Taylor nodes of the FP64 plain path: 0.0044 apart in x up to x = 6, n of them
-// over [0, x_top] beyond (the allocation-free entry point's scratch holds 1363)
-constexpr int kPlain64MaxN = 1363;
+// Nodes of the FP64 plain path's tables, per unit of x: a power of two, so that
+// a distance in node spacings has the rounding of 1 / (2 r_s) alone.  The last
+// node, x = 5.32, is what the allocation-free entry point's scratch holds; tail:
+// the cutoff lies beyond it.
+constexpr int kPlain64PerX = 256, kPlain64MaxN = 1363;
 struct Plain64 {
     int n;
-    double x_top;
+    bool tail;
 };
 Plain64 plain64(double x_c);
 int launch_plain64(double x_c, void* d_t, void* d_q, void* stream);

@@ -83,3 +83,37 @@ def test_fp64_cutoff_far_beyond_the_table(r_s, device):
     ox, om = oracle.adjoint(pos, mass, cot, L, r_s, r_c, 1.0)[:2]
     tol = 1e-13 + 4 * 2.0 ** -53 * L / (0.4 * r_s)
     assert _rms(acc, ref) < tol and _rms(gx, ox) < 3 * tol and _rms(gm, om) < tol
+
+
+@pytest.mark.parametrize("x_c", [2.25, 5.3, 5.4, 9.0, 12.0, 14.0])
+def test_fp64_pairs_over_all_separations(x_c):
+    """Isolated pairs from x = 1e-3 x_c to x_c in units 2 r_s = 1, where x is the separation itself,
+    against T and exp(-x^2) in 40 digits: each pair's force and gradients to the roundings of x (r^2's
+    and the root's: under 3 x 2^-53, times |x T'/T| < 2 x^2 + 2), 16 roundings of the factors, and
+    3e-15 for the folded tables at their far end."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.dps = 40
+    m, r_c = 10, x_c
+    L, x = 3.2 * m * r_c, np.geomspace(1e-3 * x_c, 0.999 * x_c, m ** 3)
+    grid = (np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3) + 0.25) * 3.2 * r_c
+    pos = np.empty((2 * m ** 3, 3))
+    pos[::2] = pos[1::2] = grid
+    pos[1::2, 0] += x
+    r = pos[1::2, 0] - pos[::2, 0]
+    mass = np.where(np.arange(2 * m ** 3) % 2, 0.25, 0.5)
+    cot = np.zeros_like(pos)
+    cot[:, 0] = np.where(np.arange(2 * m ** 3) % 2, 2.0, -1.0)
+    lv = psr.Leaves.build(pos, mass, L, 0.5, r_c).upload()
+    o = psr.Options(precision=psr.PSR_FP64)
+    acc = lv.forces(o).cpu().numpy()
+    gx, gm = (g.cpu().numpy() for g in lv.adjoint(torch.tensor(cot), o))
+    Q = [mp.e ** (-mp.mpf(float(v)) ** 2) for v in r]
+    T = [mp.erfc(mp.mpf(float(v))) + 2 / mp.sqrt(mp.pi) * mp.mpf(float(v)) * q for v, q in zip(r, Q)]
+    f = np.array([float(t / mp.mpf(float(v)) ** 2) for t, v in zip(T, r)])
+    # longitudinal g + r g'(r) = -2 g - Q / (2 sqrt(pi) r_s^3)
+    k = np.array([float(-2 * t / mp.mpf(float(v)) ** 3 - 4 / mp.sqrt(mp.pi) * q) for t, q, v in zip(T, Q, r)])
+    tol = (16 + 3 * (2 * r * r + 2)) * 2.0 ** -53 + np.where(r > 3.0, 3e-15, 0.0)
+    for got, want in ((acc[::2, 0], 0.25 * f), (acc[1::2, 0], -0.5 * f),
+                      (gm[::2], -2.0 * f), (gm[1::2], -1.0 * f),
+                      (gx[::2, 0], k * (0.5 * 2.0 + 0.25 * 1.0)), (gx[1::2, 0], -k * (0.5 * 2.0 + 0.25 * 1.0))):
+        assert np.all(np.abs(got / want - 1.0) < tol), float(np.max(np.abs(got / want - 1.0) / tol))

@@ -131,7 +131,9 @@ typedef struct {
                             shard_index, shard_index + shard_count, ... (the
                             schedule is largest-work first, so the shards are
                             balanced) and leaves every other output element
-                            untouched; 0 or 1 = all targets                  */
+                            untouched; 0 or 1 = all targets.  The shards
+                            give the unsharded launch's results bit for bit,
+                            as do other warps_per_block and blocks_per_sm    */
     int shard_index;     /* 0 <= shard_index < max(shard_count, 1)          */
     int reserved[4];     /* must be zero                                      */
 } psr_opts;
@@ -210,7 +212,9 @@ int psr_build_leaves(const double* pos, const double* mass, int64_t n, const psr
  * psr_build_leaves_batch - host: as psr_build_leaves for nbox independent
  * boxes in one handle; one launch then serves every box.  Particles are
  * numbered box after box (box 0's n[0] particles first).  All boxes must
- * share the ratio r_c / r_s (one interpolation table).
+ * share the ratio r_c / r_s (one interpolation table).  Each box gets the
+ * forces and gradients of that box alone, bit for bit (given one mass per box
+ * in all boxes or in none, see psr_info.equal_mass).
  */
 int psr_build_leaves_batch(int nbox, const double* const* pos, const double* const* mass,
                            const int64_t* n, const psr_box* boxes, int max_leaf, int flags,

@@ -404,6 +404,7 @@ Layout make_layout(const Leaves& h)
     L.rowptr = o;    o = align256(o + (nl + 1) * 8);
     L.pairs = o;     o = align256(o + np * 4);
     L.items = o;     o = align256(o + nl * 4);
+    L.cost = o;      o = align256(o + nl * 8);
     L.boxes = o;     o = align256(o + h.boxdev.size() * sizeof(BoxDev));
     L.table = o;     o = align256(o + 2 * (size_t)(kMaxTableN + 1) * 16);
     L.fine = o;      o = align256(o + 2 * (size_t)(kFineMaxN + 1) * 16);
@@ -736,6 +737,22 @@ int build_batch(int nbox, const double* const* pos, const double* const* mass, c
         h->item_cost.resize(nl);
         for (int64_t g = 0; g < nl; ++g) h->item_cost[g] = cost[h->items[g]];
         h->max_cost = nl ? h->item_cost[0] : 0;
+        // ---- parts of heavy rows, by box ----------------------------------
+        struct Load {
+            int64_t most = 0, all = 0, leaves = 0;
+            int max_leaf = 0;
+        };
+        std::vector<Load> load(nbox);
+        for (int64_t g = 0; g < nl; ++g) {
+            Load& b = load[lbox[g]];
+            b.most = std::max(b.most, cost[g]);
+            b.all += cost[g];
+            ++b.leaves;
+            b.max_leaf = std::max(b.max_leaf, h->leaf[4 * g + 1]);
+        }
+        for (int b = 0; b < nbox; ++b)
+            parts_rule(load[b].most, load[b].all, load[b].leaves, load[b].max_leaf, &h->boxdev[b]);
+        h->cost = std::move(cost);
         h->n_leaves = nl;
         h->n_pairs = (int64_t)h->pairs.size();
         h->has_pd = !(flags & PSR_BUILD_NO_FP64);

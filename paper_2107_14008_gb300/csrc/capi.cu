@@ -46,7 +46,7 @@ int wait_stream(cudaStream_t st, int timeout_ms)
 struct Opts {
     int precision, table_n, interp, accum, warps, bps, fold, count, kernel, tile, nshard, shard;
     bool fine = false;  // PSR_FP32_EXACT by the fine cubic table (fine_exact)
-    bool split;  // heavy items on whole blocks: the default kernel's choice
+    bool split;  // heavy rows in parts: the default kernel's choice
 };
 
 int check_opts(const psr_opts* o, Opts* out)
@@ -131,6 +131,7 @@ FwdArgs base_args(Leaves* h, const Opts& o)
     a.rowptr = reinterpret_cast<const int64_t*>(w + L.rowptr);
     a.pairs = reinterpret_cast<const uint32_t*>(w + L.pairs);
     a.items = reinterpret_cast<const int32_t*>(w + L.items);
+    a.cost = reinterpret_cast<const long long*>(w + L.cost);
     a.boxes = reinterpret_cast<const BoxDev*>(w + L.boxes);
     a.ctrl = reinterpret_cast<unsigned*>(w + L.ctrl);
     a.cot_sorted = w + L.cotf;
@@ -250,52 +251,62 @@ int ensure_table(Leaves* h, const Opts& o, bool core, cudaStream_t st, const voi
     });
 }
 
-int grid_blocks(Leaves* h, const Opts& o, int adjoint, int* blocks)
+// Blocks per SM of a launch.
+int blocks_per_sm(const Leaves* h, const Opts& o, bool adjoint, int* bps)
 {
-    int bps = o.bps;
-    if (bps == 0) {
-        int occ = 0, e;
-        if (adjoint && o.precision == PSR_FP64)
-            e = adj_f64_occupancy(o.warps, cutoff_x(h), &occ);
-        else if (adjoint)
-            e = adj_f32_occupancy(o.precision, o.interp, o.accum, o.warps, h->max_leaf, o.table_n,
+    *bps = o.bps;
+    if (o.bps) return PSR_OK;
+    int occ = 0, e;
+    if (adjoint && o.precision == PSR_FP64)
+        e = adj_f64_occupancy(o.warps, cutoff_x(h), &occ);
+    else if (adjoint)
+        e = adj_f32_occupancy(o.precision, o.interp, o.accum, o.warps, h->max_leaf, o.table_n,
                               o.tile ? o.tile : kAdjStageCap, o.kernel, &occ);
-        else if (o.precision == PSR_FP64)
-            e = fwd_f64_occupancy(o.warps, o.interp, o.table_n, cutoff_x(h), &occ);
-        else if (o.kernel == PSR_KERNEL_PAPER)
-            e = fwd_blk_occupancy(o.precision, o.interp, o.accum, h->max_leaf, o.table_n, &occ);
-        else {
-            int cap;
-            if ((e = fwd32_smem_config(o, &cap))) return e;
-            if ((e = check_tile(h, cap))) return e;
-            e = fwd_f32_occupancy(o.precision, o.interp, o.accum, o.warps, o.table_n, cap, o.kernel,
-                                  fwd_core(o.precision, o.interp, o.table_n, o.kernel, cutoff_x(h)),
-                                  &occ);
-        }
-        if (e) return cuda_fail((cudaError_t)e, "occupancy query");
-        bps = occ > 0 ? occ : 1;
-    }
-    *blocks = bps * (h->sm_count > 0 ? h->sm_count : 1);
+    else if (o.precision == PSR_FP64)
+        e = fwd_f64_occupancy(o.warps, o.interp, o.table_n, cutoff_x(h), &occ);
+    else if (o.kernel == PSR_KERNEL_PAPER)
+        e = fwd_blk_occupancy(o.precision, o.interp, o.accum, h->max_leaf, o.table_n, &occ);
+    else
+        e = fwd_f32_occupancy(o.precision, o.interp, o.accum, o.warps, o.table_n, o.tile ? o.tile : 256,
+                              o.kernel, fwd_core(o.precision, o.interp, o.table_n, o.kernel, cutoff_x(h)), &occ);
+    if (e) return cuda_fail((cudaError_t)e, "occupancy query");
+    *bps = occ > 0 ? occ : 1;
     return PSR_OK;
 }
 
-// Heavy rows shared among warps (the default kernels only), for a launch
-// whose grid is known.  The line (SplitRule): 3/2 of a share; 5/4 where a pair
-// costs more, as with every table but the linear one (cubic adjoint, 150,000 NFW
-// 4.33 -> 2.72 ms against a line of 2), and 2 for the linear adjoint of leaves of
-// up to 32, whose rows are short against the group's overheads (150,000 NFW in
-// leaves of up to 16 1.95 ms, 2.05 with 3/2; 64^3 NFW 2.74 and 2.83; in leaves of
-// up to 64, 512,000 NFW gain 5.96 -> 5.36 with 3/2).
-void set_split(const Leaves* h, const Opts& o, bool adjoint, FwdArgs* a)
+// The launch's grid and how it takes rows with parts, which the default FP32 kernels
+// and the FP64 kernels have.  Side by side where the launch is short of rows: one
+// box as its parts were chosen, but for this launch's warps and shard (the groups
+// take just the rows that have parts); a batch only if it has fewer rows than
+// warps (a group then takes every row).  Else in turn: a batch of many boxes fills
+// the chip.  There the parts cost a chunk of sources more each: 64 boxes of 8^3 to
+// 64^3 particles, three quarters of the work in rows of 2 to 8 parts, 6.25 -> 6.73 ms
+// against whole rows, whose sums would differ from the boxes' alone.
+int plan_rows(const Leaves* h, const Opts& o, bool adjoint, FwdArgs* a)
 {
-    if (!o.split && o.precision != PSR_FP64) return;
+    int bps, rc;
+    if ((rc = blocks_per_sm(h, o, adjoint, &bps))) return rc;
+    a->blocks = bps * (h->sm_count > 0 ? h->sm_count : 1);
+    a->rows = kRowsWhole;
+    if (!o.split && o.precision != PSR_FP64) return PSR_OK;
     const bool linear = o.precision == PSR_FP32_TABLE && o.interp == PSR_LINEAR;
-    const int line = !linear ? 10 : adjoint && h->max_leaf <= 32 ? 16 : 12;
-    const SplitRule r = split_rule(h->max_cost, h->evaluated, h->n_leaves, h->sm_count,
-                                   (int64_t)a->blocks * o.warps, o.warps, line);
-    a->group = r.group;
+    a->kind = o.precision == PSR_FP64 ? kPartsF64
+              : adjoint               ? (linear ? kPartsAdj : kPartsAdjTab)
+                                      : (linear ? kPartsFwd : kPartsFwdTab);
+    int parts = 1;
+    for (const BoxDev& b : h->boxdev) parts = std::max(parts, b.parts[a->kind]);
+    if (parts == 1) return PSR_OK;
+    a->rows = kRowsInTurn;
+    if (o.warps % parts) return PSR_OK;
+    SplitRule r = split_rule(h->max_cost, h->evaluated / o.nshard, (h->n_leaves + o.nshard - 1) / o.nshard,
+                             (int64_t)a->blocks * o.warps, split_line(a->kind, h->max_leaf));
+    if (r.parts == 1 || (h->nbox > 1 && r.level >= 0)) return PSR_OK;
+    a->rows = kRowsJoint;
+    a->group = parts;
+    if (h->nbox == 1) r = box_rule(a->kind, h->max_cost, h->evaluated, h->n_leaves, h->max_leaf);
     if (r.level >= 0)
         a->heavy = reinterpret_cast<const int*>(h->d_ws + h->lay.ctrl) + kCtrlHeavy + r.level;
+    return PSR_OK;
 }
 
 }  // namespace
@@ -320,8 +331,7 @@ int prepare_forward(Leaves* h, const psr_opts* opts, FwdArgs* a, int* precision)
     *a = base_args(h, o);
     if (fwd32 && (rc = fwd32_smem_config(o, &a->stage_cap))) return rc;
     if (fwd32 && (rc = check_tile(h, a->stage_cap))) return rc;
-    if ((rc = grid_blocks(h, o, 0, &a->blocks))) return rc;
-    set_split(h, o, false, a);
+    if ((rc = plan_rows(h, o, false, a))) return rc;
     a->core = fwd_core(o.precision, o.interp, o.table_n, o.kernel, cutoff_x(h));
     *precision = o.precision;
     return PSR_OK;
@@ -412,6 +422,7 @@ int psr_upload(psr_leaves* hh, void* d_ws, size_t bytes, void* stream)
         {L.rowptr, h->rowptr.data(), h->rowptr.size() * sizeof(int64_t)},
         {L.pairs, h->pairs.data(), h->pairs.size() * sizeof(uint32_t)},
         {L.items, h->items.data(), h->items.size() * sizeof(int32_t)},
+        {L.cost, h->cost.data(), h->cost.size() * sizeof(int64_t)},
         {L.boxes, h->boxdev.data(), h->boxdev.size() * sizeof(BoxDev)},
     };
     for (const Cp& c : cps) {
@@ -422,7 +433,7 @@ int psr_upload(psr_leaves* hh, void* d_ws, size_t bytes, void* stream)
     if ((e = cudaMemsetAsync(w + L.ctrl, 0, kCtrlWords * 4, st)) != cudaSuccess)
         return cuda_fail(e, "cudaMemsetAsync (ctrl)");
     for (int l = 0; l < kHeavyLevels; ++l) {
-        const int64_t heavy = heavy_cost(l, h->evaluated, sms);
+        const int64_t heavy = heavy_cost(l, h->evaluated);
         h->n_heavy[l] = (int32_t)(std::partition_point(h->item_cost.begin(), h->item_cost.end(),
                                                        [heavy](int64_t c) { return c > heavy; }) -
                                   h->item_cost.begin());
@@ -464,8 +475,7 @@ int psr_p2p_forces(psr_leaves* hh, const psr_opts* opts, void* d_acc, void* stre
     a.core = core;
     if (fwd32 && (rc = fwd32_smem_config(o, &a.stage_cap))) return rc;
     if (fwd32 && (rc = check_tile(h, a.stage_cap))) return rc;
-    if ((rc = grid_blocks(h, o, 0, &a.blocks))) return rc;
-    set_split(h, o, false, &a);
+    if ((rc = plan_rows(h, o, false, &a))) return rc;
     if (o.count) {
         cudaError_t e = cudaMemsetAsync(a.ctrl + kCtrlPairsLo, 0, 16, st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (pair counters)");
@@ -509,8 +519,7 @@ int psr_p2p_adjoint(psr_leaves* hh, const psr_opts* opts, const void* d_cot, voi
                                "use fewer warps or a smaller table");
     a.out = d_grad_pos;
     a.out_m = d_grad_mass;
-    if ((rc = grid_blocks(h, o, 1, &a.blocks))) return rc;
-    set_split(h, o, true, &a);
+    if ((rc = plan_rows(h, o, true, &a))) return rc;
     int e = (o.precision == PSR_FP64) ? launch_adj_f64(a, cutoff_x(h), st) : launch_adj_f32(a, o.precision, st);
     if (e) return cuda_fail((cudaError_t)e, "adjoint kernel launch");
     return PSR_OK;

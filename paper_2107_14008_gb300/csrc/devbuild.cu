@@ -1377,12 +1377,14 @@ __global__ void k_payload(const int32_t* __restrict__ lfirst, const int32_t* __r
 }
 
 // schedule keys: maxcost - cost ascending = cost descending; equal costs keep
-// leaf order (stable sort)
+// leaf order (stable sort); and the costs into the workspace
 __global__ void k_sched_keys(const int64_t* __restrict__ lcost, int64_t nl, long long maxcost,
-                             uint64_t* __restrict__ key, int32_t* __restrict__ val)
+                             uint64_t* __restrict__ key, int32_t* __restrict__ val,
+                             int64_t* __restrict__ cost)
 {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (g >= nl) return;
+    cost[g] = lcost[g];
     key[g] = (uint64_t)(maxcost - lcost[g]);
     val[g] = (int32_t)g;
 }
@@ -1645,6 +1647,7 @@ int device_build(const double* d_pos, const double* d_mass, int64_t n, const psr
             std::memcpy(&m0, &c[kCntMass0], sizeof m0);
             h->boxdev[0].m_eq = (float)m0;
         }
+        parts_rule(c[kCntMaxCost], h->evaluated, nl, h->max_leaf, &h->boxdev[0]);
         h->lay = make_layout(*h);
     } catch (const std::bad_alloc&) {
         delete h;
@@ -1771,7 +1774,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     int32_t* v0 = (int32_t*)(s + S.flag);
     int32_t* v1 = (int32_t*)(s + S.lid);
     k_sched_keys<<<nblk(nl, 256), 256, 0, st>>>((const int64_t*)(s + S.lcost), nl,
-                                                (long long)h->max_cost, k0, v0);
+                                                (long long)h->max_cost, k0, v0, (int64_t*)(w + L.cost));
     int bits = 1;
     while (bits < 63 && ((uint64_t)h->max_cost >> bits)) ++bits;
     uint64_t* kr;
@@ -1779,7 +1782,7 @@ int psr_device_build_finish(psr_leaves* hh, void* d_ws, size_t bytes, void* stre
     if ((e = radix_sort(k0, v0, k1, v1, nl, bits, sctl, err, &kr, &vr, st)))
         return dcuda(e, "schedule sort");
     HeavyLines heavy;
-    for (int l = 0; l < kHeavyLevels; ++l) heavy.cost[l] = heavy_cost(l, h->evaluated, sms);
+    for (int l = 0; l < kHeavyLevels; ++l) heavy.cost[l] = heavy_cost(l, h->evaluated);
     k_sched_out<<<nblk(nl, 256), 256, 0, st>>>(kr, vr, nl, (long long)h->max_cost, heavy,
                                                (int32_t*)(w + L.items), (int*)(w + L.ctrl) + kCtrlHeavy);
     if ((e = (int)cudaGetLastError())) return dcuda(e, "schedule kernel");

@@ -131,6 +131,20 @@ struct Acc3 {
         }
         fx = fy = fz = 0.0f;
     }
+    __device__ __forceinline__ PartSum<ACC> part(int i) const
+    {
+        PartSum<ACC> p;
+        p.v = i == 0 ? x : i == 1 ? y : z;
+        p.hi = i == 0 ? sx : i == 1 ? sy : sz;
+        p.lo = i == 0 ? cx : i == 1 ? cy : cz;
+        return p;
+    }
+    __device__ __forceinline__ void set(const PartSum<ACC>& a, const PartSum<ACC>& b, const PartSum<ACC>& c)
+    {
+        x = a.v; y = b.v; z = c.v;
+        sx = a.hi; sy = b.hi; sz = c.hi;
+        cx = a.lo; cy = b.lo; cz = c.lo;
+    }
 };
 
 // The target leaf's particle box in the kernel's working frame, and the
@@ -365,16 +379,15 @@ __device__ __forceinline__ int stage_chunk(const FwdArgs& a, long long e0, long 
 
 // Combine the S stream partial sums of each target through shared memory
 // (the warp's staging buffer) and write the accelerations, scaled by gout, in
-// the original particle order.  With split, the group's warps each hold the
-// sums over their part of the row: every warp leaves its target sums at the
-// start of its own region, and after a barrier one thread per target adds them
-// over the warps, in warp order, and writes them (wstride: float4 per warp).
-template <int ACC, int R>
+// the original particle order.  In a row that a group of warps shares each has the
+// sums of its part (join_parts; wstride: float4 per warp).
+template <int ACC, int R, class Work>
 __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>* acc,
                                             const bool* act, int lane, int s, int q, int S, int T,
-                                            float gout, float4* __restrict__ stage, bool split,
+                                            float gout, float4* __restrict__ stage, const Work& rw,
                                             int wstride)
 {
+    const bool joint = rw.joint();
     // Each target slot r reduces through its own region of the staging buffer
     // (768 B; two slots fit the smallest per-warp buffer, 64 + 32 float4), with
     // volatile accesses, so one slot's stores cannot overtake another's loads.
@@ -386,24 +399,18 @@ __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>
             red[3 * lane + 1] = acc[r].y;
             red[3 * lane + 2] = acc[r].z;
             __syncwarp();
-            if (s == 0 && act[r]) {
+            if (!joint && s == 0 && act[r]) {
                 double sx = acc[r].x, sy = acc[r].y, sz = acc[r].z;
                 for (int t = 1; t < S; ++t) {
                     sx += red[3 * (lane + t * T) + 0];
                     sy += red[3 * (lane + t * T) + 1];
                     sz += red[3 * (lane + t * T) + 2];
                 }
-                if (split) {  // streams t >= 1 sit above the first T entries
-                    red[3 * lane + 0] = sx;
-                    red[3 * lane + 1] = sy;
-                    red[3 * lane + 2] = sz;
-                } else {
-                    int idx = a.perm[li.x + q + T * r];
-                    float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
-                    out[0] = (float)(sx * (double)gout);
-                    out[1] = (float)(sy * (double)gout);
-                    out[2] = (float)(sz * (double)gout);
-                }
+                int idx = a.perm[li.x + q + T * r];
+                float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
+                out[0] = (float)(sx * (double)gout);
+                out[1] = (float)(sy * (double)gout);
+                out[2] = (float)(sz * (double)gout);
             }
         } else {
             volatile float* red = reinterpret_cast<volatile float*>(stage) + 192 * r;
@@ -414,7 +421,7 @@ __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>
             red[6 * lane + 4] = acc[r].sz;
             red[6 * lane + 5] = acc[r].cz;
             __syncwarp();
-            if (s == 0 && act[r]) {
+            if (!joint && s == 0 && act[r]) {
                 float sx = acc[r].sx, cx = acc[r].cx, sy = acc[r].sy, cy = acc[r].cy;
                 float sz = acc[r].sz, cz = acc[r].cz, u, v;
                 for (int t = 1; t < S; ++t) {
@@ -423,47 +430,22 @@ __device__ __forceinline__ void finish_item(const FwdArgs& a, int4 li, Acc3<ACC>
                     two_sum(sy, o[2], u, v); sy = u; cy += o[3] + v;
                     two_sum(sz, o[4], u, v); sz = u; cz += o[5] + v;
                 }
-                if (split) {
-                    volatile float* o = red + 6 * lane;
-                    o[0] = sx; o[1] = cx;
-                    o[2] = sy; o[3] = cy;
-                    o[4] = sz; o[5] = cz;
-                } else {
-                    int idx = a.perm[li.x + q + T * r];
-                    float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
-                    out[0] = (sx + cx) * gout;
-                    out[1] = (sy + cy) * gout;
-                    out[2] = (sz + cz) * gout;
-                }
+                int idx = a.perm[li.x + q + T * r];
+                float* out = reinterpret_cast<float*>(a.out) + 3LL * idx;
+                out[0] = (sx + cx) * gout;
+                out[1] = (sy + cy) * gout;
+                out[2] = (sz + cz) * gout;
             }
         }
         __syncwarp();
     }
-    if (split) {
-        group_sync(a.group);
-        const int nw = a.group, gw = (threadIdx.x >> 5) % nw;  // this warp in its group
-        for (int t = 32 * gw + lane; t < li.y; t += 32 * nw) {
-            const int r = t / T, k = t - r * T;  // slot r, lane k of each warp
-            const float4* base = stage - gw * wstride;
-            float* out = reinterpret_cast<float*>(a.out) + 3LL * a.perm[li.x + t];
-            for (int i = 0; i < 3; ++i) {
-                if (ACC == PSR_ACC_FP64) {
-                    double sum = 0.0;
-                    for (int w = 0; w < nw; ++w)
-                        sum += (reinterpret_cast<const volatile double*>(base + w * wstride) + 96 * r)[3 * k + i];
-                    out[i] = (float)(sum * (double)gout);
-                } else {
-                    float hi = 0.0f, lo = 0.0f, u, v;
-                    for (int w = 0; w < nw; ++w) {
-                        const volatile float* o =
-                            reinterpret_cast<const volatile float*>(base + w * wstride) + 192 * r + 6 * k + 2 * i;
-                        two_sum(hi, o[0], u, v); hi = u; lo += o[1] + v;
-                    }
-                    out[i] = (hi + lo) * gout;
-                }
-            }
-        }
-    }
+    if (joint)
+        join_parts<3, ACC>(
+            a, rw, li.y, S, reinterpret_cast<const char*>(stage), 16 * wstride,
+            [T](int t, int s, int i) { return 768 * (t / T) + 24 * (t % T + s * T) + 8 * i; },
+            [&](int t, int i, const PartSum<ACC>& v) {
+                reinterpret_cast<float*>(a.out)[3LL * a.perm[li.x + t] + i] = v.scaled(gout);
+            });
 }
 
 // Packed FP32 helpers (sm_100+ f32x2 instructions: two lanes of work per issue)
@@ -523,15 +505,15 @@ __device__ __forceinline__ float2 eval_T2(float2 t, float2 r2, float2 rinv, unsi
     }
 }
 
-// One target leaf on one warp.  R = targets per lane; T = ceil(n_I / R) lanes
+// One target leaf on one warp (rw: or a part of its row).  R = targets per lane; T = ceil(n_I / R) lanes
 // per stream, S = 32 / T streams.  Each stream takes staged particle PAIRS
 // s, s+S, ... and evaluates both particles of a pair at once with packed
 // FP32 (f32x2) arithmetic.
-template <int TM, int ACC, bool COUNT, bool EQM, int R>
+template <int TM, int ACC, bool COUNT, bool EQM, int R, class Work>
 __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                             float4* __restrict__ stage, float4* __restrict__ meta,
                                          unsigned long long& npairs, unsigned long long& nev,
-                                            bool split, int wstride)
+                                            Work rw, PartTotals<ACC, 9>& tot, int wstride)
 {
     const int lane = threadIdx.x & 31;
     const float4* __restrict__ pf = reinterpret_cast<const float4*>(a.pf);
@@ -575,101 +557,116 @@ __device__ __forceinline__ void fwd_item_pk(const FwdArgs& a, int I, int4 li, un
             }
         cull_box(lx, ly, lz, hx, hy, hz, x_c * sc, meta + kMetaPerWarp);
     }
-    Acc3<ACC> acc[R];
-    float2 fx[R], fy[R], fz[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) fx[r] = fy[r] = fz[r] = make_float2(0.0f, 0.0f);
     unsigned cnt = 0;
-    long long e0, re;
-    row_part(a, I, split, e0, re);
     const float eps = kEps2 * sc * sc;
     const float2 eps2 = make_float2(eps, eps);
     // table coordinate: u - 1/2 (interval tables), u (Taylor: nearest node)
     const float2 mhalf = TM == TM_TAYLOR ? make_float2(0.0f, 0.0f) : make_float2(-0.5f, -0.5f);
     const float soff = -0.5f / nmax;  // linear path: s = sat(r / x_c - 1/(2N))
-    while (e0 < re) {
-        int nst;
-        e0 += stage_chunk<1>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
-        if (COUNT && lane == 0) nev += (unsigned long long)nst * (unsigned)nI;
-        if (on) {
-            auto evalp = [&](const float4 A, const float4 B) {
-                const float2 px = make_float2(A.x, A.y), py = make_float2(A.z, A.w);
-                const float2 pz = make_float2(B.x, B.y), pm = make_float2(B.z, B.w);
+    Acc3<ACC> acc[R];
+    float4* const wbox = meta + kMetaPerWarp;
+    rw.park(wbox);
+    float2 fx[R], fy[R], fz[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) fx[r] = fy[r] = fz[r] = make_float2(0.0f, 0.0f);
+    for (;;) {  // the row, or its parts in turn
+        long long e0, re;
+        row_part(a, I, Work::at(wbox), e0, re);
+        while (e0 < re) {
+            int nst;
+            e0 += stage_chunk<1>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
+            if (COUNT && lane == 0) nev += (unsigned long long)nst * (unsigned)nI;
+            if (on) {
+                auto evalp = [&](const float4 A, const float4 B) {
+                    const float2 px = make_float2(A.x, A.y), py = make_float2(A.z, A.w);
+                    const float2 pz = make_float2(B.x, B.y), pm = make_float2(B.z, B.w);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float2 dx = add2(px, ntx[r]), dy = add2(py, nty[r]), dz = add2(pz, ntz[r]);
+                        const float2 dyz = fma2(dy, dy, fma2(dz, dz, eps2));
+                        float2 r2, rinv, w;
+                        if (TM == TM_CORE) {
+                            r2 = make_float2(fma_sat(dx.x, dx.x, dyz.x), fma_sat(dx.y, dx.y, dyz.y));
+                            rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+                            w = core_weight2(r2, rinv, nmax, tab_bias);
+                            if (!EQM) w = mul2(w, pm);
+                        } else {
+                            r2 = fma2(dx, dx, dyz);
+                            rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+                            const float2 t = TM == TM_LINEAR
+                                                 ? make_float2(fma_sat(r2.x, rinv.x, soff), fma_sat(r2.y, rinv.y, soff))
+                                                 : fma2(r2, rinv, mhalf);
+                            const float2 Tv = eval_T2<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
+                            // 1/r^3 formed beside the table lookup: two dependent
+                            // multiplies after T instead of four
+                            const float2 ri3 = mul2(mul2(rinv, rinv), rinv);
+                            w = EQM ? mul2(Tv, ri3) : mul2(mul2(pm, Tv), ri3);
+                        }
+                        fx[r] = fma2(w, dx, fx[r]);
+                        fy[r] = fma2(w, dy, fy[r]);
+                        fz[r] = fma2(w, dz, fz[r]);
+                        if (COUNT) {
+                            const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
+                            const float ua = TM == TM_CORE ? r2.x : r2.x * rinv.x;
+                            const float ub = TM == TM_CORE ? r2.y : r2.y * rinv.y;
+                            cnt += (act[r] && ua < uc && (dx.x != 0.0f || dy.x != 0.0f || dz.x != 0.0f));
+                            cnt += (act[r] && ub < uc && (dx.y != 0.0f || dy.y != 0.0f || dz.y != 0.0f));
+                        }
+                    }
+                };
+                // Two staged pairs per iteration (k and k + S, then the odd one),
+                // in the order of the plain loop: two independent dependency
+                // chains per lane, as in the scalar kernel.  32-bit shared-window
+                // addresses and volatile loads as there; with one mass the (m0,
+                // m1) half of a pair is not read (a 16-byte broadcast load takes
+                // two cycles of the shared-memory pipe, an 8-byte one takes one).
+                auto load = [&](unsigned p, float4& A, float4& B) {
+                    A = lds_f4_v(p);
+                    if (EQM) {
+                        const float2 z = lds_f2_v(p + 16u);
+                        B = make_float4(z.x, z.y, 0.0f, 0.0f);
+                    } else {
+                        B = lds_f4_v(p + 16u);
+                    }
+                };
+                unsigned sa = smem_u32(stage + 2 * s);
+                const unsigned se = smem_u32(stage + 2 * ((nst + 1) >> 1)), st1 = 32u * (unsigned)S;
+                float4 A0, B0, A1, B1;
+#pragma unroll 1
+                for (; sa + st1 < se; sa += 2u * st1) {
+                    load(sa, A0, B0);
+                    load(sa + st1, A1, B1);
+                    evalp(A0, B0);
+                    evalp(A1, B1);
+                }
+                if (sa < se) {
+                    load(sa, A0, B0);
+                    evalp(A0, B0);
+                }
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const float2 dx = add2(px, ntx[r]), dy = add2(py, nty[r]), dz = add2(pz, ntz[r]);
-                    const float2 dyz = fma2(dy, dy, fma2(dz, dz, eps2));
-                    float2 r2, rinv, w;
-                    if (TM == TM_CORE) {
-                        r2 = make_float2(fma_sat(dx.x, dx.x, dyz.x), fma_sat(dx.y, dx.y, dyz.y));
-                        rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-                        w = core_weight2(r2, rinv, nmax, tab_bias);
-                        if (!EQM) w = mul2(w, pm);
-                    } else {
-                        r2 = fma2(dx, dx, dyz);
-                        rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-                        const float2 t = TM == TM_LINEAR
-                                             ? make_float2(fma_sat(r2.x, rinv.x, soff), fma_sat(r2.y, rinv.y, soff))
-                                             : fma2(r2, rinv, mhalf);
-                        const float2 Tv = eval_T2<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
-                        // 1/r^3 formed beside the table lookup: two dependent
-                        // multiplies after T instead of four
-                        const float2 ri3 = mul2(mul2(rinv, rinv), rinv);
-                        w = EQM ? mul2(Tv, ri3) : mul2(mul2(pm, Tv), ri3);
-                    }
-                    fx[r] = fma2(w, dx, fx[r]);
-                    fy[r] = fma2(w, dy, fy[r]);
-                    fz[r] = fma2(w, dz, fz[r]);
-                    if (COUNT) {
-                        const float uc = TM == TM_EXACT ? x_c : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
-                        const float ua = TM == TM_CORE ? r2.x : r2.x * rinv.x;
-                        const float ub = TM == TM_CORE ? r2.y : r2.y * rinv.y;
-                        cnt += (act[r] && ua < uc && (dx.x != 0.0f || dy.x != 0.0f || dz.x != 0.0f));
-                        cnt += (act[r] && ub < uc && (dx.y != 0.0f || dy.y != 0.0f || dz.y != 0.0f));
-                    }
+                    float sx = fx[r].x + fx[r].y, sy = fy[r].x + fy[r].y, sz = fz[r].x + fz[r].y;
+                    acc[r].fold(sx, sy, sz);
+                    fx[r] = fy[r] = fz[r] = make_float2(0.0f, 0.0f);
                 }
-            };
-            // Two staged pairs per iteration (k and k + S, then the odd one),
-            // in the order of the plain loop: two independent dependency
-            // chains per lane, as in the scalar kernel.  32-bit shared-window
-            // addresses and volatile loads as there; with one mass the (m0,
-            // m1) half of a pair is not read (a 16-byte broadcast load takes
-            // two cycles of the shared-memory pipe, an 8-byte one takes one).
-            auto load = [&](unsigned p, float4& A, float4& B) {
-                A = lds_f4_v(p);
-                if (EQM) {
-                    const float2 z = lds_f2_v(p + 16u);
-                    B = make_float4(z.x, z.y, 0.0f, 0.0f);
-                } else {
-                    B = lds_f4_v(p + 16u);
-                }
-            };
-            unsigned sa = smem_u32(stage + 2 * s);
-            const unsigned se = smem_u32(stage + 2 * ((nst + 1) >> 1)), st1 = 32u * (unsigned)S;
-            float4 A0, B0, A1, B1;
-#pragma unroll 1
-            for (; sa + st1 < se; sa += 2u * st1) {
-                load(sa, A0, B0);
-                load(sa + st1, A1, B1);
-                evalp(A0, B0);
-                evalp(A1, B1);
             }
-            if (sa < se) {
-                load(sa, A0, B0);
-                evalp(A0, B0);
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                float sx = fx[r].x + fx[r].y, sy = fy[r].x + fy[r].y, sz = fz[r].x + fz[r].y;
-                acc[r].fold(sx, sy, sz);
-                fx[r] = fy[r] = fz[r] = make_float2(0.0f, 0.0f);
-            }
+            __syncwarp();
         }
-        __syncwarp();
+        rw = Work::at(wbox);
+        if (rw.in_turn()) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                acc[r].set(tot.add(3 * r, rw.part(), acc[r].part(0)), tot.add(3 * r + 1, rw.part(), acc[r].part(1)),
+                           tot.add(3 * r + 2, rw.part(), acc[r].part(2)));
+        }
+        if (rw.last()) break;
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = Acc3<ACC>();
+        rw.next(wbox);
     }
-    finish_item<ACC, R>(a, li, acc, act, lane, s, q, S, T,
-                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage, split, wstride);
     if (COUNT) npairs += cnt;
+    finish_item<ACC, R>(a, li, acc, act, lane, s, q, S, T,
+                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage, rw, wstride);
 }
 
 // T for one table coordinate t = u - 1/2 (see eval_T2).
@@ -693,12 +690,12 @@ __device__ __forceinline__ float eval_T1(float t, float r2, float rinv, unsigned
 // f32x2 add of register pairs (the staged (x, y) and the target's
 // (-x_k, -y_k)), the same rounding as two scalar subtractions: one
 // instruction fewer per pair (2 % on the 128^3 launch, 5 % at 96^3).
-template <int TM, int ACC, bool COUNT, bool EQM, int R>
+template <int TM, int ACC, bool COUNT, bool EQM, int R, class Work>
 __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                             float4* __restrict__ stage,
                                             float4* __restrict__ meta, unsigned long long& npairs,
                                             unsigned long long& nev,
-                                            bool split, int wstride)
+                                            Work rw, PartTotals<ACC, 9>& tot, int wstride)
 {
     const int lane = threadIdx.x & 31;
     const float4* __restrict__ pf = reinterpret_cast<const float4*>(a.pf);
@@ -740,76 +737,91 @@ __device__ __forceinline__ void fwd_item_sc(const FwdArgs& a, int I, int4 li, un
     }
     // the target box for the cull (shared memory, after the entry records)
     cull_box(lx, ly, lz, hx, hy, hz, x_c * sc, meta + kMetaPerWarp);
+    unsigned cnt = 0;
+    const float eps2 = kEps2 * sc * sc;
     Acc3<ACC> acc[R];
+    float4* const wbox = meta + kMetaPerWarp;
+    rw.park(wbox);
     float fx[R], fy[R], fz[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) fx[r] = fy[r] = fz[r] = 0.0f;
-    unsigned cnt = 0;
-    long long e0, re;
-    row_part(a, I, split, e0, re);
-    const float eps2 = kEps2 * sc * sc;
-    while (e0 < re) {
-        int nst;
-        e0 += stage_chunk<0>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
-        if (COUNT && lane == 0) nev += (unsigned long long)nst * (unsigned)nI;
-        if (on) {
-            auto eval = [&](const float4 p) {
+    for (;;) {  // the row, or its parts in turn
+        long long e0, re;
+        row_part(a, I, Work::at(wbox), e0, re);
+        while (e0 < re) {
+            int nst;
+            e0 += stage_chunk<0>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
+            if (COUNT && lane == 0) nev += (unsigned long long)nst * (unsigned)nI;
+            if (on) {
+                auto eval = [&](const float4 p) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float2 dxy = add2(make_float2(p.x, p.y), nxy[r]);
-                    const float dx = dxy.x, dy = dxy.y, dz = p.z - xz[r];
-                    const float dyz = fmaf(dy, dy, fmaf(dz, dz, eps2));
-                    const float r2 = TM == TM_CORE ? fma_sat(dx, dx, dyz) : fmaf(dx, dx, dyz);
-                    const float rinv = rsqrt_ftz(r2);
-                    float w;
-                    if (TM == TM_CORE) {
-                        w = core_weight(r2, rinv, nmax, tab_bias);
-                        if (!EQM) w *= p.w;
-                    } else {
-                        const float t = TM == TM_LINEAR ? fma_sat(r2, rinv, soff)
-                                        : TM == TM_FINE ? fmaf(r2 * rinv, tsc, -0.5f)
-                                                        : fmaf(r2, rinv, TM == TM_TAYLOR ? 0.0f : -0.5f);
-                        const float Tv = eval_T1<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
-                        // 1/r^3 formed beside the table lookup (two dependent
-                        // multiplies after T instead of four)
-                        const float ri3 = rinv * rinv * rinv;
-                        w = EQM ? Tv * ri3 : (p.w * Tv) * ri3;
+                    for (int r = 0; r < R; ++r) {
+                        const float2 dxy = add2(make_float2(p.x, p.y), nxy[r]);
+                        const float dx = dxy.x, dy = dxy.y, dz = p.z - xz[r];
+                        const float dyz = fmaf(dy, dy, fmaf(dz, dz, eps2));
+                        const float r2 = TM == TM_CORE ? fma_sat(dx, dx, dyz) : fmaf(dx, dx, dyz);
+                        const float rinv = rsqrt_ftz(r2);
+                        float w;
+                        if (TM == TM_CORE) {
+                            w = core_weight(r2, rinv, nmax, tab_bias);
+                            if (!EQM) w *= p.w;
+                        } else {
+                            const float t = TM == TM_LINEAR ? fma_sat(r2, rinv, soff)
+                                            : TM == TM_FINE ? fmaf(r2 * rinv, tsc, -0.5f)
+                                                            : fmaf(r2, rinv, TM == TM_TAYLOR ? 0.0f : -0.5f);
+                            const float Tv = eval_T1<TM>(t, r2, rinv, tab_bias, nmax, x_c, xscale);
+                            // 1/r^3 formed beside the table lookup (two dependent
+                            // multiplies after T instead of four)
+                            const float ri3 = rinv * rinv * rinv;
+                            w = EQM ? Tv * ri3 : (p.w * Tv) * ri3;
+                        }
+                        fx[r] = fmaf(w, dx, fx[r]);
+                        fy[r] = fmaf(w, dy, fy[r]);
+                        fz[r] = fmaf(w, dz, fz[r]);
+                        if (COUNT) {
+                            const float u = TM == TM_CORE ? r2 : r2 * rinv;
+                            const float uc = TM == TM_EXACT || TM == TM_FINE ? x_c
+                                             : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
+                            cnt += (act[r] && u < uc && (dx != 0.0f || dy != 0.0f || dz != 0.0f));
+                        }
                     }
-                    fx[r] = fmaf(w, dx, fx[r]);
-                    fy[r] = fmaf(w, dy, fy[r]);
-                    fz[r] = fmaf(w, dz, fz[r]);
-                    if (COUNT) {
-                        const float u = TM == TM_CORE ? r2 : r2 * rinv;
-                        const float uc = TM == TM_EXACT || TM == TM_FINE ? x_c
-                                         : TM == TM_LINEAR || TM == TM_CORE ? 1.0f : nmax;
-                        cnt += (act[r] && u < uc && (dx != 0.0f || dy != 0.0f || dz != 0.0f));
-                    }
-                }
-            };
-            // Two sources per iteration (s + 2jS and s + (2j+1)S), then the odd
-            // one: the same order as a plain loop over k = s, s+S, ..., with
-            // half its loop and address instructions (1-3 % faster launches).
-// the loop walks 32-bit shared-window addresses (one integer add per
-            // step; 1.5 % faster than pointer arithmetic on the bench workload);
-            // the loads are volatile so that none moves across the chunk's
-            // staging stores
-            unsigned sa = smem_u32(stage + s);
-            const unsigned se = smem_u32(stage + nst), st1 = 16u * (unsigned)S;
+                };
+                // Two sources per iteration (s + 2jS and s + (2j+1)S), then the odd
+                // one: the same order as a plain loop over k = s, s+S, ..., with
+                // half its loop and address instructions (1-3 % faster launches).
+                // the loop walks 32-bit shared-window addresses (one integer add per
+                // step; 1.5 % faster than pointer arithmetic on the bench workload);
+                // the loads are volatile so that none moves across the chunk's
+                // staging stores
+                unsigned sa = smem_u32(stage + s);
+                const unsigned se = smem_u32(stage + nst), st1 = 16u * (unsigned)S;
 #pragma unroll 1
-            for (; sa + st1 < se; sa += 2u * st1) {
-                const float4 p0 = lds_f4_v(sa), p1 = lds_f4_v(sa + st1);
-                eval(p0);
-                eval(p1);
-            }
-            if (sa < se) eval(lds_f4_v(sa));
+                for (; sa + st1 < se; sa += 2u * st1) {
+                    const float4 p0 = lds_f4_v(sa), p1 = lds_f4_v(sa + st1);
+                    eval(p0);
+                    eval(p1);
+                }
+                if (sa < se) eval(lds_f4_v(sa));
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r].fold(fx[r], fy[r], fz[r]);
+                for (int r = 0; r < R; ++r) acc[r].fold(fx[r], fy[r], fz[r]);
+            }
+            __syncwarp();
         }
-        __syncwarp();
+        rw = Work::at(wbox);
+        if (rw.in_turn()) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                acc[r].set(tot.add(3 * r, rw.part(), acc[r].part(0)), tot.add(3 * r + 1, rw.part(), acc[r].part(1)),
+                           tot.add(3 * r + 2, rw.part(), acc[r].part(2)));
+        }
+        if (rw.last()) break;
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = Acc3<ACC>();
+        rw.next(wbox);
     }
-    finish_item<ACC, R>(a, li, acc, act, lane, s, q, S, T,
-                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage, split, wstride);
     if (COUNT) npairs += cnt;
+    finish_item<ACC, R>(a, li, acc, act, lane, s, q, S, T,
+                        bx.g_acc * sc * sc * (EQM ? bx.m_eq : 1.0f), stage, rw, wstride);
 }
 
 // Lane-slot efficiency of R targets per lane: n_I * floor(32 / ceil(n_I/R)) / (32 R)
@@ -823,8 +835,8 @@ __device__ __forceinline__ bool prefer_two_per_lane(int n)
 }
 
 // Shared memory: the table, then one staging buffer of stage_cap particles
-// plus 32 entry records per warp.
-template <int TM, int ACC, bool COUNT, bool PK, bool EQM, bool SPLIT>
+// plus 32 entry records and the two box slots per warp.
+template <int TM, int ACC, bool COUNT, bool PK, bool EQM, int ROWS>
 __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -832,8 +844,8 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
     const int warp = threadIdx.x >> 5;
     const unsigned esize = TM == TM_TAYLOR ? 32u : TM == TM_CUBIC || TM == TM_FINE ? 16u : 8u;
     const size_t tab_bytes = TM == TM_EXACT ? 0 : (size_t)(a.table_n + 1) * esize;
-    float4* stage = reinterpret_cast<float4*>(smem + ((tab_bytes + 15) & ~(size_t)15)) +
-                    (size_t)warp * (a.stage_cap + kWarpMeta);
+    const int wstride = a.stage_cap + kWarpMeta;
+    float4* stage = reinterpret_cast<float4*>(smem + ((tab_bytes + 15) & ~(size_t)15)) + (size_t)warp * wstride;
     float4* meta = stage + a.stage_cap;
     if (TM == TM_TAYLOR) {
         const float4* g = reinterpret_cast<const float4*>(a.table);
@@ -861,11 +873,10 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
     const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
     unsigned long long npairs = 0, nev = 0;
     __shared__ int s_it[8];
-    const int wstride = a.stage_cap + kWarpMeta;
-    const int n_heavy = !SPLIT ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
-    bool split = SPLIT && n_heavy > 0;
+    const int n_heavy = ROWS != kRowsJoint ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    bool split = n_heavy > 0;
     int it;
-    while (next_item<SPLIT>(a, a.ctrl + kCtrlTicketFwd, split, n_heavy, s_it, it)) {
+    while (next_item<ROWS>(a, a.ctrl + kCtrlTicketFwd, split, n_heavy, s_it, it)) {
         int I = a.items[it];
         if (I < 0 || I >= a.n_leaves) {
             if (lane == 0) set_error(a.ctrl, kErrItemIndex);
@@ -877,6 +888,8 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
             if (lane == 0) set_error(a.ctrl, kErrParticleRange);
             continue;
         }
+        const auto rw = row_work<ROWS>(a, I, li.z, split);
+        PartTotals<ACC, 9> tot;  // kRowsInTurn
         if (PK) {
             // packed pairs where one target per lane fills the lanes as well
             // as any R; elsewhere the scalar two- or three-targets paths,
@@ -885,19 +898,19 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
             // on the bench workload)
             const int R = targets_per_lane(li.y, a.stage_cap);
             if (R == 1)
-                fwd_item_pk<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
+                fwd_item_pk<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev, rw, tot, wstride);
             else if (R == 3)
-                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev, rw, tot, wstride);
             else
-                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev, rw, tot, wstride);
         } else {
             const int R = targets_per_lane(li.y, a.stage_cap);
             if (R == 3)
-                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 3>(a, I, li, tab_bias, stage, meta, npairs, nev, rw, tot, wstride);
             else if (R == 2)
-                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 2>(a, I, li, tab_bias, stage, meta, npairs, nev, rw, tot, wstride);
             else
-                fwd_item_sc<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev, SPLIT && split, wstride);
+                fwd_item_sc<TM, ACC, COUNT, EQM, 1>(a, I, li, tab_bias, stage, meta, npairs, nev, rw, tot, wstride);
         }
     }
     if (COUNT) {
@@ -912,13 +925,13 @@ __global__ void __launch_bounds__(256, 4) p2p_fwd_f32_kernel(const FwdArgs a)
 
 // Launch and occupancy of the variant PK (explicitly instantiated in
 // p2p_fwd_f32_sc.cu and p2p_fwd_f32_pk.cu).
-template <int TM, int ACC, bool COUNT, bool PK, bool EQM, bool SPLIT>
+template <int TM, int ACC, bool COUNT, bool PK, bool EQM, int ROWS>
 static int launch_t(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
     // Both variants carry the scalar two- and three-targets-per-lane paths
     // (targets_per_lane picks per leaf; the packed variant runs its f32x2
     // loop for the leaves that take one target per lane).
-    auto k = p2p_fwd_f32_kernel<TM, ACC, COUNT, PK, EQM, SPLIT>;
+    auto k = p2p_fwd_f32_kernel<TM, ACC, COUNT, PK, EQM, ROWS>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
@@ -927,58 +940,58 @@ static int launch_t(const FwdArgs& a, size_t smem, cudaStream_t st)
     return (int)cudaGetLastError();
 }
 
-template <int TM, int ACC, bool PK, bool SPLIT>
+template <int TM, int ACC, bool PK, int ROWS>
 static int launch_s(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
     // equal masses: the mass leaves the pair sum (the pair-counting launch,
     // untimed, keeps the general form)
-    return a.count_pairs  ? launch_t<TM, ACC, true, PK, false, SPLIT>(a, smem, st)
-           : a.equal_mass ? launch_t<TM, ACC, false, PK, true, SPLIT>(a, smem, st)
-                          : launch_t<TM, ACC, false, PK, false, SPLIT>(a, smem, st);
+    return a.count_pairs  ? launch_t<TM, ACC, true, PK, false, ROWS>(a, smem, st)
+           : a.equal_mass ? launch_t<TM, ACC, false, PK, true, ROWS>(a, smem, st)
+                          : launch_t<TM, ACC, false, PK, false, ROWS>(a, smem, st);
 }
 
-template <bool PK, bool SPLIT>
+template <bool PK, int ROWS>
 static int launch_fwd_f32_t(const FwdArgs& a, int precision, size_t smem, cudaStream_t st)
 {
     if constexpr (!PK)
         if (a.fine)
-            return a.accum == PSR_ACC_FP64 ? launch_s<TM_FINE, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
-                                           : launch_s<TM_FINE, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
+            return a.accum == PSR_ACC_FP64 ? launch_s<TM_FINE, PSR_ACC_FP64, PK, ROWS>(a, smem, st)
+                                           : launch_s<TM_FINE, PSR_ACC_KAHAN32, PK, ROWS>(a, smem, st);
     if (precision == PSR_FP32_EXACT)
-        return a.accum == PSR_ACC_FP64 ? launch_s<TM_EXACT, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
-                                       : launch_s<TM_EXACT, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_EXACT, PSR_ACC_FP64, PK, ROWS>(a, smem, st)
+                                       : launch_s<TM_EXACT, PSR_ACC_KAHAN32, PK, ROWS>(a, smem, st);
     if (a.interp == PSR_LINEAR)
-        return a.accum == PSR_ACC_FP64 ? launch_s<TM_LINEAR, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
-                                       : launch_s<TM_LINEAR, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_LINEAR, PSR_ACC_FP64, PK, ROWS>(a, smem, st)
+                                       : launch_s<TM_LINEAR, PSR_ACC_KAHAN32, PK, ROWS>(a, smem, st);
     if (a.interp == PSR_TAYLOR2 || a.interp == PSR_TAYLOR4)
-        return a.accum == PSR_ACC_FP64 ? launch_s<TM_TAYLOR, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
-                                       : launch_s<TM_TAYLOR, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
-    return a.accum == PSR_ACC_FP64 ? launch_s<TM_CUBIC, PSR_ACC_FP64, PK, SPLIT>(a, smem, st)
-                                   : launch_s<TM_CUBIC, PSR_ACC_KAHAN32, PK, SPLIT>(a, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_TAYLOR, PSR_ACC_FP64, PK, ROWS>(a, smem, st)
+                                       : launch_s<TM_TAYLOR, PSR_ACC_KAHAN32, PK, ROWS>(a, smem, st);
+    return a.accum == PSR_ACC_FP64 ? launch_s<TM_CUBIC, PSR_ACC_FP64, PK, ROWS>(a, smem, st)
+                                   : launch_s<TM_CUBIC, PSR_ACC_KAHAN32, PK, ROWS>(a, smem, st);
 }
 
-// One translation unit each: <PK, SPLIT> = <false, false>, <true, false>,
+// One translation unit each: <PK, ROWS> = <false, false>, <true, false>,
 // <false, true>, <true, true> (the last only for the core form).  Launches
 // without heavy items (most large sets) keep the kernel without the block
 // phase, whose registers cost 1-3 % of a launch.
-template <bool PK, bool SPLIT>
+template <bool PK, int ROWS>
 int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStream_t st)
 {
     if (PK && a.core)
-        return a.accum == PSR_ACC_FP64 ? launch_s<TM_CORE, PSR_ACC_FP64, true, SPLIT>(a, smem, st)
-                                       : launch_s<TM_CORE, PSR_ACC_KAHAN32, true, SPLIT>(a, smem, st);
-    if constexpr (!(PK && SPLIT))
-        return launch_fwd_f32_t<PK, SPLIT>(a, precision, smem, st);
+        return a.accum == PSR_ACC_FP64 ? launch_s<TM_CORE, PSR_ACC_FP64, true, ROWS>(a, smem, st)
+                                       : launch_s<TM_CORE, PSR_ACC_KAHAN32, true, ROWS>(a, smem, st);
+    if constexpr (!PK || ROWS == kRowsWhole)
+        return launch_fwd_f32_t<PK, ROWS>(a, precision, smem, st);
     else
-        return (int)cudaErrorInvalidValue;  // not reached: only the core form is split on packed pairs
+        return (int)cudaErrorInvalidValue;  // not reached: only the core form has parts on packed pairs
 }
 
 
 template <bool PK>
 const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int core)
 {
-#define PSR_PICK_PK(ACC) ((const void*)p2p_fwd_f32_kernel<TM_CORE, ACC, false, true, false, false>)
-#define PSR_PICK(TM, ACC) ((const void*)p2p_fwd_f32_kernel<TM, ACC, false, PK, false, false>)
+#define PSR_PICK_PK(ACC) ((const void*)p2p_fwd_f32_kernel<TM_CORE, ACC, false, true, false, kRowsWhole>)
+#define PSR_PICK(TM, ACC) ((const void*)p2p_fwd_f32_kernel<TM, ACC, false, PK, false, kRowsWhole>)
     if (precision == PSR_FP32_EXACT)
         return accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
     if (PK && core)

@@ -100,16 +100,201 @@ __device__ __forceinline__ void group_sync(int warps)
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(32 * warps) : "memory");
 }
 
-// This warp's entries of a row: all of them, or with split its share among
-// the warps of its group.
-__device__ __forceinline__ void row_part(const FwdArgs& a, int I, bool split, long long& e0, long long& re)
+// How a row's sums are formed: over `parts` consecutive parts of its entries, each
+// by itself from zero, added in order lane by lane.  Which rows have parts, and how
+// many, is fixed by the row and its box alone (parts_rule), so that neither the
+// other boxes, the launch's shape nor its shard move a bit of the result.  Who
+// forms them is the launch's choice (FwdArgs::rows), and each choice has kernel
+// instances of its own.  The FP32 pair loops have no register to spare, so what an
+// item needs to know after its pair loop waits in one word of shared memory, the
+// unused last word of the warp's target box.
+__device__ __forceinline__ volatile unsigned* row_word(float4* box)
 {
+    return reinterpret_cast<volatile unsigned*>(box) + 7;
+}
+
+// no row has parts
+struct WholeRow {
+    __device__ __forceinline__ void park(float4*) const {}
+    __device__ static __forceinline__ WholeRow at(float4*) { return WholeRow{}; }
+    __device__ static constexpr bool joint() { return false; }
+    __device__ static constexpr bool in_turn() { return false; }
+    __device__ static constexpr int parts() { return 1; }
+    __device__ static constexpr int part() { return 0; }
+    __device__ static __forceinline__ int leaf(int I) { return I; }
+    __device__ static constexpr bool last() { return true; }
+    __device__ __forceinline__ void next(float4*) {}
+};
+// the warps of a group side by side, one part each (at least as many warps as
+// parts); rows without parts also by single warps
+struct JointRow {
+    unsigned v;  // parts | warp << 4 | joint << 8
+    __device__ __forceinline__ void park(float4* box) const
+    {
+        if ((threadIdx.x & 31) == 0) *row_word(box) = v;
+        __syncwarp();
+    }
+    __device__ static __forceinline__ JointRow at(float4* box) { return JointRow{*row_word(box)}; }
+    __device__ __forceinline__ bool joint() const { return v >> 8; }
+    __device__ static constexpr bool in_turn() { return false; }
+    __device__ __forceinline__ int parts() const { return (int)(v & 15u); }
+    __device__ __forceinline__ int part() const { return (int)((v >> 4) & 15u); }
+    __device__ static __forceinline__ int leaf(int I) { return I; }
+    __device__ static constexpr bool last() { return true; }
+    __device__ __forceinline__ void next(float4*) {}
+};
+// one warp all parts in turn
+struct TurnRow {
+    unsigned v;  // leaf << 5 | log2(parts) << 3 | part
+    __device__ __forceinline__ void park(float4* box) const
+    {
+        if ((threadIdx.x & 31) == 0) *row_word(box) = v;
+        __syncwarp();
+    }
+    __device__ static __forceinline__ TurnRow at(float4* box) { return TurnRow{*row_word(box)}; }
+    __device__ static constexpr bool joint() { return false; }
+    __device__ __forceinline__ bool in_turn() const { return v & 24u; }
+    __device__ __forceinline__ int parts() const { return 1 << ((v >> 3) & 3u); }
+    __device__ __forceinline__ int part() const { return (int)(v & 7u); }
+    __device__ __forceinline__ int leaf(int) const { return (int)(v >> 5); }
+    __device__ __forceinline__ bool last() const { return part() + 1 >= parts(); }
+    __device__ __forceinline__ void next(float4* box)
+    {
+        ++v;
+        __syncwarp();
+        park(box);
+    }
+};
+
+template <int ROWS>
+__device__ __forceinline__ auto row_work(const FwdArgs& a, int I, int box, bool split)
+{
+    if constexpr (ROWS == kRowsWhole) {
+        return WholeRow{};
+    } else {
+        const BoxDev& bx = a.boxes[box];
+        int parts = a.cost[I] > bx.above[a.kind] ? bx.parts[a.kind] : 1;
+        if (parts < 1 || parts > (ROWS == kRowsInTurn ? 8 : split ? a.group : 1)) {
+            set_error(a.ctrl, kErrParts);
+            parts = 1;
+        }
+        if constexpr (ROWS == kRowsJoint)
+            return JointRow{split ? (unsigned)(parts | (int)(threadIdx.x >> 5) % a.group << 4 | 256) : (unsigned)parts};
+        else
+            return TurnRow{(unsigned)I << 5 | (unsigned)(31 - __clz(parts)) << 3};
+    }
+}
+
+// The entries of this warp's present part of a row.
+template <class Work>
+__device__ __forceinline__ void row_part(const FwdArgs& a, int I, const Work& w, long long& e0, long long& re)
+{
+    I = w.leaf(I);
     e0 = a.rowptr[I];
     re = a.rowptr[I + 1];
-    if (split) {
-        const int len = (int)(re - e0), W = a.group, w = (threadIdx.x >> 5) % W;
-        re = e0 + (long long)len * (w + 1) / W;
-        e0 += (long long)len * w / W;
+    if (w.joint() || w.in_turn()) {
+        const int len = (int)(re - e0), part = w.part(), parts = w.parts();
+        re = part < parts ? e0 + (long long)len * (part + 1) / parts : e0;
+        e0 += part < parts ? (long long)len * part / parts : 0;
+    }
+}
+
+// A sum over parts, and the 8-byte word it is kept in: FP64, or a compensated
+// FP32 pair.
+template <int ACC>
+struct PartSum {
+    double v = 0.0;
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void load(const volatile char* p)
+    {
+        if (ACC == PSR_ACC_FP64) {
+            v = *reinterpret_cast<const volatile double*>(p);
+        } else {
+            hi = reinterpret_cast<const volatile float*>(p)[0];
+            lo = reinterpret_cast<const volatile float*>(p)[1];
+        }
+    }
+    __device__ __forceinline__ void add(const PartSum& o)
+    {
+        if (ACC == PSR_ACC_FP64) {
+            v += o.v;
+        } else {
+            float s, e;
+            two_sum(hi, o.hi, s, e);
+            hi = s;
+            lo += o.lo + e;
+        }
+    }
+    __device__ __forceinline__ float scaled(float g) const
+    {
+        return ACC == PSR_ACC_FP64 ? (float)(v * (double)g) : (hi + lo) * g;
+    }
+};
+
+// The sums of the parts that one warp has formed so far.  In local memory, by
+// volatile accesses: they are touched once a part, and in registers they push the
+// pair loop's values out (batch of 64 boxes 7.01 -> 6.76 ms).
+template <int ACC, int N>
+struct PartTotals {
+    volatile double v[ACC == PSR_ACC_FP64 ? N : 1];
+    volatile float hi[ACC == PSR_ACC_FP64 ? 1 : N], lo[ACC == PSR_ACC_FP64 ? 1 : N];
+    __device__ __forceinline__ PartSum<ACC> get(int i) const
+    {
+        PartSum<ACC> p;
+        if (ACC == PSR_ACC_FP64) {
+            p.v = v[i];
+        } else {
+            p.hi = hi[i];
+            p.lo = lo[i];
+        }
+        return p;
+    }
+    __device__ __forceinline__ void put(int i, const PartSum<ACC>& p)
+    {
+        if (ACC == PSR_ACC_FP64) {
+            v[i] = p.v;
+        } else {
+            hi[i] = p.hi;
+            lo[i] = p.lo;
+        }
+    }
+    // adds p to sum i (part 0: to zero) and returns it
+    __device__ __forceinline__ PartSum<ACC> add(int i, int part, const PartSum<ACC>& p)
+    {
+        PartSum<ACC> t;
+        if (part) t = get(i);
+        t.add(p);
+        put(i, t);
+        return t;
+    }
+};
+
+// End of a row that a group of warps shares: every lane of every warp has left the
+// sums of its part (NC words a target; word(t, s, i): the byte offset of target t's
+// component i in stream s) in the warp's region, `stride` bytes apart, `base` this
+// warp's.  One thread a target and component adds each lane's over the parts, then
+// the S streams, in the order in which one warp adds them, and hands the sum to
+// write(t, i, sum).  next_item's barrier frees the regions.
+template <int NC, int ACC, class Work, class Word, class Write>
+__device__ __forceinline__ void join_parts(const FwdArgs& a, const Work& w, int n_targets, int S, const char* base,
+                                           int stride, Word word, Write write)
+{
+    group_sync(a.group);
+    const int gw = (int)(threadIdx.x >> 5) % a.group;
+    base -= gw * stride;
+    for (int u = 32 * gw + (int)(threadIdx.x & 31); u < NC * n_targets; u += 32 * a.group) {
+        const int t = u / NC, i = u - NC * t;
+        PartSum<ACC> sum;
+        for (int s = 0; s < S; ++s) {
+            PartSum<ACC> lane, part;
+            for (int k = 0; k < w.parts(); ++k) {
+                part.load(base + k * stride + word(t, s, i));
+                lane.add(part);
+            }
+            if (s) sum.add(lane);
+            else sum = lane;
+        }
+        write(t, i, sum);
     }
 }
 
@@ -118,14 +303,12 @@ __device__ __forceinline__ void row_part(const FwdArgs& a, int I, bool split, lo
 // see heavy_cost) are taken by groups of a.group warps, one ticket a group
 // (split stays true; s_it: one word per group), the rest by single warps; the
 // ticket on which a group leaves the first phase goes to its first warp.
-// Returns false when no item is left.  Which items are split, and how, is
-// fixed by the schedule alone, so results do not depend on the order in which
-// blocks run.
-template <bool SPLIT>
+// Returns false when no item is left.
+template <int ROWS>
 __device__ __forceinline__ bool next_item(const FwdArgs& a, unsigned* ticket, bool& split,
                                           int n_heavy, volatile int* s_it, int& it)
 {
-    if (SPLIT && split) {
+    if (ROWS == kRowsJoint && split) {
         const int g = (threadIdx.x >> 5) / a.group;
         const bool first = threadIdx.x - g * 32 * a.group < 32;
         group_sync(a.group);  // the group's last item is combined

@@ -92,6 +92,20 @@ struct Acc4 {
             f[i] = 0.0f;
         }
     }
+    __device__ __forceinline__ PartSum<ACC> part(int i) const
+    {
+        PartSum<ACC> p;
+        p.v = d[i];
+        p.hi = s[i];
+        p.lo = c[i];
+        return p;
+    }
+    __device__ __forceinline__ void set(int i, const PartSum<ACC>& p)
+    {
+        d[i] = p.v;
+        s[i] = p.hi;
+        c[i] = p.lo;
+    }
 };
 
 // Writes one target's gradients from its four sums.
@@ -105,55 +119,34 @@ __device__ __forceinline__ void adj_write(const FwdArgs& a, int target, const fl
     if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = v[3];
 }
 
-// The target sums that the group's warps left (base: this warp's, wstride
-// float4 per warp),
-// four 8-byte words (an FP64 sum, or a compensated FP32 pair) per target
-// at off + target slot, added over the warps in order and written.  word(t, i)
-// is the byte offset of target t's component i from a warp's base.
-template <int ACC, class Word>
-__device__ __forceinline__ void adj_combine(const FwdArgs& a, int4 li, const float4* base, int wstride,
-                                            float gx, float gm, Word word)
+// A warp's region in float4: staging buffer, entry records and box slots, then the
+// accumulator block of the two-targets path.
+constexpr int kAdjAccF4 = 128;  // accumulator block per warp: 2 targets x 4 x 32 lanes x 8 B
+__device__ __forceinline__ int adj_acc_f4(const FwdArgs& a) { return 2 * a.stage_cap + kWarpMeta; }
+
+template <int ACC, class Work, class Word>
+__device__ __forceinline__ void adj_join(const FwdArgs& a, int4 li, const Work& rw, int S, const float4* stage,
+                                         int wstride, float gx, float gm, Word word)
 {
-    group_sync(a.group);
-    const int nw = a.group, gw = (threadIdx.x >> 5) % nw;
-    base -= gw * wstride;
-    for (int t = 32 * gw + (threadIdx.x & 31); t < li.y; t += 32 * nw) {
-        float v[4];
-        for (int i = 0; i < 4; ++i) {
-            const float g = i < 3 ? gx : gm;
-            const unsigned off = word(t, i);
-            if (ACC == PSR_ACC_FP64) {
-                double sum = 0.0;
-                for (int w = 0; w < nw; ++w)
-                    sum += *reinterpret_cast<const volatile double*>(
-                        reinterpret_cast<const char*>(base + w * wstride) + off);
-                v[i] = (float)(sum * (double)g);
-            } else {
-                float hi = 0.0f, lo = 0.0f, u, e;
-                for (int w = 0; w < nw; ++w) {
-                    const volatile float* o = reinterpret_cast<const volatile float*>(
-                        reinterpret_cast<const char*>(base + w * wstride) + off);
-                    two_sum(hi, o[0], u, e);
-                    hi = u;
-                    lo += o[1] + e;
-                }
-                v[i] = (hi + lo) * g;
-            }
-        }
-        adj_write(a, li.x + t, v);
-    }
+    join_parts<4, ACC>(a, rw, li.y, S, reinterpret_cast<const char*>(stage), 16 * wstride, word,
+                       [&](int t, int i, const PartSum<ACC>& s) {
+                           const int idx = a.perm[li.x + t];
+                           if (i < 3) reinterpret_cast<float*>(a.out)[3LL * idx + i] = s.scaled(gx);
+                           else if (a.out_m) reinterpret_cast<float*>(a.out_m)[idx] = s.scaled(gm);
+                       });
 }
 
 // Combine the S stream partials of each target and write dL/dx (scaled by
 // gx = G/(8 r_s^3) sc^3) and dL/dm (gm = -G/(4 r_s^2) sc^2) in the original
-// order; with split, each warp's sums cover its part of the row and the
-// group's are combined after that.
-template <int ACC, int R>
+// order; in a row that a group of warps shares each has the sums of its part
+// (join_parts).
+template <int ACC, int R, class Work>
 __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>* acc,
                                            const bool* act, int lane, int s, int q, int S, int T,
-                                           float gx, float gm, float4* __restrict__ stage, bool split,
-                                           int wstride)
+                                           float gx, float gm, float4* __restrict__ stage,
+                                           const Work& rw, int wstride)
 {
+    const bool joint = rw.joint();
     // Combine the S stream partials through the staging buffer: each target
     // slot r has its own region (1 KB) and the accesses are volatile, so no
     // slot's writes can meet another slot's reads whatever the compiler's
@@ -166,19 +159,14 @@ __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>*
 #pragma unroll
             for (int i = 0; i < 4; ++i) red[4 * lane + i] = acc[r].d[i];
             __syncwarp();
-            if (s == 0 && act[r]) {
+            if (!joint && s == 0 && act[r]) {
                 double t4[4] = {acc[r].d[0], acc[r].d[1], acc[r].d[2], acc[r].d[3]};
                 for (int t = 1; t < S; ++t)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) t4[i] += red[4 * (lane + t * T) + i];
-                if (split) {  // streams t >= 1 sit above the first T entries
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) red[4 * lane + i] = t4[i];
-                } else {
-                    const float v[4] = {(float)(t4[0] * (double)gx), (float)(t4[1] * (double)gx),
-                                        (float)(t4[2] * (double)gx), (float)(t4[3] * (double)gm)};
-                    adj_write(a, li.x + q + T * r, v);
-                }
+                const float v[4] = {(float)(t4[0] * (double)gx), (float)(t4[1] * (double)gx),
+                                    (float)(t4[2] * (double)gx), (float)(t4[3] * (double)gm)};
+                adj_write(a, li.x + q + T * r, v);
             }
         } else {
             volatile float* red = reinterpret_cast<volatile float*>(stage) + 256 * r;
@@ -188,7 +176,7 @@ __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>*
                 red[8 * lane + 2 * i + 1] = acc[r].c[i];
             }
             __syncwarp();
-            if (s == 0 && act[r]) {
+            if (!joint && s == 0 && act[r]) {
                 float hi[4], lo[4], u, v;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -203,25 +191,16 @@ __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>*
                         hi[i] = u;
                         lo[i] += o[1] + v;
                     }
-                if (split) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        red[8 * lane + 2 * i] = hi[i];
-                        red[8 * lane + 2 * i + 1] = lo[i];
-                    }
-                } else {
-                    const float v4[4] = {(hi[0] + lo[0]) * gx, (hi[1] + lo[1]) * gx,
-                                         (hi[2] + lo[2]) * gx, (hi[3] + lo[3]) * gm};
-                    adj_write(a, li.x + q + T * r, v4);
-                }
+                const float v4[4] = {(hi[0] + lo[0]) * gx, (hi[1] + lo[1]) * gx,
+                                     (hi[2] + lo[2]) * gx, (hi[3] + lo[3]) * gm};
+                adj_write(a, li.x + q + T * r, v4);
             }
         }
         __syncwarp();
     }
-    if (split)
-        adj_combine<ACC>(a, li, stage, wstride, gx, gm, [T](int t, int i) {
-            return (unsigned)(1024 * (t / T) + 32 * (t % T) + 8 * i);
-        });
+    if (joint)
+        adj_join<ACC>(a, li, rw, S, stage, wstride, gx, gm,
+                      [T](int t, int s, int i) { return 1024 * (t / T) + 32 * (t % T + s * T) + 8 * i; });
 }
 
 // Running sums of the two-targets-per-lane path in shared memory: the
@@ -233,8 +212,6 @@ __device__ __forceinline__ void adj_finish(const FwdArgs& a, int4 li, Acc4<ACC>*
 // warp's access to one slot is one conflict-free 256-byte row): one double,
 // or the compensated pair (sum, compensation).  The accesses are volatile so
 // that none is merged with or moved across another.
-constexpr int kAdjAccF4 = 128;  // accumulator block per warp (float4): 2 targets x 4 x 32 lanes x 8 B
-
 __device__ __forceinline__ unsigned acc_slot(unsigned base, int r, int i, int lane)
 {
     return base + 256u * (unsigned)(4 * r + i) + 8u * (unsigned)lane;
@@ -291,19 +268,41 @@ __device__ __forceinline__ void acc_fold_all(unsigned base, int lane, float (*f)
         }
 }
 
+// adds a part's sums, the lane's slots, to the totals and leaves those in the slots
+template <int ACC, int R>
+__device__ __forceinline__ void acc_take_all(unsigned base, int lane, int part, PartTotals<ACC, 8>& tot)
+{
+#pragma unroll
+    for (int k = 0; k < 4 * R; ++k) {
+        const unsigned a = acc_slot(base, k / 4, k % 4, lane);
+        PartSum<ACC> p;
+        if (ACC == PSR_ACC_FP64) {
+            p.v = acc_ld_f64(a);
+        } else {
+            const float2 v = acc_ld_f2(a);
+            p.hi = v.x;
+            p.lo = v.y;
+        }
+        p = tot.add(k, part, p);
+        if (ACC == PSR_ACC_FP64) asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(p.v) : "memory");
+        else asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(p.hi), "f"(p.lo) : "memory");
+    }
+}
+
 // adj_finish for sums kept in shared memory: the S stream partials of each
 // target are the slots of lanes q, q + T, ..., q + (S-1) T, combined in that
 // order (the order of adj_finish).
-template <int ACC, int R>
+template <int ACC, int R, class Work>
 __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsigned accb,
                                                 const bool* act, int lane, int s, int q, int S,
-                                                int T, float gx, float gm, const float4* acc0, bool split,
-                                                int wstride)
+                                                int T, float gx, float gm, float4* stage,
+                                                const Work& rw, int wstride)
 {
+    const bool joint = rw.joint();
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        if (s != 0 || !act[r]) continue;
+        if (joint || s != 0 || !act[r]) continue;
         if (ACC == PSR_ACC_FP64) {
             double t4[4];
 #pragma unroll
@@ -311,16 +310,9 @@ __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsig
             for (int t = 1; t < S; ++t)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) t4[i] += acc_ld_f64(acc_slot(accb, r, i, lane + t * T));
-            if (split) {  // the sums go to the slots of lane q
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    asm volatile("st.shared.f64 [%0], %1;" ::"r"(acc_slot(accb, r, i, lane)), "d"(t4[i])
-                                 : "memory");
-            } else {
-                const float v[4] = {(float)(t4[0] * (double)gx), (float)(t4[1] * (double)gx),
-                                    (float)(t4[2] * (double)gx), (float)(t4[3] * (double)gm)};
-                adj_write(a, li.x + q + T * r, v);
-            }
+            const float v[4] = {(float)(t4[0] * (double)gx), (float)(t4[1] * (double)gx),
+                                (float)(t4[2] * (double)gx), (float)(t4[3] * (double)gm)};
+            adj_write(a, li.x + q + T * r, v);
         } else {
             float hi[4], lo[4], u, v;
 #pragma unroll
@@ -337,23 +329,15 @@ __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsig
                     hi[i] = u;
                     lo[i] += w.y + v;
                 }
-            if (split) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(acc_slot(accb, r, i, lane)),
-                                 "f"(hi[i]), "f"(lo[i])
-                                 : "memory");
-            } else {
-                const float v4[4] = {(hi[0] + lo[0]) * gx, (hi[1] + lo[1]) * gx, (hi[2] + lo[2]) * gx,
-                                     (hi[3] + lo[3]) * gm};
-                adj_write(a, li.x + q + T * r, v4);
-            }
+            const float v4[4] = {(hi[0] + lo[0]) * gx, (hi[1] + lo[1]) * gx, (hi[2] + lo[2]) * gx,
+                                 (hi[3] + lo[3]) * gm};
+            adj_write(a, li.x + q + T * r, v4);
         }
     }
     __syncwarp();
-    if (split)
-        adj_combine<ACC>(a, li, acc0, wstride, gx, gm, [T](int t, int i) {
-            return (unsigned)(256 * (4 * (t / T) + i) + 8 * (t % T));
+    if (joint)
+        adj_join<ACC>(a, li, rw, S, stage, wstride, gx, gm, [T, off = 16 * adj_acc_f4(a)](int t, int s, int i) {
+            return off + 256 * (4 * (t / T) + i) + 8 * (t % T + s * T);
         });
 }
 
@@ -365,11 +349,11 @@ __device__ __forceinline__ void adj_finish_smem(const FwdArgs& a, int4 li, unsig
 // same rounding.  The rest of the pair stays scalar, where it spreads over
 // both halves of the FMA pipe (f32x2 runs on one).  With two targets per
 // lane the running sums live in shared memory (acc_fold_all).
-template <int TM, int ACC, bool EQM, int R>
+template <int TM, int ACC, bool EQM, int R, class Work>
 __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                          unsigned q_off, float4* __restrict__ stage,
-                                         float4* __restrict__ meta, unsigned accb, bool split,
-                                         int wstride)
+                                         float4* __restrict__ meta, unsigned accb, Work rw,
+                                         PartTotals<ACC, 8>& tot, int wstride)
 {
     constexpr bool SA = R == 2;  // sums in shared memory
     const int lane = threadIdx.x & 31;
@@ -400,8 +384,6 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
     float nckz[R];
     bool act[R];
     float f[R][4];
-    Acc4<ACC> acc[SA ? 1 : R];
-    if (SA) acc_zero_all<R>(accb, lane);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int t = q + T * r;
@@ -429,101 +411,122 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
             }
         cull_box(lx, ly, lz, hx, hy, hz, x_c * sc, meta + kMetaPerWarp);
     }
-    long long e0, re;
-    row_part(a, I, split, e0, re);
-    while (e0 < re) {
-        int nst;
-        e0 += stage_chunk<2>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
-        if (on) {
-            // p = (x, y, z, c_z), c = (c_x, c_y, m, m) of one staged source
-            auto eval = [&](const float4 p, const float4 c) {
+    Acc4<ACC> acc[SA ? 1 : R];
+    float4* const wbox = meta + kMetaPerWarp;
+    rw.park(wbox);
+    if (SA) acc_zero_all<R>(accb, lane);
+    for (;;) {  // the row, or its parts in turn
+        long long e0, re;
+        row_part(a, I, Work::at(wbox), e0, re);
+        while (e0 < re) {
+            int nst;
+            e0 += stage_chunk<2>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
+            if (on) {
+                // p = (x, y, z, c_z), c = (c_x, c_y, m, m) of one staged source
+                auto eval = [&](const float4 p, const float4 c) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float2 dxy = add2(make_float2(p.x, p.y), nxy[r]);
-                    const float dx = dxy.x, dy = dxy.y, dz = p.z - xi[r].z;
-                    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    // the self pair and coincident pairs contribute nothing:
-                    // on the linear path the NaN coordinate at r = 0 selects
-                    // the zero entry (T = Q = 0) and the clamped 1/r keeps
-                    // every product finite; elsewhere 1/r = 0 makes tr3 and
-                    // hh zero (T and Q stay finite)
-                    float rinv, tv;
-                    if (TM == TM_LINEAR) {
-                        const float ri = rsqrt_ftz(r2);
-                        tv = fma_sat(r2, -ri, sref);
-                        rinv = fminf(ri, kRinvMax);
-                    } else {
-                        rinv = r2 > 0.0f ? rsqrt_ftz(r2) : 0.0f;
-                        tv = TM == TM_FINE ? fmaf(r2 * rinv, tsc, -0.5f) : fmaf(r2, rinv, -0.5f);
+                    for (int r = 0; r < R; ++r) {
+                        const float2 dxy = add2(make_float2(p.x, p.y), nxy[r]);
+                        const float dx = dxy.x, dy = dxy.y, dz = p.z - xi[r].z;
+                        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                        // the self pair and coincident pairs contribute nothing:
+                        // on the linear path the NaN coordinate at r = 0 selects
+                        // the zero entry (T = Q = 0) and the clamped 1/r keeps
+                        // every product finite; elsewhere 1/r = 0 makes tr3 and
+                        // hh zero (T and Q stay finite)
+                        float rinv, tv;
+                        if (TM == TM_LINEAR) {
+                            const float ri = rsqrt_ftz(r2);
+                            tv = fma_sat(r2, -ri, sref);
+                            rinv = fminf(ri, kRinvMax);
+                        } else {
+                            rinv = r2 > 0.0f ? rsqrt_ftz(r2) : 0.0f;
+                            tv = TM == TM_FINE ? fmaf(r2 * rinv, tsc, -0.5f) : fmaf(r2, rinv, -0.5f);
+                        }
+                        float Tv, Qv;
+                        eval_TQ<TM>(tv, r2 * rinv * xscale, x_c, tab_bias, q_off, nmax, c4, Tv, Qv);
+                        const float rinv2 = rinv * rinv;
+                        const float tr3 = Tv * rinv2 * rinv;                          // T/u^3
+                        const float hh = -rinv2 * fmaf(3.0f, tr3, Qv);                // g'(r)/r
+                        // v = m_k c_j - m_j c_k
+                        // (equal masses: v = m (c_j - c_k), m applied with gx)
+                        const float2 vxy = EQM ? add2(make_float2(c.x, c.y), nck[r])
+                                               : fma2(mk2[r], make_float2(c.x, c.y),
+                                                      mul2(make_float2(c.z, c.w), nck[r]));
+                        const float vx = vxy.x, vy = vxy.y;
+                        const float vz = EQM ? p.w + nckz[r] : fmaf(xi[r].w, p.w, c.z * nckz[r]);
+                        const float hd = hh * fmaf(dx, vx, fmaf(dy, vy, dz * vz));
+                        f[r][0] = fmaf(tr3, vx, fmaf(hd, dx, f[r][0]));
+                        f[r][1] = fmaf(tr3, vy, fmaf(hd, dy, f[r][1]));
+                        f[r][2] = fmaf(tr3, vz, fmaf(hd, dz, f[r][2]));
+                        f[r][3] = fmaf(tr3, fmaf(dx, c.x, fmaf(dy, c.y, dz * p.w)), f[r][3]);
                     }
-                    float Tv, Qv;
-                    eval_TQ<TM>(tv, r2 * rinv * xscale, x_c, tab_bias, q_off, nmax, c4, Tv, Qv);
-                    const float rinv2 = rinv * rinv;
-                    const float tr3 = Tv * rinv2 * rinv;                          // T/u^3
-                    const float hh = -rinv2 * fmaf(3.0f, tr3, Qv);                // g'(r)/r
-                    // v = m_k c_j - m_j c_k
-                    // (equal masses: v = m (c_j - c_k), m applied with gx)
-                    const float2 vxy = EQM ? add2(make_float2(c.x, c.y), nck[r])
-                                           : fma2(mk2[r], make_float2(c.x, c.y),
-                                                  mul2(make_float2(c.z, c.w), nck[r]));
-                    const float vx = vxy.x, vy = vxy.y;
-                    const float vz = EQM ? p.w + nckz[r] : fmaf(xi[r].w, p.w, c.z * nckz[r]);
-                    const float hd = hh * fmaf(dx, vx, fmaf(dy, vy, dz * vz));
-                    f[r][0] = fmaf(tr3, vx, fmaf(hd, dx, f[r][0]));
-                    f[r][1] = fmaf(tr3, vy, fmaf(hd, dy, f[r][1]));
-                    f[r][2] = fmaf(tr3, vz, fmaf(hd, dz, f[r][2]));
-                    f[r][3] = fmaf(tr3, fmaf(dx, c.x, fmaf(dy, c.y, dz * p.w)), f[r][3]);
-                }
-            };
-            // Stream s takes staged sources s, s + S, ... in that order: four
-            // per iteration with one target per lane, two with two targets
-            // (then the rest one by one), which halves and quarters the loop
-            // instructions (the two-source loop was 4 % faster than the plain
-            // one with the FP64 fold, 9 % with the compensated one; four
-            // sources gain 0.7 % more).  The loop walks 32-bit shared
-            // addresses with volatile loads, as in the forward kernel (3 %
-            // faster than pointer arithmetic).
-            unsigned sa = smem_u32(stage + 2 * s);
-            const unsigned se = smem_u32(stage + 2 * nst), st1 = 32u * (unsigned)S;
-            if (R == 1) {
+                };
+                // Stream s takes staged sources s, s + S, ... in that order: four
+                // per iteration with one target per lane, two with two targets
+                // (then the rest one by one), which halves and quarters the loop
+                // instructions (the two-source loop was 4 % faster than the plain
+                // one with the FP64 fold, 9 % with the compensated one; four
+                // sources gain 0.7 % more).  The loop walks 32-bit shared
+                // addresses with volatile loads, as in the forward kernel (3 %
+                // faster than pointer arithmetic).
+                unsigned sa = smem_u32(stage + 2 * s);
+                const unsigned se = smem_u32(stage + 2 * nst), st1 = 32u * (unsigned)S;
+                if (R == 1) {
 #pragma unroll 1
-                for (; sa + 3u * st1 < se; sa += 4u * st1) {
-                    const float4 p0 = lds_f4_v(sa), c0 = lds_f4_v(sa + 16u);
-                    const float4 p1 = lds_f4_v(sa + st1), c1 = lds_f4_v(sa + st1 + 16u);
-                    const float4 p2 = lds_f4_v(sa + 2u * st1), c2 = lds_f4_v(sa + 2u * st1 + 16u);
-                    const float4 p3 = lds_f4_v(sa + 3u * st1), c3 = lds_f4_v(sa + 3u * st1 + 16u);
-                    eval(p0, c0);
-                    eval(p1, c1);
-                    eval(p2, c2);
-                    eval(p3, c3);
-                }
+                    for (; sa + 3u * st1 < se; sa += 4u * st1) {
+                        const float4 p0 = lds_f4_v(sa), c0 = lds_f4_v(sa + 16u);
+                        const float4 p1 = lds_f4_v(sa + st1), c1 = lds_f4_v(sa + st1 + 16u);
+                        const float4 p2 = lds_f4_v(sa + 2u * st1), c2 = lds_f4_v(sa + 2u * st1 + 16u);
+                        const float4 p3 = lds_f4_v(sa + 3u * st1), c3 = lds_f4_v(sa + 3u * st1 + 16u);
+                        eval(p0, c0);
+                        eval(p1, c1);
+                        eval(p2, c2);
+                        eval(p3, c3);
+                    }
 #pragma unroll 1
-                for (; sa < se; sa += st1) eval(lds_f4_v(sa), lds_f4_v(sa + 16u));
-            } else {
+                    for (; sa < se; sa += st1) eval(lds_f4_v(sa), lds_f4_v(sa + 16u));
+                } else {
 #pragma unroll 1
-                for (; sa + st1 < se; sa += 2u * st1) {
-                    const float4 p0 = lds_f4_v(sa), c0 = lds_f4_v(sa + 16u);
-                    const float4 p1 = lds_f4_v(sa + st1), c1 = lds_f4_v(sa + st1 + 16u);
-                    eval(p0, c0);
-                    eval(p1, c1);
+                    for (; sa + st1 < se; sa += 2u * st1) {
+                        const float4 p0 = lds_f4_v(sa), c0 = lds_f4_v(sa + 16u);
+                        const float4 p1 = lds_f4_v(sa + st1), c1 = lds_f4_v(sa + st1 + 16u);
+                        eval(p0, c0);
+                        eval(p1, c1);
+                    }
+                    if (sa < se) eval(lds_f4_v(sa), lds_f4_v(sa + 16u));
                 }
-                if (sa < se) eval(lds_f4_v(sa), lds_f4_v(sa + 16u));
+                if (SA) {
+                    acc_fold_all<ACC, R>(accb, lane, f);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) acc[SA ? 0 : r].fold(f[r]);
+                }
             }
+            __syncwarp();
+        }
+        rw = Work::at(wbox);
+        if (rw.in_turn()) {
             if (SA) {
-                acc_fold_all<ACC, R>(accb, lane, f);
+                acc_take_all<ACC, R>(accb, lane, rw.part(), tot);
             } else {
 #pragma unroll
-                for (int r = 0; r < R; ++r) acc[SA ? 0 : r].fold(f[r]);
+                for (int k = 0; k < 4 * R; ++k)
+                    acc[SA ? 0 : k / 4].set(k % 4, tot.add(k, rw.part(), acc[SA ? 0 : k / 4].part(k % 4)));
             }
         }
-        __syncwarp();
+        if (rw.last()) break;
+        if (SA) acc_zero_all<R>(accb, lane);
+#pragma unroll
+        for (int r = 0; r < (SA ? 1 : R); ++r) acc[r] = Acc4<ACC>();
+        rw.next(wbox);
     }
     const float gx = bx.g_adj * sc * sc * sc * (EQM ? bx.m_eq : 1.0f);
     if (SA)
         adj_finish_smem<ACC, R>(a, li, accb, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc,
-                                meta + kWarpMeta, split, wstride);
+                                stage, rw, wstride);
     else
-        adj_finish<ACC, R>(a, li, acc, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc, stage, split,
+        adj_finish<ACC, R>(a, li, acc, act, lane, s, q, S, T, gx, -bx.g_adjm * sc * sc, stage, rw,
                            wstride);
 }
 
@@ -539,10 +542,11 @@ __device__ __forceinline__ void adj_item(const FwdArgs& a, int I, int4 li, unsig
 // of the FMA pipe, whose load and the dependency chains of 24 warps per SM
 // hold it at about 60 % of issue.  One target per lane unless leaves exceed
 // 32 particles (the two-targets state spills at 80 registers).
-template <int TM, int ACC, bool EQM, int R>
+template <int TM, int ACC, bool EQM, int R, class Work>
 __device__ __forceinline__ void adj_item_pk(const FwdArgs& a, int I, int4 li, unsigned tab_bias,
                                             unsigned q_off, float4* __restrict__ stage,
-                                            float4* __restrict__ meta, bool split, int wstride)
+                                            float4* __restrict__ meta, Work rw,
+                                            PartTotals<ACC, 8>& tot, int wstride)
 {
     const int lane = threadIdx.x & 31;
     const float4* __restrict__ pf = reinterpret_cast<const float4*>(a.pf);
@@ -566,7 +570,6 @@ __device__ __forceinline__ void adj_item_pk(const FwdArgs& a, int I, int4 li, un
 
     float2 nx[R], ny[R], nz[R], mk[R], ncx[R], ncy[R], ncz[R], fx[R], fy[R], fz[R], fm[R];
     bool act[R];
-    Acc4<ACC> acc[R];
     float lx = kInf, ly = kInf, lz = kInf, hx = -kInf, hy = -kInf, hz = -kInf;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -594,79 +597,93 @@ __device__ __forceinline__ void adj_item_pk(const FwdArgs& a, int I, int4 li, un
     const float2 c4n2 = make_float2(c4n, c4n);
     // exp(-x^2) = 2^(r2 qarg): r2 is in units of x_c^2 on the linear path
     const float qarg = -kLog2E * x_c * x_c;
-    long long e0, re;
-    row_part(a, I, split, e0, re);
-    while (e0 < re) {
-        int nst;
-        e0 += stage_chunk<3>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
-        if (on) {
-            const int npair = (nst + 1) >> 1;
+    Acc4<ACC> acc[R];
+    float4* const wbox = meta + kMetaPerWarp;
+    rw.park(wbox);
+    for (;;) {  // the row, or its parts in turn
+        long long e0, re;
+        row_part(a, I, Work::at(wbox), e0, re);
+        while (e0 < re) {
+            int nst;
+            e0 += stage_chunk<3>(a, e0, re, ci, unit, sc, a.stage_cap, stage, meta, nst);
+            if (on) {
+                const int npair = (nst + 1) >> 1;
 #pragma unroll 1
-            for (int k = s; k < npair; k += S) {
-                const float4 A = stage[4 * k], B = stage[4 * k + 1];
-                const float4 C = stage[4 * k + 2], D = stage[4 * k + 3];
-                const float2 px = make_float2(A.x, A.y), py = make_float2(A.z, A.w);
-                const float2 pz = make_float2(B.x, B.y), pm = make_float2(B.z, B.w);
-                const float2 cx = make_float2(C.x, C.y), cy = make_float2(C.z, C.w);
-                const float2 cz = make_float2(D.x, D.y);
+                for (int k = s; k < npair; k += S) {
+                    const float4 A = stage[4 * k], B = stage[4 * k + 1];
+                    const float4 C = stage[4 * k + 2], D = stage[4 * k + 3];
+                    const float2 px = make_float2(A.x, A.y), py = make_float2(A.z, A.w);
+                    const float2 pz = make_float2(B.x, B.y), pm = make_float2(B.z, B.w);
+                    const float2 cx = make_float2(C.x, C.y), cy = make_float2(C.z, C.w);
+                    const float2 cz = make_float2(D.x, D.y);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float2 dx = add2(px, nx[r]), dy = add2(py, ny[r]), dz = add2(pz, nz[r]);
+                        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+                        // self and coincident pairs: 1/r = 0 zeroes their terms
+                        const float2 rinv = make_float2(r2.x > 0.0f ? rsqrt_ftz(r2.x) : 0.0f,
+                                                        r2.y > 0.0f ? rsqrt_ftz(r2.y) : 0.0f);
+                        float2 Tv, Qn;
+                        if (TM == TM_LINEAR) {
+                            // T from the table (8-byte entries, as in the forward);
+                            // -c4 exp(-x^2) from ex2, zeroed with T beyond the
+                            // cutoff (the table's zero entry): half the table's
+                            // shared-memory traffic for one MUFU and three ALU
+                            // instructions per pair
+                            const float2 sv = make_float2(fma_sat(r2.x, rinv.x, soff),
+                                                          fma_sat(r2.y, rinv.y, soff));
+                            Tv = make_float2(linear_T(sv.x, nmax, tab_bias), linear_T(sv.y, nmax, tab_bias));
+                            const float2 q2 = make_float2(ex2_ftz(r2.x * qarg), ex2_ftz(r2.y * qarg));
+                            Qn = mul2(c4n2, make_float2(Tv.x > 0.0f ? q2.x : 0.0f, Tv.y > 0.0f ? q2.y : 0.0f));
+                        } else {
+                            eval_TQ<TM>(fmaf(r2.x, rinv.x, -0.5f), r2.x * rinv.x * xscale, x_c, tab_bias,
+                                        q_off, nmax, c4n, Tv.x, Qn.x);
+                            eval_TQ<TM>(fmaf(r2.y, rinv.y, -0.5f), r2.y * rinv.y * xscale, x_c, tab_bias,
+                                        q_off, nmax, c4n, Tv.y, Qn.y);
+                        }
+                        const float2 rinv2 = mul2(rinv, rinv);
+                        const float2 tr3 = mul2(Tv, mul2(rinv2, rinv));           // T/u^3
+                        const float2 hh = mul2(rinv2, fma2(m3, tr3, Qn));         // g'(r)/r
+                        // m_k c_j - m_j c_k (equal masses: c_j - c_k, m applied with gx)
+                        const float2 vx = EQM ? add2(cx, ncx[r]) : fma2(mk[r], cx, mul2(pm, ncx[r]));
+                        const float2 vy = EQM ? add2(cy, ncy[r]) : fma2(mk[r], cy, mul2(pm, ncy[r]));
+                        const float2 vz = EQM ? add2(cz, ncz[r]) : fma2(mk[r], cz, mul2(pm, ncz[r]));
+                        const float2 hd = mul2(hh, fma2(dx, vx, fma2(dy, vy, mul2(dz, vz))));
+                        fx[r] = fma2(tr3, vx, fma2(hd, dx, fx[r]));
+                        fy[r] = fma2(tr3, vy, fma2(hd, dy, fy[r]));
+                        fz[r] = fma2(tr3, vz, fma2(hd, dz, fz[r]));
+                        fm[r] = fma2(tr3, fma2(dx, cx, fma2(dy, cy, mul2(dz, cz))), fm[r]);
+                    }
+                }
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const float2 dx = add2(px, nx[r]), dy = add2(py, ny[r]), dz = add2(pz, nz[r]);
-                    const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-                    // self and coincident pairs: 1/r = 0 zeroes their terms
-                    const float2 rinv = make_float2(r2.x > 0.0f ? rsqrt_ftz(r2.x) : 0.0f,
-                                                    r2.y > 0.0f ? rsqrt_ftz(r2.y) : 0.0f);
-                    float2 Tv, Qn;
-                    if (TM == TM_LINEAR) {
-                        // T from the table (8-byte entries, as in the forward);
-                        // -c4 exp(-x^2) from ex2, zeroed with T beyond the
-                        // cutoff (the table's zero entry): half the table's
-                        // shared-memory traffic for one MUFU and three ALU
-                        // instructions per pair
-                        const float2 sv = make_float2(fma_sat(r2.x, rinv.x, soff),
-                                                      fma_sat(r2.y, rinv.y, soff));
-                        Tv = make_float2(linear_T(sv.x, nmax, tab_bias), linear_T(sv.y, nmax, tab_bias));
-                        const float2 q2 = make_float2(ex2_ftz(r2.x * qarg), ex2_ftz(r2.y * qarg));
-                        Qn = mul2(c4n2, make_float2(Tv.x > 0.0f ? q2.x : 0.0f, Tv.y > 0.0f ? q2.y : 0.0f));
-                    } else {
-                        eval_TQ<TM>(fmaf(r2.x, rinv.x, -0.5f), r2.x * rinv.x * xscale, x_c, tab_bias,
-                                    q_off, nmax, c4n, Tv.x, Qn.x);
-                        eval_TQ<TM>(fmaf(r2.y, rinv.y, -0.5f), r2.y * rinv.y * xscale, x_c, tab_bias,
-                                    q_off, nmax, c4n, Tv.y, Qn.y);
-                    }
-                    const float2 rinv2 = mul2(rinv, rinv);
-                    const float2 tr3 = mul2(Tv, mul2(rinv2, rinv));           // T/u^3
-                    const float2 hh = mul2(rinv2, fma2(m3, tr3, Qn));         // g'(r)/r
-                    // m_k c_j - m_j c_k (equal masses: c_j - c_k, m applied with gx)
-                    const float2 vx = EQM ? add2(cx, ncx[r]) : fma2(mk[r], cx, mul2(pm, ncx[r]));
-                    const float2 vy = EQM ? add2(cy, ncy[r]) : fma2(mk[r], cy, mul2(pm, ncy[r]));
-                    const float2 vz = EQM ? add2(cz, ncz[r]) : fma2(mk[r], cz, mul2(pm, ncz[r]));
-                    const float2 hd = mul2(hh, fma2(dx, vx, fma2(dy, vy, mul2(dz, vz))));
-                    fx[r] = fma2(tr3, vx, fma2(hd, dx, fx[r]));
-                    fy[r] = fma2(tr3, vy, fma2(hd, dy, fy[r]));
-                    fz[r] = fma2(tr3, vz, fma2(hd, dz, fz[r]));
-                    fm[r] = fma2(tr3, fma2(dx, cx, fma2(dy, cy, mul2(dz, cz))), fm[r]);
+                    float f4[4] = {fx[r].x + fx[r].y, fy[r].x + fy[r].y, fz[r].x + fz[r].y,
+                                   fm[r].x + fm[r].y};
+                    acc[r].fold(f4);
+                    fx[r] = fy[r] = fz[r] = fm[r] = make_float2(0.0f, 0.0f);
                 }
             }
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                float f4[4] = {fx[r].x + fx[r].y, fy[r].x + fy[r].y, fz[r].x + fz[r].y,
-                               fm[r].x + fm[r].y};
-                acc[r].fold(f4);
-                fx[r] = fy[r] = fz[r] = fm[r] = make_float2(0.0f, 0.0f);
-            }
+            __syncwarp();
         }
-        __syncwarp();
+        rw = Work::at(wbox);
+        if (rw.in_turn()) {
+#pragma unroll
+            for (int k = 0; k < 4 * R; ++k) acc[k / 4].set(k % 4, tot.add(k, rw.part(), acc[k / 4].part(k % 4)));
+        }
+        if (rw.last()) break;
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = Acc4<ACC>();
+        rw.next(wbox);
     }
     adj_finish<ACC, R>(a, li, acc, act, lane, s, q, S, T,
-                       bx.g_adj * sc * sc * sc * (EQM ? bx.m_eq : 1.0f), -bx.g_adjm * sc * sc, stage, split,
+                       bx.g_adj * sc * sc * sc * (EQM ? bx.m_eq : 1.0f), -bx.g_adjm * sc * sc, stage, rw,
                        wstride);
 }
 
 // Shared memory: the table (T and Q), then per warp a staging buffer of
 // stage_cap particles x 2 float4, 32 entry records and the two box slots,
 // then the accumulator block of the two-targets path (kAdjAccF4).
-template <int TM, int ACC, bool WIDE, bool PK, bool EQM, bool SPLIT>
+template <int TM, int ACC, bool WIDE, bool PK, bool EQM, int ROWS>
 __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -674,8 +691,8 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
     const int warp = threadIdx.x >> 5;
     const size_t tab_bytes = TM == TM_EXACT ? 0
                            : (size_t)(a.table_n + 1) * (TM == TM_LINEAR ? 16 : 32);
-    float4* stage = reinterpret_cast<float4*>(smem + tab_bytes) +
-                    (size_t)warp * (2 * a.stage_cap + kWarpMeta + kAdjAccF4);
+    const int wstride = 2 * a.stage_cap + kWarpMeta + kAdjAccF4;
+    float4* stage = reinterpret_cast<float4*>(smem + tab_bytes) + (size_t)warp * wstride;
     float4* meta = stage + 2 * a.stage_cap;
     const unsigned accb = smem_u32(meta + kWarpMeta);
     if (TM != TM_EXACT) {
@@ -712,11 +729,10 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
     const unsigned q_off = (unsigned)(a.table_n + 1) * 16u;
     const int4* __restrict__ leaf = reinterpret_cast<const int4*>(a.leaf);
     __shared__ int s_it[8];
-    const int wstride = 2 * a.stage_cap + kWarpMeta + kAdjAccF4;
-    const int n_heavy = !SPLIT ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
-    bool split = SPLIT && n_heavy > 0;
+    const int n_heavy = ROWS != kRowsJoint ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    bool split = n_heavy > 0;
     int it;
-    while (next_item<SPLIT>(a, a.ctrl + kCtrlTicketAdj, split, n_heavy, s_it, it)) {
+    while (next_item<ROWS>(a, a.ctrl + kCtrlTicketAdj, split, n_heavy, s_it, it)) {
         int I = a.items[it];
         if (I < 0 || I >= a.n_leaves) {
             if (lane == 0) set_error(a.ctrl, kErrItemIndex);
@@ -728,19 +744,21 @@ __global__ void __launch_bounds__(256, 3) p2p_adj_f32_kernel(const FwdArgs a)
             if (lane == 0) set_error(a.ctrl, kErrParticleRange);
             continue;
         }
+        const auto rw = row_work<ROWS>(a, I, li.z, split);
+        PartTotals<ACC, 8> tot;  // kRowsInTurn
         if (PK) {
             if (WIDE && prefer_two_per_lane(li.y))
-                adj_item_pk<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, SPLIT && split, wstride);
+                adj_item_pk<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, rw, tot, wstride);
             else
-                adj_item_pk<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, SPLIT && split, wstride);
+                adj_item_pk<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, rw, tot, wstride);
         } else if (WIDE && prefer_two_per_lane(li.y)) {
             // leaves of 11-12 and 17-20 particles up to 32 (and all larger
             // ones); at equal lane fill one target per lane is faster (its
             // state fits the registers and its loop takes four sources per
             // iteration): sending the ties to two targets cost 1.4 %
-            adj_item<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, accb, SPLIT && split, wstride);
+            adj_item<TM, ACC, EQM, 2>(a, I, li, tab_bias, q_off, stage, meta, accb, rw, tot, wstride);
         } else {
-            adj_item<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, accb, SPLIT && split, wstride);
+            adj_item<TM, ACC, EQM, 1>(a, I, li, tab_bias, q_off, stage, meta, accb, rw, tot, wstride);
         }
     }
     persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
@@ -753,15 +771,17 @@ size_t adj_f32_smem(int precision, int interp, int table_n, int warps, int cap)
     return tab + (size_t)warps * (2 * cap + kWarpMeta + kAdjAccF4) * 16;
 }
 
-template <int TM, int ACC, bool EQM, bool SPLIT>
+template <int TM, int ACC, bool EQM, int ROWS>
 static int launch_adj_e(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
     // always with the two-targets-per-lane path (mid-size leaves fill more lanes)
     // (the packed variant carries it only for leaves above 32 particles: its
     // per-target state would spill)
-    auto k = SPLIT || TM == TM_FINE || a.variant != PSR_KERNEL_PACKED ? p2p_adj_f32_kernel<TM, ACC, true, false, EQM, SPLIT>
-             : a.max_leaf > 32              ? p2p_adj_f32_kernel<TM == TM_FINE ? TM_CUBIC : TM, ACC, true, true, EQM, false>
-                                            : p2p_adj_f32_kernel<TM == TM_FINE ? TM_CUBIC : TM, ACC, false, true, EQM, false>;
+    constexpr int PTM = TM == TM_FINE ? TM_CUBIC : TM;
+    auto k = ROWS != kRowsWhole || TM == TM_FINE || a.variant != PSR_KERNEL_PACKED
+                 ? p2p_adj_f32_kernel<TM, ACC, true, false, EQM, ROWS>
+             : a.max_leaf > 32 ? p2p_adj_f32_kernel<PTM, ACC, true, true, EQM, kRowsWhole>
+                               : p2p_adj_f32_kernel<PTM, ACC, false, true, EQM, kRowsWhole>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
@@ -771,14 +791,19 @@ static int launch_adj_e(const FwdArgs& a, size_t smem, cudaStream_t st)
 }
 
 // equal masses: m leaves the pair sums (v = m (c_j - c_k))
+template <int TM, int ACC, int ROWS>
+static int launch_adj_r(const FwdArgs& a, size_t smem, cudaStream_t st)
+{
+    return a.equal_mass ? launch_adj_e<TM, ACC, true, ROWS>(a, smem, st)
+                        : launch_adj_e<TM, ACC, false, ROWS>(a, smem, st);
+}
+
 template <int TM, int ACC>
 static int launch_adj_t(const FwdArgs& a, size_t smem, cudaStream_t st)
 {
-    if (a.group > 1)
-        return a.equal_mass ? launch_adj_e<TM, ACC, true, true>(a, smem, st)
-                            : launch_adj_e<TM, ACC, false, true>(a, smem, st);
-    return a.equal_mass ? launch_adj_e<TM, ACC, true, false>(a, smem, st)
-                        : launch_adj_e<TM, ACC, false, false>(a, smem, st);
+    return a.rows == kRowsJoint    ? launch_adj_r<TM, ACC, kRowsJoint>(a, smem, st)
+           : a.rows == kRowsInTurn ? launch_adj_r<TM, ACC, kRowsInTurn>(a, smem, st)
+                                   : launch_adj_r<TM, ACC, kRowsWhole>(a, smem, st);
 }
 
 int launch_adj_f32(const FwdArgs& a, int precision, void* stream)
@@ -810,9 +835,9 @@ int adj_f32_occupancy(int precision, int interp, int accum, int warps, int max_l
     const void* f;
     const size_t smem = adj_f32_smem(precision, interp, table_n, warps, cap);
 #define PSR_PICK(TM, ACC) (variant != PSR_KERNEL_PACKED \
-                               ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, false, false, false> \
-                               : wide ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, true, false, false> \
-                                      : (const void*)p2p_adj_f32_kernel<TM, ACC, false, true, false, false>)
+                               ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, false, false, kRowsWhole> \
+                               : wide ? (const void*)p2p_adj_f32_kernel<TM, ACC, true, true, false, kRowsWhole> \
+                                      : (const void*)p2p_adj_f32_kernel<TM, ACC, false, true, false, kRowsWhole>)
     if (precision == PSR_FP32_EXACT)
         f = accum == PSR_ACC_FP64 ? PSR_PICK(TM_EXACT, PSR_ACC_FP64) : PSR_PICK(TM_EXACT, PSR_ACC_KAHAN32);
     else if (interp == PSR_LINEAR)

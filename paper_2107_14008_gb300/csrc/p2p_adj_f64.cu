@@ -9,9 +9,10 @@
 
 namespace psr {
 
-template <bool EQM, bool TAIL, int R>
+template <bool EQM, bool TAIL, int R, class Work>
 __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, const double* tab,
-                                           const double* tabq, const Warp64& w64, bool split)
+                                           const double* tabq, const Warp64& w64, Work rw,
+                                           PartTotals<PSR_ACC_FP64, 12>& tot)
 {
     const int lane = threadIdx.x & 31;
     const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
@@ -43,7 +44,7 @@ __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, con
 #pragma unroll
     for (int r = 0; r < R; ++r) ti[r] = target64(xi[r], w64.box, kx);
     long long e0, re;
-    row_part(a, I, split, e0, re);
+    row_part(a, I, rw, e0, re);
     const int len = (int)(re - e0);
     for (int e = 0; e < len;) {
         int nst;
@@ -90,19 +91,23 @@ __device__ __forceinline__ void adj64_item(const FwdArgs& a, int I, int4 li, con
         }
         __syncwarp();
     }
+    if (rw.in_turn()) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) g[r][i] = tot.add(4 * r + i, rw.part(), PartSum<PSR_ACC_FP64>{g[r][i]}).v;
+    }
+    if (!rw.last()) return;
     const double G = bx.G, gx = EQM ? G * pd[li.x].w : G;
-    finish64<4, R>(a, li, g, act, lane, s, S, T, w64.near, split, kWarp64Bytes,
-                   [&](int target, const double* v) {
+    finish64<4, R>(a, li, g, act, lane, s, S, T, w64.near, rw, kWarp64Bytes,
+                   [&](int target, int i, double v) {
                        const int idx = a.perm[target];
-                       double* o = reinterpret_cast<double*>(a.out) + 3LL * idx;
-                       o[0] = gx * v[0];
-                       o[1] = gx * v[1];
-                       o[2] = gx * v[2];
-                       if (a.out_m) reinterpret_cast<double*>(a.out_m)[idx] = -G * v[3];
+                       if (i < 3) reinterpret_cast<double*>(a.out)[3LL * idx + i] = gx * v;
+                       else if (a.out_m) reinterpret_cast<double*>(a.out_m)[idx] = -G * v;
                    });
 }
 
-template <bool EQM, bool TAIL>
+template <bool EQM, bool TAIL, int ROWS>
 __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem64[];
@@ -117,27 +122,46 @@ __global__ void __launch_bounds__(256, 2) p2p_adj_f64_kernel(const FwdArgs a)
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const Warp64 w64(smem64 + 16 * words + (threadIdx.x >> 5) * kWarp64Bytes);
-    const int n_heavy = a.group <= 1 ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    const int n_heavy = ROWS != kRowsJoint ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
     bool split = n_heavy > 0;
     int it;
-    while (next_item<true>(a, a.ctrl + kCtrlTicketAdj, split, n_heavy, s_it, it)) {
+    while (next_item<ROWS>(a, a.ctrl + kCtrlTicketAdj, split, n_heavy, s_it, it)) {
         int I;
         int4 li;
         if (!item64(a, it, lane, I, li)) continue;
         const int R = targets_per_lane(li.y, 128);
-        if (R == 1) adj64_item<EQM, TAIL, 1>(a, I, li, tab, tabq, w64, split);
-        else if (R == 2) adj64_item<EQM, TAIL, 2>(a, I, li, tab, tabq, w64, split);
-        else adj64_item<EQM, TAIL, 3>(a, I, li, tab, tabq, w64, split);
+        auto rw = row_work<ROWS>(a, I, li.z, split);
+        PartTotals<PSR_ACC_FP64, 12> tot;  // kRowsInTurn
+        for (;;) {  // parts in turn
+            if (R == 1) adj64_item<EQM, TAIL, 1>(a, I, li, tab, tabq, w64, rw, tot);
+            else if (R == 2) adj64_item<EQM, TAIL, 2>(a, I, li, tab, tabq, w64, rw, tot);
+            else adj64_item<EQM, TAIL, 3>(a, I, li, tab, tabq, w64, rw, tot);
+            if (rw.last()) break;
+            if constexpr (ROWS == kRowsInTurn) ++rw.v;
+        }
     }
     persistent_exit(a.ctrl + kCtrlTicketAdj, a.ctrl + kCtrlDoneAdj);
 }
 
 namespace {
 
-auto pick_adj64(double x_c, bool eqm)
+template <bool TAIL, int ROWS>
+auto pick_adj64_r(bool eqm)
 {
-    if (plain64(x_c).tail) return eqm ? p2p_adj_f64_kernel<true, true> : p2p_adj_f64_kernel<false, true>;
-    return eqm ? p2p_adj_f64_kernel<true, false> : p2p_adj_f64_kernel<false, false>;
+    return eqm ? p2p_adj_f64_kernel<true, TAIL, ROWS> : p2p_adj_f64_kernel<false, TAIL, ROWS>;
+}
+
+template <bool TAIL>
+auto pick_adj64_t(int rows, bool eqm)
+{
+    return rows == kRowsJoint    ? pick_adj64_r<TAIL, kRowsJoint>(eqm)
+           : rows == kRowsInTurn ? pick_adj64_r<TAIL, kRowsInTurn>(eqm)
+                                 : pick_adj64_r<TAIL, kRowsWhole>(eqm);
+}
+
+auto pick_adj64(double x_c, int rows, bool eqm)
+{
+    return plain64(x_c).tail ? pick_adj64_t<true>(rows, eqm) : pick_adj64_t<false>(rows, eqm);
 }
 
 }  // namespace
@@ -157,7 +181,7 @@ int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)
     if (e != cudaSuccess) return (int)e;
     a.t64_max = plain64(x_c).n;
     const size_t smem = adj_f64_smem(x_c, a.warps_per_block);
-    auto k = pick_adj64(x_c, a.equal_mass);
+    auto k = pick_adj64(x_c, a.rows, a.equal_mass);
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     k<<<a.blocks, a.warps_per_block * 32, smem, st>>>(a);
@@ -167,7 +191,7 @@ int launch_adj_f64(const FwdArgs& args, double x_c, void* stream)
 int adj_f64_occupancy(int warps, double x_c, int* out)
 {
     const size_t smem = adj_f64_smem(x_c, warps);
-    auto k = pick_adj64(x_c, false);
+    auto k = pick_adj64(x_c, kRowsWhole, false);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k, warps * 32, smem);

@@ -340,51 +340,37 @@ __device__ __forceinline__ void near_pairs(const float4* __restrict__ near, int 
 
 // Adds the S stream partials (NC components per target slot) of each target
 // through the warp's staging buffer, in stream order, and hands each target's
-// sums to write(target, sums); with split, the sums of the group's warps are
-// added after that, in warp order (stride: bytes between the warps' buffers).
-template <int NC, int R, class Write>
-__device__ __forceinline__ void finish64(const FwdArgs& a, int4 li, const double (*acc)[NC], const bool* act,
-                                         int lane, int s, int S, int T, float4* __restrict__ stage,
-                                         bool split, int stride, Write write)
+// sums to write(target, component, sum); in a row that a group of warps shares each has the
+// sums of its part (join_parts; stride: bytes between the warps' regions).
+template <int NC, int R, class Work, class Write>
+__device__ __forceinline__ void finish64(const FwdArgs& a, int4 li, const double (*acc)[NC], const bool* act, int lane, int s, int S,
+                                         int T, float4* __restrict__ stage, const Work& rw, int stride,
+                                         Write write)
 {
+    const bool joint = rw.joint();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         volatile double* red = reinterpret_cast<volatile double*>(stage) + 32 * NC * r;
 #pragma unroll
         for (int i = 0; i < NC; ++i) red[NC * lane + i] = acc[r][i];
         __syncwarp();
-        if (s == 0 && act[r]) {
+        if (!joint && s == 0 && act[r]) {
             double v[NC];
 #pragma unroll
             for (int i = 0; i < NC; ++i) v[i] = acc[r][i];
             for (int t = 1; t < S; ++t)
 #pragma unroll
                 for (int i = 0; i < NC; ++i) v[i] += red[NC * (lane + t * T) + i];
-            if (split) {  // streams t >= 1 sit above the first T entries
 #pragma unroll
-                for (int i = 0; i < NC; ++i) red[NC * lane + i] = v[i];
-            } else {
-                write(li.x + lane + T * r, v);
-            }
+            for (int i = 0; i < NC; ++i) write(li.x + lane + T * r, i, v[i]);
         }
         __syncwarp();
     }
-    if (!split) return;
-    group_sync(a.group);
-    const int nw = a.group, gw = (threadIdx.x >> 5) % nw;
-    const char* base = reinterpret_cast<const char*>(stage) - gw * stride;
-    for (int t = 32 * gw + lane; t < li.y; t += 32 * nw) {
-        double v[NC];
-#pragma unroll
-        for (int i = 0; i < NC; ++i) v[i] = 0.0;
-        for (int w = 0; w < nw; ++w) {
-            const volatile double* o = reinterpret_cast<const volatile double*>(base + w * stride) +
-                                       32 * NC * (t / T) + NC * (t % T);
-#pragma unroll
-            for (int i = 0; i < NC; ++i) v[i] += o[i];
-        }
-        write(li.x + t, v);
-    }
+    if (joint)
+        join_parts<NC, PSR_ACC_FP64>(
+            a, rw, li.y, S, reinterpret_cast<const char*>(stage), stride,
+            [T](int t, int s, int i) { return 8 * (32 * NC * (t / T) + NC * (t % T + s * T) + i); },
+            [&](int t, int i, const PartSum<PSR_ACC_FP64>& p) { write(li.x + t, i, p.v); });
 }
 
 // a checked schedule entry; false (and the error word) if it is out of range

@@ -6,7 +6,7 @@
 
 namespace psr {
 
-template <bool PK, bool SPLIT>
+template <bool PK, int ROWS>
 int launch_fwd_f32_variant(const FwdArgs& a, int precision, size_t smem, cudaStream_t st);
 template <bool PK>
 const void* fwd_f32_kernel_ptr(int precision, int interp, int accum, int core);
@@ -160,11 +160,15 @@ int launch_fwd_f32(const FwdArgs& a, int precision, void* stream)
 {
     size_t smem = fwd_f32_smem(precision, a.interp, a.table_n, a.warps_per_block, a.stage_cap);
     cudaStream_t st = (cudaStream_t)stream;
-    if (a.variant == PSR_KERNEL_PACKED)
-        return a.group > 1 ? launch_fwd_f32_variant<true, true>(a, precision, smem, st)
-                       : launch_fwd_f32_variant<true, false>(a, precision, smem, st);
-    return a.group > 1 ? launch_fwd_f32_variant<false, true>(a, precision, smem, st)
-                   : launch_fwd_f32_variant<false, false>(a, precision, smem, st);
+    const bool pk = a.variant == PSR_KERNEL_PACKED;
+    if (a.rows == kRowsJoint)
+        return pk ? launch_fwd_f32_variant<true, kRowsJoint>(a, precision, smem, st)
+                  : launch_fwd_f32_variant<false, kRowsJoint>(a, precision, smem, st);
+    if (a.rows == kRowsInTurn)
+        return pk ? launch_fwd_f32_variant<true, kRowsInTurn>(a, precision, smem, st)
+                  : launch_fwd_f32_variant<false, kRowsInTurn>(a, precision, smem, st);
+    return pk ? launch_fwd_f32_variant<true, kRowsWhole>(a, precision, smem, st)
+              : launch_fwd_f32_variant<false, kRowsWhole>(a, precision, smem, st);
 }
 
 int fwd_f32_occupancy(int precision, int interp, int accum, int warps, int table_n, int cap,

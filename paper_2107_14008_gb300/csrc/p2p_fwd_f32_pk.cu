@@ -1,8 +1,8 @@
-// FP32 forward kernel, packed pairs (its own translation unit so that
-// the variants compile in parallel).
+// FP32 forward kernel, packed pairs, whole rows (its own translation unit
+// so that the variants compile in parallel).
 #include "fwd_f32_common.cuh"
 
 namespace psr {
-template int launch_fwd_f32_variant<true, false>(const FwdArgs&, int, size_t, cudaStream_t);
+template int launch_fwd_f32_variant<true, kRowsWhole>(const FwdArgs&, int, size_t, cudaStream_t);
 template const void* fwd_f32_kernel_ptr<true>(int, int, int, int);
 }  // namespace psr

@@ -1,0 +1,7 @@
+// FP32 forward kernel, packed pairs of the core form, rows with parts on groups of warps (its own translation unit
+// so that the variants compile in parallel).
+#include "fwd_f32_common.cuh"
+
+namespace psr {
+template int launch_fwd_f32_variant<true, kRowsJoint>(const FwdArgs&, int, size_t, cudaStream_t);
+}  // namespace psr

@@ -86,14 +86,15 @@ int launch_plain64(double x_c, void* d_t, void* d_q, void* stream)
     return (int)cudaGetLastError();
 }
 
-// One target leaf (or, with split, this warp's part of its row).  EQM: every
-// particle of the box has one mass, applied once per target.  COUNT: pairs
+// One target leaf (rw: this warp's parts of its row).  EQM: every particle of
+// the box has one mass, applied once per target.  COUNT: pairs
 // within the cutoff and pairs evaluated are counted, over every tile pair (no
 // cull).
-template <bool COUNT, bool EQM, int DEG, bool TAIL, int R>
+template <bool COUNT, bool EQM, int DEG, bool TAIL, int R, class Work>
 __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, const double* tab,
                                            const Warp64& w64, unsigned long long& npairs,
-                                           unsigned long long& nev, bool split)
+                                           unsigned long long& nev, Work rw,
+                                           PartTotals<PSR_ACC_FP64, 9>& tot)
 {
     const int lane = threadIdx.x & 31;
     const double4* __restrict__ pd = reinterpret_cast<const double4*>(a.pd);
@@ -122,7 +123,7 @@ __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, con
     for (int r = 0; r < R; ++r) ti[r] = target64(xi[r], w64.box, kx);
     unsigned cnt = 0;
     long long e0, re;
-    row_part(a, I, split, e0, re);
+    row_part(a, I, rw, e0, re);
     const int len = (int)(re - e0);
     for (int e = 0; e < len;) {
         int nst;
@@ -156,18 +157,22 @@ __device__ __forceinline__ void fwd64_item(const FwdArgs& a, int I, int4 li, con
         __syncwarp();
     }
     if (COUNT) npairs += cnt;
+    if (rw.in_turn()) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) acc[r][i] = tot.add(3 * r + i, rw.part(), PartSum<PSR_ACC_FP64>{acc[r][i]}).v;
+    }
+    if (!rw.last()) return;
     const double g = EQM ? bx.G * pd[li.x].w : bx.G;
-    finish64<3, R>(a, li, acc, act, lane, s, S, T, w64.near, split, kWarp64Bytes,
-                   [&](int target, const double* v) {
-                       double* out = reinterpret_cast<double*>(a.out) + 3LL * a.perm[target];
-                       out[0] = g * v[0];
-                       out[1] = g * v[1];
-                       out[2] = g * v[2];
+    finish64<3, R>(a, li, acc, act, lane, s, S, T, w64.near, rw, kWarp64Bytes,
+                   [&](int target, int i, double v) {
+                       reinterpret_cast<double*>(a.out)[3LL * a.perm[target] + i] = g * v;
                    });
 }
 
 // DEG 5: the plain path (TAIL: the cutoff lies beyond its table), 4: the Taylor levels.
-template <bool COUNT, bool EQM, int DEG, bool TAIL>
+template <bool COUNT, bool EQM, int DEG, bool TAIL, int ROWS>
 __global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem64[];
@@ -179,17 +184,23 @@ __global__ void __launch_bounds__(256, 2) p2p_fwd_f64_kernel(const FwdArgs a)
     const int lane = threadIdx.x & 31;
     const Warp64 w64(smem64 + 8 * words + (threadIdx.x >> 5) * kWarp64Bytes);
     unsigned long long npairs = 0, nev = 0;
-    const int n_heavy = a.group <= 1 ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
+    const int n_heavy = ROWS != kRowsJoint ? 0 : a.heavy ? min(*a.heavy, a.n_items) : a.n_items;
     bool split = n_heavy > 0;
     int it;
-    while (next_item<true>(a, a.ctrl + kCtrlTicketFwd, split, n_heavy, s_it, it)) {
+    while (next_item<ROWS>(a, a.ctrl + kCtrlTicketFwd, split, n_heavy, s_it, it)) {
         int I;
         int4 li;
         if (!item64(a, it, lane, I, li)) continue;
         const int R = targets_per_lane(li.y, 128);
-        if (R == 1) fwd64_item<COUNT, EQM, DEG, TAIL, 1>(a, I, li, tab, w64, npairs, nev, split);
-        else if (R == 2) fwd64_item<COUNT, EQM, DEG, TAIL, 2>(a, I, li, tab, w64, npairs, nev, split);
-        else fwd64_item<COUNT, EQM, DEG, TAIL, 3>(a, I, li, tab, w64, npairs, nev, split);
+        auto rw = row_work<ROWS>(a, I, li.z, split);
+        PartTotals<PSR_ACC_FP64, 9> tot;  // kRowsInTurn
+        for (;;) {  // parts in turn
+            if (R == 1) fwd64_item<COUNT, EQM, DEG, TAIL, 1>(a, I, li, tab, w64, npairs, nev, rw, tot);
+            else if (R == 2) fwd64_item<COUNT, EQM, DEG, TAIL, 2>(a, I, li, tab, w64, npairs, nev, rw, tot);
+            else fwd64_item<COUNT, EQM, DEG, TAIL, 3>(a, I, li, tab, w64, npairs, nev, rw, tot);
+            if (rw.last()) break;
+            if constexpr (ROWS == kRowsInTurn) ++rw.v;
+        }
     }
     if (COUNT) {
         for (int off = 16; off > 0; off >>= 1) npairs += __shfl_xor_sync(kFull, npairs, off);
@@ -205,19 +216,27 @@ namespace {
 
 bool taylor64(int interp) { return interp == PSR_TAYLOR2 || interp == PSR_TAYLOR4; }
 
-template <int DEG, bool TAIL>
-const void* pick64_t(bool count, bool eqm)
+template <int DEG, bool TAIL, int ROWS>
+const void* pick64_r(bool count, bool eqm)
 {
-    return count ? (const void*)p2p_fwd_f64_kernel<true, false, DEG, TAIL>
-           : eqm ? (const void*)p2p_fwd_f64_kernel<false, true, DEG, TAIL>
-                 : (const void*)p2p_fwd_f64_kernel<false, false, DEG, TAIL>;
+    return count ? (const void*)p2p_fwd_f64_kernel<true, false, DEG, TAIL, ROWS>
+           : eqm ? (const void*)p2p_fwd_f64_kernel<false, true, DEG, TAIL, ROWS>
+                 : (const void*)p2p_fwd_f64_kernel<false, false, DEG, TAIL, ROWS>;
 }
 
-const void* pick64(int interp, double x_c, bool count, bool eqm)
+template <int DEG, bool TAIL>
+const void* pick64_t(int rows, bool count, bool eqm)
 {
-    return taylor64(interp)    ? pick64_t<4, false>(count, eqm)
-           : plain64(x_c).tail ? pick64_t<5, true>(count, eqm)
-                               : pick64_t<5, false>(count, eqm);
+    return rows == kRowsJoint    ? pick64_r<DEG, TAIL, kRowsJoint>(count, eqm)
+           : rows == kRowsInTurn ? pick64_r<DEG, TAIL, kRowsInTurn>(count, eqm)
+                                 : pick64_r<DEG, TAIL, kRowsWhole>(count, eqm);
+}
+
+const void* pick64(int interp, double x_c, int rows, bool count, bool eqm)
+{
+    return taylor64(interp)    ? pick64_t<4, false>(rows, count, eqm)
+           : plain64(x_c).tail ? pick64_t<5, true>(rows, count, eqm)
+                               : pick64_t<5, false>(rows, count, eqm);
 }
 
 }  // namespace
@@ -233,7 +252,7 @@ int launch_fwd_f64(const FwdArgs& args, double x_c, void* stream)
     FwdArgs a = args;
     a.t64_max = taylor64(a.interp) ? a.table_n : plain64(x_c).n;
     const size_t smem = fwd_f64_smem(a.interp, a.table_n, x_c, a.warps_per_block);
-    const void* k = pick64(a.interp, x_c, a.count_pairs, a.equal_mass);
+    const void* k = pick64(a.interp, x_c, a.rows, a.count_pairs, a.equal_mass);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     void* params[] = {&a};
@@ -243,7 +262,7 @@ int launch_fwd_f64(const FwdArgs& args, double x_c, void* stream)
 
 int fwd_f64_occupancy(int warps, int interp, int table_n, double x_c, int* out)
 {
-    const void* f = pick64(interp, x_c, false, false);
+    const void* f = pick64(interp, x_c, kRowsWhole, false, false);
     const size_t smem = fwd_f64_smem(interp, table_n, x_c, warps);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;

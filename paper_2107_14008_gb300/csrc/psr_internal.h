@@ -25,6 +25,10 @@ constexpr int kFineMaxN = 1024;      // intervals of PSR_FP32_EXACT's fine table
 constexpr int kMaxTaylorN = 2048;    // Taylor tables: 32-byte entries
 constexpr int kTaylorPaperN = 384;   // x_c / 384 = 3 / 512 at x_c = 2.25, the paper's spacing
 
+// Kinds of launch with a rule of their own for the parts of rows (parts_rule):
+// the FP32 forward and adjoint with the linear table and with others, FP64.
+enum : int { kPartsFwd, kPartsFwdTab, kPartsAdj, kPartsAdjTab, kPartsF64, kPartsKinds };
+
 // Per-box constants as the kernels see them (plain old data, 16B aligned).
 struct alignas(16) BoxDev {
     double L, r_s, r_c, G;      // FP64 path
@@ -37,8 +41,11 @@ struct alignas(16) BoxDev {
     float g_adjm;   // G / (4 r_s^2): adjoint mass gradient factor
     float m_eq;     // the mass every particle of the box has (as FP32), 0 if they differ
     float pad3;
+    // rows of more than above[kind] evaluated pairs are summed in parts[kind] parts
+    int64_t above[kPartsKinds];
+    int parts[kPartsKinds], pad4;
 };
-static_assert(sizeof(BoxDev) == 96, "BoxDev layout");
+static_assert(sizeof(BoxDev) == 160, "BoxDev layout");
 
 // Byte offsets of the regions of the device workspace (256-byte aligned).
 struct Layout {
@@ -50,6 +57,7 @@ struct Layout {
     size_t rowptr;   // int64[nl+1]  CSR of pair entries by target leaf
     size_t pairs;    // uint32[np]   (source leaf << 5) | shift code
     size_t items;    // int32[nl]    target leaves in schedule order
+    size_t cost;     // int64[nl]    evaluated pairs of each leaf's row
     size_t boxes;    // BoxDev[nbox]
     size_t table;    // float4[2 * (kMaxTableN + 1)]: T table, then exp(-x^2)
     size_t core;     // float2[kMaxTableN + 1]: core form of the forward's linear table
@@ -83,6 +91,7 @@ enum : unsigned {
     kErrParticleRange = 2u,
     kErrItemIndex = 4u,
     kErrShiftCode = 8u,
+    kErrParts = 32u,     // a row of more parts than its group has warps
     kErrLookback = 16u,  // a look-back of the device build's scans or sorts ran out
 };
 
@@ -116,7 +125,8 @@ struct Leaves {
     std::vector<int64_t> rowptr;
     std::vector<uint32_t> pairs;
     std::vector<int32_t> items;
-    std::vector<int64_t> item_cost;  // evaluated pairs of each item, in schedule order
+    std::vector<int64_t> cost;       // evaluated pairs of each leaf's row
+    std::vector<int64_t> item_cost;  // the same in schedule order
     int32_t n_heavy[4] = {0, 0, 0, 0};  // host copy of ctrl[kCtrlHeavy..] (psr_upload)
     int64_t evaluated = 0;
     int64_t max_cost = 0;  // the largest leaf's evaluated pairs
@@ -152,46 +162,81 @@ Layout make_layout(const Leaves& h);
 size_t table_entry_bytes(int interp);  // p2p_fwd_f32.cu
 BoxDev box_constants(const psr_box& b);  // per-box kernel constants
 
-// Heavy items: those of the schedule's head that are worth sharing among the
-// warps of a group.  The schedule keeps the counts of items whose work exceeds
-// 1/2, 1, 2 and 4 times a warp's share of the launch with 32 warps per SM.
+// Heavy rows.  Where a launch's largest row exceeds a warp's share of the work, a
+// row on one warp outlasts the others, or the chip is never filled: such rows
+// are summed in parts, which a group of warps forms side by side.  The parts are
+// a matter of the arithmetic (each is summed by itself, and the parts are added in
+// order), so the rule looks at the row and its box alone: a box gives the same
+// forces, bit for bit, in a batch and alone, in a shard and whole, whatever the
+// launch's shape.  Whether warps form the parts side by side or one warp forms
+// them in turn is up to the launch (group_rule).
+
+// Work of a row above which it is heavy, at level l: 1/2, 1, 2 and 4 times a warp's
+// share with 32 warps per SM.
 constexpr int kHeavyLevels = 4;
-inline int64_t heavy_cost(int level, int64_t evaluated, int sms)
+constexpr int kPartsSms = 152;  // the chip the parts are meant for
+inline int64_t heavy_cost(int level, int64_t evaluated)
 {
-    return (evaluated << level) / (64 * (int64_t)(sms > 0 ? sms : 1));
+    return (evaluated << level) / (64 * (int64_t)kPartsSms);
 }
 
-// Whether and how a launch on `warps` resident warps shares heavy rows.
-// group: warps per heavy item, 1 for none; level: which count of heavy items
-// applies, -1 for all items.  A launch shares rows only where the largest item
-// exceeds `line` / 8 of a warp's share of the work: then a row on one warp
-// outlasts the others, or the chip is never filled; below it the largest-first
-// order hides the longest row, and the group phase's registers cost 1-3 % (128^3
-// NFW in leaves of up to 64: 9.53 -> 9.66 ms).  Items above about half a share
-// are shared, all of them when there are fewer leaves than warps, and the group
-// is large enough to bring the largest item's parts to 3/2 of a share, with at
-// least 2500 pairs in a part (the group's barriers and the row's start-up
-// latency cost about as much as 1500).  Forward, one warp per row against this:
-// 5000 uniform particles 0.235 -> 0.081 ms, 32^3 0.28 -> 0.12, 110,000 NFW 2.57
-// -> 1.1, 64^3 NFW 2.3 -> 1.5; adjoint 32^3 0.28 -> 0.20.  Groups of 8 wherever
-// rows are shared at all: 60,000 uniform in leaves of up to 16 0.28 ms against
-// 0.17 with groups of 2 and 0.19 with one warp per row.
+// The parts of a set's heavy rows when `warps` warps share its work, and the level
+// of heavy_cost above which rows are heavy (-1: all are).  No parts unless the
+// largest row exceeds `line` / 8 of a share; below it the largest-first order
+// hides the longest row, and the group phase's registers cost 1-3 % (128^3 NFW in
+// leaves of up to 64: 9.53 -> 9.66 ms).  Rows above about half a share are heavy,
+// all of them when there are fewer leaves than warps, and the parts are as many
+// (2, 4 or 8) as bring the largest row's to 3/2 of a share, with at least 2500
+// pairs in a part (the group's barriers and the row's start-up latency cost about
+// as much as 1500).  Forward, one warp per row against this: 5000 uniform
+// particles 0.235 -> 0.081 ms, 32^3 0.28 -> 0.12, 110,000 NFW 2.57 -> 1.1, 64^3 NFW
+// 2.3 -> 1.5; adjoint 32^3 0.28 -> 0.20.  Eight parts wherever there are any: 60,000
+// uniform in leaves of up to 16 0.28 ms against 0.17 with two and 0.19 with none.
 struct SplitRule {
-    int group, level;
+    int parts, level;
 };
-inline SplitRule split_rule(int64_t max_cost, int64_t evaluated, int64_t n_leaves, int sms, int64_t warps,
-                            int block_warps, int line)
+inline SplitRule split_rule(int64_t max_cost, int64_t evaluated, int64_t n_leaves, int64_t warps, int line)
 {
     SplitRule r{1, -1};
     const int64_t share = evaluated / (warps > 0 ? warps : 1);
     if (max_cost <= line * share / 8) return r;
-    while (r.group < 8 && 2 * max_cost > 3 * r.group * share && max_cost >= 5000 * r.group) r.group *= 2;
-    while (r.group > 1 && block_warps % r.group) r.group /= 2;
+    while (r.parts < 8 && 2 * max_cost > 3 * r.parts * share && max_cost >= 5000 * r.parts) r.parts *= 2;
     if (n_leaves >= warps)
-        for (r.level = 0; r.level + 1 < kHeavyLevels && 3 * heavy_cost(r.level, evaluated, sms) < share;)
+        for (r.level = 0; r.level + 1 < kHeavyLevels && 3 * heavy_cost(r.level, evaluated) < share;)
             ++r.level;
     return r;
 }
+
+// The line of a kind of launch: 3/2 of a share; 5/4 where a pair costs more, as
+// with every table but the linear one (cubic adjoint, 150,000 NFW 4.33 -> 2.72 ms
+// against a line of 2), and 2 for the linear adjoint of leaves of up to 32, whose
+// rows are short against the group's overheads (150,000 NFW in leaves of up to 16
+// 1.95 ms, 2.05 with 3/2; 64^3 NFW 2.74 and 2.83; in leaves of up to 64, 512,000 NFW
+// gain 5.96 -> 5.36 with 3/2).
+inline int split_line(int kind, int max_leaf)
+{
+    return kind == kPartsAdj ? (max_leaf <= 32 ? 16 : 12) : kind == kPartsFwd ? 12 : 10;
+}
+
+// A box's parts, for each kind as a launch of that kind on the box alone has them:
+// 32, 24 and 16 warps per SM for the FP32 forward, the FP32 adjoint and FP64.
+inline SplitRule box_rule(int kind, int64_t max_cost, int64_t evaluated, int64_t n_leaves, int max_leaf)
+{
+    const int warps = kind == kPartsFwd || kind == kPartsFwdTab ? 32 : kind == kPartsF64 ? 16 : 24;
+    return split_rule(max_cost, evaluated, n_leaves, (int64_t)kPartsSms * warps, split_line(kind, max_leaf));
+}
+inline void parts_rule(int64_t max_cost, int64_t evaluated, int64_t n_leaves, int max_leaf, BoxDev* b)
+{
+    for (int k = 0; k < kPartsKinds; ++k) {
+        const SplitRule r = box_rule(k, max_cost, evaluated, n_leaves, max_leaf);
+        b->parts[k] = r.parts;
+        b->above[k] = r.level < 0 ? -1 : heavy_cost(r.level, evaluated);
+    }
+}
+
+// How a launch takes rows with parts: there are none; groups of warps form them side
+// by side; one warp forms them in turn.
+enum : int { kRowsWhole = 0, kRowsJoint = 1, kRowsInTurn = 2 };
 
 // kernels (launchers defined in the .cu files; return cudaError_t as int)
 struct FwdArgs {
@@ -228,8 +273,11 @@ struct FwdArgs {
     int item_stride; // this launch takes schedule entries ticket * stride + offset
     int item_offset;
     int t64_max;       // FP64 kernels: last node of the table
-    const int* heavy;  // how many items groups of warps take (null: all)
-    int group;         // warps per group (divides warps_per_block); 0 or 1: none
+    const long long* cost;  // evaluated pairs of each row
+    int rows;          // kRowsWhole, kRowsJoint or kRowsInTurn
+    int kind;          // whose parts rows have (kParts...)
+    const int* heavy;  // kRowsJoint: how many items groups of warps take (null: all)
+    int group;         //   and the warps per group (divides warps_per_block)
     int fine;        // PSR_FP32_EXACT by the fine cubic table (interp and table_n are its)
     int core;        // FP32 forward: a.table is the core form of the linear table
     int equal_mass;  // every box has one particle mass: the FP32 kernels take it out of the sums

@@ -307,7 +307,8 @@ int psr_p2p_forces_noalloc(psr_leaves* h, const psr_opts* opts, void* d_acc, voi
  * kernel for this leaf set.  Starting from *base (precision, table, interp
  * and accumulation are kept), times every candidate of
  *   kernel      PSR_KERNEL_SCALAR | PSR_KERNEL_PACKED  (sources per lane
- *               and iteration: 1 | 2)
+ *               and iteration: 1 | 2), and PSR_KERNEL_AUTO where that is
+ *               neither (it shares heavy rows among warps)
  *   warps       4 | 8 per block
  *   source_tile 64 | 128 | 256 staged source particles per warp
  * that fits shared memory and the largest leaf, with CUDA events on

@@ -46,7 +46,7 @@ int wait_stream(cudaStream_t st, int timeout_ms)
 struct Opts {
     int precision, table_n, interp, accum, warps, bps, fold, count, kernel, tile, nshard, shard;
     bool fine = false;  // PSR_FP32_EXACT by the fine cubic table (fine_exact)
-    bool split;  // heavy rows in parts: the default kernel's choice
+    bool split;  // heavy rows in parts: the default kernel's, by either name
 };
 
 int check_opts(const psr_opts* o, Opts* out)
@@ -187,10 +187,10 @@ void fine_exact(const Leaves* h, Opts& o)
 // packed pairs were level or slower).
 void resolve_kernel(const Leaves* h, Opts& o)
 {
+    const bool core = fwd_core(o.precision, o.interp, o.table_n, PSR_KERNEL_PACKED, cutoff_x(h));
+    if (o.kernel == PSR_KERNEL_PACKED && core) o.split = true;  // the default's kernel: the same results
     if (o.kernel != PSR_KERNEL_AUTO) return;
-    o.kernel = fwd_core(o.precision, o.interp, o.table_n, PSR_KERNEL_PACKED, cutoff_x(h))
-                   ? PSR_KERNEL_PACKED
-                   : PSR_KERNEL_SCALAR;
+    o.kernel = core ? PSR_KERNEL_PACKED : PSR_KERNEL_SCALAR;
 }
 
 // Builds the table of `key` in its region by launch(), unless it is there for
@@ -549,10 +549,13 @@ int psr_autotune(psr_leaves* hh, const psr_opts* base, void* d_acc, void* stream
     }
     float best_t = -1.0f;
     psr_opts best_o = b;
-    const int kernels[2] = {PSR_KERNEL_SCALAR, PSR_KERNEL_PACKED};
+    // the default shares heavy rows and takes PSR_FP32_EXACT's fine table, which the
+    // named kernels do not: a candidate of its own, unless it is the packed one
+    const int kernels[3] = {PSR_KERNEL_SCALAR, PSR_KERNEL_PACKED, PSR_KERNEL_AUTO};
+    const int nk = fwd_core(chk.precision, chk.interp, chk.table_n, PSR_KERNEL_PACKED, cutoff_x(h)) ? 2 : 3;
     const int warps[2] = {4, 8};
     const int tiles[3] = {64, 128, 256};
-    for (int ki = 0; ki < 2 && rc == PSR_OK; ++ki)
+    for (int ki = 0; ki < nk && rc == PSR_OK; ++ki)
         for (int wi = 0; wi < 2 && rc == PSR_OK; ++wi)
             for (int ti = 0; ti < 3 && rc == PSR_OK; ++ti) {
                 psr_opts c = b;

@@ -10,7 +10,7 @@
 //                     PSR_PM_NO_DECONVOLVE, and by N^3 (cuFFT does not
 //                     normalise), zero at k = 0; then -i k_c for each axis c
 //                     (Nyquist plane of axis c zeroed), three spectra
-//   4. cuFFT C2R, the three axes as one batch
+//   4. cuFFT C2R, the three axes as one batch (from N = 896 on one by one)
 //   5. k_cic_interp   CIC interpolation of the three component meshes at the
 //                     particles, written to (or added into) the output
 //
@@ -44,6 +44,7 @@ using namespace psr;
 struct psr_pm {
     int n;
     cufftHandle r2c, c2r;
+    int batch;    // axes that one inverse transform takes
     size_t work;  // bytes of the larger cuFFT work area
 };
 
@@ -267,6 +268,10 @@ int psr_pm_create(int n_pm, psr_pm** out)
     psr_pm* pm = new (std::nothrow) psr_pm();
     if (!pm) return pfail(PSR_E_NOMEM, "out of host memory");
     pm->n = n_pm;
+    // three axes at once while their 3 N^3 reals stay below 2^31 (N < 895), one by
+    // one beyond: the plan's counts are 32-bit
+    const int64_t cells = (int64_t)n_pm * n_pm * n_pm;
+    pm->batch = 3 * cells < ((int64_t)1 << 31) ? 3 : 1;
     size_t w1 = 0, w2 = 0;
     int dims[3] = {n_pm, n_pm, n_pm}, spec[3] = {n_pm, n_pm, n_pm / 2 + 1};
     cufftResult r;
@@ -283,7 +288,7 @@ int psr_pm_create(int n_pm, psr_pm** out)
         (r = cufftSetAutoAllocation(pm->c2r, 0)) != CUFFT_SUCCESS ||
         (r = cufftMakePlan3d(pm->r2c, n_pm, n_pm, n_pm, CUFFT_R2C, &w1)) != CUFFT_SUCCESS ||
         (r = cufftMakePlanMany(pm->c2r, 3, dims, spec, 1, n_pm * n_pm * (n_pm / 2 + 1), dims, 1,
-                               n_pm * n_pm * n_pm, CUFFT_C2R, 3, &w2)) != CUFFT_SUCCESS) {
+                               n_pm * n_pm * n_pm, CUFFT_C2R, pm->batch, &w2)) != CUFFT_SUCCESS) {
         cufftDestroy(pm->r2c);
         cufftDestroy(pm->c2r);
         delete pm;
@@ -350,7 +355,9 @@ int psr_pm_forces(psr_pm* pm, const double* d_pos, const double* d_mass, int64_t
         phik, ak, N, kf, (float)(box->r_s * box->r_s), (float)(4.0 * M_PI * box->G),
         (float)(0.5 * delta), (flags & PSR_PM_NO_DECONVOLVE) ? 0 : 1, (float)(1.0 / (double)nr));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_err(e, "field kernel");
-    if ((r = cufftExecC2R(pm->c2r, ak, g)) != CUFFT_SUCCESS) return fft_err(r, "cufftExecC2R");
+    for (int c = 0; c < 3; c += pm->batch)
+        if ((r = cufftExecC2R(pm->c2r, ak + c * nc, g + c * nr)) != CUFFT_SUCCESS)
+            return fft_err(r, "cufftExecC2R");
     k_pm_gather<<<nblk(nr / 4, 256), 256, 0, st>>>(g, nr, g4);
     k_cic_interp<<<nblk(n, 256), 256, 0, st>>>(d_pos, n, L, 1.0 / delta, N, g4, d_acc,
                                                (flags & PSR_PM_ACCUMULATE) ? 1 : 0);

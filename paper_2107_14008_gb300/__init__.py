@@ -454,8 +454,7 @@ def _autograd_function():
         def forward(ctx, pos, mass, L, r_s, r_c, G=1.0, opts=None, max_leaf=32):
             opts = opts or Options()
             if opts.kernel == PSR_KERNEL_AUTO and pos.dtype == torch.float64:
-                # FP64 tensors get the FP32 sums of the scalar kernels, whose
-                # order and rounding do not change with the default kernel's
+                # the kernel whose order of sums its name fixes: see forces()
                 opts = replace(opts, kernel=PSR_KERNEL_SCALAR)
             if pos.is_cuda:
                 lv = Leaves.device_build(pos, mass, L, r_s, r_c, G, max_leaf, fp64=opts.fp64)
@@ -499,5 +498,12 @@ def __getattr__(name):
 
 
 def forces(pos, mass, L, r_s, r_c, G=1.0, opts=None, max_leaf=32):
-    """Differentiable accelerations of particles `pos` (torch, CUDA)."""
+    """Differentiable accelerations of particles `pos` (torch, CUDA), in pos's dtype.
+
+    opts as in Leaves.forces, with one exception: float64 tensors get PSR_KERNEL_AUTO as
+    PSR_KERNEL_SCALAR, forward and backward.  Their FP32 sums are read to more digits than the
+    default kernel's form keeps (its table form and its parts of heavy rows move results by 1e-7,
+    within FP32's error but far above float64's), so they come from the kernel whose order of sums
+    is fixed by its name, at up to three times the default's time on small sets.  A kernel that the
+    caller names is kept, and float32 tensors get the same bits as Leaves.forces and adjoint."""
     return _Namespace.P2PForce.apply(pos, mass, L, r_s, r_c, G, opts, max_leaf)

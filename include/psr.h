@@ -157,10 +157,12 @@ typedef struct {
                                 then counts the near (P2P) entries only        */
     double theta;            /* acceptance parameter of that split, else 0    */
     int64_t rows_walked_twice; /* device builds: target leaves whose pair row
-                                the count walk could not keep in the pair
-                                cache, walked again by psr_device_build_finish
-                                (every row when the cache's per-row slot is
-                                below 16 runs); else 0                       */
+                                has more runs than its slot of the pair cache
+                                (every row when a slot is below 16 runs);
+                                psr_device_build_finish walks them again.  For
+                                a split, runs of the undivided row: the near
+                                and the far part are kept apart, and rows that
+                                fit undivided may be walked again too; else 0 */
     int equal_mass;          /* 1 if within every box all particles have one
                                 mass: the FP32 kernels then apply it once per
                                 target instead of once per pair (the paper's
@@ -358,7 +360,8 @@ int psr_pair_count(psr_leaves* h, void* cuda_stream, int timeout_ms, int64_t* co
  * particle box (those pairs are zero by the truncation of Eq. tr), so their
  * count lies between psr_pair_count's and the leaf-pair tiles' total
  * (psr_info.evaluated_pairs); PSR_KERNEL_PAPER evaluates every tile
- * pair, and so do the FP64 kernels on a counting launch.  Errors: PSR_E_STATE, PSR_E_TIMEOUT.
+ * pair, and so do the FP64 kernels on a counting launch.
+ * Errors: PSR_E_STATE, PSR_E_TIMEOUT.
  */
 int psr_evaluated_count(psr_leaves* h, void* cuda_stream, int timeout_ms, int64_t* count);
 

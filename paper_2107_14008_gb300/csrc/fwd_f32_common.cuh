@@ -17,8 +17,8 @@
 // for the leaves that take one target per lane).  The
 // S partial sums of each target are combined through shared memory at the
 // end.  Warps take target leaves from an atomic ticket in largest-work-first
-// order (persistent grid, no inter-block waits); the split instances share a
-// heavy leaf between 2, 4 or 8 warps of a block.
+// order (persistent grid, no inter-block waits); heavy rows have parts, which a
+// group of warps of a block forms side by side or one warp in turn (row_work).
 //
 // Precision.  Pair arithmetic is FP32 in leaf-local coordinates scaled by
 // 1/(2 r_s); the offset between two leaf centres (with the periodic image) is
@@ -77,9 +77,9 @@ __device__ __forceinline__ float linear_T(float s, float nmax, unsigned tab_bias
 // at or beyond the cutoff has q = 1, 1/r = 1 and reaches the sentinel entry
 // H(N) = 1: its weight is exactly 0.  Entries are (-A_k, -D_k), H = A_k + q D_k
 // on q N in [k, k + 1) (the index by an FMA rounded down), shifted by half the
-// chord's error so that the error is balanced.  Bound by the shared-memory
-// pipe (about 5.8 cycles per warp lane pair, 3.4 of them the table entry's,
-// 79 % of the launch) with issue behind it (71 %).  128^3 NFW set: 10.27 ms
+// chord's error so that the error is balanced.  Nothing is saturated (shared-
+// memory pipe 76 %, issue 71 %, FMA 53 % of a 96^3 launch): the loop waits on its
+// chain of rsqrt, table load and sum at 8 warps per scheduler.  128^3 NFW set: 10.27 ms
 // with T by its own table and scalar streams, 9.58 with this form (16 instead
 // of 18 instructions per pair), 9.32 with it on packed pairs.  H by a degree-9
 // polynomial instead (no table) is bound by the FMA pipe: 11.1 ms.

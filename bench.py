@@ -795,7 +795,7 @@ def run_psr(args):
             "value": within / (mst / 1e3) / 1e9, "ms_per_step": mst,
             "rel_rms_vs_plain_fp64_path": float(np.sqrt(np.sum(dt_ * dt_) / np.sum(ref64 ** 2))),
             "path": "FP64, T from the paper's Taylor T[4] table in FP64 (384 nodes), "
-                    "1/r by Newton-Raphson from an FP32 estimate"}
+                    "1/r by a series from the FP64 rsqrt estimate"}
         lv.check()
 
     # adjoint (FP32 table) on the same leaf set, same timing rules
